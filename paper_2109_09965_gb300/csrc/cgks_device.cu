@@ -238,51 +238,37 @@ void enqueue_hi_eval(Batch *b, const TF *W, const TF *Wx, TF *Fout) {
   // so the default (linear weights, smooth flux) kernels stay as lean as before
   const bool chr = b->sh.weno_eps > 0.0 && b->sh.weno_vars == CGKS_WENO_CHARACTERISTIC;
   const bool weno = b->sh.weno_eps > 0.0 && !chr, full = b->sh.flux_hi == CGKS_FLUX_FULL;
+  const int rs = b->tune.shape(TK_RECON), fs = b->tune.shape(TK_FACE);
+  auto recon = [&](auto kern) {
+    launch(b, KI_RECON, kern, dim3(nblk(b->N, shape_bs(rs))), dim3(shape_bs(rs)), fmesh<TF>(b),
+           fparams<TF>(b), W, Wx, B.coef);
+  };
+  auto face = [&](auto kern, int threads) {   // threads: of a face
+    launch(b, KI_FACE, kern, dim3(nblk(threads * b->F, shape_bs(fs))), dim3(shape_bs(fs)), fmesh<TF>(b),
+           fparams<TF>(b), W, Wx, (const TF *)B.coef, Fout, (const Ctl *)b->ctl,
+           (const unsigned long long *)b->dt_bits);
+  };
   if (b->sh.per_slot_flux) {
     // one launch per flux class present; each skips the other class's solves
     tuned_launch(b->tune, TK_RECON, b->stream, [&] {
-      with_shape(b->tune.shape(TK_RECON), [&](auto sh) {
-        constexpr int S = decltype(sh)::value;
-        const dim3 g(nblk(b->N, shape_bs(S) * shape_ipt(S))), blk(shape_bs(S));
-        if (b->n_smooth) launch(b, KI_RECON, k_recon<TF, S, false>, g, blk, fmesh<TF>(b), fparams<TF>(b), W, Wx, B.coef);
-        if (b->n_lim) launch(b, KI_RECON, k_recon<TF, S, true>, g, blk, fmesh<TF>(b), fparams<TF>(b), W, Wx, B.coef);
-      });
+      if (b->n_smooth) recon(k_recon<TF, false>);
+      if (b->n_lim) recon(k_recon<TF, true>);
     });
     tuned_launch(b->tune, TK_FACE, b->stream, [&] {
-      with_shape(b->tune.shape(TK_FACE), [&](auto sh) {
-        constexpr int S = decltype(sh)::value;
-        const dim3 g(nblk(b->F, shape_bs(S) * shape_ipt(S))), blk(shape_bs(S));
-        auto go = [&](auto kern) {
-          launch(b, KI_FACE, kern, g, blk, fmesh<TF>(b), fparams<TF>(b), W, Wx, (const TF *)B.coef, Fout,
-                 (const Ctl *)b->ctl, (const unsigned long long *)b->dt_bits);
-        };
-        if (b->n_smooth) go(k_face<TF, S, false, false>);
-        if (b->n_lim) go(k_face<TF, S, true, false>);
-      });
+      if (b->n_smooth) face(k_face<TF, false, false>, face_threads<TF, false>());
+      if (b->n_lim) face(k_face<TF, true, false>, face_threads<TF, true>());
     });
     return;
   }
   tuned_launch(b->tune, TK_RECON, b->stream, [&] {
-    with_shape(b->tune.shape(TK_RECON), [&](auto sh) {
-      constexpr int S = decltype(sh)::value;
-      const dim3 g(nblk(b->N, shape_bs(S) * shape_ipt(S))), blk(shape_bs(S));
-      if (weno) launch(b, KI_RECON, k_recon<TF, S, true>, g, blk, fmesh<TF>(b), fparams<TF>(b), W, Wx, B.coef);
-      else launch(b, KI_RECON, k_recon<TF, S, false>, g, blk, fmesh<TF>(b), fparams<TF>(b), W, Wx, B.coef);
-    });
+    if (weno) recon(k_recon<TF, true>);
+    else recon(k_recon<TF, false>);
   });
   tuned_launch(b->tune, TK_FACE, b->stream, [&] {
-    with_shape(b->tune.shape(TK_FACE), [&](auto sh) {
-      constexpr int S = decltype(sh)::value;
-      const dim3 g(nblk(b->F, shape_bs(S) * shape_ipt(S))), blk(shape_bs(S));
-      auto go = [&](auto kern) {
-        launch(b, KI_FACE, kern, g, blk, fmesh<TF>(b), fparams<TF>(b), W, Wx, (const TF *)B.coef, Fout,
-               (const Ctl *)b->ctl, (const unsigned long long *)b->dt_bits);
-      };
-      if (full && chr) go(k_face<TF, S, true, true>);
-      else if (full) go(k_face<TF, S, true, false>);
-      else if (chr) go(k_face<TF, S, false, true>);
-      else go(k_face<TF, S, false, false>);
-    });
+    if (full && chr) face(k_face<TF, true, true>, face_threads<TF, true>());
+    else if (full) face(k_face<TF, true, false>, face_threads<TF, true>());
+    else if (chr) face(k_face<TF, false, true>, face_threads<TF, false>());
+    else face(k_face<TF, false, false>, face_threads<TF, false>());
   });
 }
 
@@ -367,12 +353,11 @@ void enqueue_lo_solve(Batch *b) {
   for (int k = 0; k < b->sh.n_implicit; ++k) {
     launch(b, KI_LOCELL, k_lo_cell<TF>, gc, blk, static_cast<int>(b->Ncap), fparams<TF>(b), k == 0 ? 1 : 0,
            (const double *)b->Wn, b->U, (const TF *)B.dU, B.prim, mirror<TF>(B.U));
+    const int fsh = b->tune.shape(TK_LOFACE);
     tuned_launch(b->tune, TK_LOFACE, b->stream, [&] {
-      with_shape(b->tune.shape(TK_LOFACE), [&](auto sh) {
-        constexpr int S = decltype(sh)::value;
-        launch(b, KI_LOFACE, k_lo_face<TF, S>, dim3(nblk(b->F, shape_bs(S) * shape_ipt(S))), dim3(shape_bs(S)),
-               fmesh<TF>(b), fparams<TF>(b), (const TF *)B.U, (const TF *)B.prim, B.Flo, B.lam, B.E0, B.E1);
-      });
+      launch(b, KI_LOFACE, k_lo_face<TF>, dim3(nblk(b->F, shape_bs(fsh))), dim3(shape_bs(fsh)),
+             fmesh<TF>(b), fparams<TF>(b), (const TF *)B.U, (const TF *)B.prim, B.Flo, B.lam, B.E0,
+             B.E1);
     });
     launch(b, KI_LORHS, k_lo_rhs<TF>, gc, blk, b->dm, b->dp, k == 0 ? 1 : 0, colour0, (const TF *)B.Flo,
            (const TF *)B.lam, (const double *)b->Rp0, b->Src, B.Rk, B.invD, dU0, B.lamS);
@@ -394,13 +379,10 @@ void enqueue_lo_solve(Batch *b) {
       const bool use_list = R.n == 0;
       const int grid = use_list ? nblk(cnt, sweep_cpb(ssh)) : R.blk[R.n];
       tuned_launch(b->tune, TK_SWEEP, b->stream, [&] {
-        with_shape(ssh, [&](auto sh) {
-          constexpr int S = decltype(sh)::value;
-          launch(b, KI_SWEEP, k_sweep<TF, S>, dim3(grid), dim3(shape_bs(S)), fmesh<TF>(b), fparams<TF>(b), R,
-                 use_list ? (const int *)b->list + b->list_off[c] : (const int *)nullptr, cnt, (const TF *)B.U,
-                 (const TF *)B.prim, (const TF *)B.Rk, (const TF *)B.invD, (const TF *)B.lamS,
-                 (const TF *)B.E0, (const TF *)B.E1, B.dU);
-        });
+        launch(b, KI_SWEEP, k_sweep<TF>, dim3(grid), dim3(shape_bs(ssh)), fmesh<TF>(b), fparams<TF>(b),
+               R, use_list ? (const int *)b->list + b->list_off[c] : (const int *)nullptr, cnt, (const TF *)B.U,
+               (const TF *)B.prim, (const TF *)B.Rk, (const TF *)B.invD, (const TF *)B.lamS, (const TF *)B.E0,
+               (const TF *)B.E1, B.dU);
       });
     }
   }
@@ -545,6 +527,7 @@ void fill_shared_params(const Shared &sh, ParamsT<T> &P) {
   P.kc.K = static_cast<T>(K);
   P.kc.c2K = static_cast<T>(2.0 / (K + 2.0));
   P.kc.c4K = static_cast<T>(4.0 / (K + 2.0));
+  P.kc.hN = static_cast<T>(0.5 * (K + 2.0));
   P.flux_lo = sh.flux_lo;
   P.flux_hi = sh.flux_hi;
   P.tau_c1 = static_cast<T>(sh.tau_c1);

@@ -135,26 +135,23 @@ void hi_eval(Solver3 *s, const TF *W, const TF *Wx, TF *Fout) {
   // nonlinear weights and the full flux are separate instantiations (the
   // default kernels stay as before)
   const bool weno = s->P.weno_eps > 0.0, full = s->P.flux_hi == CGKS_FLUX_FULL;
+  const int rs = s->tune.shape(TK_RECON), fs = s->tune.shape(TK_FACE);
   tuned_launch(s->tune, TK_RECON, s->stream, [&] {
-    with_shape(s->tune.shape(TK_RECON), [&](auto sh) {
-      constexpr int S = decltype(sh)::value;
-      const dim3 gr(nblk(s->N, shape_bs(S) * shape_ipt(S))), blk(shape_bs(S));
-      if (weno)
-        launch(s, KI_RECON, k_recon_weno<TF, S>, gr, blk, fmesh<TF>(s), fpar<TF>(s), W, Wx, B.coef,
-               (const unsigned char *)s->g.wenok);
-      else launch(s, KI_RECON, k_recon<TF, S>, gr, blk, fmesh<TF>(s), fpar<TF>(s), W, Wx, B.coef);
-    });
+    const dim3 gr(nblk(s->N, shape_bs(rs))), blk(shape_bs(rs));
+    if (weno)
+      launch(s, KI_RECON, k_recon_weno<TF>, gr, blk, fmesh<TF>(s), fpar<TF>(s), W, Wx, B.coef,
+             (const unsigned char *)s->g.wenok);
+    else launch(s, KI_RECON, k_recon<TF>, gr, blk, fmesh<TF>(s), fpar<TF>(s), W, Wx, B.coef);
   });
   tuned_launch(s->tune, TK_FACE, s->stream, [&] {
-    with_shape(s->tune.shape(TK_FACE), [&](auto sh) {
-      constexpr int S = decltype(sh)::value;
-      const dim3 gr(nblk(s->F, shape_bs(S) * shape_ipt(S))), blk(shape_bs(S));
-      if (full)
-        launch(s, KI_FACE, k_face_full<TF, S>, gr, blk, fmesh<TF>(s), fpar<TF>(s), W, (const TF *)B.coef, Fout,
-               (const Ctl *)s->ctl, (const unsigned long long *)s->dt_bits);
-      else
-        launch(s, KI_FACE, k_face<TF, S>, gr, blk, fmesh<TF>(s), fpar<TF>(s), W, (const TF *)B.coef, Fout);
-    });
+    auto go = [&](int threads, auto kern, auto... rest) {   // threads: of a face
+      launch(s, KI_FACE, kern, dim3(nblk(threads * s->F, shape_bs(fs))), dim3(shape_bs(fs)),
+             fmesh<TF>(s), fpar<TF>(s), W, (const TF *)B.coef, Fout, rest...);
+    };
+    if (full) go(1, k_face_full<TF>, (const Ctl *)s->ctl, (const unsigned long long *)s->dt_bits);
+    else if constexpr (is_f32<TF>()) go(1, k_face<TF>);
+    else if (face_lanes(s->F) == 4) go(4, k_face_smooth<4>);
+    else go(1, k_face_smooth<1>);
   });
 }
 
@@ -188,24 +185,19 @@ void lo_solve(Solver3 *s) {
   for (int k = 0; k < s->P.n_implicit; ++k) {
     launch(s, KI_LOCELL, k_lo_cell<TF>, gc, blk, static_cast<int>(s->N), fpar<TF>(s), k == 0 ? 1 : 0,
            (const double *)s->Wn, s->U, (const TF *)B.dU, B.rec);
+    const int fs = s->tune.shape(TK_LOFACE), ss = s->tune.shape(TK_SWEEP);
     tuned_launch(s->tune, TK_LOFACE, s->stream, [&] {
-      with_shape(s->tune.shape(TK_LOFACE), [&](auto sh) {
-        constexpr int S = decltype(sh)::value;
-        launch(s, KI_LOFACE, k_lo_face<TF, S>, dim3(nblk(s->F, shape_bs(S) * shape_ipt(S))), dim3(shape_bs(S)),
-               fmesh<TF>(s), fpar<TF>(s), (const TF *)B.rec, B.Flo, B.E0, B.E1);
-      });
+      launch(s, KI_LOFACE, k_lo_face<TF>, dim3(nblk(s->F, shape_bs(fs))), dim3(shape_bs(fs)),
+             fmesh<TF>(s), fpar<TF>(s), (const TF *)B.rec, B.Flo, B.E0, B.E1);
     });
     launch(s, KI_LORHS, k_lo_rhs<TF>, gc, blk, s->dm, s->dp, k == 0 ? 1 : 0, colour0_end, (const TF *)B.Flo,
            (const double *)s->Rp0, s->Src, B.Rk, B.invD, B.dU, B.lamS);
     for (int c : s->sweep_seq) {
       const int beg = s->colour_start[c], cnt = s->colour_start[c + 1] - beg;
       tuned_launch(s->tune, TK_SWEEP, s->stream, [&] {
-        with_shape(s->tune.shape(TK_SWEEP), [&](auto sh) {
-          constexpr int S = decltype(sh)::value;
-          launch(s, KI_SWEEP, k_sweep<TF, S>, dim3(nblk(cnt, sweep_cpb(S))), dim3(shape_bs(S)), fmesh<TF>(s),
-                 fpar<TF>(s), beg, cnt, (const TF *)B.rec, (const TF *)B.Rk, (const TF *)B.invD,
-                 (const TF *)B.lamS, (const TF *)B.E0, (const TF *)B.E1, B.dU);
-        });
+        launch(s, KI_SWEEP, k_sweep<TF>, dim3(nblk(cnt, sweep_cpb(ss))), dim3(shape_bs(ss)), fmesh<TF>(s), fpar<TF>(s),
+               beg, cnt, (const TF *)B.rec, (const TF *)B.Rk, (const TF *)B.invD, (const TF *)B.lamS,
+               (const TF *)B.E0, (const TF *)B.E1, B.dU);
       });
     }
   }
@@ -325,6 +317,7 @@ void fill_params(const cgks_params &p, ParamsT<T> &P) {
   P.kc.K = static_cast<T>(K);
   P.kc.c2K = static_cast<T>(2.0 / (K + 3.0));
   P.kc.c4K = static_cast<T>(4.0 / (K + 3.0));
+  P.kc.hN = static_cast<T>(0.5 * (K + 3.0));
   P.flux_lo = p.flux_lo;
   P.tau_c1 = static_cast<T>(p.tau_c1);
   P.tau_c2 = static_cast<T>(p.tau_c2);

@@ -311,13 +311,13 @@ __device__ __forceinline__ void recon_at(const MeshT<T> &m, const ParamsT<T> &P,
   for (int q = 0; q < kNM; ++q)
     for (int v = 0; v < 4; ++v) coef[(q * 4 + v) * n + i] = c[q][v];
 }
-template <typename T, int SH, bool WENO = false>
-__global__ void __launch_bounds__(shape_bs(SH), shape_minb(SH)) k_recon(MeshT<T> m, ParamsT<T> P,
+template <typename T, bool WENO>
+__global__ void __launch_bounds__(kMaxShapeBlock) k_recon(MeshT<T> m, ParamsT<T> P,
                                                                         const T *__restrict__ W,
                                                                         const T *__restrict__ Wx,
                                                                         T *__restrict__ coef) {
   pdl_enter();
-  for_items<SH>(m.nc, [&](int i) {
+  for_items(m.nc, [&](int i) {
     if (P.slim) {
       const int sid = m.csid[i];
       if (sid >= 0 && (P.slim[sid] != 0) != WENO) return;
@@ -355,6 +355,26 @@ __device__ __forceinline__ void poly_point(const MeshT<T> &m, const T *__restric
     val[v] = W[v * n + i] + c[0][v] * x + c[1][v] * y + c[2][v] * p2 + c[3][v] * p3 + c[4][v] * p4;
     gx[v] = (c[0][v] + T(2) * c[2][v] * x + c[3][v] * y) * ih;
     gy[v] = (c[1][v] + c[3][v] * x + T(2) * c[4][v] * y) * ih;
+  }
+}
+
+// the same with the gradient left in the cell's scaled coordinates (to be
+// multiplied by 1/h): from coef, or from the given coefficients where lim
+template <bool CHAR>
+__device__ __forceinline__ void side_scaled(const MeshT<double> &m, const double *__restrict__ W,
+                                            const double *__restrict__ coef, const double (*lc)[4], bool lim, int i,
+                                            double x, double y, double val[4], double gx[4], double gy[4]) {
+  const int n = m.nc;
+  const double p2 = x * x - m.m2[i], p3 = x * y - m.m2[n + i], p4 = y * y - m.m2[2 * n + i];
+  const double x2 = x + x, y2 = y + y;
+#pragma unroll
+  for (int v = 0; v < 4; ++v) {
+    double c[kNM];
+#pragma unroll
+    for (int q = 0; q < kNM; ++q) c[q] = CHAR && lim ? lc[q][v] : coef[(q * 4 + v) * n + i];
+    val[v] = W[v * n + i] + c[0] * x + c[1] * y + c[2] * p2 + c[3] * p3 + c[4] * p4;
+    gx[v] = c[0] + c[2] * x2 + c[3] * y;
+    gy[v] = c[1] + c[3] * x + c[4] * y2;
   }
 }
 
@@ -454,8 +474,13 @@ __device__ __forceinline__ void lo_ghost(const ParamsT<T> &P, int tag, T nx, T n
 // K2: gas-kinetic flux and interface state at the two Gauss points of every
 // face; writes the weighted sums F0, F1, Wc, Wt (global frame) per face:
 //   out[(k*4 + v)*nf + f], k = 0 F0, 1 F1, 2 Wc, 3 Wt.
+// Two forms.  face_raw_at: both Gauss points of a face in one thread, raw
+// moments in the face frame; the full flux, and the FP32 of the mixed path
+// (whose rounding it fixes: the implicit solves of a V-cycle carry a changed
+// FP32 rounding into every cell, and the mixed results are to stay what they
+// are).  face_smooth_at: the FP64 smooth flux.
 template <typename T, bool FULL, bool CHAR>
-__device__ __forceinline__ void face_at(const MeshT<T> &m, const ParamsT<T> &P, const T *__restrict__ W,
+__device__ __forceinline__ void face_raw_at(const MeshT<T> &m, const ParamsT<T> &P, const T *__restrict__ W,
                                         const T *__restrict__ Wx, const T *__restrict__ coef, T *__restrict__ out,
                                         const Ctl *ctl, const unsigned long long *dt_bits, const int f) {
   const int sid = m.fsid[f];
@@ -546,15 +571,112 @@ __device__ __forceinline__ void face_at(const MeshT<T> &m, const ParamsT<T> &P, 
   for (int k = 0; k < 4; ++k)
     for (int v = 0; v < 4; ++v) out[(k * 4 + v) * nf + f] = acc[k][v];
 }
-template <typename T, int SH, bool FULL = false, bool CHAR = false>
-__global__ void __launch_bounds__(shape_bs(SH), shape_minb(SH)) k_face(MeshT<T> m, ParamsT<T> P,
-                                                                       const T *__restrict__ W,
-                                                                       const T *__restrict__ Wx,
-                                                                       const T *__restrict__ coef,
-                                                                       T *__restrict__ out, const Ctl *ctl,
-                                                                       const unsigned long long *dt_bits) {
+// The FP64 smooth flux.  One thread evaluates Gauss point k of face f; in the
+// pair of lanes of a face lane 0 collects and stores F0 and F1, lane 1 Wc and
+// Wt.  GB300's FP64 units take 64 clocks of a sub-core per warp instruction
+// whatever the number of active lanes, so the FP64 instructions of a thread
+// are what the kernel costs: the gradients of the two sides are averaged in
+// the global frame before the moments need them, the moments close about the
+// mean velocity (gks_smooth), erf and exp share one argument (half01), and
+// one point per thread halves the serial chain of a small mesh.  Bound by the
+// FP64 pipe.  Before (face_raw_at) and now: 319 -> 140 us on 90,368 faces,
+// 66 -> 23 us on 208.
+__device__ __forceinline__ void pair_sum_store(const double F0[4], const double F1[4], const double Wc[4],
+                                               const double Wt[4], int k, unsigned pair, double *__restrict__ out,
+                                               int nf, int f) {
+  double a[8];
+#pragma unroll
+  for (int v = 0; v < 4; ++v) {
+    const double s0 = k ? F0[v] : Wc[v], s1 = k ? F1[v] : Wt[v];
+    a[v] = (k ? Wc[v] : F0[v]) + __shfl_xor_sync(pair, s0, 1);
+    a[4 + v] = (k ? Wt[v] : F1[v]) + __shfl_xor_sync(pair, s1, 1);
+  }
+#pragma unroll
+  for (int q = 0; q < 8; ++q) out[(k * 8 + q) * nf + f] = 0.5 * a[q];
+}
+template <bool CHAR>
+__device__ __forceinline__ void face_smooth_at(const MeshT<double> &m, const ParamsT<double> &P,
+                                               const double *__restrict__ W, const double *__restrict__ Wx,
+                                               const double *__restrict__ coef, double *__restrict__ out, const int f,
+                                               const int k) {
+  const int sid = m.fsid[f];
+  if (sid < 0) return;   // free face space of a batch
+  if (P.slim && P.slim[sid] != 0) return;   // the other flux class's launch
+  const unsigned pair = 3u << (threadIdx.x & 30);      // the lanes of this face
+  const int nf = m.nf;
+  const int c0 = m.fc0[f], c1 = m.fc1[f];
+  const double nx = m.fn[f], ny = m.fn[nf + f], ajump = m.fjump[f];
+  // characteristic WENO: the two sides' polynomials limited for this face
+  double cs0[CHAR ? kNM : 1][4], cs1[CHAR ? kNM : 1][4];
+  bool lim0 = false, lim1 = false;
+  if constexpr (CHAR) {
+    double wref[4];
+    for (int v = 0; v < 4; ++v) wref[v] = c1 >= 0 ? 0.5 * (W[v * m.nc + c0] + W[v * m.nc + c1]) : W[v * m.nc + c0];
+    lim0 = m.wenok[c0] != 0;
+    if (lim0) char_side(m, P, W, Wx, coef, c0, wref, nx, ny, cs0);
+    lim1 = c1 >= 0 && m.wenok[c1] != 0;
+    if (lim1) char_side(m, P, W, Wx, coef, c1, wref, nx, ny, cs1);
+  }
+  // the two sides: value and scaled gradient, global frame
+  double wL[4], gL[2][4], wR[4], gR[2][4], wl[4], wr[4];
+  side_scaled<CHAR>(m, W, coef, cs0, lim0, c0, m.fxi[(2 * k) * nf + f], m.fxi[(2 * k + 1) * nf + f], wL, gL[0], gL[1]);
+  D::rot_in(nx, ny, wL, wl);
+  const double ihL = m.ih[c0];
+  double ihR = ihL;
+  if (c1 >= 0) {
+    side_scaled<CHAR>(m, W, coef, cs1, lim1, c1, m.fxi[(4 + 2 * k) * nf + f], m.fxi[(5 + 2 * k) * nf + f], wR, gR[0],
+                      gR[1]);
+    D::rot_in(nx, ny, wR, wr);
+    ihR = m.ih[c1];
+  } else {
+    const int tag = -1 - c1, kind = P.bc_kind[tag];
+    if (kind == CGKS_BC_FARFIELD || kind == CGKS_BC_DIRICHLET) {
+      if (kind == CGKS_BC_FARFIELD) {
+        // Riemann-invariant state from the cell mean and the free stream
+        double wm[4], wi[4];
+        for (int v = 0; v < 4; ++v) wm[v] = W[v * m.nc + c0];
+        D::rot_in(nx, ny, wm, wi);
+        farfield_ghost(P, tag, nx, ny, wi, wr);
+      } else {
+        dirichlet_ghost(P, tag, nx, ny, wr);
+      }
+      D::rot_out(nx, ny, wr, wR);
+      for (int v = 0; v < 4; ++v) gR[0][v] = gR[1][v] = 0.0;
+    } else if (kind == CGKS_BC_OUTFLOW) {
+      for (int v = 0; v < 4; ++v) { wR[v] = wL[v]; wr[v] = wl[v]; gR[0][v] = gL[0][v]; gR[1][v] = gL[1][v]; }
+    } else {
+      wall_ghost_global(P, tag, nx, ny, wL, gL[0], gL[1], wR, gR[0], gR[1]);   // linear in the gradient
+      D::rot_in(nx, ny, wR, wr);
+    }
+  }
+  // W^c from the two half ranges; its slopes: the mean of the sides plus,
+  // along n, alpha / delta times the jump
+  double wc[4], Wc[4], G[2][4], F0[4], F1[4], Wt[4];
+  D::half_state<double, false>(P.kc, wl, +1, wc);
+  D::half_state<double, true>(P.kc, wr, -1, wc);
+  D::rot_out(nx, ny, wc, Wc);
+  const double hl = 0.5 * ihL, hr = 0.5 * ihR, ax = ajump * nx, ay = ajump * ny;
+#pragma unroll
+  for (int v = 0; v < 4; ++v) {
+    const double d = wR[v] - wL[v];
+    G[0][v] = hl * gL[0][v] + hr * gR[0][v] + ax * d;
+    G[1][v] = hl * gL[1][v] + hr * gR[1][v] + ay * d;
+  }
+  D::gks_smooth(P.kc, P.mu[sid], nx, ny, Wc, G, F0, F1, Wt);
+  pair_sum_store(F0, F1, Wc, Wt, k, pair, out, nf, f);
+}
+// threads a face takes
+template <typename T, bool FULL> __host__ __device__ constexpr int face_threads() { return FULL || is_f32<T>() ? 1 : 2; }
+template <typename T, bool FULL, bool CHAR>
+__global__ void __launch_bounds__(kMaxShapeBlock) k_face(MeshT<T> m, ParamsT<T> P, const T *__restrict__ W,
+                                                         const T *__restrict__ Wx, const T *__restrict__ coef,
+                                                         T *__restrict__ out, const Ctl *ctl,
+                                                         const unsigned long long *dt_bits) {
   pdl_enter();
-  for_items<SH>(m.nf, [&](int f) { face_at<T, FULL, CHAR>(m, P, W, Wx, coef, out, ctl, dt_bits, f); });
+  if constexpr (face_threads<T, FULL>() == 2)
+    for_items(2 * m.nf, [&](int i) { face_smooth_at<CHAR>(m, P, W, Wx, coef, out, i >> 1, i & 1); });
+  else
+    for_items(m.nf, [&](int f) { face_raw_at<T, FULL, CHAR>(m, P, W, Wx, coef, out, ctl, dt_bits, f); });
   pdl_exit();
 }
 
@@ -789,13 +911,13 @@ __device__ __forceinline__ void lo_face_at(const MeshT<T> &m, const ParamsT<T> &
       for (int v = 0; v < 4; ++v) E1[v * nf + f] = Fb[v];
   }
 }
-template <typename T, int SH>
-__global__ void __launch_bounds__(shape_bs(SH), shape_minb(SH)) k_lo_face(MeshT<T> m, ParamsT<T> P,
+template <typename T>
+__global__ void __launch_bounds__(kMaxShapeBlock) k_lo_face(MeshT<T> m, ParamsT<T> P,
                                                                           const T *__restrict__ U,
                                                                           const T *__restrict__ prim,
                                                                           T *__restrict__ Flo, T *__restrict__ lam,
                                                                           T *__restrict__ E0, T *__restrict__ E1) {
-  for_items_pdl<SH>(m.nf, [&](int f) { return lo_face_geo(m, P, f); },
+  for_items_pdl(m.nf, [&](int f) { return lo_face_geo(m, P, f); },
                     [&](int f, const LoFaceGeo<T> &g) { lo_face_at(m, P, g, U, prim, Flo, lam, E0, E1, f); });
   pdl_exit();
 }
@@ -973,10 +1095,10 @@ __device__ __forceinline__ void sweep_cell(const MeshT<T> &m, const ParamsT<T> &
                                            const T *__restrict__ E0, const T *__restrict__ E1, T *dU) {
   sweep_cell_from(m, P, g, i, s, U, prim, Rk, invD, lamS, E0, E1, dU, false, dU);
 }
-// cells per block of a sweep launch of shape SH
-__host__ __device__ constexpr int sweep_cpb(int sh) { return shape_bs(sh) / kMaxFace * shape_ipt(sh); }
-template <typename T, int SH>
-__global__ void __launch_bounds__(shape_bs(SH), shape_minb(SH)) k_sweep(MeshT<T> m, ParamsT<T> P,
+// cells per block of a sweep launch of a shape
+__host__ __device__ constexpr int sweep_cpb(int sh) { return shape_bs(sh) / kMaxFace; }
+template <typename T>
+__global__ void __launch_bounds__(kMaxShapeBlock) k_sweep(MeshT<T> m, ParamsT<T> P,
                                                                         const __grid_constant__ Ranges R,
                                                                         const int *__restrict__ list, int count,
                                                                         const T *__restrict__ U,
@@ -986,24 +1108,18 @@ __global__ void __launch_bounds__(shape_bs(SH), shape_minb(SH)) k_sweep(MeshT<T>
                                                                         const T *__restrict__ lamS,
                                                                         const T *__restrict__ E0,
                                                                         const T *__restrict__ E1, T *__restrict__ dU) {
-  constexpr int kGroups = shape_bs(SH) / kMaxFace, kCpb = sweep_cpb(SH), kIpt = shape_ipt(SH);
-  const int s = threadIdx.x & (kMaxFace - 1);
-  // one copy of the per-cell code for every shape (the same arithmetic);
-  // the first item's mesh data is read before the wait, later items' after
-#pragma unroll 1
-  for (int k = 0; k < kIpt; ++k) {
-    const int cl = k * kGroups + static_cast<int>(threadIdx.x) / kMaxFace;
-    int i;
-    if (list) {
-      const int g = static_cast<int>(blockIdx.x) * kCpb + cl;
-      i = g < count ? list[g] : -1;
-    } else {
-      i = range_cell(R, cl, kCpb);
-    }
-    const SweepGeo<T> geo = sweep_geo(m, i, s);
-    pdl_enter();
-    sweep_cell(m, P, geo, i, s, U, prim, Rk, invD, lamS, E0, E1, dU);
+  const int cpb = blockDim.x / kMaxFace, s = threadIdx.x & (kMaxFace - 1);
+  const int cl = static_cast<int>(threadIdx.x) / kMaxFace;
+  int i;
+  if (list) {
+    const int g = static_cast<int>(blockIdx.x) * cpb + cl;
+    i = g < count ? list[g] : -1;
+  } else {
+    i = range_cell(R, cl, cpb);
   }
+  const SweepGeo<T> geo = sweep_geo(m, i, s);   // mesh data, before the wait for the predecessor
+  pdl_enter();
+  sweep_cell(m, P, geo, i, s, U, prim, Rk, invD, lamS, E0, E1, dU);
   pdl_exit();
 }
 

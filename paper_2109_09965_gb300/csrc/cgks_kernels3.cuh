@@ -298,21 +298,43 @@ __device__ __forceinline__ void recon_at(const MeshT<T> &m, const ParamsT<T> &P,
 #pragma unroll
     for (int v = 0; v < NV; ++v) coef[(q * NV + v) * n + i] = c[q][v];
 }
-template <typename T, int SH>
-__global__ void __launch_bounds__(shape_bs(SH), shape_minb(SH))
+template <typename T>
+__global__ void __launch_bounds__(kMaxShapeBlock)
     k_recon(MeshT<T> m, ParamsT<T> P, const T *__restrict__ W, const T *__restrict__ Wx, T *__restrict__ coef) {
   pdl_enter();
-  for_items<SH>(m.nc, [&](int i) { recon_at<T, false>(m, P, W, Wx, coef, nullptr, i); });
+  for_items(m.nc, [&](int i) { recon_at<T, false>(m, P, W, Wx, coef, nullptr, i); });
   pdl_exit();
 }
 // with the compact WENO step; wenok[i] = 1 where the stencil gave a quadratic
-template <typename T, int SH>
-__global__ void __launch_bounds__(shape_bs(SH), shape_minb(SH))
+template <typename T>
+__global__ void __launch_bounds__(kMaxShapeBlock)
     k_recon_weno(MeshT<T> m, ParamsT<T> P, const T *__restrict__ W, const T *__restrict__ Wx, T *__restrict__ coef,
                  const unsigned char *__restrict__ wenok) {
   pdl_enter();
-  for_items<SH>(m.nc, [&](int i) { recon_at<T, true>(m, P, W, Wx, coef, wenok, i); });
+  for_items(m.nc, [&](int i) { recon_at<T, true>(m, P, W, Wx, coef, wenok, i); });
   pdl_exit();
+}
+
+// value and gradient of cell i's quadratic at scaled offset x; the gradient
+// is left in the cell's scaled coordinates (times 1/h = ih for the physical one)
+__device__ __forceinline__ void recon_scaled(const MeshT<double> &m, const double *__restrict__ W, const double *__restrict__ coef,
+                                             int i, const double x[3], double val[NV], double g[3][NV]) {
+  const int n = m.nc;
+  const double a = x[0], b = x[1], e = x[2];
+  const double a2 = a + a, b2 = b + b, e2 = e + e;
+  const double p[6] = { a * a - m.m2[i], a * b - m.m2[n + i], a * e - m.m2[2 * n + i], b * b - m.m2[3 * n + i],
+                   b * e - m.m2[4 * n + i], e * e - m.m2[5 * n + i] };
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    double c[kNM3];
+#pragma unroll
+    for (int q = 0; q < kNM3; ++q) c[q] = coef[(q * NV + v) * n + i];
+    val[v] = W[v * n + i] + c[0] * a + c[1] * b + c[2] * e + c[3] * p[0] + c[4] * p[1] + c[5] * p[2] + c[6] * p[3] +
+             c[7] * p[4] + c[8] * p[5];
+    g[0][v] = c[0] + c[3] * a2 + c[4] * b + c[5] * e;
+    g[1][v] = c[1] + c[4] * a + c[6] * b2 + c[7] * e;
+    g[2][v] = c[2] + c[5] * a + c[7] * b + c[8] * e2;
+  }
 }
 
 // value and gradient of cell i's quadratic at scaled offset x
@@ -340,9 +362,11 @@ __device__ __forceinline__ void recon_point(const MeshT<T> &m, const T *__restri
 // K2: smooth GKS flux and interface state at the Gauss points of every face:
 // out[f][k*5 + v], k = 0 F0, 1 F1, 2 Wc, 3 Wt, weighted sums, global frame:
 // one run of kFO values per face (AoS), so that the cells gathering a face
-// read it in one piece
+// read it in one piece.
+// Two forms, as in 2-D: face_raw_at (raw moments in the face frame: the full
+// flux and the FP32 of the mixed path) and face_smooth_at (FP64 smooth flux).
 template <typename T, bool FULL>
-__device__ __forceinline__ void face_at(const MeshT<T> &m, const ParamsT<T> &P, const T *__restrict__ W,
+__device__ __forceinline__ void face_raw_at(const MeshT<T> &m, const ParamsT<T> &P, const T *__restrict__ W,
                                         const T *__restrict__ coef, T *__restrict__ out, const Ctl *ctl,
                                         const unsigned long long *dt_bits, const int f) {
   const int nf = m.nf;
@@ -440,20 +464,129 @@ __device__ __forceinline__ void face_at(const MeshT<T> &m, const ParamsT<T> &P, 
     for (int v = 0; v < NV; ++v) o[k * NV + v] = acc[k][v];
   vstore<T, kFO>(out + static_cast<size_t>(f) * kFO, o);
 }
-template <typename T, int SH>
-__global__ void __launch_bounds__(shape_bs(SH), shape_minb(SH))
-    k_face(MeshT<T> m, ParamsT<T> P, const T *__restrict__ W, const T *__restrict__ coef, T *__restrict__ out) {
+// The FP64 smooth flux by the 2-D face_smooth_at's scheme.  LANES threads
+// share a face's 3 or 4 Gauss points.
+template <int LANES>
+__device__ __forceinline__ void face_smooth_at(const MeshT<double> &m, const ParamsT<double> &P,
+                                               const double *__restrict__ W, const double *__restrict__ coef,
+                                               double *__restrict__ out, const int f, const int lane) {
+  using T = double;
+  const int nf = m.nf;
+  const int c0 = m.fc0[f], c1 = m.fc1[f], ng = m.fng[f];
+  const T ajump = m.fjump[f];
+  const D3::Frame<T> F = frame_of(m, f);
+  T acc[4][NV];
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+#pragma unroll
+    for (int v = 0; v < NV; ++v) acc[k][v] = T(0);
+  const int tag = c1 < 0 ? -1 - c1 : 0;
+  const bool farfield = c1 < 0 && P.bc_kind[tag] == CGKS_BC_FARFIELD;
+  const T ihL = m.ih[c0], ihR = c1 >= 0 ? m.ih[c1] : ihL;
+#pragma unroll 1
+  for (int k = lane; k < ng; k += LANES) {
+    T x0[3], wL[NV], gL[3][NV], wR[NV], gR[3][NV];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) x0[d] = m.fxi[(3 * k + d) * nf + f];
+    recon_scaled(m, W, coef, c0, x0, wL, gL);
+    T wl[NV], wr[NV];
+    D3::rot_in(F, wL, wl);
+    if (c1 >= 0) {
+      T x1[3];
+#pragma unroll
+      for (int d = 0; d < 3; ++d) x1[d] = m.fxi[(12 + 3 * k + d) * nf + f];
+      recon_scaled(m, W, coef, c1, x1, wR, gR);
+      D3::rot_in(F, wR, wr);
+    } else if (farfield) {
+      T wm[NV], wi[NV];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) wm[v] = W[v * m.nc + c0];
+      D3::rot_in(F, wm, wi);
+      farfield_ghost(P, tag, F, wi, wr);
+      D3::rot_out(F, wr, wR);
+#pragma unroll
+      for (int d = 0; d < 3; ++d)
+#pragma unroll
+        for (int v = 0; v < NV; ++v) gR[d][v] = T(0);
+    } else {
+      wall_ghost(P, tag, F, wL, gL, wR, gR);
+      D3::rot_in(F, wR, wr);
+    }
+    T F0[NV], F1[NV], Wc[NV], Wt[NV];
+    // W^c from the two half ranges; its slopes: the mean of the sides
+    // plus, along n, alpha / delta times the jump
+    T wc[NV], G[3][NV];
+    D3::half_state<T, false>(P.kc, wl, +1, wc);
+    D3::half_state<T, true>(P.kc, wr, -1, wc);
+    D3::rot_out(F, wc, Wc);
+    const T hl = T(0.5) * ihL, hr = T(0.5) * ihR;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const T aj = ajump * F.e[0][d];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) G[d][v] = hl * gL[d][v] + hr * gR[d][v] + aj * (wR[v] - wL[v]);
+    }
+    D3::gks_smooth(P.kc, P.mu, F.e[0], Wc, G, F0, F1, Wt);
+    const T wk = m.fw[k * nf + f];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      acc[0][v] += wk * F0[v];
+      acc[1][v] += wk * F1[v];
+      acc[2][v] += wk * Wc[v];
+      acc[3][v] += wk * Wt[v];
+    }
+  }
+  T *o = out + static_cast<size_t>(f) * kFO;
+  if constexpr (LANES == 1) {
+    T r[kFO];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+      for (int v = 0; v < NV; ++v) r[k * NV + v] = acc[k][v];
+    vstore<T, kFO>(o, r);
+  } else {
+    // lane l collects and stores output l: halves exchanged, then quarters
+    static_assert(LANES == 4, "one lane per output");
+    const unsigned quad = 0xfu << (threadIdx.x & 28);
+    const bool b1 = lane & 2, b0 = lane & 1;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      const T p = (b1 ? acc[2][v] : acc[0][v]) + __shfl_xor_sync(quad, b1 ? acc[0][v] : acc[2][v], 2);
+      const T q = (b1 ? acc[3][v] : acc[1][v]) + __shfl_xor_sync(quad, b1 ? acc[1][v] : acc[3][v], 2);
+      o[lane * NV + v] = (b0 ? q : p) + __shfl_xor_sync(quad, b0 ? p : q, 1);
+    }
+  }
+}
+// Threads per face: one on a large mesh wastes no lane on the missing fourth
+// point of a triangle; four on a small one spread its few faces over the FP64
+// units (608 sub-cores).  28,850 faces (hexahedra): 174 us with 4, 191 with 1;
+// 282,880 (mostly triangles): 1281 us with 4, 1162 with 1 (before, raw moments
+// in one thread: 358 and 2809 us).
+constexpr int64_t kFaceLanes4 = 100000;
+inline int face_lanes(int64_t n_faces) { return n_faces < kFaceLanes4 ? 4 : 1; }
+template <typename T>
+__global__ void __launch_bounds__(kMaxShapeBlock)
+    k_face(MeshT<T> m, ParamsT<T> P, const T *__restrict__ W, const T *__restrict__ coef,
+           T *__restrict__ out) {
   pdl_enter();
-  for_items<SH>(m.nf, [&](int f) { face_at<T, false>(m, P, W, coef, out, nullptr, nullptr, f); });
+  for_items(m.nf, [&](int f) { face_raw_at<T, false>(m, P, W, coef, out, nullptr, nullptr, f); });
+  pdl_exit();
+}
+template <int LANES>
+__global__ void __launch_bounds__(kMaxShapeBlock)
+    k_face_smooth(MeshT<double> m, ParamsT<double> P, const double *__restrict__ W,
+                  const double *__restrict__ coef, double *__restrict__ out) {
+  pdl_enter();
+  for_items(LANES * m.nf, [&](int i) { face_smooth_at<LANES>(m, P, W, coef, out, i / LANES, i % LANES); });
   pdl_exit();
 }
 // the full flux of Eq. (2nd-flux): the same face loop, with the step's dt
-template <typename T, int SH>
-__global__ void __launch_bounds__(shape_bs(SH), shape_minb(SH))
-    k_face_full(MeshT<T> m, ParamsT<T> P, const T *__restrict__ W, const T *__restrict__ coef, T *__restrict__ out,
-                const Ctl *ctl, const unsigned long long *dt_bits) {
+template <typename T>
+__global__ void __launch_bounds__(kMaxShapeBlock)
+    k_face_full(MeshT<T> m, ParamsT<T> P, const T *__restrict__ W, const T *__restrict__ coef,
+                T *__restrict__ out, const Ctl *ctl, const unsigned long long *dt_bits) {
   pdl_enter();
-  for_items<SH>(m.nf, [&](int f) { face_at<T, true>(m, P, W, coef, out, ctl, dt_bits, f); });
+  for_items(m.nf, [&](int f) { face_raw_at<T, true>(m, P, W, coef, out, ctl, dt_bits, f); });
   pdl_exit();
 }
 
@@ -727,12 +860,12 @@ __device__ __forceinline__ void lo_face_at(const MeshT<T> &m, const ParamsT<T> &
     }
   }
 }
-template <typename T, int SH>
-__global__ void __launch_bounds__(shape_bs(SH), shape_minb(SH))
+template <typename T>
+__global__ void __launch_bounds__(kMaxShapeBlock)
     k_lo_face(MeshT<T> m, ParamsT<T> P, const T *__restrict__ rec, T *__restrict__ Flo,
               T *__restrict__ E0, T *__restrict__ E1) {
   pdl_enter();
-  for_items<SH>(m.nf, [&](int f) { lo_face_at(m, P, rec, Flo, E0, E1, f); });
+  for_items(m.nf, [&](int f) { lo_face_at(m, P, rec, Flo, E0, E1, f); });
   pdl_exit();
 }
 
@@ -868,25 +1001,19 @@ __device__ __forceinline__ void sweep_cell(const MeshT<T> &m, const ParamsT<T> &
     dU[static_cast<size_t>(i) * kDU + s] = (Rk[s * n + i] - mine) * invD[i];
   }
 }
-// cells per block of a sweep launch of shape SH
-__host__ __device__ constexpr int sweep_cpb(int sh) { return shape_bs(sh) / kSweepLanes * shape_ipt(sh); }
-template <typename T, int SH>
-__global__ void __launch_bounds__(shape_bs(SH), shape_minb(SH))
+// cells per block of a sweep launch of a shape
+__host__ __device__ constexpr int sweep_cpb(int sh) { return shape_bs(sh) / kSweepLanes; }
+template <typename T>
+__global__ void __launch_bounds__(kMaxShapeBlock)
     k_sweep(MeshT<T> m, ParamsT<T> P, int begin, int count, const T *__restrict__ rec,
             const T *__restrict__ Rk, const T *__restrict__ invD, const T *__restrict__ lamS,
             const T *__restrict__ E0, const T *__restrict__ E1, T *__restrict__ dU) {
-  constexpr int kGroups = shape_bs(SH) / kSweepLanes, kIpt = shape_ipt(SH);
   const int s = threadIdx.x & (kSweepLanes - 1);
-  // one copy of the per-cell code for every shape (the same arithmetic);
-  // the first item's mesh data is read before the wait, later items' after
-#pragma unroll 1
-  for (int k = 0; k < kIpt; ++k) {
-    const int g = (static_cast<int>(blockIdx.x) * kIpt + k) * kGroups + static_cast<int>(threadIdx.x) / kSweepLanes;
-    const int i = g < count ? begin + g : -1;
-    const SweepGeo<T> geo = sweep_geo(m, i, s);
-    pdl_enter();
-    sweep_cell(m, P, geo, i, s, rec, Rk, invD, lamS, E0, E1, dU);
-  }
+  const int g = static_cast<int>(blockIdx.x * blockDim.x + threadIdx.x) / kSweepLanes;
+  const int i = g < count ? begin + g : -1;
+  const SweepGeo<T> geo = sweep_geo(m, i, s);   // mesh data, before the wait for the predecessor
+  pdl_enter();
+  sweep_cell(m, P, geo, i, s, rec, Rk, invD, lamS, E0, E1, dU);
   pdl_exit();
 }
 

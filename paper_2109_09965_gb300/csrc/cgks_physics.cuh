@@ -12,14 +12,14 @@
 
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 namespace cgks {
 namespace dev {
 
 constexpr int NV = 4;
 
-template <typename T> __device__ __forceinline__ T d_erfc(T x);
-template <> __device__ __forceinline__ double d_erfc<double>(double x) { return erfc(x); }
-template <> __device__ __forceinline__ float d_erfc<float>(float x) { return erfcf(x); }
+__device__ __forceinline__ float d_erfc(float x) { return erfcf(x); }
 template <typename T> __device__ __forceinline__ T d_exp(T x);
 template <> __device__ __forceinline__ double d_exp<double>(double x) { return exp(x); }
 template <> __device__ __forceinline__ float d_exp<float>(float x) { return expf(x); }
@@ -50,10 +50,10 @@ __device__ __forceinline__ void rot_out(T nx, T ny, const T l[NV], T g[NV]) {
 }
 
 // Constants of the kinetic model with K internal degrees of freedom,
-// computed once on the host: c2K = 2/(K+2), c4K = 4/(K+2).
+// computed once on the host: c2K = 2/(K+2), c4K = 4/(K+2), hN = (K+2)/2.
 template <typename T>
 struct KC {
-  T K, c2K, c4K;
+  T K, c2K, c4K, hN;
 };
 constexpr double kInvSqrtPi = 0.56418958354775628694807945156;
 
@@ -81,19 +81,92 @@ template <typename T> __device__ __forceinline__ T d_rsqrt(T x);
 template <> __device__ __forceinline__ double d_rsqrt<double>(double x) { return rsqrt(x); }
 template <> __device__ __forceinline__ float d_rsqrt<float>(float x) { return rsqrtf(x); }
 
+// Reciprocal and reciprocal square root.  GB300 issues two FP64 lanes per
+// clock per SM, so the number of FP64 instructions is what an FP64 kernel
+// costs: the FP64 forms take the hardware's estimate (relative error 2^-22)
+// and one third-order step of Newton's family (Householder's iteration),
+// whose error is of the order of the cube, 2^-66.
+//   1/x:        e = 1 - x r,    r <- r + r (e + e^2)             3 FP64
+//   1/sqrt(x):  e = 1 - x r^2,  r <- r + r e (1/2 + 3/8 e)       5 FP64
+// against 8-9 for the IEEE quotient and the library's rsqrt.  Normal
+// arguments; zero, infinity and NaN give NaN or infinity (the state check
+// marks them as it did).  FP32 keeps the library's.
+__device__ __forceinline__ float d_rcp(float x) { return 1.0f / x; }
+__device__ __forceinline__ double d_rcp(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+__device__ __forceinline__ double d_rsqrt3(double x) {
+  double r;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double e = fma(-x * r, r, 1.0);
+  return fma(r * e, fma(0.375, e, 0.5), r);
+}
+
+// sqrt(lambda) and 1/sqrt(pi lambda) of a Maxwellian with 1/(2 lambda) = i2l
+__device__ __forceinline__ void sqrt_lambda(float i2l, float &sl, float &isp) {
+  const float lam = 0.5f / i2l;
+  sl = sqrtf(lam);
+  isp = rsqrtf(lam) * static_cast<float>(kInvSqrtPi);
+}
+__device__ __forceinline__ void sqrt_lambda(double i2l, double &sl, double &isp) {
+  const double t = 2.0 * i2l;
+  sl = d_rsqrt3(t);
+  isp = t * sl * kInvSqrtPi;
+}
+
+// The first two half-range moments, <1> = (1 + sgn erf(z)) / 2 and <u>, over
+// u > 0 (sgn = +1) or u < 0 (-1), z = sl U.  In FP64, for |z| < 1 (normal Mach
+// number below 1.19), erf(z) / (2 z) and exp(-z^2) come from polynomials in
+// t = z^2, the interpolants at the Chebyshev nodes of [0, 1] (degrees 11 and
+// 12, relative errors 8e-18): 24 FP64 instructions in place of about 90 of the
+// library pair; beyond, and for NaN, the library's functions.  FP32 keeps the
+// library's: its arithmetic is not what the mixed path waits for.
+__device__ __forceinline__ void half01(double U, double sl, double isp, int sgn, double &m0, double &m1) {
+  const double z = sl * U, t = z * z;
+  double ex;
+  if (static_cast<unsigned>(__double2hiint(t)) < 0x3ff00000u) {
+    double p = -3.8979494135010711208e-10, q = 1.2719039650810422692e-09;
+    p = fma(p, t, 6.8600322733888428021e-09);  q = fma(q, t, -2.2905624278899245573e-08);
+    p = fma(p, t, -8.1042419009358529508e-08); q = fma(q, t, 2.7213633679812669228e-07);
+    p = fma(p, t, 8.2237123516586812051e-07);  q = fma(q, t, -2.7521178006932174539e-06);
+    p = fma(p, t, -7.4623684537098301688e-06); q = fma(q, t, 2.4798998659720724886e-05);
+    p = fma(p, t, 6.0276474524198539583e-05);  q = fma(q, t, -1.9841141919339012344e-04);
+    p = fma(p, t, -4.2741629876948460403e-04); q = fma(q, t, 1.3888884549085944042e-03);
+    p = fma(p, t, 2.6119888035582113661e-03);  q = fma(q, t, -8.3333332344813161057e-03);
+    p = fma(p, t, -1.343308532161888518e-02);  q = fma(q, t, 4.1666666652193343912e-02);
+    p = fma(p, t, 5.6418958354725031328e-02);  q = fma(q, t, -1.6666666666540416823e-01);
+    p = fma(p, t, -1.8806319451591770219e-01); q = fma(q, t, 4.999999999999427302e-01);
+    p = fma(p, t, 5.6418958354775628327e-01);  q = fma(q, t, -9.9999999999999897845e-01);
+    ex = fma(q, t, 9.9999999999999999698e-01);
+    m0 = fma(sgn > 0 ? z : -z, p, 0.5);
+  } else {
+    m0 = 0.5 * erfc(sgn > 0 ? -z : z);
+    ex = exp(-t);
+  }
+  const double e = 0.5 * (ex * isp);
+  m1 = fma(U, m0, sgn > 0 ? e : -e);
+}
+
 // Half-range moments <u^k>, k = 0..KMAX, over u > 0 (sgn = +1) or u < 0
 // (-1), of the Maxwellian with mean U, 1/(2 lambda) = i2l, sqrt(lambda) = sl
 // and 1/sqrt(pi lambda) = isp.
 template <typename T, int KMAX>
 __device__ __forceinline__ void half_moments(T U, T i2l, T sl, T isp, int sgn, T mu[KMAX + 1]) {
-  T z = sl * U;
-  T e = d_exp(-z * z) * isp;
-  if (sgn > 0) {
-    mu[0] = T(0.5) * d_erfc(-z);
-    mu[1] = U * mu[0] + T(0.5) * e;
+  if constexpr (std::is_same<T, double>::value) {
+    half01(U, sl, isp, sgn, mu[0], mu[1]);
   } else {
-    mu[0] = T(0.5) * d_erfc(z);
-    mu[1] = U * mu[0] - T(0.5) * e;
+    T z = sl * U;
+    T e = d_exp(-z * z) * isp;
+    if (sgn > 0) {
+      mu[0] = T(0.5) * d_erfc(-z);
+      mu[1] = U * mu[0] + T(0.5) * e;
+    } else {
+      mu[0] = T(0.5) * d_erfc(z);
+      mu[1] = U * mu[0] - T(0.5) * e;
+    }
   }
 #pragma unroll
   for (int k = 2; k <= KMAX; ++k) mu[k] = U * mu[k - 1] + T(k - 1) * i2l * mu[k - 2];
@@ -163,7 +236,10 @@ __device__ __forceinline__ void micro_slope(const SlopeSolver<T> &S, const T b[N
   s[0] = b[0] - S.U * s[1] - S.V * s[2] - T(0.5) * s[3] * S.q;
 }
 
-// Smooth gas-kinetic flux at one Gauss point, Eq. (2nd-smooth-flux):
+// Smooth gas-kinetic flux at one Gauss point, Eq. (2nd-smooth-flux), by raw
+// moments in the face frame: the FP32 form of the 2-D mixed path, whose
+// results it keeps (a flux rounded differently moves the FP32 gradients by as
+// much as their own error); the FP64 form is gks_smooth.
 //   f = g^c - tau (a_n u + a_t v + A) g^c + A g^c t,   tau = mu / p^c
 // with W^c from the half-range moments of g^l (u>0) and g^r (u<0), the
 // equilibrium slopes from the mean of the side derivatives plus, along n,
@@ -218,6 +294,86 @@ __device__ __forceinline__ void gks_point_local(const KC<T> &kc, T mu_visc, T aj
     F0[v] = gc.rho * (feq[v] - tau * (gn2[v] + gtuv[v] + gAu[v]));
     F1[v] = gc.rho * gAu[v];
     Wt[v] = gc.rho * gA[v];
+  }
+}
+
+// One side of a Gauss point in the face frame: its share of W^c (the
+// half-range moments <psi> of its Maxwellian over u > 0 for sgn = +1, u < 0
+// for -1), added to or stored in Wc.
+template <typename T, bool ADD>
+__device__ __forceinline__ void half_state(const KC<T> &kc, const T W[NV], int sgn, T Wc[NV]) {
+  const T ir = d_rcp(W[0]);
+  const T U = W[1] * ir, V = W[2] * ir;
+  const T th = kc.c2K * ((W[3] - T(0.5) * (W[1] * U + W[2] * V)) * ir);   // 1 / (2 lambda)
+  T sl, isp, m[2];
+  sqrt_lambda(th, sl, isp);
+  half_moments<T, 1>(U, th, sl, isp, sgn, m);
+  const T a = W[0] * m[0], b = W[0] * m[1];
+  const T E = T(0.5) * (b * U + a * (V * V + (kc.K + T(2)) * th));
+  if (ADD) { Wc[0] += a; Wc[1] += b; Wc[2] += a * V; Wc[3] += E; }
+  else { Wc[0] = a; Wc[1] = b; Wc[2] = a * V; Wc[3] = E; }
+}
+
+// Smooth gas-kinetic flux at one Gauss point, Eq. (2nd-smooth-flux):
+//   f = g^c - tau (a_n u + a_t v + A) g^c + A g^c t,   tau = mu / p^c,
+// for the interface state W^c = Wc and its spatial derivatives G[j] along
+// x and y, in the global frame (n the face normal).  F0 + t F1 = flux,
+// Wc + t Wt = interface state.
+// The moments are taken about the mean velocity, where they close: with
+// theta = 1/(2 lambda) and N = K + 2 degrees of freedom the micro-slope of a
+// direction is the one of (rho, U, theta),
+//   a = d rho / rho + c.dU / theta + ((c^2 + xi^2) / theta - N) d theta / (2 theta),
+// the condition <A + a.u> = 0 gives A as the same expression of the Euler
+// time derivatives
+//   d_t rho = -rho (U.grad rho / rho + div U), d_t U = -U.grad U - grad p / rho,
+//   d_t theta = -U.grad theta - (2/N) theta div U,
+// so that <A psi> and <u A psi> are the time derivatives of the conservative
+// variables and of the Euler flux, and -tau <u (a.u + A) psi> is the viscous
+// traction mu (dU/dn + grad U_n - (2/N) div U n) with the heat flux
+// mu (N/2 + 1) d theta / dn.  About 110 FP64 instructions where the tables
+// of raw moments took about 650.
+template <typename T>
+__device__ __forceinline__ void gks_smooth(const KC<T> &kc, T mu_visc, T nx, T ny, const T Wc[NV],
+                                           const T G[2][NV], T F0[NV], T F1[NV], T Wt[NV]) {
+  const T c2 = kc.c2K, hN = kc.hN;
+  const T rho = Wc[0], ir = d_rcp(rho);
+  const T u = Wc[1] * ir, v = Wc[2] * ir, E = Wc[3] * ir;
+  const T th = c2 * (E - T(0.5) * (u * u + v * v)), H = E + th;
+  T r[2], ux[2], vx[2], Tx[2];
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    r[j] = G[j][0] * ir;
+    ux[j] = G[j][1] * ir - u * r[j];
+    vx[j] = G[j][2] * ir - v * r[j];
+    Tx[j] = c2 * (G[j][3] * ir - E * r[j] - u * ux[j] - v * vx[j]);
+  }
+  const T div = ux[0] + vx[1];
+  const T rt = -(u * r[0] + v * r[1] + div);
+  const T ut = -(u * ux[0] + v * ux[1] + th * r[0] + Tx[0]);
+  const T vt = -(u * vx[0] + v * vx[1] + th * r[1] + Tx[1]);
+  const T Tt = -(u * Tx[0] + v * Tx[1] + c2 * th * div);
+  const T un = u * nx + v * ny, mn = rho * un, p = rho * th;
+  const T a0 = rho * rt, ek = u * ut + v * vt, ei = ek + hN * Tt;
+  Wt[0] = a0;
+  Wt[1] = u * a0 + rho * ut;
+  Wt[2] = v * a0 + rho * vt;
+  Wt[3] = E * a0 + rho * ei;
+  const T mt = Wt[1] * nx + Wt[2] * ny, pt = th * a0 + rho * Tt;
+  F1[0] = mt;
+  F1[1] = u * mt + mn * ut + nx * pt;
+  F1[2] = v * mt + mn * vt + ny * pt;
+  F1[3] = H * mt + mn * (ei + Tt);
+  F0[0] = mn;
+  F0[1] = mn * u + p * nx;
+  F0[2] = mn * v + p * ny;
+  F0[3] = mn * H;
+  if (mu_visc != T(0)) {
+    const T s = ux[1] + vx[0], d = c2 * div;
+    const T sx = mu_visc * ((T(2) * ux[0] - d) * nx + s * ny);
+    const T sy = mu_visc * (s * nx + (T(2) * vx[1] - d) * ny);
+    F0[1] -= sx;
+    F0[2] -= sy;
+    F0[3] -= u * sx + v * sy + mu_visc * (hN + T(1)) * (Tx[0] * nx + Tx[1] * ny);
   }
 }
 

@@ -5,7 +5,7 @@
 // face).  Conservative variables (rho, rho u_n, rho u_t1, rho u_t2, rho E).
 // Moments normalised by rho; K = (5 - 3 gamma)/(gamma - 1) internal degrees
 // of freedom, so <xi^2> = K/(2 lambda), <xi^4> = K(K+2)/(4 lambda^2).
-// kc holds K, c2K = 2/(K+3), c4K = 4/(K+3).  The micro-slope solve
+// kc holds K, c2K = 2/(K+3), c4K = 4/(K+3), hN = (K+3)/2.  The micro-slope solve
 // <a psi> = b uses its closed form.
 #pragma once
 
@@ -131,7 +131,8 @@ __device__ __forceinline__ void micro_slope(const SlopeSolver<T> &S, const T b[N
   s[0] = b[0] - S.U * s[1] - S.V * s[2] - S.W * s[3] - T(0.5) * s[4] * S.q;
 }
 
-// Smooth GKS flux at one Gauss point, Eq. (2nd-smooth-flux), local frame:
+// Smooth GKS flux at one Gauss point, Eq. (2nd-smooth-flux), local frame,
+// by raw moments: the FP32 form of the mixed path (see the 2-D one)
 //   f = g^c - tau (a_n u + a_t1 v + a_t2 w + A) g^c + A g^c t,  tau = mu / p^c
 // W^c from the half-range moments of g^l (u > 0) and g^r (u < 0); the
 // equilibrium slopes from the mean of the side derivatives (dl[k], dr[k]:
@@ -188,6 +189,81 @@ __device__ __forceinline__ void gks_point_local(const KC<T> &kc, T mu_visc, T aj
     F0[v] = gc.rho * (feq[v] - tau * (gn2[v] + g1u[v] + g2u[v] + gAu[v]));
     F1[v] = gc.rho * gAu[v];
     Wt[v] = gc.rho * gA[v];
+  }
+}
+
+// One side of a Gauss point in the face frame: its share of W^c over u > 0
+// (sgn = +1) or u < 0 (-1), added to or stored in Wc.
+template <typename T, bool ADD>
+__device__ __forceinline__ void half_state(const KC<T> &kc, const T W[NV], int sgn, T Wc[NV]) {
+  const T ir = dev::d_rcp(W[0]);
+  const T U = W[1] * ir, V = W[2] * ir, Z = W[3] * ir;
+  const T th = kc.c2K * ((W[4] - T(0.5) * (W[1] * U + W[2] * V + W[3] * Z)) * ir);   // 1 / (2 lambda)
+  T sl, isp, m[2];
+  dev::sqrt_lambda(th, sl, isp);
+  half_moments<T, 1>(U, th, sl, isp, sgn, m);
+  const T a = W[0] * m[0], b = W[0] * m[1];
+  const T E = T(0.5) * (b * U + a * (V * V + Z * Z + (kc.K + T(3)) * th));
+  if (ADD) { Wc[0] += a; Wc[1] += b; Wc[2] += a * V; Wc[3] += a * Z; Wc[4] += E; }
+  else { Wc[0] = a; Wc[1] = b; Wc[2] = a * V; Wc[3] = a * Z; Wc[4] = E; }
+}
+
+// Smooth GKS flux at one Gauss point, Eq. (2nd-smooth-flux), from the
+// interface state Wc and its derivatives G[j] along x, y, z, global frame,
+// n the face normal: the moments about the mean velocity in closed form, as
+// the 2-D dev::gks_smooth explains (N = K + 3 degrees of freedom).
+template <typename T>
+__device__ __forceinline__ void gks_smooth(const KC<T> &kc, T mu_visc, const T n[3], const T Wc[NV],
+                                           const T G[3][NV], T F0[NV], T F1[NV], T Wt[NV]) {
+  const T c2 = kc.c2K, hN = kc.hN;
+  const T rho = Wc[0], ir = dev::d_rcp(rho);
+  const T u[3] = { Wc[1] * ir, Wc[2] * ir, Wc[3] * ir };
+  const T E = Wc[4] * ir;
+  const T th = c2 * (E - T(0.5) * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2])), H = E + th;
+  T r[3], du[3][3], Tx[3];   // du[j][k] = d u_k / d x_j
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    r[j] = G[j][0] * ir;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) du[j][k] = G[j][1 + k] * ir - u[k] * r[j];
+    Tx[j] = c2 * (G[j][4] * ir - E * r[j] - u[0] * du[j][0] - u[1] * du[j][1] - u[2] * du[j][2]);
+  }
+  const T div = du[0][0] + du[1][1] + du[2][2];
+  const T rt = -(u[0] * r[0] + u[1] * r[1] + u[2] * r[2] + div);
+  T ut[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+    ut[k] = -(u[0] * du[0][k] + u[1] * du[1][k] + u[2] * du[2][k] + th * r[k] + Tx[k]);
+  const T Tt = -(u[0] * Tx[0] + u[1] * Tx[1] + u[2] * Tx[2] + c2 * th * div);
+  const T un = u[0] * n[0] + u[1] * n[1] + u[2] * n[2], mn = rho * un, p = rho * th;
+  const T a0 = rho * rt, ei = u[0] * ut[0] + u[1] * ut[1] + u[2] * ut[2] + hN * Tt;
+  Wt[0] = a0;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) Wt[1 + k] = u[k] * a0 + rho * ut[k];
+  Wt[4] = E * a0 + rho * ei;
+  const T mt = Wt[1] * n[0] + Wt[2] * n[1] + Wt[3] * n[2], pt = th * a0 + rho * Tt;
+  F1[0] = mt;
+  F0[0] = mn;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    F1[1 + k] = u[k] * mt + mn * ut[k] + n[k] * pt;
+    F0[1 + k] = mn * u[k] + p * n[k];
+  }
+  F1[4] = H * mt + mn * (ei + Tt);
+  F0[4] = mn * H;
+  if (mu_visc != T(0)) {
+    T w = mu_visc * (hN + T(1)) * (Tx[0] * n[0] + Tx[1] * n[1] + Tx[2] * n[2]);
+    const T d = c2 * div;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      T s = -d * n[k];
+#pragma unroll
+      for (int j = 0; j < 3; ++j) s += (du[j][k] + du[k][j]) * n[j];
+      s *= mu_visc;
+      F0[1 + k] -= s;
+      w += u[k] * s;
+    }
+    F0[4] -= w;
   }
 }
 

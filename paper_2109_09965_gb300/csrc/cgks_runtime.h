@@ -166,19 +166,6 @@ void tuned_launch(Tuner &tu, int tk, cudaStream_t st, Launch &&go) {
   tu.used[tk] = true;
 }
 
-// call f(std::integral_constant<int, s>) for the runtime shape index s
-template <typename F>
-void with_shape(int s, F &&f) {
-  switch (s) {
-    case 1: f(std::integral_constant<int, 1>{}); break;
-    case 2: f(std::integral_constant<int, 2>{}); break;
-    case 3: f(std::integral_constant<int, 3>{}); break;
-    case 4: f(std::integral_constant<int, 4>{}); break;
-    default: f(std::integral_constant<int, 0>{}); break;
-  }
-}
-static_assert(kNShape == 5, "with_shape covers every shape");
-
 // ---- the 3-D solver (cgks_device3.cu) ----
 struct Solver3;
 int s3_create(const HostMesh3 &m, const cgks_params *p, cudaStream_t stream, Timer *timer, Solver3 **out);

@@ -1,10 +1,11 @@
 // Launch shapes of the tunable kernels (shared by the kernels and the
 // runtimes).  A shape is (threads per block, items per thread, minimum
-// resident blocks per SM).  An item is a cell or a face; for the colour
-// sweeps, where a lane group serves one cell, it is a cell per lane group.
-// Item k of thread t of block b is (b * ipt + k) * bs + t, so every item is
-// computed by the same arithmetic whatever the shape: the shape changes only
-// which thread does the work, never the result.
+// resident blocks per SM); an item is a cell or a face (a face's Gauss point,
+// a lane group's cell), one per thread in every shape.  The block size is a
+// launch argument, so one compiled kernel serves every shape: it changes only
+// which thread does the work, never the result.  (A compilation per shape let
+// the compiler fuse multiplies and adds differently in each; a runtime count
+// of items per thread cost the short FP32 kernels 5-20%.)
 #pragma once
 
 #include "../../include/cgks.h"
@@ -15,14 +16,13 @@
 namespace cgks {
 
 constexpr int kNShape = CGKS_TUNE_SHAPES;
+constexpr int kMaxShapeBlock = 256;   // the largest block of any shape
 
 __host__ __device__ constexpr int shape_bs(int s) {
-  return (s == 1 || s == 4) ? 64 : s == 2 ? 256 : 128;
+  return s == 1 ? 64 : s == 2 ? 256 : s == 3 ? 96 : s == 4 ? 192 : 128;
 }
-__host__ __device__ constexpr int shape_ipt(int s) { return (s == 3 || s == 4) ? 2 : 1; }
-// minimum resident blocks per SM (a register cap for the compiler); 1 = none.
-// No shape caps registers: under a cap the compiler may fuse multiplies and
-// adds differently, and a shape must never change a result.
+__host__ __device__ constexpr int shape_ipt(int) { return 1; }
+// minimum resident blocks per SM; 1 = no register cap
 __host__ __device__ constexpr int shape_minb(int) { return 1; }
 
 // tunable kernels
@@ -33,31 +33,25 @@ static_assert(TK_COUNT == CGKS_TUNE_KERNELS, "tunable kernel count");
 constexpr int kDefaultShape[TK_COUNT] = { 2, 0, 2, 0 };
 
 #ifdef __CUDACC__
-// the items of this thread in a launch of shape SH over n items
-template <int SH, typename F>
+// the item of this thread in a launch over n items
+template <typename F>
 __device__ __forceinline__ void for_items(const int n, F &&f) {
-#pragma unroll 1
-  for (int k = 0; k < shape_ipt(SH); ++k) {
-    const int i = (static_cast<int>(blockIdx.x) * shape_ipt(SH) + k) * shape_bs(SH) + static_cast<int>(threadIdx.x);
-    if (i < n) f(i);
-  }
+  const int i = static_cast<int>(blockIdx.x * blockDim.x + threadIdx.x);
+  if (i < n) f(i);
 }
 
 // The same, for a kernel launched as a programmatic dependent launch: geo(i)
 // reads the item's mesh data (which no kernel of a cycle writes), then the
 // thread waits for the predecessor kernel before f(i, g) touches anything
 // else.  Every thread waits, so the grid completes only after its
-// predecessor has.  One copy of the per-item code serves every shape.
-template <int SH, typename G, typename F>
+// predecessor has.
+template <typename G, typename F>
 __device__ __forceinline__ void for_items_pdl(const int n, G &&geo, F &&f) {
-#pragma unroll 1
-  for (int k = 0; k < shape_ipt(SH); ++k) {
-    const int i = (static_cast<int>(blockIdx.x) * shape_ipt(SH) + k) * shape_bs(SH) + static_cast<int>(threadIdx.x);
-    if (i < n) {
-      const auto g = geo(i);
-      pdl_enter();
-      f(i, g);
-    }
+  const int i = static_cast<int>(blockIdx.x * blockDim.x + threadIdx.x);
+  if (i < n) {
+    const auto g = geo(i);
+    pdl_enter();
+    f(i, g);
   }
   pdl_enter();   // threads without items wait too: this grid ends after its predecessor
 }

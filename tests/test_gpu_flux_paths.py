@@ -1,0 +1,82 @@
+"""Branches of the high-order flux that depend on the state or the mesh size,
+against the CPU oracle: the half-range integrals on both sides of |z| = 1
+(normal Mach number 1.19, where the polynomials hand over to the library's
+erfc and exp), and the two ways a 3-D face's Gauss points are spread over
+threads (one thread per face from 100,000 faces, four below).
+
+Bars as in the other parity tests: FP64 1e-12 relative L2 (the same formulas
+in double), mixed 1e-5.
+"""
+import numpy as np
+import pytest
+
+from paper_2109_09965_gb300 import meshgen as MG
+
+pytestmark = pytest.mark.gpu
+GAM = 1.4
+TOL = {"fp64": 1e-12, "mixed": 1e-5}
+
+
+def rel(a, b):
+    return np.linalg.norm(a - b) / max(np.linalg.norm(b), 1e-300)
+
+
+def state(mesh, ma0, ma1):
+    """Stream along a diagonal whose Mach number runs from ma0 to ma1 across
+    the box, with a smooth perturbation."""
+    D = mesh.dim
+    ptr = mesh.cell_ptr
+    x = np.add.reduceat(mesh.nodes[mesh.cell_nodes], ptr[:-1], axis=0) / np.diff(ptr)[:, None]
+    s = 0.02 * np.sin(2.0 * x[:, 0] + 0.3) * np.cos(1.5 * x[:, 1])
+    r, p = 1.0 + s, (1.0 + 0.7 * s) / GAM
+    d = np.array([1.0, 0.4, -0.3][:D]) / np.linalg.norm([1.0, 0.4, -0.3][:D])
+    u = (ma0 + (ma1 - ma0) * x[:, :1]) * d + 0.1 * s[:, None]
+    E = p / (GAM - 1.0) + 0.5 * r * (u * u).sum(1)
+    return np.concatenate([r[:, None], r[:, None] * u, E[:, None]], axis=1)
+
+
+def compare(mesh, spec, W, precision, cycles):
+    from paper_2109_09965_gb300 import cgks
+    if mesh.dim == 2:
+        from oracle import oracle as O
+        om = O.OracleSolver(O.OracleMesh(mesh), spec)
+    else:
+        from oracle import oracle3 as O
+        om = O.OracleSolver3(O.OracleMesh3(mesh), spec)
+    s = cgks.Solver(cgks.Mesh(mesh), dict(spec, precision=precision))
+    s.set_state(W)
+    om.set_state(W)
+    s.explicit_steps(2)
+    om.explicit_steps(2)
+    if cycles:
+        s.pmg_cycle(cycles)
+        om.pmg_cycles(cycles)
+    (a, ax), (b, bx) = s.get_state(), om.get_state()
+    s.close()
+    assert rel(a, b) < TOL[precision]
+    assert rel(ax, bx) < (1e-11 if precision == "fp64" else 1e-4)   # gradients lose one order in h
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("dim", [2, 3])
+@pytest.mark.parametrize("ma, cycles", [((0.0, 0.2), 1), ((0.9, 1.6), 1), ((1.8, 2.6), 0), ((1.4, 0.8), 1)])
+def test_half_range_integrals_across_the_hand_over(dim, ma, cycles, precision):
+    if dim == 2:
+        mesh = MG.box(9, 7, jitter=0.15, seed=2, cells="tri", tags=(0, 0, 0, 0))
+        u = (ma[1], 0.0)
+    else:
+        mesh = MG.box3(3, 3, 3, jitter=0.1, seed=2, cells="prism", tags=(0,) * 6)
+        u = (ma[1], 0.0, 0.0)
+    spec = dict(gamma=GAM, mu=0.002, cfl_hi=0.3, bcs=[dict(kind="farfield", rho=1.0, u=u, p=1 / GAM)])
+    compare(mesh, spec, state(mesh, *ma), precision, cycles)   # the oracle's V-cycle too diverges at 1.8 to 2.6
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("flux", ["smooth", "full"])
+def test_one_thread_per_face_matches_the_oracle(flux, precision):
+    mesh = MG.box3(28, 28, 28, jitter=0.1, seed=4, cells="prism", tags=(0, 0, 0, 0, 1, 1))
+    spec = dict(gamma=GAM, mu=0.002, cfl_hi=0.3, flux_hi=flux,
+                bcs=[dict(kind="farfield", rho=1.0, u=(0.3, 0.0, 0.0), p=1 / GAM), dict(kind="slip")])
+    from paper_2109_09965_gb300 import cgks
+    assert cgks.Mesh(mesh).n_faces >= 100000
+    compare(mesh, spec, state(mesh, 0.2, 0.3), precision, 0)

@@ -37,11 +37,11 @@ inline int nblk(int64_t n, int b) { return static_cast<int>((n + b - 1) / b); }
 // double state, in mixed mode they are float mirrors)
 template <typename T>
 struct Bufs {
-  T *W = nullptr, *Wx = nullptr, *Wn = nullptr, *Ws = nullptr, *Wxs = nullptr, *U = nullptr;
+  T *W = nullptr, *Wx = nullptr, *Wn = nullptr, *Ws = nullptr, *Wxs = nullptr;
   T *coef = nullptr, *FA = nullptr, *FB = nullptr;
-  T *prim = nullptr, *Flo = nullptr, *lam = nullptr, *E0 = nullptr, *E1 = nullptr;
-  T *Rk = nullptr, *invD = nullptr, *dU = nullptr, *lamS = nullptr;
-  T *dU2 = nullptr;   // second increment buffer of the partitioned sweep (ping-pong with dU)
+  T *base = nullptr, *base2 = nullptr;     // low level: base records of alternating implicit steps
+  T *Flo = nullptr, *Rk = nullptr, *invD = nullptr, *delta = nullptr, *lamS = nullptr;
+  T *delta2 = nullptr;   // second increment buffer of the partitioned sweep (ping-pong with delta)
 };
 
 // batch-wide settings (every solve of a batch shares them)
@@ -73,7 +73,7 @@ struct Member {
 
 // device tables of a batch (views into its arena)
 struct DevArrays {
-  double *vol, *ivol, *per, *ih, *m2, *op, *fn, *fS, *fjump, *fxi, *snx, *sny, *shs, *fidl = nullptr;
+  double *vol, *ivol, *per, *ih, *m2, *op, *fn, *fS, *fjump, *fxi, *snx, *sny, *fidl = nullptr;
   double *mu, *bcuw, *bcrho, *bcu, *bcp;
   int *cface, *cnbr, *fc0, *fc1, *csid, *fsid, *bckind;
   unsigned char *ccol, *wenok;
@@ -100,6 +100,7 @@ struct Batch {
   std::vector<int> sweep_seq;        // colour order after the first pass
   std::vector<int> list_off;         // [n_colours + 1] offsets into the sweep cell list
   std::vector<Ranges> ranges[kNShape];  // per sweep shape, per colour: per-solve cell ranges (n = 0: the list)
+  std::vector<int> lanes;               // [n_colours] lanes per cell of the colour's sweeps
   ParamsT<double> dp{};
   ParamsT<float> fp{};
   MeshT<double> dm{};
@@ -296,8 +297,14 @@ void enqueue_hi_step(Batch *b, double *Wout, TF *Wout_m, bool want_res) {
 }
 
 // low-order solve from U = W_p0 (= Wn), R_p0 in Rp0; result in U.  Per
-// implicit step: cell primitives (and U += dU), KFVS faces, right-hand side
-// with the first colour pass, then the remaining colour passes.
+// implicit step: KFVS faces, right-hand side with the first colour pass, then
+// the remaining colour passes; the last pass of each colour advances U and
+// writes the next step's base records.  A pass over all cells makes the first
+// base records, and takes the last passes' place where they do not visit
+// every cell (one colour, no sweeps) or run in one launch (partitioned).
+bool last_pass_advances(const Batch *b) {
+  return b->sh.sweep_order != CGKS_SWEEP_PARTITIONED && b->sh.n_sweeps > 0 && b->n_colours > 1;
+}
 template <typename TF>
 void enqueue_lo_fused(Batch *b) {
   Bufs<TF> &B = bufs<TF>(b);
@@ -312,8 +319,7 @@ void enqueue_lo_fused(Batch *b) {
   for (int q = 0; q < a.n_seq; ++q) a.seq[q] = b->sweep_seq[q];
   a.cr.rstart = b->r_start; a.cr.rbegin = b->r_begin; a.cr.rpre = b->r_pre;
   a.Wp0 = b->Wn; a.Rp0 = b->Rp0; a.U = b->U; a.Src = b->Src;
-  a.dU = B.dU; a.prim = B.prim; a.Um = mirror<TF>(B.U); a.Flo = B.Flo; a.lam = B.lam; a.E0 = B.E0; a.E1 = B.E1;
-  a.Rk = B.Rk; a.invD = B.invD; a.lamS = B.lamS;
+  a.delta = B.delta; a.base = B.base; a.Flo = B.Flo; a.Rk = B.Rk; a.invD = B.invD; a.lamS = B.lamS;
   a.gb = b->gb; a.err = b->status; a.n_err = static_cast<int>(b->S);
   a.spin_limit = b->sh.spin_limit > 0 ? b->sh.spin_limit : kSpinLimit;
   // a launch that timed out leaves the barrier's arrival count behind: start
@@ -346,52 +352,71 @@ void enqueue_lo_solve(Batch *b) {
   const dim3 gc(nblk(b->N, kCellBlock)), blk(kCellBlock);
   const bool part = b->sh.sweep_order == CGKS_SWEEP_PARTITIONED;
   // colour sweeps: k_lo_rhs relaxes colour 0 of the first pass.  Partitioned:
-  // k_lo_rhs zeroes the increments, the sweeps ping-pong between dU and
-  // dU2 starting so that the last one writes dU
+  // k_lo_rhs zeroes the increments, the sweeps ping-pong between delta and
+  // delta2 starting so that the last one writes delta
   const int colour0 = !part && b->sh.n_sweeps > 0 ? 1 : 0;
-  TF *dU0 = part && (b->sh.n_sweeps & 1) ? B.dU2 : B.dU;
+  const bool adv = last_pass_advances(b);
+  TF *del0 = part && (b->sh.n_sweeps & 1) ? B.delta2 : B.delta;
+  TF *base = B.base, *next = B.base2;
+  auto cells = [&](int first) {
+    launch(b, KI_LOCELL, k_lo_cell<TF>, gc, blk, static_cast<int>(b->Ncap), fparams<TF>(b), first,
+           (const double *)b->Wn, b->U, (const TF *)B.delta, base);
+  };
+  // the last visit of each colour in the sequence
+  std::vector<int> last(b->n_colours, -1);
+  for (size_t q = 0; q < b->sweep_seq.size(); ++q) last[b->sweep_seq[q]] = static_cast<int>(q);
   for (int k = 0; k < b->sh.n_implicit; ++k) {
-    launch(b, KI_LOCELL, k_lo_cell<TF>, gc, blk, static_cast<int>(b->Ncap), fparams<TF>(b), k == 0 ? 1 : 0,
-           (const double *)b->Wn, b->U, (const TF *)B.dU, B.prim, mirror<TF>(B.U));
+    if (k == 0 || !adv) cells(k == 0 ? 1 : 0);
     const int fsh = b->tune.shape(TK_LOFACE);
     tuned_launch(b->tune, TK_LOFACE, b->stream, [&] {
       launch(b, KI_LOFACE, k_lo_face<TF>, dim3(nblk(b->F, shape_bs(fsh))), dim3(shape_bs(fsh)),
-             fmesh<TF>(b), fparams<TF>(b), (const TF *)B.U, (const TF *)B.prim, B.Flo, B.lam, B.E0,
-             B.E1);
+             fmesh<TF>(b), fparams<TF>(b), (const TF *)base, B.Flo);
     });
-    launch(b, KI_LORHS, k_lo_rhs<TF>, gc, blk, b->dm, b->dp, k == 0 ? 1 : 0, colour0, (const TF *)B.Flo,
-           (const TF *)B.lam, (const double *)b->Rp0, b->Src, B.Rk, B.invD, dU0, B.lamS);
+    launch(b, KI_LORHS, k_lo_rhs<TF>, gc, blk, b->dm, b->dp, fparams<TF>(b).gamma, k == 0 ? 1 : 0, colour0,
+           (const TF *)base, (const TF *)B.Flo, (const double *)b->Rp0, b->Src, B.Rk, B.invD, del0, B.lamS);
     if (part) {
-      TF *in = dU0, *out = dU0 == B.dU ? B.dU2 : B.dU;
+      TF *in = del0, *out = del0 == B.delta ? B.delta2 : B.delta;
       for (int sw = 0; sw < b->sh.n_sweeps; ++sw) {
         launch_cluster(b, KI_SWEEP, k_sweep_part<TF>, dim3(b->n_parts * kPartCluster), dim3(kPartBlock),
                        kPartCluster, fmesh<TF>(b), fparams<TF>(b), (const int *)b->ptab, b->n_colours,
-                       (const TF *)B.U, (const TF *)B.prim, (const TF *)B.Rk, (const TF *)B.invD,
-                       (const TF *)B.lamS, (const TF *)B.E0, (const TF *)B.E1, (const TF *)in, out);
+                       (const TF *)base, (const TF *)B.Rk, (const TF *)B.invD, (const TF *)B.lamS, (const TF *)in,
+                       out);
         std::swap(in, out);
       }
       continue;
     }
     const int ssh = b->tune.shape(TK_SWEEP);
-    for (int c : b->sweep_seq) {
+    for (size_t q = 0; q < b->sweep_seq.size(); ++q) {
+      const int c = b->sweep_seq[q];
       const int cnt = b->list_off[c + 1] - b->list_off[c];
       const Ranges &R = b->ranges[ssh][c];
       const bool use_list = R.n == 0;
-      const int grid = use_list ? nblk(cnt, sweep_cpb(ssh)) : R.blk[R.n];
+      const int grid = use_list ? nblk(cnt, shape_bs(ssh) / b->lanes[c]) : R.blk[R.n];
       tuned_launch(b->tune, TK_SWEEP, b->stream, [&] {
-        launch(b, KI_SWEEP, k_sweep<TF>, dim3(grid), dim3(shape_bs(ssh)), fmesh<TF>(b), fparams<TF>(b),
-               R, use_list ? (const int *)b->list + b->list_off[c] : (const int *)nullptr, cnt, (const TF *)B.U,
-               (const TF *)B.prim, (const TF *)B.Rk, (const TF *)B.invD, (const TF *)B.lamS, (const TF *)B.E0,
-               (const TF *)B.E1, B.dU);
+        auto go = [&](auto kern) {
+          launch(b, KI_SWEEP, kern, dim3(grid), dim3(shape_bs(ssh)), fmesh<TF>(b), fparams<TF>(b), R,
+                 use_list ? (const int *)b->list + b->list_off[c] : (const int *)nullptr, cnt, (const TF *)base,
+                 (const TF *)B.Rk, (const TF *)B.invD, (const TF *)B.lamS, B.delta, b->U, next);
+        };
+        const bool end = adv && last[c] == static_cast<int>(q);
+        if constexpr (!is_f32<TF>()) {
+          if (b->lanes[c] == 1) {
+            if (end) go(k_sweep<TF, true, 1>);
+            else go(k_sweep<TF, false, 1>);
+            return;
+          }
+        }
+        if (end) go(k_sweep<TF, true, 4>);
+        else go(k_sweep<TF, false, 4>);
       });
     }
+    if (adv) std::swap(base, next);
   }
   // U^{n_implicit} = U + dU of the last step
-  if (b->sh.n_implicit > 0)
-    launch(b, KI_LOCELL, k_lo_cell<TF>, gc, blk, static_cast<int>(b->Ncap), fparams<TF>(b), 0, (const double *)b->Wn, b->U,
-           (const TF *)B.dU, B.prim, mirror<TF>(B.U));
-  else
+  if (b->sh.n_implicit == 0)
     cudaMemcpyAsync(b->U, b->Wn, sizeof(double) * 4 * b->Ncap, cudaMemcpyDeviceToDevice, b->stream);
+  else if (!adv)
+    cells(0);
 }
 
 template <typename TF>
@@ -444,7 +469,8 @@ long long count_launches(const Batch *b, bool cycle) {
   const long long sweeps = b->sh.sweep_order == CGKS_SWEEP_PARTITIONED
                                ? static_cast<long long>(b->sh.n_sweeps)
                                : static_cast<long long>(b->sweep_seq.size());
-  long long lo = b->lo_fused_ok ? 1 : b->sh.n_implicit * (3 + sweeps) + (b->sh.n_implicit > 0 ? 1 : 0);
+  const long long cells = last_pass_advances(b) ? 1 : b->sh.n_implicit + 1;
+  long long lo = b->lo_fused_ok ? 1 : b->sh.n_implicit > 0 ? b->sh.n_implicit * (2 + sweeps) + cells : 0;
   return dt + hi + per_eval + 1 + lo + 2;
 }
 
@@ -523,11 +549,12 @@ void fill_shared_params(const Shared &sh, ParamsT<T> &P) {
   P.gamma = static_cast<T>(sh.gamma);
   P.K = static_cast<T>(K);
   P.cfl_hi = static_cast<T>(sh.cfl_hi);
-  P.cfl_lo = static_cast<T>(sh.cfl_lo);
+  P.icfl_lo = static_cast<T>(1.0 / sh.cfl_lo);
   P.kc.K = static_cast<T>(K);
   P.kc.c2K = static_cast<T>(2.0 / (K + 2.0));
   P.kc.c4K = static_cast<T>(4.0 / (K + 2.0));
   P.kc.hN = static_cast<T>(0.5 * (K + 2.0));
+  P.kc.sq2g = static_cast<T>(std::sqrt(2.0 * sh.gamma));
   P.flux_lo = sh.flux_lo;
   P.flux_hi = sh.flux_hi;
   P.tau_c1 = static_cast<T>(sh.tau_c1);
@@ -560,7 +587,7 @@ void plan_arena(Batch *b, int64_t N, int64_t F, int S, int64_t L, bool mixed, st
   P8(&b->U, 4 * N); P8(&b->Rp0, 4 * N); P8(&b->Src, 4 * N); P8(&b->stage, 12 * N);
   P8(&b->partial, 2 * std::max<int64_t>(N / kCellBlock, 1)); P8(&b->last, 4); P8(&b->res, S);
   P8(&d.vol, N); P8(&d.ivol, N); P8(&d.per, N); P8(&d.ih, N); P8(&d.m2, 3 * N); P8(&d.op, kNCol * kNM * N);
-  P8(&d.snx, kMaxFace * N); P8(&d.sny, kMaxFace * N); P8(&d.shs, kMaxFace * N);
+  P8(&d.snx, kMaxFace * N); P8(&d.sny, kMaxFace * N);
   P8(&d.fn, 2 * F); P8(&d.fS, F); P8(&d.fjump, F); P8(&d.fxi, 8 * F); P8(&d.fidl, F);
   P8(&d.mu, S); P8(&d.bcuw, 2 * T); P8(&d.bcrho, T); P8(&d.bcu, 2 * T); P8(&d.bcp, T);
   PI(&d.cface, kMaxFace * N); PI(&d.cnbr, kMaxFace * N); PI(&d.fc0, F); PI(&d.fc1, F); PI(&d.csid, N); PI(&d.fsid, F);
@@ -582,16 +609,16 @@ void plan_arena(Batch *b, int64_t N, int64_t F, int S, int64_t L, bool mixed, st
   if (!mixed) {
     Bufs<double> &X = b->bd;
     P8(&X.coef, 20 * N); P8(&X.FA, 16 * F); P8(&X.FB, 16 * F);
-    P8(&X.prim, D::NPRIM * N); P8(&X.Flo, 4 * F); P8(&X.lam, F); P8(&X.E0, 4 * F); P8(&X.E1, 4 * F);
-    P8(&X.Rk, 4 * N); P8(&X.invD, N); P8(&X.dU, 4 * N); P8(&X.lamS, kMaxFace * N);
-    if (b->sh.sweep_order == CGKS_SWEEP_PARTITIONED) P8(&X.dU2, 4 * N);
+    P8(&X.base, kBase * N); P8(&X.base2, kBase * N); P8(&X.Flo, lo_run<double>() * F);
+    P8(&X.Rk, 4 * N); P8(&X.invD, N); P8(&X.delta, del_run<double>() * N); P8(&X.lamS, kMaxFace * N);
+    if (b->sh.sweep_order == CGKS_SWEEP_PARTITIONED) P8(&X.delta2, del_run<double>() * N);
   } else {
     Bufs<float> &X = b->bf;
-    P4(&X.W, 4 * N); P4(&X.Wx, 8 * N); P4(&X.Wn, 4 * N); P4(&X.Ws, 4 * N); P4(&X.Wxs, 8 * N); P4(&X.U, 4 * N);
+    P4(&X.W, 4 * N); P4(&X.Wx, 8 * N); P4(&X.Wn, 4 * N); P4(&X.Ws, 4 * N); P4(&X.Wxs, 8 * N);
     P4(&X.coef, 20 * N); P4(&X.FA, 16 * F); P4(&X.FB, 16 * F);
-    P4(&X.prim, D::NPRIM * N); P4(&X.Flo, 4 * F); P4(&X.lam, F);
-    P4(&X.Rk, 4 * N); P4(&X.invD, N); P4(&X.dU, 4 * N); P4(&X.lamS, kMaxFace * N);
-    if (b->sh.sweep_order == CGKS_SWEEP_PARTITIONED) P4(&X.dU2, 4 * N);
+    P4(&X.base, kBase * N); P4(&X.base2, kBase * N); P4(&X.Flo, lo_run<float>() * F);
+    P4(&X.Rk, 4 * N); P4(&X.invD, N); P4(&X.delta, del_run<float>() * N); P4(&X.lamS, kMaxFace * N);
+    if (b->sh.sweep_order == CGKS_SWEEP_PARTITIONED) P4(&X.delta2, del_run<float>() * N);
     P4(&d.f_ivol, N); P4(&d.f_ih, N); P4(&d.f_m2, 3 * N); P4(&d.f_op, kNCol * kNM * N);
     P4(&d.f_snx, kMaxFace * N); P4(&d.f_sny, kMaxFace * N); P4(&d.f_shs, kMaxFace * N);
     P4(&d.f_fn, 2 * F); P4(&d.f_fS, F); P4(&d.f_fjump, F); P4(&d.f_fxi, 8 * F); P4(&d.f_fidl, F);
@@ -632,16 +659,12 @@ void clear_cells(Batch *b, int64_t c0, int64_t c1) {
       b->mixed ? b->bf.Wn : nullptr, b->mixed ? b->bf.Ws : nullptr, b->mixed ? b->bf.Wxs : nullptr);
   // the second increment buffer of the partitioned sweep is written only at
   // partition cells: clear it (and the first) where cells become inert
-  for (int v = 0; v < 4; ++v) {
-    if (b->bd.dU2) {
-      cudaMemsetAsync(b->bd.dU + v * b->Ncap + c0, 0, sizeof(double) * (c1 - c0), b->stream);
-      cudaMemsetAsync(b->bd.dU2 + v * b->Ncap + c0, 0, sizeof(double) * (c1 - c0), b->stream);
-    }
-    if (b->bf.dU2) {
-      cudaMemsetAsync(b->bf.dU + v * b->Ncap + c0, 0, sizeof(float) * (c1 - c0), b->stream);
-      cudaMemsetAsync(b->bf.dU2 + v * b->Ncap + c0, 0, sizeof(float) * (c1 - c0), b->stream);
-    }
-  }
+  auto clear = [&](auto *p) {
+    constexpr int n = del_run<std::decay_t<decltype(*p)>>();
+    if (p) cudaMemsetAsync(p + n * c0, 0, sizeof(*p) * n * (c1 - c0), b->stream);
+  };
+  if (b->bd.delta2) { clear(b->bd.delta); clear(b->bd.delta2); }
+  if (b->bf.delta2) { clear(b->bf.delta); clear(b->bf.delta2); }
 }
 
 // Allocate a batch with capacity for Ncap cells, Fcap faces and S slots;
@@ -673,7 +696,7 @@ int create_batch(const Shared &sh, int64_t Ncap, int64_t Fcap, int S, cudaStream
   }
   if (!b->mixed) {
     Bufs<double> &X = b->bd;
-    X.W = b->W; X.Wx = b->Wx; X.Wn = b->Wn; X.Ws = b->Ws; X.Wxs = b->Wxs; X.U = b->U;
+    X.W = b->W; X.Wx = b->Wx; X.Wn = b->Wn; X.Ws = b->Ws; X.Wxs = b->Wxs;
   }
   // kernel-side views
   fill_shared_params(sh, b->dp);
@@ -688,7 +711,7 @@ int create_batch(const Shared &sh, int64_t Ncap, int64_t Fcap, int S, cudaStream
   MeshT<double> &dm = b->dm;
   dm.nc = static_cast<int>(Ncap); dm.nf = static_cast<int>(Fcap);
   dm.vol = d.vol; dm.ivol = d.ivol; dm.per = d.per; dm.ih = d.ih; dm.m2 = d.m2; dm.op = d.op;
-  dm.fn = d.fn; dm.fS = d.fS; dm.fjump = d.fjump; dm.fxi = d.fxi; dm.snx = d.snx; dm.sny = d.sny; dm.shs = d.shs;
+  dm.fn = d.fn; dm.fS = d.fS; dm.fjump = d.fjump; dm.fxi = d.fxi; dm.snx = d.snx; dm.sny = d.sny;
   dm.fidl = d.fidl;
   dm.cface = d.cface; dm.cnbr = d.cnbr; dm.fc0 = d.fc0; dm.fc1 = d.fc1; dm.csid = d.csid; dm.fsid = d.fsid;
   dm.ccol = d.ccol; dm.wenok = d.wenok;
@@ -711,10 +734,9 @@ int create_batch(const Shared &sh, int64_t Ncap, int64_t Fcap, int S, cudaStream
             cudaMemsetAsync(b->gb, 0, sizeof(GridBarrier), st) == cudaSuccess &&
             cudaMemsetAsync(b->slim, 0, sizeof(int) * S, st) == cudaSuccess;
   if (ok) {
-    if (b->mixed) ok = cudaMemsetAsync(b->bf.dU, 0, sizeof(float) * 4 * Ncap, st) == cudaSuccess;
-    else ok = cudaMemsetAsync(b->bd.dU, 0, sizeof(double) * 4 * Ncap, st) == cudaSuccess;
-    if (ok && b->bf.dU2) ok = cudaMemsetAsync(b->bf.dU2, 0, sizeof(float) * 4 * Ncap, st) == cudaSuccess;
-    if (ok && b->bd.dU2) ok = cudaMemsetAsync(b->bd.dU2, 0, sizeof(double) * 4 * Ncap, st) == cudaSuccess;
+    const size_t bytes = (b->mixed ? sizeof(float) * del_run<float>() : sizeof(double) * del_run<double>()) * Ncap;
+    for (void *p : { (void *)b->bf.delta, (void *)b->bd.delta, (void *)b->bf.delta2, (void *)b->bd.delta2 })
+      if (ok && p) ok = cudaMemsetAsync(p, 0, bytes, st) == cudaSuccess;
   }
   if (ok) {
     clear_cells(b, 0, Ncap);
@@ -779,6 +801,10 @@ int insert_solve(Batch *b, int s, const Member &m, int64_t cell_off, int64_t fac
       snx[sl * np + i] = sg * hm.fn[f];
       sny[sl * np + i] = sg * hm.fn[nf + f];
       shs[sl * np + i] = 0.5 * hm.fS[f];
+      if (!b->mixed) {   // FP64 sweeps take n S/2
+        snx[sl * np + i] *= shs[sl * np + i];
+        sny[sl * np + i] *= shs[sl * np + i];
+      }
     }
   }
   for (int c = 0; c < hm.n_colours; ++c)
@@ -815,7 +841,7 @@ int insert_solve(Batch *b, int s, const Member &m, int64_t cell_off, int64_t fac
   const int64_t T = kTagsPerSolve;
   up(d.vol, vol, np, N, co); up(d.ivol, ivol, np, N, co); up(d.per, per, np, N, co); up(d.ih, ih, np, N, co);
   up(d.m2, m2, np, N, co); up(d.op, op, np, N, co); up(d.snx, snx, np, N, co); up(d.sny, sny, np, N, co);
-  up(d.shs, shs, np, N, co); up(d.cface, cface, np, N, co); up(d.cnbr, cnbr, np, N, co);
+  up(d.cface, cface, np, N, co); up(d.cnbr, cnbr, np, N, co);
   up(d.csid, csid, np, N, co); up(b->perm, perm, np, N, co); up(d.ccol, ccol, np, N, co);
   up(d.wenok, wenok, np, N, co);
   up(d.fn, fn, nf, F, fo); up(d.fS, fS, nf, F, fo); up(d.fjump, fjump, nf, F, fo); up(d.fxi, fxi, nf, F, fo);
@@ -909,6 +935,15 @@ int finalize_batch(Batch *b) {
   b->sweep_seq = seq;
   for (auto &rs : b->ranges) rs.assign(C, Ranges{});
   b->list_off.assign(C + 1, 0);
+  b->lanes.assign(C, 4);
+  for (int c = 0; c < C; ++c) {
+    int cnt = 0;
+    for (int s : order) {
+      const HostMesh &hm = *b->mem[s].mesh;
+      if (c < hm.n_colours) cnt += hm.colour_start[c + 1] - hm.colour_start[c];
+    }
+    b->lanes[c] = b->mixed ? sweep_lanes<float>(cnt) : sweep_lanes<double>(cnt);
+  }
   std::vector<int> list;
   bool need_list = false;
   for (int c = 0; c < C; ++c) {
@@ -930,7 +965,7 @@ int finalize_batch(Batch *b) {
         R.blk[nr] = blocks;
         R.begin[nr] = beg;
         R.end[nr] = end;
-        blocks += nblk(end - beg, sweep_cpb(sh));
+        blocks += nblk(end - beg, shape_bs(sh) / b->lanes[c]);
         ++nr;
       }
       if (nr >= 0) { R.n = nr; R.blk[nr] = blocks; }

@@ -25,10 +25,10 @@ inline int nblk(int64_t n, int b) { return static_cast<int>((n + b - 1) / b); }
 
 template <typename T>
 struct Bufs3 {
-  T *W = nullptr, *Wx = nullptr, *Wn = nullptr, *Ws = nullptr, *Wxs = nullptr, *U = nullptr;
-  T *coef = nullptr, *FA = nullptr, *FB = nullptr, *rec = nullptr;
-  T *Flo = nullptr;   // [F][kLo]: low-level flux and lambda_p per face
-  T *E0 = nullptr, *E1 = nullptr, *Rk = nullptr, *invD = nullptr, *dU = nullptr, *lamS = nullptr;
+  T *W = nullptr, *Wx = nullptr, *Wn = nullptr, *Ws = nullptr, *Wxs = nullptr;
+  T *coef = nullptr, *FA = nullptr, *FB = nullptr;
+  T *base = nullptr, *base2 = nullptr;   // low level: base records of alternating implicit steps
+  T *Flo = nullptr, *Rk = nullptr, *invD = nullptr, *delta = nullptr, *lamS = nullptr;
 };
 
 struct Geo3 {
@@ -177,35 +177,58 @@ void hi_step(Solver3 *s, double *Wout, TF *Wout_m, bool want_res) {
   if (want_res) enqueue_res(s);
 }
 
+bool last_pass_advances(const Solver3 *s) { return s->P.n_sweeps > 0 && s->n_colours > 1; }
+
 template <typename TF>
 void lo_solve(Solver3 *s) {
   Bufs3<TF> &B = bufs<TF>(s);
   const dim3 gc(nblk(s->N, kCellBlock)), blk(kCellBlock);
   const int colour0_end = s->P.n_sweeps > 0 ? s->colour_start[1] : 0;
+  // the last pass of each colour advances U and writes the next step's base
+  // records; where the passes do not visit every cell, a pass over all does
+  const bool adv = last_pass_advances(s);
+  TF *base = B.base, *next = B.base2;
+  auto cells = [&](int first) {
+    launch(s, KI_LOCELL, k_lo_cell<TF>, gc, blk, static_cast<int>(s->N), fpar<TF>(s), first, (const double *)s->Wn,
+           s->U, (const TF *)B.delta, base);
+  };
+  std::vector<int> last(s->n_colours, -1);
+  for (size_t q = 0; q < s->sweep_seq.size(); ++q) last[s->sweep_seq[q]] = static_cast<int>(q);
   for (int k = 0; k < s->P.n_implicit; ++k) {
-    launch(s, KI_LOCELL, k_lo_cell<TF>, gc, blk, static_cast<int>(s->N), fpar<TF>(s), k == 0 ? 1 : 0,
-           (const double *)s->Wn, s->U, (const TF *)B.dU, B.rec);
+    if (k == 0 || !adv) cells(k == 0 ? 1 : 0);
     const int fs = s->tune.shape(TK_LOFACE), ss = s->tune.shape(TK_SWEEP);
     tuned_launch(s->tune, TK_LOFACE, s->stream, [&] {
       launch(s, KI_LOFACE, k_lo_face<TF>, dim3(nblk(s->F, shape_bs(fs))), dim3(shape_bs(fs)),
-             fmesh<TF>(s), fpar<TF>(s), (const TF *)B.rec, B.Flo, B.E0, B.E1);
+             fmesh<TF>(s), fpar<TF>(s), (const TF *)base, B.Flo);
     });
-    launch(s, KI_LORHS, k_lo_rhs<TF>, gc, blk, s->dm, s->dp, k == 0 ? 1 : 0, colour0_end, (const TF *)B.Flo,
-           (const double *)s->Rp0, s->Src, B.Rk, B.invD, B.dU, B.lamS);
-    for (int c : s->sweep_seq) {
+    launch(s, KI_LORHS, k_lo_rhs<TF>, gc, blk, s->dm, s->dp, fpar<TF>(s).gamma, k == 0 ? 1 : 0, colour0_end,
+           (const TF *)base, (const TF *)B.Flo, (const double *)s->Rp0, s->Src, B.Rk, B.invD, B.delta, B.lamS);
+    for (size_t q = 0; q < s->sweep_seq.size(); ++q) {
+      const int c = s->sweep_seq[q];
       const int beg = s->colour_start[c], cnt = s->colour_start[c + 1] - beg;
       tuned_launch(s->tune, TK_SWEEP, s->stream, [&] {
-        launch(s, KI_SWEEP, k_sweep<TF>, dim3(nblk(cnt, sweep_cpb(ss))), dim3(shape_bs(ss)), fmesh<TF>(s), fpar<TF>(s),
-               beg, cnt, (const TF *)B.rec, (const TF *)B.Rk, (const TF *)B.invD, (const TF *)B.lamS,
-               (const TF *)B.E0, (const TF *)B.E1, B.dU);
+        const int lanes = sweep_lanes<TF>(cnt);
+        auto go = [&](auto kern) {
+          launch(s, KI_SWEEP, kern, dim3(nblk(static_cast<int64_t>(cnt) * lanes, shape_bs(ss))), dim3(shape_bs(ss)),
+                 fmesh<TF>(s), fpar<TF>(s), beg, cnt, (const TF *)base, (const TF *)B.Rk, (const TF *)B.invD,
+                 (const TF *)B.lamS, B.delta, s->U, next);
+        };
+        const bool end = adv && last[c] == static_cast<int>(q);
+        if (lanes == 1) {
+          if (end) go(k_sweep<TF, true, 1>);
+          else go(k_sweep<TF, false, 1>);
+        } else {
+          if (end) go(k_sweep<TF, true, kSweepLanes>);
+          else go(k_sweep<TF, false, kSweepLanes>);
+        }
       });
     }
+    if (adv) std::swap(base, next);
   }
-  if (s->P.n_implicit > 0)
-    launch(s, KI_LOCELL, k_lo_cell<TF>, gc, blk, static_cast<int>(s->N), fpar<TF>(s), 0, (const double *)s->Wn, s->U,
-           (const TF *)B.dU, B.rec);
-  else
+  if (s->P.n_implicit == 0)
     cudaMemcpyAsync(s->U, s->Wn, sizeof(double) * NV * s->N, cudaMemcpyDeviceToDevice, s->stream);
+  else if (!adv)
+    cells(0);
 }
 
 template <typename TF>
@@ -238,7 +261,9 @@ void enqueue_step(Solver3 *s, double dt_fixed) {
 long long count_launches(const Solver3 *s, bool cycle) {
   const long long hi = 3 + (s->P.time_scheme == CGKS_S2O4 ? 3 : 0);
   if (!cycle) return 2 + hi + 1;
-  const long long lo = s->P.n_implicit * (3 + static_cast<long long>(s->sweep_seq.size())) + (s->P.n_implicit > 0);
+  const long long cells = last_pass_advances(s) ? 1 : s->P.n_implicit + 1;
+  const long long lo =
+      s->P.n_implicit > 0 ? s->P.n_implicit * (2 + static_cast<long long>(s->sweep_seq.size())) + cells : 0;
   return 2 + hi + 3 + lo + 2;
 }
 
@@ -284,15 +309,15 @@ void plan(Solver3 *s, std::vector<Piece3> &pc) {
   pc.push_back({ reinterpret_cast<void **>(&s->dt_bits), sizeof(unsigned long long) });
   if (!s->mixed) {
     Bufs3<double> &X = s->bd;
-    P8(&X.coef, kNM3 * NV * N); P8(&X.FA, 4 * NV * F); P8(&X.FB, 4 * NV * F); P8(&X.rec, kRec * N);
-    P8(&X.Flo, kLo * F); P8(&X.E0, kEu * F); P8(&X.E1, kEu * F); P8(&X.Rk, NV * N); P8(&X.invD, N);
-    P8(&X.dU, kDU * N); P8(&X.lamS, kMaxFace3 * N);
+    P8(&X.coef, kNM3 * NV * N); P8(&X.FA, 4 * NV * F); P8(&X.FB, 4 * NV * F);
+    P8(&X.base, kBase * N); P8(&X.base2, kBase * N); P8(&X.Flo, lo_run<double>() * F); P8(&X.Rk, NV * N);
+    P8(&X.invD, N); P8(&X.delta, del_run<double>() * N); P8(&X.lamS, kMaxFace3 * N);
   } else {
     Bufs3<float> &X = s->bf;
     P4(&X.W, NV * N); P4(&X.Wx, 3 * NV * N); P4(&X.Wn, NV * N); P4(&X.Ws, NV * N); P4(&X.Wxs, 3 * NV * N);
     P4(&X.coef, kNM3 * NV * N); P4(&X.FA, 4 * NV * F); P4(&X.FB, 4 * NV * F);
-    P4(&X.rec, kRec * N); P4(&X.Flo, kLo * F); P4(&X.Rk, NV * N); P4(&X.invD, N);
-    P4(&X.dU, kDU * N); P4(&X.lamS, kMaxFace3 * N);
+    P4(&X.base, kBase * N); P4(&X.base2, kBase * N); P4(&X.Flo, lo_run<float>() * F); P4(&X.Rk, NV * N);
+    P4(&X.invD, N); P4(&X.delta, del_run<float>() * N); P4(&X.lamS, kMaxFace3 * N);
     P4(&g.f_ivol, N); P4(&g.f_ih, N); P4(&g.f_m2, 6 * N); P4(&g.f_op, kNCol3 * kNM3 * N); P4(&g.f_fe, 9 * F);
     P4(&g.f_fS, F); P4(&g.f_fjump, F); P4(&g.f_fw, 4 * F); P4(&g.f_fxi, 24 * F); P4(&g.f_fidl, F); P4(&g.f_sn, 3 * kMaxFace3 * N);
     P4(&g.f_shs, kMaxFace3 * N); P4(&g.f_bcuw, 3 * CGKS_MAX_BC); P4(&g.f_bcrho, CGKS_MAX_BC);
@@ -312,12 +337,13 @@ void fill_params(const cgks_params &p, ParamsT<T> &P) {
   P.gamma = static_cast<T>(p.gamma);
   P.K = static_cast<T>(K);
   P.cfl_hi = static_cast<T>(p.cfl_hi);
-  P.cfl_lo = static_cast<T>(p.cfl_lo);
+  P.icfl_lo = static_cast<T>(1.0 / p.cfl_lo);
   P.mu = static_cast<T>(p.mu);
   P.kc.K = static_cast<T>(K);
   P.kc.c2K = static_cast<T>(2.0 / (K + 3.0));
   P.kc.c4K = static_cast<T>(4.0 / (K + 3.0));
   P.kc.hN = static_cast<T>(0.5 * (K + 3.0));
+  P.kc.sq2g = static_cast<T>(std::sqrt(2.0 * p.gamma));
   P.flux_lo = p.flux_lo;
   P.tau_c1 = static_cast<T>(p.tau_c1);
   P.tau_c2 = static_cast<T>(p.tau_c2);
@@ -405,7 +431,7 @@ int s3_create(const HostMesh3 &m, const cgks_params *p, cudaStream_t stream, Tim
   }
   if (!s->mixed) {
     Bufs3<double> &X = s->bd;
-    X.W = s->W; X.Wx = s->Wx; X.Wn = s->Wn; X.Ws = s->Ws; X.Wxs = s->Wxs; X.U = s->U;
+    X.W = s->W; X.Wx = s->Wx; X.Wn = s->Wn; X.Ws = s->Ws; X.Wxs = s->Wxs;
   }
   // ---- host tables
   const int64_t N = s->N, F = s->F;
@@ -414,7 +440,8 @@ int s3_create(const HostMesh3 &m, const cgks_params *p, cudaStream_t stream, Tim
   std::vector<double> op;
   std::vector<unsigned char> wenok;
   build_operator3(m, wall, op, &wenok);
-  std::vector<double> ivol(N), ih(N), hdt(N), fe(9 * F), fjump(F), fidl(F), sn(3 * kMaxFace3 * N, 0.0), shs(kMaxFace3 * N, 0.0);
+  std::vector<double> ivol(N), ih(N), hdt(N), fe(9 * F), fjump(F), fidl(F), sn(3 * kMaxFace3 * N, 0.0), sns(3 * kMaxFace3 * N, 0.0),
+      shs(kMaxFace3 * N, 0.0);   // sn: normal (FP32), sns: times S/2 (FP64)
   for (int64_t i = 0; i < N; ++i) {
     ivol[i] = 1.0 / m.vol[i];
     ih[i] = 1.0 / m.h[i];
@@ -441,8 +468,12 @@ int s3_create(const HostMesh3 &m, const cgks_params *p, cudaStream_t stream, Tim
       if (fs == kNoFace) continue;
       const int32_t f = fs >= 0 ? fs : ~fs;
       const double sg = fs >= 0 ? 1.0 : -1.0;
-      for (int d = 0; d < 3; ++d) sn[(3 * sl + d) * N + i] = sg * m.fn[d * F + f];
       shs[sl * N + i] = 0.5 * m.fS[f];
+      for (int d = 0; d < 3; ++d) {
+        const int64_t at = (3 * sl + d) * N + i;
+        sn[at] = sg * m.fn[d * F + f];
+        sns[at] = sn[at] * shs[sl * N + i];
+      }
     }
   std::vector<double> bcuw(3 * CGKS_MAX_BC, 0.0), bcrho(CGKS_MAX_BC, 1.0), bcu(3 * CGKS_MAX_BC, 0.0),
       bcp(CGKS_MAX_BC, 1.0);
@@ -464,7 +495,7 @@ int s3_create(const HostMesh3 &m, const cgks_params *p, cudaStream_t stream, Tim
   up(g.hdt, hdt.data(), 8 * N); up(g.m2, m.m2.data(), 8 * 6 * N); up(g.op, op.data(), 8 * op.size());
   up(g.fe, fe.data(), 8 * fe.size()); up(g.fS, m.fS.data(), 8 * F); up(g.fjump, fjump.data(), 8 * F);
   up(g.fidl, fidl.data(), 8 * F);
-  up(g.fw, m.fw.data(), 8 * 4 * F); up(g.fxi, m.fxi.data(), 8 * 24 * F); up(g.sn, sn.data(), 8 * sn.size());
+  up(g.fw, m.fw.data(), 8 * 4 * F); up(g.fxi, m.fxi.data(), 8 * 24 * F); up(g.sn, sns.data(), 8 * sns.size());
   up(g.shs, shs.data(), 8 * shs.size()); up(g.bcuw, bcuw.data(), 8 * bcuw.size());
   up(g.bcrho, bcrho.data(), 8 * bcrho.size()); up(g.bcu, bcu.data(), 8 * bcu.size());
   up(g.bcp, bcp.data(), 8 * bcp.size()); up(g.fng, m.fng.data(), 4 * F); up(g.cface, m.cface.data(), 4 * kMaxFace3 * N);
@@ -485,8 +516,9 @@ int s3_create(const HostMesh3 &m, const cgks_params *p, cudaStream_t stream, Tim
                cudaMemsetAsync(s->status, 0, sizeof(int), stream) == cudaSuccess &&
                cudaMemsetAsync(s->Rp0, 0, sizeof(double) * NV * N, stream) == cudaSuccess &&
                cudaMemsetAsync(s->last, 0, sizeof(double) * 4, stream) == cudaSuccess &&
-               (s->mixed ? cudaMemsetAsync(s->bf.dU, 0, sizeof(float) * kDU * N, stream)
-                         : cudaMemsetAsync(s->bd.dU, 0, sizeof(double) * kDU * N, stream)) == cudaSuccess;
+               (s->mixed ? cudaMemsetAsync(s->bf.delta, 0, sizeof(float) * del_run<float>() * N, stream)
+                         : cudaMemsetAsync(s->bd.delta, 0, sizeof(double) * del_run<double>() * N, stream)) ==
+                   cudaSuccess;
   ok = ok && cudaStreamSynchronize(stream) == cudaSuccess;
   if (!ok) { s3_destroy(S.release()); return CGKS_ECUDA; }
   fill_params(*p, s->dp);

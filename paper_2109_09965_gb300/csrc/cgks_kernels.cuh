@@ -25,6 +25,7 @@
 #include "cgks_physics.cuh"
 #include "cgks_pdl.cuh"
 #include "cgks_shapes.h"
+#include "cgks_vec.cuh"
 
 namespace cgks {
 namespace kern {
@@ -41,7 +42,7 @@ __host__ __device__ constexpr bool is_f32() { return std::is_same<T, float>::val
 // Shared model constants and pointers to per-solve / per-tag tables.
 template <typename T>
 struct ParamsT {
-  T gamma, K, cfl_hi, cfl_lo;
+  T gamma, K, cfl_hi, icfl_lo;   // icfl_lo = 1 / CFL of the low-order level
   D::KC<T> kc;
   const T *mu;                   // [S] dynamic viscosity per solve
   const int *bc_kind;            // [16 S] boundary kind per global tag
@@ -67,7 +68,7 @@ struct MeshT {
   const T *op;                               // [kNCol*kNM][nc]
   const T *fn, *fS, *fjump, *fxi;            // fn [2][nf], fjump = alpha/delta, fxi [8][nf]
   const T *fidl;                             // 1/delta: the centre distance along n (boundary: twice to the face)
-  const T *snx, *sny, *shs;                  // [4][nc] per face slot: outward normal of the cell, S/2
+  const T *snx, *sny, *shs;                  // [4][nc] per face slot: outward normal of the cell (FP64: times S/2), S/2 (FP32)
   const int *cface, *cnbr;                   // [4][nc]
   const int *fc0, *fc1;
   const int *csid, *fsid;                    // solve of each cell (-1: padding) and face
@@ -127,7 +128,7 @@ __global__ void k_reset_dt(Ctl *ctl, unsigned long long *dt_bits, int S, double 
 // (min is order independent).  h = 2|Omega|/perimeter, speed |U| + c + 2 nu / h.
 // Solves are padded to whole blocks, so a block never spans two solves and
 // its first cell is a real one: one atomic per block.
-__global__ void __launch_bounds__(kCellBlock) k_dt(MeshT<double> m, ParamsT<double> P, const double *__restrict__ W,
+__global__ void __launch_bounds__(kCellBlock) k_dt(MeshT<double> m, ParamsT<double> P, const double *W,
                                                    unsigned long long *dt_bits) {
   pdl_enter();
   __shared__ double wmin[kCellBlock / 32];
@@ -313,9 +314,9 @@ __device__ __forceinline__ void recon_at(const MeshT<T> &m, const ParamsT<T> &P,
 }
 template <typename T, bool WENO>
 __global__ void __launch_bounds__(kMaxShapeBlock) k_recon(MeshT<T> m, ParamsT<T> P,
-                                                                        const T *__restrict__ W,
-                                                                        const T *__restrict__ Wx,
-                                                                        T *__restrict__ coef) {
+                                                                        const T *W,
+                                                                        const T *Wx,
+                                                                        T *coef) {
   pdl_enter();
   for_items(m.nc, [&](int i) {
     if (P.slim) {
@@ -668,9 +669,9 @@ __device__ __forceinline__ void face_smooth_at(const MeshT<double> &m, const Par
 // threads a face takes
 template <typename T, bool FULL> __host__ __device__ constexpr int face_threads() { return FULL || is_f32<T>() ? 1 : 2; }
 template <typename T, bool FULL, bool CHAR>
-__global__ void __launch_bounds__(kMaxShapeBlock) k_face(MeshT<T> m, ParamsT<T> P, const T *__restrict__ W,
-                                                         const T *__restrict__ Wx, const T *__restrict__ coef,
-                                                         T *__restrict__ out, const Ctl *ctl,
+__global__ void __launch_bounds__(kMaxShapeBlock) k_face(MeshT<T> m, ParamsT<T> P, const T *W,
+                                                         const T *Wx, const T *coef,
+                                                         T *out, const Ctl *ctl,
                                                          const unsigned long long *dt_bits) {
   pdl_enter();
   if constexpr (face_threads<T, FULL>() == 2)
@@ -691,12 +692,12 @@ enum UpdMode { kS1O2 = 0, kS2O4Stage = 1, kS2O4Final = 2, kResidual = 3 };
 // per-block density-residual partial sums; plus the state check.
 template <typename TF>
 __global__ void __launch_bounds__(kCellBlock) k_update(MeshT<double> m, ParamsT<double> P, int mode,
-                                                       const double *__restrict__ Wbase, const TF *__restrict__ FA,
-                                                       const TF *__restrict__ FB, const Ctl *ctl,
+                                                       const double *Wbase, const TF *FA,
+                                                       const TF *FB, const Ctl *ctl,
                                                        const unsigned long long *dt_bits, int *status,
-                                                       double *__restrict__ Wout, double *__restrict__ Wxout,
-                                                       double *__restrict__ partial, double *__restrict__ Rout,
-                                                       TF *__restrict__ Wout_m, TF *__restrict__ Wxout_m) {
+                                                       double *Wout, double *Wxout,
+                                                       double *partial, double *Rout,
+                                                       TF *Wout_m, TF *Wxout_m) {
   pdl_enter();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int n = m.nc, nf = m.nf;
@@ -735,6 +736,7 @@ __global__ void __launch_bounds__(kCellBlock) k_update(MeshT<double> m, ParamsT<
       for (int v = 0; v < 4; ++v) Rout[v * n + i] = R[v];
     if (mode != kResidual) {
       double iv = m.ivol[i];
+      const double old = Wbase[i];   // Wout may be Wbase (explicit steps update in place)
       double w[4];
       for (int v = 0; v < 4; ++v) {
         w[v] = Wbase[v * n + i] + dt / m.vol[i] * R[v];
@@ -748,8 +750,8 @@ __global__ void __launch_bounds__(kCellBlock) k_update(MeshT<double> m, ParamsT<
         }
       }
       if (!state_ok(P.gamma, w)) atomicOr(&status[sid], kBadState);
-      num = fabs(w[0] - Wbase[i]);
-      den = Wbase[i];
+      num = fabs(w[0] - old);
+      den = old;
     }
   }
   if (partial) block_sum2(num, den, &partial[2 * blockIdx.x]);
@@ -759,8 +761,8 @@ __global__ void __launch_bounds__(kCellBlock) k_update(MeshT<double> m, ParamsT<
 // Sum each solve's block partials in a fixed order (one block per solve
 // slot; blk[2s], blk[2s+1] its cell blocks): Res_s = num / den.  Slot 0
 // also appends to the residual history.
-__global__ void k_res_final(const double *__restrict__ partial, const int *__restrict__ blk, Ctl *ctl,
-                            double *__restrict__ res, double *hist, int cap, double *last) {
+__global__ void k_res_final(const double *partial, const int *__restrict__ blk, Ctl *ctl,
+                            double *res, double *hist, int cap, double *last) {
   pdl_enter();
   const int s = blockIdx.x;
   double a = 0.0, b = 0.0;
@@ -785,42 +787,108 @@ __global__ void k_res_final(const double *__restrict__ partial, const int *__res
 }
 
 // ---------------------------- low-order level ----------------------------
-// K5a: per-cell start of an implicit step: U = W_p0 (first step) or
-// U += dU (Algorithm 1's update, in FP64), then the primitives of U (and
-// its float mirror in mixed mode).
+// Records of the low level, one run of values per cell or face, so that a
+// neighbour's data costs whole sectors:
+//   base  [kBase] per cell, the state U at the start of an implicit step, the
+//         part a sweep reads first: in FP64 rho, u, v, H = rho E + p; p,
+//         1/(2 lambda), sqrt(lambda), 1/sqrt(pi lambda), c, rho u, rho v, rho E;
+//         in FP32 rho, rho u, rho v, rho E, u, v, p, 0; 1/(2 lambda),
+//         sqrt(lambda), 1/sqrt(pi lambda), c;
+//   delta [del_run] per cell, its increment dU; in FP64 then du, dv and dp,
+//         the exact changes of velocity and pressure it makes, 0;
+//   Flo   [lo_run] per face: the flux, lambda_p, padding.
+// The device functions serve the per-phase kernels and the persistent
+// launch; CG reads what other blocks of a launch wrote through L2.
+constexpr int kBase = 12;
+template <typename T> __host__ __device__ constexpr int del_run() { return is_f32<T>() ? 4 : 8; }
+template <typename T> __host__ __device__ constexpr int lo_run() { return is_f32<T>() ? 8 : 6; }
+
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
+// positions in a base record
+template <typename T>
+struct BaseAt {
+  static constexpr bool f = is_f32<T>();
+  static constexpr int m = f ? 1 : 9, E = f ? 3 : 11, u = f ? 4 : 1, p = f ? 6 : 4, i2l = f ? 8 : 5, sl = f ? 9 : 6,
+                       isp = f ? 10 : 7, c = f ? 11 : 8;
+};
+template <typename T>
+__device__ __forceinline__ D::Prim<T> base_prim(const T r[kBase]) {
+  using A = BaseAt<T>;
+  D::Prim<T> q;
+  q.rho = r[0]; q.u = r[A::u]; q.v = r[A::u + 1]; q.p = r[A::p];
+  q.i2l = r[A::i2l]; q.sl = r[A::sl]; q.isp = r[A::isp]; q.c = r[A::c];
+  return q;
+}
+// base record of the FP64 state u
 template <typename TF>
-__global__ void __launch_bounds__(kCellBlock) k_lo_cell(int n, ParamsT<TF> P, int first, const double *__restrict__ Wp0,
-                                                        double *__restrict__ U, const TF *__restrict__ dU,
-                                                        TF *__restrict__ prim, TF *__restrict__ Um) {
-  pdl_enter();
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  TF w[4];
+__device__ __forceinline__ void base_record(const ParamsT<TF> &P, const double u[4], TF r[kBase]) {
+  using A = BaseAt<TF>;
+  const TF w[4] = { static_cast<TF>(u[0]), static_cast<TF>(u[1]), static_cast<TF>(u[2]), static_cast<TF>(u[3]) };
+  const D::Prim<TF> q = D::prim_of(w, P.gamma, P.kc);
+  if constexpr (is_f32<TF>()) r[7] = TF(0);
+  else r[3] = w[3] + q.p;
+  r[0] = w[0];
+  r[A::m] = w[1]; r[A::m + 1] = w[2]; r[A::E] = w[3];
+  r[A::u] = q.u; r[A::u + 1] = q.v; r[A::p] = q.p;
+  r[A::i2l] = q.i2l; r[A::sl] = q.sl; r[A::isp] = q.isp; r[A::c] = q.c;
+}
+// The delta record of an increment d on a cell with base (rho, u, v, H).  FP64:
+//   du = (dm - u d rho) / (rho + d rho),
+//   dp = (gamma - 1)(dE - d(|m|^2 / 2 rho)), d(m.u) = dm.(u + du) + rho u.du,
+// every term proportional to the increment (no cancellation between two
+// nearly equal states), with one reciprocal per relaxed cell.
+// (Fused multiply-adds are written out: the sweep's two forms below must round
+// alike.)
+__device__ __forceinline__ void delta_record(double gamma, const double b[4], const double d[4], double r[8]) {
+  const double ir = D::d_rcp(b[0] + d[0]);
+  const double du = fma(-b[1], d[0], d[1]) * ir, dv = fma(-b[2], d[0], d[2]) * ir;
+  const double k1 = fma(d[2], b[2] + dv, __dmul_rn(d[1], b[1] + du));
+  const double dk = fma(b[0], fma(b[2], dv, __dmul_rn(b[1], du)), k1);
+  const double g1 = gamma - 1.0;
+  r[0] = d[0]; r[1] = d[1]; r[2] = d[2]; r[3] = d[3];
+  r[4] = du; r[5] = dv; r[6] = fma(g1, d[3], __dmul_rn(-0.5 * g1, dk)); r[7] = 0.0;
+}
+__device__ __forceinline__ void store_delta(double gamma, const double b[4], const double d[4], double *delta, int i) {
+  double r[8];
+  delta_record(gamma, b, d, r);
+  vstore<double, 8>(delta + static_cast<size_t>(i) * 8, r);
+}
+__device__ __forceinline__ void store_delta(float, const float *, const float d[4], float *delta, int i) {
+  vstore<float, 4>(delta + static_cast<size_t>(i) * 4, d);
+}
+
+// K5a: per-cell start of an implicit step: U = W_p0 (first step) or
+// U += dU (Algorithm 1's update, in FP64), then the base record of U.
+template <typename TF, bool CG>
+__device__ __forceinline__ void lo_cell_at(int n, const ParamsT<TF> &P, int first, const double *__restrict__ Wp0,
+                                           double *U, const TF *delta, TF *base, int i) {
+  TF d[4] = { TF(0), TF(0), TF(0), TF(0) };
+  if (!first) vload<TF, 4, CG>(delta + static_cast<size_t>(i) * del_run<TF>(), d);
+  double u[4];
+#pragma unroll
   for (int v = 0; v < 4; ++v) {
-    double u = first ? Wp0[v * n + i] : U[v * n + i] + static_cast<double>(dU[v * n + i]);
-    U[v * n + i] = u;
-    w[v] = static_cast<TF>(u);
-    if (Um) Um[v * n + i] = w[v];
+    u[v] = first ? Wp0[v * n + i] : ld<CG>(&U[v * n + i]) + static_cast<double>(d[v]);
+    U[v * n + i] = u[v];
   }
-  D::Prim<TF> q = D::prim_of(w, P.gamma, P.kc);
-  prim[0 * n + i] = q.rho; prim[1 * n + i] = q.u; prim[2 * n + i] = q.v; prim[3 * n + i] = q.p;
-  prim[4 * n + i] = q.i2l; prim[5 * n + i] = q.sl; prim[6 * n + i] = q.isp; prim[7 * n + i] = q.c;
-  prim[8 * n + i] = q.ir;
+  TF r[kBase];
+  base_record(P, u, r);
+  vstore<TF, kBase>(base + static_cast<size_t>(i) * kBase, r);
+}
+template <typename TF>
+__global__ void __launch_bounds__(kCellBlock) k_lo_cell(int n, ParamsT<TF> P, int first, const double *Wp0,
+                                                        double *U, const TF *delta,
+                                                        TF *base) {
+  pdl_enter();
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  lo_cell_at<TF, false>(n, P, first, Wp0, U, delta, base, i);
   pdl_exit();
 }
 
-template <typename T>
-__device__ __forceinline__ D::Prim<T> load_prim(const T *__restrict__ prim, int n, int i) {
-  D::Prim<T> q;
-  q.rho = prim[0 * n + i]; q.u = prim[1 * n + i]; q.v = prim[2 * n + i]; q.p = prim[3 * n + i];
-  q.i2l = prim[4 * n + i]; q.sl = prim[5 * n + i]; q.isp = prim[6 * n + i]; q.c = prim[7 * n + i];
-  q.ir = prim[8 * n + i];
-  return q;
-}
-
-// K5b: first-order KFVS flux, spectral radius lambda_p = max of both sides,
-// and (FP64 mode) the Euler normal fluxes F_n(U_c0), F_n(U_c1) the
-// relaxation reuses.
+// K5b: first-order KFVS (or Lax-Friedrichs) flux and the spectral radius
+// lambda_p = max of both sides.
 template <typename T>
 struct LoFaceGeo {
   int sid, c0, c1;
@@ -839,51 +907,53 @@ __device__ __forceinline__ LoFaceGeo<T> lo_face_geo(const MeshT<T> &m, const Par
   g.c1 = m.fc1[f];
   g.nx = m.fn[f];
   g.ny = m.fn[nf + f];
-  g.S = m.fS[f];
   g.mu = P.mu[g.sid];
-  g.iva = m.ivol[g.c0];
-  g.ivb = g.c1 >= 0 ? m.ivol[g.c1] : g.iva;
+  if (g.mu != T(0)) {   // the viscous part of lambda_p
+    g.S = m.fS[f];
+    g.iva = m.ivol[g.c0];
+    g.ivb = g.c1 >= 0 ? m.ivol[g.c1] : g.iva;
+  }
   return g;
 }
-template <typename T>
+template <typename T, bool CG>
 __device__ __forceinline__ void lo_face_at(const MeshT<T> &m, const ParamsT<T> &P, const LoFaceGeo<T> &g,
-                                           const T *__restrict__ U, const T *__restrict__ prim,
-                                           T *__restrict__ Flo, T *__restrict__ lam, T *__restrict__ E0,
-                                           T *__restrict__ E1, const int f) {
+                                           const T *base, T *__restrict__ Flo, const int f) {
   if (g.sid < 0) return;   // free face space of a batch
-  const int n = m.nc, nf = m.nf;
-  const int c0 = g.c0, c1 = g.c1;
-  const T nx = g.nx, ny = g.ny, S = g.S;
-  const T mu = g.mu;
-  D::Prim<T> a = load_prim(prim, n, c0), b;
-  const T ivb = g.ivb;
-  T wa[4], wb[4];   // states of the two sides (global frame); wb is the ghost on a boundary
-  const bool need_w = P.flux_lo == CGKS_FLUX_LF || E0 != nullptr;
+  const int c1 = g.c1;
+  const T nx = g.nx, ny = g.ny, mu = g.mu;
+  T ra[kBase], rb[kBase];
+  vload<T, kBase, CG>(base + static_cast<size_t>(g.c0) * kBase, ra);
+  const D::Prim<T> a = base_prim(ra);
+  D::Prim<T> b;
+  using A = BaseAt<T>;
+  const T wa[4] = { ra[0], ra[A::m], ra[A::m + 1], ra[A::E] };   // states of the two sides (global frame)
+  T wb[4];                                                       // the ghost on a boundary
   if (c1 >= 0) {
-    b = load_prim(prim, n, c1);
-    if (need_w)
-      for (int v = 0; v < 4; ++v) { wa[v] = U[v * n + c0]; wb[v] = U[v * n + c1]; }
+    vload<T, kBase, CG>(base + static_cast<size_t>(c1) * kBase, rb);
+    b = base_prim(rb);
+    wb[0] = rb[0]; wb[1] = rb[A::m]; wb[2] = rb[A::m + 1]; wb[3] = rb[A::E];
   } else {
-    for (int v = 0; v < 4; ++v) wa[v] = U[v * n + c0];
     lo_ghost(P, -1 - c1, nx, ny, wa, wb);
     b = D::prim_of(wb, P.gamma, P.kc);
   }
   const T una = a.u * nx + a.v * ny, uta = -a.u * ny + a.v * nx;
   const T unb = b.u * nx + b.v * ny, utb = -b.u * ny + b.v * nx;
-  const T la = fabs(una) + a.c + T(2) * (mu * a.ir) * S * g.iva;
-  const T lb = fabs(unb) + b.c + T(2) * (mu * b.ir) * S * ivb;
-  const T lmax = la > lb ? la : lb;
-  lam[f] = lmax;
-  // Euler normal fluxes of the two sides (the L-F flux, the FP64 cache)
-  T Fa[4], Fb[4];
-  if (need_w) {
-    Fa[0] = a.rho * una; Fa[1] = wa[1] * una + a.p * nx; Fa[2] = wa[2] * una + a.p * ny; Fa[3] = (wa[3] + a.p) * una;
-    Fb[0] = b.rho * unb; Fb[1] = wb[1] * unb + b.p * nx; Fb[2] = wb[2] * unb + b.p * ny; Fb[3] = (wb[3] + b.p) * unb;
+  T la = fabs(una) + a.c, lb = fabs(unb) + b.c, ira = T(0), irb = T(0);
+  if (mu != T(0)) {
+    ira = D::d_rcp(a.rho);
+    irb = D::d_rcp(b.rho);
+    la += T(2) * (mu * ira) * g.S * g.iva;
+    lb += T(2) * (mu * irb) * g.S * g.ivb;
   }
+  const T lmax = la > lb ? la : lb;
   T F[4];
   if (P.flux_lo == CGKS_FLUX_LF) {
     // Lax-Friedrichs alternative of Section 3 with the implicit operator's
     // lambda_p: (F_n(U_l) + F_n(U_r)) / 2 - lambda_p (U_r - U_l) / 2
+    // (products rounded by themselves: the mixed path's FP32 results stay what they are)
+    const T Fa[4] = { mul_rn(a.rho, una), wa[1] * una + a.p * nx, wa[2] * una + a.p * ny, mul_rn(wa[3] + a.p, una) };
+    const T Fb[4] = { mul_rn(b.rho, unb), wb[1] * unb + b.p * nx, wb[2] * unb + b.p * ny, mul_rn(wb[3] + b.p, unb) };
+#pragma unroll
     for (int v = 0; v < 4; ++v) F[v] = T(0.5) * (Fa[v] + Fb[v]) - T(0.5) * lmax * (wb[v] - wa[v]);
   } else {
     T Fl[4];
@@ -898,78 +968,106 @@ __device__ __forceinline__ void lo_face_at(const MeshT<T> &m, const ParamsT<T> &
     const T dux = b.u - a.u, duy = b.v - a.v;
     const T dn = (dux * nx + duy * ny) / T(3);
     const T tx = md * (dux + dn * nx), ty = md * (duy + dn * ny);
-    const T qn = -md * P.gamma / (P.gamma - T(1)) * (b.p * b.ir - a.p * a.ir);
+    const T qn = -md * P.gamma / (P.gamma - T(1)) * (b.p * irb - a.p * ira);
     F[1] -= tx;
     F[2] -= ty;
     F[3] -= tx * (T(0.5) * (a.u + b.u)) + ty * (T(0.5) * (a.v + b.v)) - qn;
   }
-  for (int v = 0; v < 4; ++v) Flo[v * nf + f] = F[v];
-  if (E0) {
-    // Euler normal flux of the cell means (interior faces: both sides)
-    for (int v = 0; v < 4; ++v) E0[v * nf + f] = Fa[v];
-    if (c1 >= 0)
-      for (int v = 0; v < 4; ++v) E1[v * nf + f] = Fb[v];
-  }
+  constexpr int N = lo_run<T>();
+  T o[N];
+#pragma unroll
+  for (int v = 0; v < 4; ++v) o[v] = F[v];
+  o[4] = lmax;
+#pragma unroll
+  for (int v = 5; v < N; ++v) o[v] = T(0);
+  vstore<T, N>(Flo + static_cast<size_t>(f) * N, o);
 }
 template <typename T>
-__global__ void __launch_bounds__(kMaxShapeBlock) k_lo_face(MeshT<T> m, ParamsT<T> P,
-                                                                          const T *__restrict__ U,
-                                                                          const T *__restrict__ prim,
-                                                                          T *__restrict__ Flo, T *__restrict__ lam,
-                                                                          T *__restrict__ E0, T *__restrict__ E1) {
+__global__ void __launch_bounds__(kMaxShapeBlock) k_lo_face(MeshT<T> m, ParamsT<T> P, const T *base, T *Flo) {
   for_items_pdl(m.nf, [&](int f) { return lo_face_geo(m, P, f); },
-                    [&](int f, const LoFaceGeo<T> &g) { lo_face_at(m, P, g, U, prim, Flo, lam, E0, E1, f); });
+                [&](int f, const LoFaceGeo<T> &g) { lo_face_at<T, false>(m, P, g, base, Flo, f); });
   pdl_exit();
 }
 
 // K6: low-order right-hand side R^k = R_lo(U^k) + S (FP64 sums), 1/D_i
-// (FP64 inversion), each slot's lambda for the sweeps, and the first colour
-// pass of the relaxation: with dU = 0 everywhere the update of a colour-0
-// cell reduces to R_i / D_i; all other cells start at 0.  first: also
-// forms the forcing S = R_p0 - R_lo(W_p0) (Section 3, step 3).
-template <typename TF>
-__global__ void __launch_bounds__(kCellBlock) k_lo_rhs(MeshT<double> m, ParamsT<double> P, int first, int colour0,
-                                                       const TF *__restrict__ Flo, const TF *__restrict__ lam,
-                                                       const double *__restrict__ Rp0, double *__restrict__ Src,
-                                                       TF *__restrict__ Rk, TF *__restrict__ invD, TF *__restrict__ dU,
-                                                       TF *__restrict__ lamS) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= m.nc) { pdl_enter(); return; }
-  const int n = m.nc, nf = m.nf;
-  // mesh data first (nothing in a cycle writes it), then wait for the predecessor
-  int fsl[kMaxFace];
-  double Sl[kMaxFace];
+// (FP64), each slot's lambda for the sweeps (in FP64 times S/2), and the first colour pass
+// of the relaxation: with dU = 0 everywhere the update of a colour-0 cell
+// reduces to R_i / D_i; all other cells start at 0.  first: also forms the
+// forcing S = R_p0 - R_lo(W_p0) (Section 3, step 3).
+struct RhsGeo {
+  int fs[kMaxFace];
+  double S[kMaxFace];
+  bool c0;
+};
+__device__ __forceinline__ RhsGeo rhs_geo(const MeshT<double> &m, int i, int colour0) {
+  RhsGeo g;
 #pragma unroll
   for (int s = 0; s < kMaxFace; ++s) {
-    fsl[s] = m.cface[s * n + i];
-    Sl[s] = fsl[s] == kNoFace ? 0.0 : m.fS[fsl[s] >= 0 ? fsl[s] : ~fsl[s]];
+    g.fs[s] = m.cface[s * m.nc + i];
+    g.S[s] = g.fs[s] == kNoFace ? 0.0 : m.fS[g.fs[s] >= 0 ? g.fs[s] : ~g.fs[s]];
   }
-  const bool c0 = colour0 && m.ccol[i] == 0;
-  pdl_enter();
+  g.c0 = colour0 && m.ccol[i] == 0;
+  return g;
+}
+template <typename TF, bool CG>
+__device__ __forceinline__ void lo_rhs_at(const MeshT<double> &m, const ParamsT<double> &P, TF gamma, const RhsGeo &g,
+                                          int first, const TF *base, const TF *Flo, const double *__restrict__ Rp0,
+                                          double *Src, TF *Rk, TF *invD, TF *delta, TF *lamS, int i) {
+  const int n = m.nc;
+  constexpr int N = lo_run<TF>();
   double R[4] = { 0, 0, 0, 0 }, sum = 0.0;
 #pragma unroll
   for (int s = 0; s < kMaxFace; ++s) {
-    int fs = fsl[s];
+    const int fs = g.fs[s];
     if (fs == kNoFace) { lamS[s * n + i] = TF(0); continue; }
-    int f = fs >= 0 ? fs : ~fs;
-    double sg = fs >= 0 ? 1.0 : -1.0;
-    double S = Sl[s];
-    for (int v = 0; v < 4; ++v) R[v] -= sg * S * static_cast<double>(Flo[v * nf + f]);
-    TF l = lam[f];
-    lamS[s * n + i] = l;
-    sum += static_cast<double>(l) * S;
+    const double S = g.S[s], Sg = fs >= 0 ? -S : S;
+    TF fl[N];
+    double x[N];
+    vload<TF, N, CG>(Flo + static_cast<size_t>(fs >= 0 ? fs : ~fs) * N, fl);
+    widen<5>(fl, x);
+#pragma unroll
+    for (int v = 0; v < 4; ++v) R[v] += Sg * x[v];
+    sum += x[4] * S;
+    if constexpr (is_f32<TF>()) lamS[s * n + i] = fl[4];
+    else lamS[s * n + i] = fl[4] * (0.5 * S);
   }
   // dt_i = CFL_lo |Omega| / sum;  D_i = |Omega| / dt_i + sum / 2 (padding cells: 0)
-  const double id = sum > 0.0 ? 1.0 / (sum / P.cfl_lo + 0.5 * sum) : 0.0;
+  const double id = sum > 0.0 ? D::d_rcp(sum * (P.icfl_lo + 0.5)) : 0.0;
   invD[i] = static_cast<TF>(id);
+  TF d[4];
+#pragma unroll
   for (int v = 0; v < 4; ++v) {
     double src;
     if (first) { src = Rp0[v * n + i] - R[v]; Src[v * n + i] = src; }
-    else src = Src[v * n + i];
-    double r = R[v] + src;
+    else src = ld<CG>(&Src[v * n + i]);
+    const double r = R[v] + src;
     Rk[v * n + i] = static_cast<TF>(r);
-    dU[v * n + i] = c0 ? static_cast<TF>(r * id) : TF(0);
+    d[v] = static_cast<TF>(r * id);
   }
+  if (g.c0) {
+    TF b[4];
+    vload<TF, 4, CG>(base + static_cast<size_t>(i) * kBase, b);
+    store_delta(gamma, b, d, delta, i);
+  } else {
+    TF z[del_run<TF>()];
+#pragma unroll
+    for (int v = 0; v < del_run<TF>(); ++v) z[v] = TF(0);
+    vstore<TF, del_run<TF>()>(delta + static_cast<size_t>(i) * del_run<TF>(), z);
+  }
+}
+template <typename TF>
+__global__ void __launch_bounds__(kCellBlock) k_lo_rhs(MeshT<double> m, ParamsT<double> P, TF gamma, int first,
+                                                       int colour0, const TF *base,
+                                                       const TF *Flo, const double *Rp0,
+                                                       double *Src, TF *Rk,
+                                                       TF *invD, TF *delta,
+                                                       TF *lamS) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= m.nc) { pdl_enter(); return; }
+  // mesh data first (nothing in a cycle writes it), then wait for the predecessor
+  const RhsGeo g = rhs_geo(m, i, colour0);
+  pdl_enter();
+  lo_rhs_at<TF, false>(m, P, gamma, g, first, base, Flo, Rp0, Src, Rk, invD, delta, lamS, i);
   pdl_exit();
 }
 
@@ -1003,113 +1101,132 @@ __device__ __forceinline__ int range_cell(const Ranges &R, int cl, int cpb) {
 // spanning every solve of the batch), Eq. (implicit-local):
 //   dU_i = (R_i - sum_p S_p [F^-(U_ip + dU_ip) - F^-(U_ip)]) / D_i,
 //   F^-(U) = (F_n(U) - lambda_p U) / 2, ghost increments zero.
-// FP64: F_n(U_ip) from the face cache of this implicit step.  Mixed: the
-// difference F_n(U_ip + dU_ip) - F_n(U_ip) in the exact increment form.
-// Four lanes per cell, one per face slot: each lane evaluates its
-// neighbour's term, the four terms are summed by shuffles within the lane
-// group, and lane v writes component v.  Cells of one colour never
-// neighbour each other, so the dU_ip read here are not written by this
-// launch.
-// static (mesh) data of one lane of a sweep: the neighbour across face
-// slot s of cell i and the slot geometry; read before the kernel waits on
-// its predecessor, since no kernel of a cycle writes it
+// FP64: the bracket in increment form, Q = (rho, rho u, rho v, rho E + p),
+//   F_n(U + dU) - F_n(U) = dQ u_n' + Q du_n + dp (0, n, 0),  u_n' = u_n + du_n,
+// from the neighbour's base and delta records, with n S/2 and lambda S/2 per
+// slot.  The velocity and pressure changes of an increment are formed once,
+// by the cell that makes it (store_delta), not by each of its neighbours: 17
+// FP64 instructions per neighbour and 21 per cell, no division, where each
+// face slot took about 45 with an IEEE division.  FP32 (the mixed path) keeps
+// its expressions and the order of its sums (euler_flux_delta; pairs of
+// slots), which fix its rounding.
+// Two forms with the same roundings (the four slots' brackets are summed in
+// pairs).  One thread per cell: an FP64 instruction costs a warp the same
+// however many lanes are active, so no lane is spent on absent slots, sums or
+// the cell's own part; for FP64 launches with more cells than fill the FP64
+// units (sweep_lanes).  Four lanes per cell, one per slot: for fewer cells,
+// where the chain of FP64 instructions of one warp is what a launch waits for
+// (about 42 instead of 90), and for FP32, where it is the chain of loads.
+// Cells of one colour never neighbour each other, so the deltas read here are
+// not written by this launch.
+
+// static (mesh) data of slot s of cell i; read before the kernel waits on its
+// predecessor, since no kernel of a cycle writes it
 template <typename T>
-struct SweepGeo {
-  int j, f;
-  bool is0;
+struct SlotGeo {
+  int j;
   T nx, ny, hS;
 };
 template <typename T>
-__device__ __forceinline__ SweepGeo<T> sweep_geo(const MeshT<T> &m, const int i, const int s) {
-  const int n = m.nc;
-  SweepGeo<T> g;
-  g.j = i >= 0 ? m.cnbr[s * n + i] : -1;
-  g.f = 0;
-  g.is0 = true;
-  g.nx = g.ny = g.hS = T(0);
+__device__ __forceinline__ SlotGeo<T> slot_geo(const MeshT<T> &m, const int i, const int s) {
+  SlotGeo<T> g;
+  g.j = i >= 0 ? m.cnbr[s * m.nc + i] : -1;
   if (g.j >= 0) {
-    g.nx = m.snx[s * n + i];
-    g.ny = m.sny[s * n + i];
-    g.hS = m.shs[s * n + i];
-    if constexpr (!is_f32<T>()) {
-      const int fs = m.cface[s * n + i];
-      g.is0 = fs >= 0;
-      g.f = g.is0 ? fs : ~fs;
-    }
+    g.nx = m.snx[s * m.nc + i];
+    g.ny = m.sny[s * m.nc + i];
+    if constexpr (is_f32<T>()) g.hS = m.shs[s * m.nc + i];
   }
   return g;
 }
-// The relaxation of cell i by its 4-lane group; the neighbour's increment
-// is read from dn (through L2 when l2 is set: values another CTA of the
-// launch wrote), the cell's new increment written to dU.
+// what a sweep reads of a neighbour, and of slot s
 template <typename T>
-__device__ __forceinline__ void sweep_cell_from(const MeshT<T> &m, const ParamsT<T> &P, const SweepGeo<T> &g,
-                                                const int i, const int s, const T *__restrict__ U,
-                                                const T *__restrict__ prim, const T *__restrict__ Rk,
-                                                const T *__restrict__ invD, const T *__restrict__ lamS,
-                                                const T *__restrict__ E0, const T *__restrict__ E1,
-                                                const T *dn, const bool l2, T *dU) {
-  const int n = m.nc, nf = m.nf;
-  const int j = g.j;
-  // every lane stays to the shuffles; lanes of absent cells or slots add 0
-  T c[4] = { T(0), T(0), T(0), T(0) };
-  if (j >= 0) {
-    const T nx = g.nx, ny = g.ny, hS = g.hS, lp = lamS[s * n + i];
-    T uj[4], du[4];
+struct SlotData {
+  static constexpr int NB = is_f32<T>() ? 8 : 4;
+  T b[NB], q[del_run<T>()], ls;
+};
+template <typename T, bool CG, bool CGD>
+__device__ __forceinline__ void slot_load(const MeshT<T> &m, int i, int s, int j, const T *base, const T *lamS,
+                                          const T *del, SlotData<T> &x) {
+  vload<T, SlotData<T>::NB, CG>(base + static_cast<size_t>(j) * kBase, x.b);
+  vload<T, del_run<T>(), CGD>(del + static_cast<size_t>(j) * del_run<T>(), x.q);
+  x.ls = ld<CG>(&lamS[s * m.nc + i]);
+}
+// the slot's bracket times S / 2
+__device__ __forceinline__ void slot_bracket(float gamma, const SlotGeo<float> &g, const SlotData<float> &x,
+                                             float c[4]) {
+  float dF[4];
+  D::euler_flux_delta(gamma, x.b, x.b[4], x.b[5], x.b[6], x.q, g.nx, g.ny, dF);
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      uj[v] = U[v * n + j];
-      du[v] = l2 ? __ldcg(&dn[v * n + j]) : dn[v * n + j];
-    }
-    if constexpr (is_f32<T>()) {
-      T dF[4];
-      D::euler_flux_delta(P.gamma, uj, prim[1 * n + j], prim[2 * n + j], prim[3 * n + j], du, nx, ny, dF);
+  for (int v = 0; v < 4; ++v) c[v] = __fmul_rn(g.hS, dF[v] - x.ls * x.q[v]);
+}
+__device__ __forceinline__ void slot_bracket(double, const SlotGeo<double> &g, const SlotData<double> &x,
+                                             double c[4]) {
+  const double *b = x.b, *q = x.q;
+  const double dun = fma(q[5], g.ny, __dmul_rn(q[4], g.nx));
+  const double un1 = fma(b[2], g.ny, fma(b[1], g.nx, dun));
+  const double w = un1 - x.ls, t = __dmul_rn(b[0], dun);
+  c[0] = fma(q[0], w, t);
+  c[1] = fma(q[6], g.nx, fma(b[1], t, __dmul_rn(q[1], w)));
+  c[2] = fma(q[6], g.ny, fma(b[2], t, __dmul_rn(q[2], w)));
+  c[3] = fma(b[3], dun, fma(q[6], un1, __dmul_rn(q[3], w)));
+}
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+
+// One thread per cell: the new increment of cell i in d, its delta record
+// written to out.  The neighbours' delta records are read from del_of(j)
+// (through L2 when CGD is set), the rest through L2 when CG is.
+template <typename T, bool CG, bool CGD, typename DelOf>
+__device__ __forceinline__ void sweep_cell(const MeshT<T> &m, T gamma, const SlotGeo<T> g[kMaxFace], const int i,
+                                           const T *base, const T *Rk, const T *invD, const T *lamS, DelOf &&del_of,
+                                           T *out, T d[4]) {
+  const int n = m.nc;
+  T r[4], bi[4] = { T(0), T(0), T(0), T(0) };
 #pragma unroll
-      for (int v = 0; v < 4; ++v) c[v] = hS * (dF[v] - lp * du[v]);
-    } else {
-      const int f = g.f;
-      T up[4], fa[4];
+  for (int v = 0; v < 4; ++v) r[v] = ld<CG>(&Rk[v * n + i]);
+  if constexpr (!is_f32<T>()) vload<T, 4, CG>(base + static_cast<size_t>(i) * kBase, bi);
+  const T iD = ld<CG>(&invD[i]);
+  // every neighbour's loads are in flight before the first is used
+  SlotData<T> x[kMaxFace];
 #pragma unroll
-      for (int v = 0; v < 4; ++v) up[v] = uj[v] + du[v];
-      D::euler_flux(P.gamma, up, nx, ny, fa);
+  for (int s = 0; s < kMaxFace; ++s)
+    if (g[s].j >= 0) slot_load<T, CG, CGD>(m, i, s, g[s].j, base, lamS, del_of(g[s].j), x[s]);
+  T c[kMaxFace][4];
 #pragma unroll
-      for (int v = 0; v < 4; ++v) {
-        const T fb = g.is0 ? E1[v * nf + f] : -E0[v * nf + f];
-        c[v] = hS * ((fa[v] - fb) - lp * du[v]);   // (U + dU) - U = dU
-      }
-    }
+  for (int s = 0; s < kMaxFace; ++s) {
+#pragma unroll
+    for (int v = 0; v < 4; ++v) c[s][v] = T(0);
+    if (g[s].j >= 0) slot_bracket(gamma, g[s], x[s], c[s]);
   }
-  // lane s needs component s summed over the group: a transposing
-  // reduction (3 additions per lane instead of an all-reduce of 4 values)
-  const bool b0 = s & 1, b1 = s & 2;
-  const T k0 = (b0 ? c[1] : c[0]) + __shfl_xor_sync(0xffffffffu, b0 ? c[0] : c[1], 1);   // component b0
-  const T k1 = (b0 ? c[3] : c[2]) + __shfl_xor_sync(0xffffffffu, b0 ? c[2] : c[3], 1);   // component b0 + 2
-  const T mine = (b1 ? k1 : k0) + __shfl_xor_sync(0xffffffffu, b1 ? k0 : k1, 2);
-  if (i >= 0) dU[s * n + i] = (Rk[s * n + i] - mine) * invD[i];
+  const bool four = g[3].j >= 0;   // (adding an absent slot's 0 changes nothing)
+#pragma unroll
+  for (int v = 0; v < 4; ++v) {
+    const T hi = four ? add_rn(c[2][v], c[3][v]) : c[2][v];
+    d[v] = (r[v] - add_rn(add_rn(c[0][v], c[1][v]), hi)) * iD;
+  }
+  store_delta(gamma, bi, d, out, i);
 }
-template <typename T>
-__device__ __forceinline__ void sweep_cell(const MeshT<T> &m, const ParamsT<T> &P, const SweepGeo<T> &g,
-                                           const int i, const int s, const T *__restrict__ U,
-                                           const T *__restrict__ prim, const T *__restrict__ Rk,
-                                           const T *__restrict__ invD, const T *__restrict__ lamS,
-                                           const T *__restrict__ E0, const T *__restrict__ E1, T *dU) {
-  sweep_cell_from(m, P, g, i, s, U, prim, Rk, invD, lamS, E0, E1, dU, false, dU);
-}
-// cells per block of a sweep launch of a shape
-__host__ __device__ constexpr int sweep_cpb(int sh) { return shape_bs(sh) / kMaxFace; }
-template <typename T>
+// Lanes per cell of a sweep over cnt cells.  An FP64 launch takes as long as
+// the warps of one sub-core (608 of them) issue one after another: about 43
+// instructions for each 8 cells with four lanes, 91 for each 32 with one, so
+// four are shorter up to two warps a sub-core, 9,728 cells.  Event-timed, us
+// per launch, four / one: colours of 1,000 cells 8.0 / 10.6, 2,900 8.2 / 11.1,
+// 28,480 15.1 / 13.0 (before: 14.5).
+constexpr int kSweepOneLane = 9728;
+template <typename T> int sweep_lanes(int cnt) { return !is_f32<T>() && cnt >= kSweepOneLane ? 1 : 4; }
+// The cells of one colour form one contiguous range per solve; a block works
+// on blockDim / LANES cells of a range.
+// LAST: the cell's last relaxation of the implicit step.  It then also
+// advances its state, U += dU (FP64), and writes the base record of the next
+// implicit step (to a second buffer: later colours of this step still read
+// the present one), which takes the place of a pass over all cells.
+template <typename T, bool LAST, int LANES>
 __global__ void __launch_bounds__(kMaxShapeBlock) k_sweep(MeshT<T> m, ParamsT<T> P,
-                                                                        const __grid_constant__ Ranges R,
-                                                                        const int *__restrict__ list, int count,
-                                                                        const T *__restrict__ U,
-                                                                        const T *__restrict__ prim,
-                                                                        const T *__restrict__ Rk,
-                                                                        const T *__restrict__ invD,
-                                                                        const T *__restrict__ lamS,
-                                                                        const T *__restrict__ E0,
-                                                                        const T *__restrict__ E1, T *__restrict__ dU) {
-  const int cpb = blockDim.x / kMaxFace, s = threadIdx.x & (kMaxFace - 1);
-  const int cl = static_cast<int>(threadIdx.x) / kMaxFace;
+                                                          const __grid_constant__ Ranges R,
+                                                          const int *__restrict__ list, int count, const T *base,
+                                                          const T *Rk, const T *invD, const T *lamS, T *delta,
+                                                          double *U, T *base_next) {
+  const int n = m.nc, cpb = blockDim.x / LANES, cl = static_cast<int>(threadIdx.x) / LANES;
   int i;
   if (list) {
     const int g = static_cast<int>(blockIdx.x) * cpb + cl;
@@ -1117,9 +1234,83 @@ __global__ void __launch_bounds__(kMaxShapeBlock) k_sweep(MeshT<T> m, ParamsT<T>
   } else {
     i = range_cell(R, cl, cpb);
   }
-  const SweepGeo<T> geo = sweep_geo(m, i, s);   // mesh data, before the wait for the predecessor
-  pdl_enter();
-  sweep_cell(m, P, geo, i, s, U, prim, Rk, invD, lamS, E0, E1, dU);
+  if constexpr (LANES == 1) {
+    if (i < 0) { pdl_enter(); return; }   // waits too: this grid ends after its predecessor
+    SlotGeo<T> geo[kMaxFace];
+#pragma unroll
+    for (int s = 0; s < kMaxFace; ++s) geo[s] = slot_geo(m, i, s);
+    pdl_enter();
+    T d[4];
+    sweep_cell<T, false, false>(m, P.gamma, geo, i, base, Rk, invD, lamS, [&](int) -> const T * { return delta; },
+                                delta, d);
+    if constexpr (LAST) {
+      double u[4];
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        u[v] = U[v * n + i] + static_cast<double>(d[v]);
+        U[v * n + i] = u[v];
+      }
+      T rec[kBase];
+      base_record(P, u, rec);
+      vstore<T, kBase>(base_next + static_cast<size_t>(i) * kBase, rec);
+    }
+  } else {
+    static_assert(LANES == kMaxFace, "a lane per slot");
+    const int s = threadIdx.x & (kMaxFace - 1);
+    const SlotGeo<T> geo = slot_geo(m, i, s);
+    pdl_enter();
+    T bi[4] = { T(0), T(0), T(0), T(0) }, r = T(0), iD = T(0);
+    double us = 0.0;
+    if (i >= 0) {
+      r = Rk[s * n + i];
+      iD = invD[i];
+      if constexpr (!is_f32<T>()) vload<T, 4>(base + static_cast<size_t>(i) * kBase, bi);
+      if (LAST) us = U[s * n + i];
+    }
+    T c[4] = { T(0), T(0), T(0), T(0) };
+    if (geo.j >= 0) {
+      SlotData<T> x;
+      slot_load<T, false, false>(m, i, s, geo.j, base, lamS, delta, x);
+      slot_bracket(P.gamma, geo, x, c);
+    }
+    // lane s needs component s summed over the group: a transposing
+    // reduction (3 additions per lane instead of an all-reduce of 4 values);
+    // every lane stays to the shuffles, absent cells and slots add 0
+    const bool b0 = s & 1, b1 = s & 2;
+    const T k0 = add_rn(b0 ? c[1] : c[0], __shfl_xor_sync(0xffffffffu, b0 ? c[0] : c[1], 1));   // component b0
+    const T k1 = add_rn(b0 ? c[3] : c[2], __shfl_xor_sync(0xffffffffu, b0 ? c[2] : c[3], 1));   // component b0 + 2
+    const T mine = add_rn(b1 ? k1 : k0, __shfl_xor_sync(0xffffffffu, b1 ? k0 : k1, 2));
+    const T ds = (r - mine) * iD;
+    if constexpr (is_f32<T>()) {
+      if (i >= 0) delta[static_cast<size_t>(i) * 4 + s] = ds;
+    } else {
+      T d[4], rec[8];
+#pragma unroll
+      for (int v = 0; v < 4; ++v) d[v] = __shfl_sync(0xffffffffu, ds, v, 4);
+      delta_record(P.gamma, bi, d, rec);
+      if (i >= 0) {
+        const T lo = s == 0 ? rec[0] : s == 1 ? rec[2] : s == 2 ? rec[4] : rec[6];
+        const T hi = s == 0 ? rec[1] : s == 1 ? rec[3] : s == 2 ? rec[5] : rec[7];
+        const T two[2] = { lo, hi };
+        vstore<T, 2>(delta + static_cast<size_t>(i) * 8 + 2 * s, two);
+      }
+    }
+    if constexpr (LAST) {
+      us += static_cast<double>(ds);
+      if (i >= 0) U[s * n + i] = us;
+      double u[4];
+#pragma unroll
+      for (int v = 0; v < 4; ++v) u[v] = __shfl_sync(0xffffffffu, us, v, 4);
+      T rec[kBase];
+      base_record(P, u, rec);
+      if (i >= 0 && s < 3) {
+        T part[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) part[v] = s == 0 ? rec[v] : s == 1 ? rec[4 + v] : rec[8 + v];
+        vstore<T, 4>(base_next + static_cast<size_t>(i) * kBase + 4 * s, part);
+      }
+    }
+  }
   pdl_exit();
 }
 
@@ -1129,15 +1320,15 @@ __global__ void __launch_bounds__(kMaxShapeBlock) k_sweep(MeshT<T> m, ParamsT<T>
 // thread-block cluster owns one partition: its CTAs share out each
 // colour's cells of the partition, and a cluster barrier (release /
 // acquire at cluster scope) separates consecutive colours, so a cell sees
-// the increments its partition's earlier colours just wrote to dU_out
+// the increments its partition's earlier colours just wrote to delta_out
 // (read through L2).  Neighbours in other partitions, and cells of this
-// partition not yet relaxed in this sweep, are read from dU_in, the
+// partition not yet relaxed in this sweep, are read from delta_in, the
 // increments at the start of the sweep: partitions exchange once per
 // sweep, lagged, like the paper's threads.  Every cell of every partition
-// is written to dU_out.  The colour C-1 ending the forward pass is not
+// is written to delta_out.  The colour C-1 ending the forward pass is not
 // relaxed again at the start of the backward pass: with its inputs
 // unchanged it would recompute the same values.
-constexpr int kPartBlock = 256;        // threads per CTA: 64 cells per pass of a CTA
+constexpr int kPartBlock = 256;        // threads per CTA: one cell per thread and pass
 constexpr int kPartCluster = 8;        // CTAs per partition (portable cluster size)
 constexpr int kMaxPartColours = 16;
 
@@ -1161,12 +1352,10 @@ __device__ __forceinline__ void cluster_sync() {
 // partition q; C colours
 template <typename T>
 __global__ void __launch_bounds__(kPartBlock) k_sweep_part(MeshT<T> m, ParamsT<T> P, const int *__restrict__ ptab,
-                                                           int C, const T *__restrict__ U,
-                                                           const T *__restrict__ prim, const T *__restrict__ Rk,
-                                                           const T *__restrict__ invD,
-                                                           const T *__restrict__ lamS, const T *__restrict__ E0,
-                                                           const T *__restrict__ E1, const T *__restrict__ dU_in,
-                                                           T *dU_out) {
+                                                           int C, const T *base,
+                                                           const T *Rk, const T *invD,
+                                                           const T *lamS,
+                                                           const T *delta_in, T *delta_out) {
   __shared__ int sb[kMaxPartColours], se[kMaxPartColours];
   const unsigned K = cluster_nctarank(), rank = cluster_ctarank();
   const int q = static_cast<int>(blockIdx.x / K);
@@ -1175,26 +1364,25 @@ __global__ void __launch_bounds__(kPartBlock) k_sweep_part(MeshT<T> m, ParamsT<T
     se[threadIdx.x] = ptab[2 * (q * C + threadIdx.x) + 1];
   }
   __syncthreads();
-  constexpr int G = kPartBlock / kMaxFace;          // cells per pass of a CTA
-  const int s = threadIdx.x & (kMaxFace - 1);
-  const int cl = static_cast<int>(threadIdx.x) / kMaxFace;
   pdl_enter();
   const int steps = 2 * C - 1;
   for (int step = 0; step < steps; ++step) {
     const bool fwd = step < C;
     const int c = fwd ? step : 2 * C - 2 - step;
     const int b = sb[c], e = se[c];
-    // the CTA's passes are uniform over its threads (the shuffles need
-    // whole lane groups)
-    for (int base = b + static_cast<int>(rank) * G; base < e; base += static_cast<int>(K) * G) {
-      const int i = base + cl < e ? base + cl : -1;
-      const SweepGeo<T> g = sweep_geo(m, i, s);
-      bool fresh = false;
-      if (g.j >= 0) {
-        const int cj = m.ccol[g.j];
-        fresh = cj < C && g.j >= sb[cj] && g.j < se[cj] && (!fwd || cj < c);
-      }
-      sweep_cell_from(m, P, g, i, s, U, prim, Rk, invD, lamS, E0, E1, fresh ? dU_out : dU_in, fresh, dU_out);
+    for (int i = b + static_cast<int>(rank) * kPartBlock + static_cast<int>(threadIdx.x); i < e;
+         i += static_cast<int>(K) * kPartBlock) {
+      SlotGeo<T> g[kMaxFace];
+#pragma unroll
+      for (int k = 0; k < kMaxFace; ++k) g[k] = slot_geo(m, i, k);
+      T d[4];
+      sweep_cell<T, false, true>(m, P.gamma, g, i, base, Rk, invD, lamS,
+                                 [&](int j) -> const T * {
+                                   const int cj = m.ccol[j];
+                                   const bool fresh = cj < C && j >= sb[cj] && j < se[cj] && (!fwd || cj < c);
+                                   return fresh ? delta_out : delta_in;
+                                 },
+                                 delta_out, d);
     }
     if (step + 1 < steps) cluster_sync();
   }
@@ -1204,10 +1392,10 @@ __global__ void __launch_bounds__(kPartBlock) k_sweep_part(MeshT<T> m, ParamsT<T
 // K9: prolongation W = W_p0 + (U - W_p0) (Section 3, step 5), density
 // residual against the state at the start of the cycle, state check.
 template <typename TF>
-__global__ void __launch_bounds__(kCellBlock) k_prolong(MeshT<double> m, ParamsT<double> P, double *__restrict__ W,
-                                                        const double *__restrict__ Wp0, const double *__restrict__ U,
-                                                        int *status, double *__restrict__ partial,
-                                                        TF *__restrict__ Wm) {
+__global__ void __launch_bounds__(kCellBlock) k_prolong(MeshT<double> m, ParamsT<double> P, double *W,
+                                                        const double *Wp0, const double *U,
+                                                        int *status, double *partial,
+                                                        TF *Wm) {
   pdl_enter();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int n = m.nc;

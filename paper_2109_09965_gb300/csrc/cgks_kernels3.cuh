@@ -21,12 +21,10 @@ namespace cgks {
 namespace kern3 {
 
 namespace D3 = cgks::dev3;
+namespace dev = cgks::dev;
 constexpr int NV = 5;
 constexpr int kCellBlock = 256;
-constexpr int kSweepLanes = 8;                     // lanes per cell (6 face slots)
 constexpr int kFO = 4 * NV;                        // face outputs of the high level: F0, F1, Wc, Wt
-constexpr int kLo = 8;                             // low-level face run: flux (NV), lambda_p, 2 pad
-constexpr int kEu = 6;                             // Euler flux cache run of one face side: NV, 1 pad
 constexpr int kBadState = 1;
 
 template <typename T>
@@ -34,7 +32,7 @@ __host__ __device__ constexpr bool is_f32() { return std::is_same<T, float>::val
 
 template <typename T>
 struct ParamsT {
-  T gamma, K, cfl_hi, cfl_lo, mu;
+  T gamma, K, cfl_hi, icfl_lo, mu;   // icfl_lo = 1 / CFL of the low-order level
   D3::KC<T> kc;
   const int *bc_kind;          // [16]
   const T *bc_uw;              // [16][3] wall velocity (global)
@@ -51,7 +49,7 @@ struct MeshT {
   const T *vol, *ivol, *ih, *hdt, *m2, *op;       // m2 [6][nc], op [27*9][nc]
   const T *fe, *fS, *fjump, *fw, *fxi;            // fe [9][nf] (n, t1, t2), fw [4][nf], fxi [24][nf]
   const T *fidl;                                  // 1/delta: centre distance along n (boundary: twice to the face)
-  const T *sn, *shs;                              // [6*3][nc] outward normal per slot, [6][nc] S/2
+  const T *sn, *shs;                              // [6*3][nc] outward normal per slot (FP64: times S/2), [6][nc] S/2
   const int *fng, *cface, *cnbr, *fc0, *fc1;
 };
 
@@ -109,7 +107,7 @@ __global__ void k_reset_dt(Ctl *ctl, unsigned long long *dt_bits, double dt_fixe
 }
 
 // explicit step: min over cells of h / (|U| + c + 2 nu / h), h = 3|Omega| / sum S
-__global__ void __launch_bounds__(kCellBlock) k_dt(MeshT<double> m, ParamsT<double> P, const double *__restrict__ W,
+__global__ void __launch_bounds__(kCellBlock) k_dt(MeshT<double> m, ParamsT<double> P, const double *W,
                                                    unsigned long long *dt_bits) {
   pdl_enter();
   __shared__ double wmin[kCellBlock / 32];
@@ -300,7 +298,7 @@ __device__ __forceinline__ void recon_at(const MeshT<T> &m, const ParamsT<T> &P,
 }
 template <typename T>
 __global__ void __launch_bounds__(kMaxShapeBlock)
-    k_recon(MeshT<T> m, ParamsT<T> P, const T *__restrict__ W, const T *__restrict__ Wx, T *__restrict__ coef) {
+    k_recon(MeshT<T> m, ParamsT<T> P, const T *W, const T *Wx, T *coef) {
   pdl_enter();
   for_items(m.nc, [&](int i) { recon_at<T, false>(m, P, W, Wx, coef, nullptr, i); });
   pdl_exit();
@@ -308,8 +306,8 @@ __global__ void __launch_bounds__(kMaxShapeBlock)
 // with the compact WENO step; wenok[i] = 1 where the stencil gave a quadratic
 template <typename T>
 __global__ void __launch_bounds__(kMaxShapeBlock)
-    k_recon_weno(MeshT<T> m, ParamsT<T> P, const T *__restrict__ W, const T *__restrict__ Wx, T *__restrict__ coef,
-                 const unsigned char *__restrict__ wenok) {
+    k_recon_weno(MeshT<T> m, ParamsT<T> P, const T *W, const T *Wx, T *coef,
+                 const unsigned char *wenok) {
   pdl_enter();
   for_items(m.nc, [&](int i) { recon_at<T, true>(m, P, W, Wx, coef, wenok, i); });
   pdl_exit();
@@ -566,16 +564,16 @@ constexpr int64_t kFaceLanes4 = 100000;
 inline int face_lanes(int64_t n_faces) { return n_faces < kFaceLanes4 ? 4 : 1; }
 template <typename T>
 __global__ void __launch_bounds__(kMaxShapeBlock)
-    k_face(MeshT<T> m, ParamsT<T> P, const T *__restrict__ W, const T *__restrict__ coef,
-           T *__restrict__ out) {
+    k_face(MeshT<T> m, ParamsT<T> P, const T *W, const T *coef,
+           T *out) {
   pdl_enter();
   for_items(m.nf, [&](int f) { face_raw_at<T, false>(m, P, W, coef, out, nullptr, nullptr, f); });
   pdl_exit();
 }
 template <int LANES>
 __global__ void __launch_bounds__(kMaxShapeBlock)
-    k_face_smooth(MeshT<double> m, ParamsT<double> P, const double *__restrict__ W,
-                  const double *__restrict__ coef, double *__restrict__ out) {
+    k_face_smooth(MeshT<double> m, ParamsT<double> P, const double *W,
+                  const double *coef, double *out) {
   pdl_enter();
   for_items(LANES * m.nf, [&](int i) { face_smooth_at<LANES>(m, P, W, coef, out, i / LANES, i % LANES); });
   pdl_exit();
@@ -583,8 +581,8 @@ __global__ void __launch_bounds__(kMaxShapeBlock)
 // the full flux of Eq. (2nd-flux): the same face loop, with the step's dt
 template <typename T>
 __global__ void __launch_bounds__(kMaxShapeBlock)
-    k_face_full(MeshT<T> m, ParamsT<T> P, const T *__restrict__ W, const T *__restrict__ coef,
-                T *__restrict__ out, const Ctl *ctl, const unsigned long long *dt_bits) {
+    k_face_full(MeshT<T> m, ParamsT<T> P, const T *W, const T *coef,
+                T *out, const Ctl *ctl, const unsigned long long *dt_bits) {
   pdl_enter();
   for_items(m.nf, [&](int f) { face_raw_at<T, true>(m, P, W, coef, out, ctl, dt_bits, f); });
   pdl_exit();
@@ -600,12 +598,12 @@ enum UpdMode { kS1O2 = 0, kS2O4Stage = 1, kS2O4Final = 2, kResidual = 3 };
 // whole run, the final S2O4 stage two.
 template <typename TF, int mode>
 __global__ void __launch_bounds__(kCellBlock) k_update(MeshT<double> m, ParamsT<double> P,
-                                                       const double *__restrict__ Wbase, const TF *__restrict__ FA,
-                                                       const TF *__restrict__ FB, const Ctl *ctl,
+                                                       const double *Wbase, const TF *FA,
+                                                       const TF *FB, const Ctl *ctl,
                                                        const unsigned long long *dt_bits, int *status,
-                                                       double *__restrict__ Wout, double *__restrict__ Wxout,
-                                                       double *__restrict__ partial, double *__restrict__ Rout,
-                                                       TF *__restrict__ Wout_m, TF *__restrict__ Wxout_m) {
+                                                       double *Wout, double *Wxout,
+                                                       double *partial, double *Rout,
+                                                       TF *Wout_m, TF *Wxout_m) {
   pdl_enter();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int n = m.nc;
@@ -625,11 +623,10 @@ __global__ void __launch_bounds__(kCellBlock) k_update(MeshT<double> m, ParamsT<
       if (fs == kNoFace) continue;
       const int f = fs >= 0 ? fs : ~fs;
       const double sg = fs >= 0 ? 1.0 : -1.0;
-      // the slot's area and outward normal from the per-cell slot arrays
-      // (coalesced; the same values as S_f and sg n_f, exactly)
+      // the slot's area and sgn S n_f from the per-cell slot arrays (coalesced)
       const double S = 2.0 * m.shs[s * n + i];
-      const double nx = sg * m.sn[(3 * s) * n + i], ny = sg * m.sn[(3 * s + 1) * n + i],
-                   nz = sg * m.sn[(3 * s + 2) * n + i];
+      const double nx = 2.0 * m.sn[(3 * s) * n + i], ny = 2.0 * m.sn[(3 * s + 1) * n + i],
+                   nz = 2.0 * m.sn[(3 * s + 2) * n + i];
       // the face's run of F0, F1, Wc, Wt (and the second stage's, when used);
       // the residual reads the leading F0, F1 part only
       constexpr int kRes = (2 * NV + VecOf<TF>::W - 1) / VecOf<TF>::W * VecOf<TF>::W;
@@ -645,9 +642,9 @@ __global__ void __launch_bounds__(kCellBlock) k_update(MeshT<double> m, ParamsT<
         R[v] -= sg * S * (a0 * static_cast<double>(a[v]) + a1 * f1);
         if constexpr (mode != kResidual) {
           const double wp = static_cast<double>(a[2 * NV + v]) + b1 * static_cast<double>(wt[3 * NV + v]);
-          g[0][v] += sg * S * nx * wp;
-          g[1][v] += sg * S * ny * wp;
-          g[2][v] += sg * S * nz * wp;
+          g[0][v] += nx * wp;
+          g[1][v] += ny * wp;
+          g[2][v] += nz * wp;
         }
       }
     }
@@ -656,6 +653,7 @@ __global__ void __launch_bounds__(kCellBlock) k_update(MeshT<double> m, ParamsT<
       for (int v = 0; v < NV; ++v) Rout[v * n + i] = R[v];
     if constexpr (mode != kResidual) {
       const double iv = m.ivol[i];
+      const double old = Wbase[i];   // Wout may be Wbase (explicit steps update in place)
       double w[NV];
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
@@ -669,15 +667,15 @@ __global__ void __launch_bounds__(kCellBlock) k_update(MeshT<double> m, ParamsT<
         }
       }
       if (!state_ok(P.gamma, w)) atomicOr(status, kBadState);
-      num = fabs(w[0] - Wbase[i]);
-      den = Wbase[i];
+      num = fabs(w[0] - old);
+      den = old;
     }
   }
   if (partial) block_sum2(num, den, &partial[2 * blockIdx.x]);
   pdl_exit();
 }
 
-__global__ void k_res_final(const double *__restrict__ partial, int nblocks, Ctl *ctl, double *hist, int cap,
+__global__ void k_res_final(const double *partial, int nblocks, Ctl *ctl, double *hist, int cap,
                             double *last) {
   pdl_enter();
   double a = 0.0, b = 0.0;
@@ -696,44 +694,102 @@ __global__ void k_res_final(const double *__restrict__ partial, int nblocks, Ctl
 }
 
 // ---------------------------- low-order level ----------------------------
-// Cell record of the low level, one per cell and implicit step: the
-// conservative state U in the flux precision and its primitives, 16 values
-// in one aligned run, so a neighbour's data costs one or two cache sectors
-// instead of one sector per value:
-//   [0..4] U, [5] u, [6] v, [7] w, [8] p, [9] rho, [10] 1/(2 lambda),
-//   [11] sqrt(lambda), [12] 1/sqrt(pi lambda), [13] c, [14] 1/rho, [15] 0.
-// A sweep reads only the first 8 (U and the velocity: 32 bytes in FP32).
-// The increments dU are stored the same way, 8 values per cell ([0..4],
-// then zeros).
-constexpr int kRec = 16, kDU = 8;
+// Records of the low level, as in 2-D (cgks_kernels.cuh):
+//   base  [kBase] per cell, the part a sweep reads first: in FP64 rho, u, v,
+//         w, H = rho E + p; p, 1/(2 lambda), sqrt(lambda), 1/sqrt(pi lambda),
+//         c, rho u, rho v, rho w, rho E, 0, 0; in FP32 U (5), u, v, w; p,
+//         1/(2 lambda), sqrt(lambda), 1/sqrt(pi lambda), c, 0, 0, 0;
+//   delta [del_run] per cell: dU; in FP64 then du, dv, dw, dp, the changes of
+//         velocity and pressure it makes; 0;
+//   Flo   [lo_run] per face: the flux, lambda_p, padding.
+constexpr int kBase = 16;
+template <typename T> __host__ __device__ constexpr int del_run() { return is_f32<T>() ? 8 : 10; }
+template <typename T> __host__ __device__ constexpr int lo_run() { return is_f32<T>() ? 8 : 6; }
+
+// positions in a base record
 template <typename T>
-__device__ __forceinline__ D3::Prim<T> rec_prim(const T r[kRec]) {
+struct BaseAt {
+  static constexpr bool f = is_f32<T>();
+  static constexpr int u = f ? 5 : 1, H = 4, p = f ? 8 : 5, i2l = f ? 9 : 6, sl = f ? 10 : 7, isp = f ? 11 : 8,
+                       c = f ? 12 : 9, m = f ? 1 : 10, E = f ? 4 : 13;
+};
+template <typename T>
+__device__ __forceinline__ D3::Prim<T> base_prim(const T r[kBase]) {
+  using A = BaseAt<T>;
   D3::Prim<T> q;
-  q.u = r[5]; q.v = r[6]; q.w = r[7]; q.p = r[8]; q.rho = r[9];
-  q.i2l = r[10]; q.sl = r[11]; q.isp = r[12]; q.c = r[13]; q.ir = r[14];
+  q.rho = r[0]; q.u = r[A::u]; q.v = r[A::u + 1]; q.w = r[A::u + 2];
+  q.p = r[A::p]; q.i2l = r[A::i2l]; q.sl = r[A::sl]; q.isp = r[A::isp]; q.c = r[A::c];
   return q;
 }
-
-// U^{k+1} = U^k + dU (FP64), cell record of U^{k+1}; first: U = W_p0
+// base record of the FP64 state u
 template <typename TF>
-__global__ void __launch_bounds__(kCellBlock) k_lo_cell(int n, ParamsT<TF> P, int first, const double *__restrict__ Wp0,
-                                                        double *__restrict__ U, const TF *__restrict__ dU,
-                                                        TF *__restrict__ rec) {
+__device__ __forceinline__ void base_record(const ParamsT<TF> &P, const double u[NV], TF r[kBase]) {
+  using A = BaseAt<TF>;
+  TF w[NV];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) w[v] = static_cast<TF>(u[v]);
+  const D3::Prim<TF> q = D3::prim_of(w, P.gamma, P.kc);
+#pragma unroll
+  for (int v = 13; v < kBase; ++v) r[v] = TF(0);
+  if constexpr (!is_f32<TF>()) r[A::H] = w[4] + q.p;
+  r[0] = w[0];
+  r[A::u] = q.u; r[A::u + 1] = q.v; r[A::u + 2] = q.w;
+  r[A::p] = q.p; r[A::i2l] = q.i2l; r[A::sl] = q.sl; r[A::isp] = q.isp; r[A::c] = q.c;
+  r[A::m] = w[1]; r[A::m + 1] = w[2]; r[A::m + 2] = w[3]; r[A::E] = w[4];
+}
+template <typename TF>
+__device__ __forceinline__ void store_base(const ParamsT<TF> &P, const double u[NV], TF *base, int i) {
+  TF r[kBase];
+  base_record(P, u, r);
+  vstore<TF, kBase>(base + static_cast<size_t>(i) * kBase, r);
+}
+// the delta record of an increment d on a cell with base b = (rho, u, v, w),
+// see the 2-D store_delta
+__device__ __forceinline__ void delta_record(double gamma, const double b[4], const double d[NV], double r[10]) {
+  const double ir = dev::d_rcp(b[0] + d[0]);
+  double du[3], a = 0.0, e = 0.0;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    du[k] = (d[1 + k] - b[1 + k] * d[0]) * ir;
+    a += d[1 + k] * (b[1 + k] + du[k]);
+    e += b[1 + k] * du[k];
+  }
+  const double g1 = gamma - 1.0;
+#pragma unroll
+  for (int v = 0; v < NV; ++v) r[v] = d[v];
+  r[5] = du[0]; r[6] = du[1]; r[7] = du[2];
+  r[8] = g1 * d[4] - 0.5 * g1 * (a + b[0] * e);
+  r[9] = 0.0;
+}
+__device__ __forceinline__ void delta_record(float, const float *, const float d[NV], float r[8]) {
+#pragma unroll
+  for (int v = 0; v < NV; ++v) r[v] = d[v];
+  r[5] = r[6] = r[7] = 0.0f;
+}
+template <typename T>
+__device__ __forceinline__ void store_delta(T gamma, const T b[4], const T d[NV], T *delta, int i) {
+  T r[del_run<T>()];
+  delta_record(gamma, b, d, r);
+  vstore<T, del_run<T>()>(delta + static_cast<size_t>(i) * del_run<T>(), r);
+}
+
+// U^{k+1} = U^k + dU (FP64), base record of U^{k+1}; first: U = W_p0
+template <typename TF>
+__global__ void __launch_bounds__(kCellBlock) k_lo_cell(int n, ParamsT<TF> P, int first, const double *Wp0,
+                                                        double *U, const TF *delta,
+                                                        TF *base) {
   pdl_enter();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  TF d[kDU];
-  if (!first) vload<TF, kDU>(dU + static_cast<size_t>(i) * kDU, d);
-  TF w[NV];
+  TF d[del_run<TF>()];
+  if (!first) vload<TF, del_run<TF>()>(delta + static_cast<size_t>(i) * del_run<TF>(), d);
+  double u[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
-    const double u = first ? Wp0[v * n + i] : U[v * n + i] + static_cast<double>(d[v]);
-    U[v * n + i] = u;
-    w[v] = static_cast<TF>(u);
+    u[v] = first ? Wp0[v * n + i] : U[v * n + i] + static_cast<double>(d[v]);
+    U[v * n + i] = u[v];
   }
-  const D3::Prim<TF> q = D3::prim_of(w, P.gamma, P.kc);
-  const TF r[kRec] = { w[0], w[1], w[2], w[3], w[4], q.u, q.v, q.w, q.p, q.rho, q.i2l, q.sl, q.isp, q.c, q.ir, TF(0) };
-  vstore<TF, kRec>(rec + static_cast<size_t>(i) * kRec, r);
+  store_base(P, u, base, i);
   pdl_exit();
 }
 
@@ -765,30 +821,26 @@ __device__ __forceinline__ void lo_ghost(const ParamsT<T> &P, int tag, const D3:
   D3::rot_out(F, wgl, wg);
 }
 
-// KFVS flux, lambda_p = max of both sides, Euler flux cache (FP64 mode)
+// KFVS (or Lax-Friedrichs) flux, lambda_p = max of both sides
 template <typename T>
-__device__ __forceinline__ void lo_face_at(const MeshT<T> &m, const ParamsT<T> &P, const T *__restrict__ rec,
-                                           T *__restrict__ Flo, T *__restrict__ E0,
-                                           T *__restrict__ E1, const int f) {
-  const int nf = m.nf;
+__device__ __forceinline__ void lo_face_at(const MeshT<T> &m, const ParamsT<T> &P, const T *__restrict__ base,
+                                           T *__restrict__ Flo, const int f) {
   const int c0 = m.fc0[f], c1 = m.fc1[f];
-  const T S = m.fS[f];
   const D3::Frame<T> F = frame_of(m, f);
-  T ra[kRec], rb[kRec];
-  vload<T, kRec>(rec + static_cast<size_t>(c0) * kRec, ra);
-  D3::Prim<T> a = rec_prim(ra), b;
-  T ivb;
+  T ra[kBase], rb[kBase];
+  vload<T, kBase>(base + static_cast<size_t>(c0) * kBase, ra);
+  const D3::Prim<T> a = base_prim(ra);
+  D3::Prim<T> b;
+  using A = BaseAt<T>;
+  const T wa[NV] = { ra[0], ra[A::m], ra[A::m + 1], ra[A::m + 2], ra[A::E] };
+  T wb[NV];
   if (c1 >= 0) {
-    vload<T, kRec>(rec + static_cast<size_t>(c1) * kRec, rb);
-    b = rec_prim(rb);
-    ivb = m.ivol[c1];
+    vload<T, kBase>(base + static_cast<size_t>(c1) * kBase, rb);
+    b = base_prim(rb);
+    wb[0] = rb[0]; wb[1] = rb[A::m]; wb[2] = rb[A::m + 1]; wb[3] = rb[A::m + 2]; wb[4] = rb[A::E];
   } else {
-    T wg[NV];
-    lo_ghost(P, -1 - c1, F, ra, wg);
-#pragma unroll
-    for (int v = 0; v < NV; ++v) rb[v] = wg[v];
-    b = D3::prim_of(wg, P.gamma, P.kc);
-    ivb = m.ivol[c0];
+    lo_ghost(P, -1 - c1, F, wa, wb);
+    b = D3::prim_of(wb, P.gamma, P.kc);
   }
   T la3[3], lb3[3];
 #pragma unroll
@@ -796,23 +848,27 @@ __device__ __forceinline__ void lo_face_at(const MeshT<T> &m, const ParamsT<T> &
     la3[k] = a.u * F.e[k][0] + a.v * F.e[k][1] + a.w * F.e[k][2];
     lb3[k] = b.u * F.e[k][0] + b.v * F.e[k][1] + b.w * F.e[k][2];
   }
-  const T la = fabs(la3[0]) + a.c + T(2) * (P.mu * a.ir) * S * m.ivol[c0];
-  const T lb = fabs(lb3[0]) + b.c + T(2) * (P.mu * b.ir) * S * ivb;
+  T la = fabs(la3[0]) + a.c, lb = fabs(lb3[0]) + b.c, ira = T(0), irb = T(0);
+  if (P.mu != T(0)) {
+    const T S = m.fS[f];
+    ira = dev::d_rcp(a.rho);
+    irb = dev::d_rcp(b.rho);
+    la += T(2) * (P.mu * ira) * S * m.ivol[c0];
+    lb += T(2) * (P.mu * irb) * S * m.ivol[c1 >= 0 ? c1 : c0];
+  }
   const T lmax = la > lb ? la : lb;
-  // Euler normal fluxes of the two sides (the L-F flux, the FP64 cache)
   const T nx = F.e[0][0], ny = F.e[0][1], nz = F.e[0][2];
-  const T una = la3[0], unb = lb3[0];
-  T Fa[NV], Fb[NV];
-  Fa[0] = a.rho * una; Fa[1] = ra[1] * una + a.p * nx; Fa[2] = ra[2] * una + a.p * ny;
-  Fa[3] = ra[3] * una + a.p * nz; Fa[4] = (ra[4] + a.p) * una;
-  Fb[0] = b.rho * unb; Fb[1] = rb[1] * unb + b.p * nx; Fb[2] = rb[2] * unb + b.p * ny;
-  Fb[3] = rb[3] * unb + b.p * nz; Fb[4] = (rb[4] + b.p) * unb;
   T Fg[NV];
   if (P.flux_lo == CGKS_FLUX_LF) {
     // Lax-Friedrichs alternative of Section 3 with the implicit operator's
     // lambda_p: (F_n(U_l) + F_n(U_r)) / 2 - lambda_p (U_r - U_l) / 2
+    const T una = la3[0], unb = lb3[0];
+    const T Fa[NV] = { a.rho * una, wa[1] * una + a.p * nx, wa[2] * una + a.p * ny, wa[3] * una + a.p * nz,
+                       (wa[4] + a.p) * una };
+    const T Fb[NV] = { b.rho * unb, wb[1] * unb + b.p * nx, wb[2] * unb + b.p * ny, wb[3] * unb + b.p * nz,
+                       (wb[4] + b.p) * unb };
 #pragma unroll
-    for (int v = 0; v < NV; ++v) Fg[v] = T(0.5) * (Fa[v] + Fb[v]) - T(0.5) * lmax * (rb[v] - ra[v]);
+    for (int v = 0; v < NV; ++v) Fg[v] = T(0.5) * (Fa[v] + Fb[v]) - T(0.5) * lmax * (wb[v] - wa[v]);
   } else {
     T Fl[NV];
     D3::kfvs(P.K, a.rho, la3[0], la3[1], la3[2], a.i2l, a.sl, a.isp, b.rho, lb3[0], lb3[1], lb3[2], b.i2l, b.sl,
@@ -835,194 +891,286 @@ __device__ __forceinline__ void lo_face_at(const MeshT<T> &m, const ParamsT<T> &
       Fg[1 + d] -= tau;
       work += tau * um[d];
     }
-    const T qn = -md * P.gamma / (P.gamma - T(1)) * (b.p * b.ir - a.p * a.ir);
+    const T qn = -md * P.gamma / (P.gamma - T(1)) * (b.p * irb - a.p * ira);
     Fg[4] -= work - qn;
   }
   // one run per face (AoS): the flux and lambda_p, read together by the
   // right-hand side of each cell
-  T o[kLo];
+  constexpr int N = lo_run<T>();
+  T o[N];
 #pragma unroll
   for (int v = 0; v < NV; ++v) o[v] = Fg[v];
   o[NV] = lmax;
-  o[NV + 1] = o[NV + 2] = T(0);
-  vstore<T, kLo>(Flo + static_cast<size_t>(f) * kLo, o);
-  if constexpr (!is_f32<T>())
-  if (E0) {   // the FP64 path's cache (the mixed path has none)
-    T e[kEu];
-    e[NV] = T(0);
 #pragma unroll
-    for (int v = 0; v < NV; ++v) e[v] = Fa[v];
-    vstore<T, kEu>(E0 + static_cast<size_t>(f) * kEu, e);
-    if (c1 >= 0) {
-#pragma unroll
-      for (int v = 0; v < NV; ++v) e[v] = Fb[v];
-      vstore<T, kEu>(E1 + static_cast<size_t>(f) * kEu, e);
-    }
-  }
+  for (int v = NV + 1; v < N; ++v) o[v] = T(0);
+  vstore<T, N>(Flo + static_cast<size_t>(f) * N, o);
 }
 template <typename T>
 __global__ void __launch_bounds__(kMaxShapeBlock)
-    k_lo_face(MeshT<T> m, ParamsT<T> P, const T *__restrict__ rec, T *__restrict__ Flo,
-              T *__restrict__ E0, T *__restrict__ E1) {
+    k_lo_face(MeshT<T> m, ParamsT<T> P, const T *base, T *Flo) {
   pdl_enter();
-  for_items(m.nf, [&](int f) { lo_face_at(m, P, rec, Flo, E0, E1, f); });
+  for_items(m.nf, [&](int f) { lo_face_at(m, P, base, Flo, f); });
   pdl_exit();
 }
 
-// right-hand side R^k = R_lo + S (FP64 sums), 1/D_i (FP64), lambda per slot,
-// first colour pass (dU = R / D on colour 0, zero elsewhere)
+// right-hand side R^k = R_lo + S (FP64 sums), 1/D_i (FP64), lambda per slot (in
+// FP64 times S/2), first colour pass (dU = R / D on colour 0, zero elsewhere)
 template <typename TF>
-__global__ void __launch_bounds__(kCellBlock) k_lo_rhs(MeshT<double> m, ParamsT<double> P, int first, int colour0_end,
-                                                       const TF *__restrict__ Flo,
-                                                       const double *__restrict__ Rp0, double *__restrict__ Src,
-                                                       TF *__restrict__ Rk, TF *__restrict__ invD, TF *__restrict__ dU,
-                                                       TF *__restrict__ lamS) {
-  pdl_enter();
+__global__ void __launch_bounds__(kCellBlock) k_lo_rhs(MeshT<double> m, ParamsT<double> P, TF gamma, int first,
+                                                       int colour0_end, const TF *base,
+                                                       const TF *Flo,
+                                                       const double *Rp0, double *Src,
+                                                       TF *Rk, TF *invD,
+                                                       TF *delta, TF *lamS) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= m.nc) return;
+  if (i >= m.nc) { pdl_enter(); return; }
   const int n = m.nc;
-  double R[NV] = { 0, 0, 0, 0, 0 }, sum = 0.0;
-  for (int s = 0; s < kMaxFace3; ++s) {
-    const int fs = m.cface[s * n + i];
-    if (fs == kNoFace) { lamS[s * n + i] = TF(0); continue; }
-    const int f = fs >= 0 ? fs : ~fs;
-    const double sg = fs >= 0 ? 1.0 : -1.0;
-    const double S = 2.0 * m.shs[s * n + i];   // S_f, from the per-cell slot array (coalesced)
-    TF fl[kLo];
-    vload<TF, kLo>(Flo + static_cast<size_t>(f) * kLo, fl);   // flux and lambda_p
+  // mesh data first (nothing in a cycle writes it), then wait for the predecessor
+  int fsl[kMaxFace3];
+  double Sh[kMaxFace3];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) R[v] -= sg * S * static_cast<double>(fl[v]);
-    const TF l = fl[NV];
-    lamS[s * n + i] = l;
-    sum += static_cast<double>(l) * S;
+  for (int s = 0; s < kMaxFace3; ++s) {
+    fsl[s] = m.cface[s * n + i];
+    Sh[s] = m.shs[s * n + i];
   }
-  const double id = 1.0 / (sum / P.cfl_lo + 0.5 * sum);
+  pdl_enter();
+  constexpr int N = lo_run<TF>();
+  double R[NV] = { 0, 0, 0, 0, 0 }, sum = 0.0;
+  TF fl[kMaxFace3][N];
+#pragma unroll
+  for (int s = 0; s < kMaxFace3; ++s) {
+    const int fs = fsl[s];
+    if (fs == kNoFace) continue;
+    vload<TF, N>(Flo + static_cast<size_t>(fs >= 0 ? fs : ~fs) * N, fl[s]);   // flux and lambda_p
+  }
+#pragma unroll
+  for (int s = 0; s < kMaxFace3; ++s) {
+    const int fs = fsl[s];
+    if (fs == kNoFace) { lamS[s * n + i] = TF(0); continue; }
+    const double h = Sh[s], hg = fs >= 0 ? -h : h;
+    double x[NV + 1];
+    widen<NV + 1>(fl[s], x);
+#pragma unroll
+    for (int v = 0; v < NV; ++v) R[v] += hg * x[v];
+    if constexpr (is_f32<TF>()) lamS[s * n + i] = fl[s][NV];
+    else lamS[s * n + i] = fl[s][NV] * h;
+    sum += x[NV] * h;
+  }
+  // sums of S/2 times the values: R / 2 and sum / 2
+  const double id = dev::d_rcp(sum * (2.0 * P.icfl_lo + 1.0));
   invD[i] = static_cast<TF>(id);
-  const bool c0 = i < colour0_end;
-  TF d[kDU];
+  TF d[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
     double src;
-    if (first) { src = Rp0[v * n + i] - R[v]; Src[v * n + i] = src; }
+    const double Rv = 2.0 * R[v];
+    if (first) { src = Rp0[v * n + i] - Rv; Src[v * n + i] = src; }
     else src = Src[v * n + i];
-    const double r = R[v] + src;
+    const double r = Rv + src;
     Rk[v * n + i] = static_cast<TF>(r);
-    d[v] = c0 ? static_cast<TF>(r * id) : TF(0);
+    d[v] = static_cast<TF>(r * id);
   }
+  if (i < colour0_end) {
+    TF b[4];
+    vload<TF, 4>(base + static_cast<size_t>(i) * kBase, b);
+    store_delta(gamma, b, d, delta, i);
+  } else {
+    TF z[del_run<TF>()];
 #pragma unroll
-  for (int v = NV; v < kDU; ++v) d[v] = TF(0);
-  vstore<TF, kDU>(dU + static_cast<size_t>(i) * kDU, d);
+    for (int v = 0; v < del_run<TF>(); ++v) z[v] = TF(0);
+    vstore<TF, del_run<TF>()>(delta + static_cast<size_t>(i) * del_run<TF>(), z);
+  }
   pdl_exit();
 }
 
 // point relaxation of the cells [begin, begin + count) of one colour, Eq.
-// (implicit-local): 8 lanes per cell, one per face slot (6 used); the five
-// terms are summed over the lane group by shuffles, lane v writes
-// component v.
-// static (mesh) data of one lane of a sweep: neighbour across face slot s
-// of cell i and the slot geometry; read before the kernel waits on its
-// predecessor, since no kernel of a cycle writes it
+// (implicit-local), as the 2-D k_sweep: FP64 in the increment form of the
+// bracket from the neighbours' base and delta records, 22 FP64 instructions
+// per neighbour and 33 per cell (before: about 55 per face slot, one IEEE
+// division each); FP32 with the expressions and the order of sums that fix
+// its rounding.
+// LANES: one thread per cell, or eight (one per face slot, six used) where a
+// colour has too few cells to fill the device (sweep_lanes).
+// LAST: the cell's last relaxation of the implicit step also advances U and
+// writes the next step's base record (second buffer).
 template <typename T>
-struct SweepGeo {
-  int j, f;
-  bool is0;
-  T nn[3], hS;
+struct SlotData {
+  static constexpr int NB = is_f32<T>() ? 8 : 5;   // part of a base record a sweep reads
+  T b[NB], q[del_run<T>()], ls, nn[3], hS;
 };
 template <typename T>
-__device__ __forceinline__ SweepGeo<T> sweep_geo(const MeshT<T> &m, const int i, const int s) {
+__device__ __forceinline__ void slot_load(const MeshT<T> &m, int i, int s, int j, const T *base, const T *lamS,
+                                          const T *delta, SlotData<T> &x) {
   const int n = m.nc;
-  SweepGeo<T> g;
-  g.j = (i >= 0 && s < kMaxFace3) ? m.cnbr[s * n + i] : -1;
-  g.f = 0;
-  g.is0 = true;
-  g.nn[0] = g.nn[1] = g.nn[2] = g.hS = T(0);
-  if (g.j >= 0) {
-    g.nn[0] = m.sn[(3 * s) * n + i];
-    g.nn[1] = m.sn[(3 * s + 1) * n + i];
-    g.nn[2] = m.sn[(3 * s + 2) * n + i];
-    g.hS = m.shs[s * n + i];
-    if constexpr (!is_f32<T>()) {
-      const int fs = m.cface[s * n + i];
-      g.is0 = fs >= 0;
-      g.f = g.is0 ? fs : ~fs;
-    }
+  if constexpr (is_f32<T>()) {
+    vload<T, 8>(base + static_cast<size_t>(j) * kBase, x.b);
+    x.hS = m.shs[s * n + i];
+  } else {
+    vload<T, 4>(base + static_cast<size_t>(j) * kBase, x.b);
+    x.b[4] = base[static_cast<size_t>(j) * kBase + 4];
   }
-  return g;
+  vload<T, del_run<T>()>(delta + static_cast<size_t>(j) * del_run<T>(), x.q);
+  x.ls = lamS[s * n + i];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) x.nn[k] = m.sn[(3 * s + k) * n + i];
 }
-template <typename T>
-__device__ __forceinline__ void sweep_cell(const MeshT<T> &m, const ParamsT<T> &P, const SweepGeo<T> &g,
-                                           const int i, const int s, const T *__restrict__ rec,
-                                           const T *__restrict__ Rk, const T *__restrict__ invD,
-                                           const T *__restrict__ lamS, const T *__restrict__ E0,
-                                           const T *__restrict__ E1, T *__restrict__ dU) {
-  const int n = m.nc, nf = m.nf;
-  const int j = g.j;
-  T c[NV] = { T(0), T(0), T(0), T(0), T(0) };
-  if (j >= 0) {
-    const T hS = g.hS, lp = lamS[s * n + i];
-    // the neighbour's U and velocity (the first 8 values of its record; 6
-    // in FP64, which needs U only) and its increment
-    constexpr int kUsed = is_f32<T>() ? 8 : 6;
-    T rj[kUsed], dj[kDU];
-    vload<T, kUsed>(rec + static_cast<size_t>(j) * kRec, rj);
-    vload<T, kDU>(dU + static_cast<size_t>(j) * kDU, dj);
-    T uj[NV], du[NV];
+__device__ __forceinline__ void slot_bracket(float gamma, const SlotData<float> &x, float c[NV]) {
+  const float *uj = x.b, *du = x.q;
+  // pressure of U_j, the expression of its primitives
+  const float pj = (gamma - 1.0f) * (uj[4] - 0.5f * uj[0] * (uj[5] * uj[5] + uj[6] * uj[6] + uj[7] * uj[7]));
+  float dF[NV];
+  D3::euler_flux_delta(gamma, uj, uj[5], uj[6], uj[7], pj, du, x.nn, dF);
 #pragma unroll
-    for (int v = 0; v < NV; ++v) { uj[v] = rj[v]; du[v] = dj[v]; }
-    if constexpr (is_f32<T>()) {
-      T dF[NV];
-      // pressure of U_j, the expression of its primitives
-      const T pj = (P.gamma - T(1)) * (uj[4] - T(0.5) * uj[0] * (rj[5] * rj[5] + rj[6] * rj[6] + rj[7] * rj[7]));
-      D3::euler_flux_delta(P.gamma, uj, rj[5], rj[6], rj[7], pj, du, g.nn, dF);
+  for (int v = 0; v < NV; ++v) c[v] = __fmul_rn(x.hS, dF[v] - x.ls * du[v]);
+}
+// r minus the slot's bracket
+__device__ __forceinline__ void slot_subtract(const SlotData<double> &x, double r[NV]) {
+  const double *b = x.b, *q = x.q, *nn = x.nn;
+  const double dun = q[5] * nn[0] + q[6] * nn[1] + q[7] * nn[2], dp = q[8];
+  const double un1 = dun + b[1] * nn[0] + b[2] * nn[1] + b[3] * nn[2];
+  const double w = un1 - x.ls, t = b[0] * dun;
+  r[0] = r[0] - q[0] * w - t;
 #pragma unroll
-      for (int v = 0; v < NV; ++v) c[v] = hS * (dF[v] - lp * du[v]);
-    } else {
-      const int f = g.f;
-      T up[NV], fa[NV], e[kEu];
-      vload<T, kEu>((g.is0 ? E1 : E0) + static_cast<size_t>(f) * kEu, e);
+  for (int k = 0; k < 3; ++k) r[1 + k] = r[1 + k] - q[1 + k] * w - b[1 + k] * t - dp * nn[k];
+  r[4] = r[4] - q[4] * w - dp * un1 - b[4] * dun;
+}
+constexpr int kSweepLanes = 8;
+// FP64: a launch takes as long as the warps of one sub-core (608 of them) issue
+// one after another: about 70 instructions for each 4 cells with eight lanes,
+// 150 for each 32 with one, so eight are shorter up to two warps a sub-core,
+// 4,864 cells.  Event-timed, us per launch, eight / one: colours of 3,960 cells
+// 11.7 / 13.3; 15,360 25.0 / 14.6; 25,000 to 51,463 42.6 / 18.8 (before: 41.4).
+// FP32 is bound by the latency of its gathers and then by their number: 3,960
+// 6.5 / 7.7; 12,779 7.2 / 7.7; 15,360 8.3 / 8.0; 211,181 17.0 / 15.9.
+constexpr int kOneLane64 = 4864, kOneLane32 = 14000;
+template <typename T> int sweep_lanes(int cnt) { return cnt >= (is_f32<T>() ? kOneLane32 : kOneLane64) ? 1 : kSweepLanes; }
+template <typename T, bool LAST, int LANES>
+__global__ void __launch_bounds__(kMaxShapeBlock)
+    k_sweep(MeshT<T> m, ParamsT<T> P, int begin, int count, const T *base, const T *Rk, const T *invD, const T *lamS,
+            T *delta, double *U, T *base_next) {
+  const int n = m.nc;
+  constexpr int ND = del_run<T>();
+  const int g = static_cast<int>(blockIdx.x * blockDim.x + threadIdx.x) / LANES;
+  const int i = g < count ? begin + g : -1;
+  if constexpr (LANES == 1) {
+    constexpr int CH = is_f32<T>() ? 6 : 3;   // slots whose loads are in flight together (registers)
+    if (i < 0) { pdl_enter(); return; }   // waits too: this grid ends after its predecessor
+    // the neighbours (mesh data) before the wait for the predecessor
+    int nb[kMaxFace3];
 #pragma unroll
-      for (int v = 0; v < NV; ++v) up[v] = uj[v] + du[v];
-      D3::euler_flux(P.gamma, up, g.nn, fa);
+    for (int s = 0; s < kMaxFace3; ++s) nb[s] = m.cnbr[s * n + i];
+    pdl_enter();
+    T r[NV], bi[4] = { T(0), T(0), T(0), T(0) }, d[NV];
 #pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        const T fb = g.is0 ? e[v] : -e[v];
-        c[v] = hS * ((fa[v] - fb) - lp * du[v]);   // (U + dU) - U = dU
+    for (int v = 0; v < NV; ++v) r[v] = Rk[v * n + i];
+    if constexpr (!is_f32<T>()) vload<T, 4>(base + static_cast<size_t>(i) * kBase, bi);
+    const T iD = invD[i];
+    T c[is_f32<T>() ? kMaxFace3 : 1][NV];
+#pragma unroll
+    for (int s0 = 0; s0 < kMaxFace3; s0 += CH) {
+      SlotData<T> x[CH];
+#pragma unroll
+      for (int s = 0; s < CH; ++s)
+        if (nb[s0 + s] >= 0) slot_load(m, i, s0 + s, nb[s0 + s], base, lamS, delta, x[s]);
+#pragma unroll
+      for (int s = 0; s < CH; ++s) {
+        if constexpr (is_f32<T>()) {
+#pragma unroll
+          for (int v = 0; v < NV; ++v) c[s0 + s][v] = T(0);
+          if (nb[s0 + s] >= 0) slot_bracket(P.gamma, x[s], c[s0 + s]);
+        } else {
+          if (nb[s0 + s] >= 0) slot_subtract(x[s], r);
+        }
       }
     }
-  }
 #pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    c[v] += __shfl_xor_sync(0xffffffffu, c[v], 1);
-    c[v] += __shfl_xor_sync(0xffffffffu, c[v], 2);
-    c[v] += __shfl_xor_sync(0xffffffffu, c[v], 4);
-  }
-  if (i >= 0 && s < NV) {
+    for (int v = 0; v < NV; ++v) {
+      if constexpr (is_f32<T>()) {
+        const T lo = __fadd_rn(__fadd_rn(c[0][v], c[1][v]), __fadd_rn(c[2][v], c[3][v]));
+        d[v] = (r[v] - __fadd_rn(lo, __fadd_rn(c[4][v], c[5][v]))) * iD;
+      } else {
+        d[v] = r[v] * iD;
+      }
+    }
+    store_delta(P.gamma, bi, d, delta, i);
+    if constexpr (LAST) {
+      double u[NV];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        u[v] = U[v * n + i] + static_cast<double>(d[v]);
+        U[v * n + i] = u[v];
+      }
+      store_base(P, u, base_next, i);
+    }
+  } else {
+    const int s = threadIdx.x & (LANES - 1);
+    const int j = (i >= 0 && s < kMaxFace3) ? m.cnbr[s * n + i] : -1;
+    pdl_enter();
+    T bi[4] = { T(0), T(0), T(0), T(0) }, r = T(0), iD = T(0);
+    double us = 0.0;
+    if (i >= 0 && s < NV) {
+      r = Rk[s * n + i];
+      iD = invD[i];
+      if (LAST) us = U[s * n + i];
+    }
+    if constexpr (!is_f32<T>())
+      if (i >= 0) vload<T, 4>(base + static_cast<size_t>(i) * kBase, bi);
+    T c[NV] = { T(0), T(0), T(0), T(0), T(0) };
+    if (j >= 0) {
+      SlotData<T> x;
+      slot_load(m, i, s, j, base, lamS, delta, x);
+      if constexpr (is_f32<T>()) slot_bracket(P.gamma, x, c);
+      else slot_subtract(x, c);   // minus the bracket
+    }
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      c[v] += __shfl_xor_sync(0xffffffffu, c[v], 1);
+      c[v] += __shfl_xor_sync(0xffffffffu, c[v], 2);
+      c[v] += __shfl_xor_sync(0xffffffffu, c[v], 4);
+    }
     const T mine = s == 0 ? c[0] : s == 1 ? c[1] : s == 2 ? c[2] : s == 3 ? c[3] : c[4];
-    dU[static_cast<size_t>(i) * kDU + s] = (Rk[s * n + i] - mine) * invD[i];
+    const T ds = (is_f32<T>() ? r - mine : r + mine) * iD;
+    if constexpr (is_f32<T>()) {
+      if (i >= 0) delta[static_cast<size_t>(i) * ND + s] = s < NV ? ds : T(0);
+    } else {
+      T d[NV], rec[ND];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) d[v] = __shfl_sync(0xffffffffu, ds, v, LANES);
+      delta_record(P.gamma, bi, d, rec);
+#pragma unroll
+      for (int v = 0; v < ND / 2; ++v)
+        if (i >= 0 && s == v) {
+          const T two[2] = { rec[2 * v], rec[2 * v + 1] };
+          vstore<T, 2>(delta + static_cast<size_t>(i) * ND + 2 * v, two);
+        }
+    }
+    if constexpr (LAST) {
+      us += static_cast<double>(ds);
+      if (i >= 0 && s < NV) U[s * n + i] = us;
+      double u[NV];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) u[v] = __shfl_sync(0xffffffffu, us, v, LANES);
+      T rec[kBase];
+      base_record(P, u, rec);
+#pragma unroll
+      for (int v = 0; v < LANES; ++v)
+        if (i >= 0 && s == v) {
+          const T two[2] = { rec[2 * v], rec[2 * v + 1] };
+          T *o = base_next + static_cast<size_t>(i) * kBase + 2 * v;
+          o[0] = two[0];
+          o[1] = two[1];
+        }
+    }
   }
-}
-// cells per block of a sweep launch of a shape
-__host__ __device__ constexpr int sweep_cpb(int sh) { return shape_bs(sh) / kSweepLanes; }
-template <typename T>
-__global__ void __launch_bounds__(kMaxShapeBlock)
-    k_sweep(MeshT<T> m, ParamsT<T> P, int begin, int count, const T *__restrict__ rec,
-            const T *__restrict__ Rk, const T *__restrict__ invD, const T *__restrict__ lamS,
-            const T *__restrict__ E0, const T *__restrict__ E1, T *__restrict__ dU) {
-  const int s = threadIdx.x & (kSweepLanes - 1);
-  const int g = static_cast<int>(blockIdx.x * blockDim.x + threadIdx.x) / kSweepLanes;
-  const int i = g < count ? begin + g : -1;
-  const SweepGeo<T> geo = sweep_geo(m, i, s);   // mesh data, before the wait for the predecessor
-  pdl_enter();
-  sweep_cell(m, P, geo, i, s, rec, Rk, invD, lamS, E0, E1, dU);
   pdl_exit();
 }
 
 // W = W_p0 + (U - W_p0), density residual partials, state check
 template <typename TF>
-__global__ void __launch_bounds__(kCellBlock) k_prolong(MeshT<double> m, ParamsT<double> P, double *__restrict__ W,
-                                                        const double *__restrict__ Wp0, const double *__restrict__ U,
-                                                        int *status, double *__restrict__ partial,
-                                                        TF *__restrict__ Wm) {
+__global__ void __launch_bounds__(kCellBlock) k_prolong(MeshT<double> m, ParamsT<double> P, double *W,
+                                                        const double *Wp0, const double *U,
+                                                        int *status, double *partial,
+                                                        TF *Wm) {
   pdl_enter();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int n = m.nc;

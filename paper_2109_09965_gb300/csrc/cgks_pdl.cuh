@@ -10,7 +10,10 @@
 // predecessor (reads and writes alike).  Every thread waits, so a kernel
 // completes only after its predecessor has, and the chain orders each
 // kernel after all earlier ones.  Before the wait a kernel may read only
-// mesh data, which nothing writes while cycles run.  pdl_exit() at the
+// mesh data, which nothing writes while cycles run.  For the same reason the
+// kernels take what the cycle writes through plain const pointers, not
+// __restrict__ ones: the compiler may treat loads through those as invariant
+// and move them above the wait.  pdl_exit() at the
 // end of the kernel body lets the next kernel launch (blocks that return
 // early count as done); where the trigger falls affects only timing, since
 // the next kernel waits for this one to complete whatever happens.

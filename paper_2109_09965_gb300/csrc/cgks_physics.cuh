@@ -50,10 +50,11 @@ __device__ __forceinline__ void rot_out(T nx, T ny, const T l[NV], T g[NV]) {
 }
 
 // Constants of the kinetic model with K internal degrees of freedom,
-// computed once on the host: c2K = 2/(K+2), c4K = 4/(K+2), hN = (K+2)/2.
+// computed once on the host: c2K = 2/(K+2), c4K = 4/(K+2), hN = (K+2)/2,
+// sq2g = sqrt(2 gamma).
 template <typename T>
 struct KC {
-  T K, c2K, c4K, hN;
+  T K, c2K, c4K, hN, sq2g;
 };
 constexpr double kInvSqrtPi = 0.56418958354775628694807945156;
 
@@ -529,26 +530,30 @@ __device__ void gks_full_point_local(const KC<T> &kc, T mu_visc, T ajump, T dt, 
 
 // Cell-average primitives used by the low level (one set per cell and
 // implicit step): rho, u, v, p, 1/(2 lambda), sqrt(lambda), 1/sqrt(pi
-// lambda), sound speed c, 1/rho.
-constexpr int NPRIM = 9;
+// lambda), sound speed c.
 template <typename T>
 struct Prim {
-  T rho, u, v, p, i2l, sl, isp, c, ir;
+  T rho, u, v, p, i2l, sl, isp, c;
 };
+// c = sqrt(gamma p / rho); in FP64 from sqrt(lambda): p / rho = 1/(2 lambda)
+__device__ __forceinline__ float sound_speed(const KC<float> &, float gamma, float p, float ir, float, float) {
+  return sqrtf(gamma * p * ir);
+}
+__device__ __forceinline__ double sound_speed(const KC<double> &kc, double, double, double, double i2l, double sl) {
+  return kc.sq2g * (i2l * sl);
+}
 template <typename T>
 __device__ __forceinline__ Prim<T> prim_of(const T W[NV], T gamma, const KC<T> &kc) {
   Prim<T> q;
+  const T ir = d_rcp(W[0]);
   q.rho = W[0];
-  q.ir = T(1) / W[0];
-  q.u = W[1] * q.ir;
-  q.v = W[2] * q.ir;
-  T eps = W[3] - T(0.5) * q.rho * (q.u * q.u + q.v * q.v);
+  q.u = W[1] * ir;
+  q.v = W[2] * ir;
+  const T eps = W[3] - T(0.5) * q.rho * (q.u * q.u + q.v * q.v);
   q.p = (gamma - T(1)) * eps;
-  q.i2l = kc.c2K * eps * q.ir;
-  T lam = T(0.5) / q.i2l;
-  q.sl = d_sqrt(lam);
-  q.isp = d_rsqrt(lam) * T(kInvSqrtPi);
-  q.c = d_sqrt(gamma * q.p * q.ir);
+  q.i2l = kc.c2K * eps * ir;
+  sqrt_lambda(q.i2l, q.sl, q.isp);
+  q.c = sound_speed(kc, gamma, q.p, ir, q.i2l, q.sl);
   return q;
 }
 
@@ -566,19 +571,6 @@ __device__ __forceinline__ void kfvs_prims(T K, T rl, T unl, T utl, T i2ll, T sl
   F[1] = rl * ml[2] + rr * mr[2];
   F[2] = rl * ml[1] * utl + rr * mr[1] * utr;
   F[3] = rl * T(0.5) * (ml[3] + ml[1] * el) + rr * T(0.5) * (mr[3] + mr[1] * er);
-}
-
-// Euler normal flux F(U).n, global frame.
-template <typename T>
-__device__ __forceinline__ void euler_flux(T gamma, const T W[NV], T nx, T ny, T F[NV]) {
-  T ir = T(1) / W[0];
-  T u = W[1] * ir, v = W[2] * ir;
-  T p = (gamma - T(1)) * (W[3] - T(0.5) * W[0] * (u * u + v * v));
-  T un = u * nx + v * ny;
-  F[0] = W[0] * un;
-  F[1] = W[1] * un + p * nx;
-  F[2] = W[2] * un + p * ny;
-  F[3] = (W[3] + p) * un;
 }
 
 // F_n(U + dU) - F_n(U) of the Euler normal flux, written so that every

@@ -414,27 +414,24 @@ __device__ void gks_full_point_local(const KC<T> &kc, T mu_visc, T ajump, T dt, 
 }
 
 // cell primitives of the low level: rho, u, v, w, p, 1/(2 lambda),
-// sqrt(lambda), 1/sqrt(pi lambda), c, 1/rho
-constexpr int NPRIM = 10;
+// sqrt(lambda), 1/sqrt(pi lambda), c
 template <typename T>
 struct Prim {
-  T rho, u, v, w, p, i2l, sl, isp, c, ir;
+  T rho, u, v, w, p, i2l, sl, isp, c;
 };
 template <typename T>
 __device__ __forceinline__ Prim<T> prim_of(const T W[NV], T gamma, const KC<T> &kc) {
   Prim<T> q;
+  const T ir = dev::d_rcp(W[0]);
   q.rho = W[0];
-  q.ir = T(1) / W[0];
-  q.u = W[1] * q.ir;
-  q.v = W[2] * q.ir;
-  q.w = W[3] * q.ir;
+  q.u = W[1] * ir;
+  q.v = W[2] * ir;
+  q.w = W[3] * ir;
   const T eps = W[4] - T(0.5) * q.rho * (q.u * q.u + q.v * q.v + q.w * q.w);
   q.p = (gamma - T(1)) * eps;
-  q.i2l = kc.c2K * eps * q.ir;
-  const T lam = T(0.5) / q.i2l;
-  q.sl = d_sqrt(lam);
-  q.isp = d_rsqrt(lam) * T(dev::kInvSqrtPi);
-  q.c = d_sqrt(gamma * q.p * q.ir);
+  q.i2l = kc.c2K * eps * ir;
+  dev::sqrt_lambda(q.i2l, q.sl, q.isp);
+  q.c = dev::sound_speed(kc, gamma, q.p, ir, q.i2l, q.sl);
   return q;
 }
 
@@ -452,19 +449,6 @@ __device__ __forceinline__ void kfvs(T K, T rl, T unl, T v1l, T v2l, T i2ll, T s
   F[2] = rl * ml[1] * v1l + rr * mr[1] * v1r;
   F[3] = rl * ml[1] * v2l + rr * mr[1] * v2r;
   F[4] = rl * T(0.5) * (ml[3] + ml[1] * el) + rr * T(0.5) * (mr[3] + mr[1] * er);
-}
-
-template <typename T>
-__device__ __forceinline__ void euler_flux(T gamma, const T W[NV], const T n[3], T F[NV]) {
-  const T ir = T(1) / W[0];
-  const T u = W[1] * ir, v = W[2] * ir, w = W[3] * ir;
-  const T p = (gamma - T(1)) * (W[4] - T(0.5) * W[0] * (u * u + v * v + w * w));
-  const T un = u * n[0] + v * n[1] + w * n[2];
-  F[0] = W[0] * un;
-  F[1] = W[1] * un + p * n[0];
-  F[2] = W[2] * un + p * n[1];
-  F[3] = W[3] * un + p * n[2];
-  F[4] = (W[4] + p) * un;
 }
 
 // F_n(W + dW) - F_n(W), every term proportional to the increment

@@ -80,3 +80,40 @@ def test_one_thread_per_face_matches_the_oracle(flux, precision):
     from paper_2109_09965_gb300 import cgks
     assert cgks.Mesh(mesh).n_faces >= 100000
     compare(mesh, spec, state(mesh, 0.2, 0.3), precision, 0)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("scheme", [dict(n_sweeps=0), dict(n_sweeps=1), dict(n_implicit=1), dict(n_implicit=3, n_sweeps=3)])
+def test_low_level_passes_that_advance_the_state(scheme, precision):
+    """The last colour passes write the next implicit step's state; without
+    sweeps, and with other counts of steps and sweeps, a pass over all cells
+    does or the buffers end the other way round."""
+    mesh = MG.box(9, 7, jitter=0.15, seed=5, cells="mixed", quad_mask=lambda i, j: (2 * i + j) % 5 == 0,
+                  tags=(0, 1, 1, 1))
+    spec = dict(gamma=GAM, mu=0.01, cfl_hi=0.3, **scheme,
+                bcs=[dict(kind="slip"), dict(kind="farfield", rho=1.0, u=(0.2, 0.0), p=1 / GAM)])
+    compare(mesh, spec, state(mesh, 0.1, 0.2), precision, 2)
+    mesh = MG.box3(3, 3, 3, jitter=0.1, seed=2, cells="prism", tags=(0,) * 6)
+    spec = dict(spec, bcs=[dict(kind="farfield", rho=1.0, u=(0.2, 0.0, 0.0), p=1 / GAM)])
+    compare(mesh, spec, state(mesh, 0.1, 0.2), precision, 2)
+
+
+def test_one_and_four_lanes_per_cell_round_alike():
+    """A solve whose colours are swept with four lanes per cell alone and with
+    one in a large batch gives the same bits."""
+    from paper_2109_09965_gb300 import cgks
+    spec = dict(gamma=GAM, mu=0.15 / 1000, bcs=[dict(kind="noslip"), dict(kind="noslip", uw=(0.15, 0.0))])
+    meshes = [MG.cavity(n, seed=3 + n) for n in (21, 34, 160)]      # 51,200 cells: colours above 20,000
+    states = [state(m, 0.0, 0.1) for m in meshes]
+    srv = cgks.Server(2 << 30, precision="fp64", max_active=4, max_cycles=100)
+    gms = [cgks.Mesh(m) for m in meshes]
+    ids = [srv.submit(g, spec, W, 1e-300, 5) for g, W in zip(gms, states)]
+    while srv.step():
+        pass
+    for g, W, i in zip(gms, states, ids):
+        s = cgks.Solver(g, spec)
+        s.set_state(W)
+        s.pmg_cycle(5)
+        assert np.array_equal(srv.poll(i)[1], s.get_state()[0])
+        s.close()
+    srv.close()

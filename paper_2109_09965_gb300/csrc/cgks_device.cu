@@ -256,8 +256,8 @@ void enqueue_hi_eval(Batch *b, const TF *W, const TF *Wx, TF *Fout) {
       if (b->n_lim) recon(k_recon<TF, true>);
     });
     tuned_launch(b->tune, TK_FACE, b->stream, [&] {
-      if (b->n_smooth) face(k_face<TF, false, false>, face_threads<TF, false>());
-      if (b->n_lim) face(k_face<TF, true, false>, face_threads<TF, true>());
+      if (b->n_smooth) face(k_face<TF, false, false>, face_threads<TF>());
+      if (b->n_lim) face(k_face<TF, true, false>, face_threads<TF>());
     });
     return;
   }
@@ -266,10 +266,10 @@ void enqueue_hi_eval(Batch *b, const TF *W, const TF *Wx, TF *Fout) {
     else recon(k_recon<TF, false>);
   });
   tuned_launch(b->tune, TK_FACE, b->stream, [&] {
-    if (full && chr) face(k_face<TF, true, true>, face_threads<TF, true>());
-    else if (full) face(k_face<TF, true, false>, face_threads<TF, true>());
-    else if (chr) face(k_face<TF, false, true>, face_threads<TF, false>());
-    else face(k_face<TF, false, false>, face_threads<TF, false>());
+    if (full && chr) face(k_face<TF, true, true>, face_threads<TF>());
+    else if (full) face(k_face<TF, true, false>, face_threads<TF>());
+    else if (chr) face(k_face<TF, false, true>, face_threads<TF>());
+    else face(k_face<TF, false, false>, face_threads<TF>());
   });
 }
 

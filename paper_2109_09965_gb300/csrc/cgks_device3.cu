@@ -144,14 +144,20 @@ void hi_eval(Solver3 *s, const TF *W, const TF *Wx, TF *Fout) {
     else launch(s, KI_RECON, k_recon<TF>, gr, blk, fmesh<TF>(s), fpar<TF>(s), W, Wx, B.coef);
   });
   tuned_launch(s->tune, TK_FACE, s->stream, [&] {
-    auto go = [&](int threads, auto kern, auto... rest) {   // threads: of a face
-      launch(s, KI_FACE, kern, dim3(nblk(threads * s->F, shape_bs(fs))), dim3(shape_bs(fs)),
-             fmesh<TF>(s), fpar<TF>(s), W, (const TF *)B.coef, Fout, rest...);
+    auto go = [&](int threads, auto kern) {   // threads: of a face
+      launch(s, KI_FACE, kern, dim3(nblk(threads * s->F, shape_bs(fs))), dim3(shape_bs(fs)), fmesh<TF>(s), fpar<TF>(s),
+             W, (const TF *)B.coef, Fout, (const Ctl *)s->ctl, (const unsigned long long *)s->dt_bits);
     };
-    if (full) go(1, k_face_full<TF>, (const Ctl *)s->ctl, (const unsigned long long *)s->dt_bits);
-    else if constexpr (is_f32<TF>()) go(1, k_face<TF>);
-    else if (face_lanes(s->F) == 4) go(4, k_face_smooth<4>);
-    else go(1, k_face_smooth<1>);
+    if constexpr (is_f32<TF>()) {
+      if (full) go(1, k_face<TF, true>);
+      else go(1, k_face<TF, false>);
+    } else if (face_lanes(s->F) == 4) {
+      if (full) go(4, k_face_points<true, 4>);
+      else go(4, k_face_points<false, 4>);
+    } else {
+      if (full) go(1, k_face_points<true, 1>);
+      else go(1, k_face_points<false, 1>);
+    }
   });
 }
 

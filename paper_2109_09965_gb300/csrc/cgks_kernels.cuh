@@ -212,36 +212,41 @@ __host__ __device__ __forceinline__ bool is_wall_kind(int k) { return k == CGKS_
 //   + (4 c2 c3 + 4 c3 c4) M_xy + 4 c2^2 + c3^2 + 4 c4^2.
 // Weights w_k ~ gamma_k / (beta_k + eps)^2 (gamma_0 = g0, the rest
 // (1 - g0) / m); result (w_0/gamma_0)(P2 - sum gamma_k P1_k) + sum w_k P1_k.
+// Candidate 0 is the cell's own; candidate 1 + s, of face slot s, counts where
+// bit 1 + s of on is set (slots by a constant index: no local memory).
+__device__ __forceinline__ float quot(float a, float b) { return a / b; }
+__device__ __forceinline__ double quot(double a, double b) { return a * D::d_rcp(b); }
 template <typename T>
-__device__ __forceinline__ void weno_combine(const ParamsT<T> &P, T mxx, T mxy, T myy, int nk, const T lin[5][2][4],
-                                             T c[kNM][4]) {
+__device__ __forceinline__ void weno_combine(const ParamsT<T> &P, T mxx, T mxy, T myy, unsigned on,
+                                             const T lin[5][2][4], T c[kNM][4]) {
+  const int nk = __popc(on);
   const T g0 = P.weno_g0, eps = P.weno_eps;
-  const T gk = (T(1) - g0) / T(nk);
+  const T gk = quot(T(1) - g0, T(nk));
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
     const T c0 = c[0][v], c1 = c[1][v], c2 = c[2][v], c3 = c[3][v], c4 = c[4][v];
     const T b0 = c0 * c0 + c1 * c1 + (T(4) * c2 * c2 + c3 * c3) * mxx + (c3 * c3 + T(4) * c4 * c4) * myy +
                  (T(4) * c2 * c3 + T(4) * c3 * c4) * mxy + T(4) * c2 * c2 + c3 * c3 + T(4) * c4 * c4;
-    T w0 = g0 / ((b0 + eps) * (b0 + eps));
+    T w0 = quot(g0, (b0 + eps) * (b0 + eps));
     T wk[5], ws = w0;
     T lin0 = T(0), lin1 = T(0);
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
-      if (k < nk) {
+      if (on >> k & 1) {
         const T a0 = lin[k][0][v], a1 = lin[k][1][v];
         const T b = a0 * a0 + a1 * a1;
-        wk[k] = gk / ((b + eps) * (b + eps));
+        wk[k] = quot(gk, (b + eps) * (b + eps));
         ws += wk[k];
         lin0 += gk * a0;
         lin1 += gk * a1;
       }
     }
-    const T iws = T(1) / ws;
-    const T f0 = w0 * iws / g0;
+    const T iws = quot(T(1), ws);
+    const T f0 = quot(w0 * iws, g0);
     T sel0 = T(0), sel1 = T(0);
 #pragma unroll
     for (int k = 0; k < 5; ++k)
-      if (k < nk) {
+      if (on >> k & 1) {
         sel0 += wk[k] * iws * lin[k][0][v];
         sel1 += wk[k] * iws * lin[k][1][v];
       }
@@ -268,11 +273,12 @@ __device__ __forceinline__ void recon_at(const MeshT<T> &m, const ParamsT<T> &P,
   }
   // linear WENO candidates: h times the cell-mean gradients of the cell and its face neighbours
   T lin[WENO ? 5 : 1][2][4];
-  int nk = 1;
+  unsigned on = 1;
   if constexpr (WENO) {
     const T hi = T(1) / m.ih[i];
     for (int v = 0; v < 4; ++v) { lin[0][0][v] = hi * gxi[v]; lin[0][1][v] = hi * gyi[v]; }
   }
+#pragma unroll
   for (int s = 0; s < kMaxFace; ++s) {
     int fs = m.cface[s * n + i];
     if (fs == kNoFace) continue;
@@ -286,8 +292,8 @@ __device__ __forceinline__ void recon_at(const MeshT<T> &m, const ParamsT<T> &P,
       }
       if constexpr (WENO) {
         const T hi = T(1) / m.ih[i];
-        for (int v = 0; v < 4; ++v) { lin[nk][0][v] = hi * b1[v]; lin[nk][1][v] = hi * b2[v]; }
-        ++nk;
+        for (int v = 0; v < 4; ++v) { lin[1 + s][0][v] = hi * b1[v]; lin[1 + s][1][v] = hi * b2[v]; }
+        on |= 2u << s;
       }
     } else {
       int f = fs >= 0 ? fs : ~fs;
@@ -308,7 +314,7 @@ __device__ __forceinline__ void recon_at(const MeshT<T> &m, const ParamsT<T> &P,
   // gradient (too few neighbours, rank deficiency) carry no quadratic terms
   // in the operator and keep it; the others may be limited
   if constexpr (WENO)
-    if (m.wenok[i]) weno_combine(P, m.m2[i], m.m2[n + i], m.m2[2 * n + i], nk, lin, c);
+    if (m.wenok[i]) weno_combine(P, m.m2[i], m.m2[n + i], m.m2[2 * n + i], on, lin, c);
   for (int q = 0; q < kNM; ++q)
     for (int v = 0; v < 4; ++v) coef[(q * 4 + v) * n + i] = c[q][v];
 }
@@ -359,24 +365,26 @@ __device__ __forceinline__ void poly_point(const MeshT<T> &m, const T *__restric
   }
 }
 
-// the same with the gradient left in the cell's scaled coordinates (to be
-// multiplied by 1/h): from coef, or from the given coefficients where lim
-template <bool CHAR>
+// the same from given coefficients, the gradient left in the cell's scaled
+// coordinates (to be multiplied by 1/h)
 __device__ __forceinline__ void side_scaled(const MeshT<double> &m, const double *__restrict__ W,
-                                            const double *__restrict__ coef, const double (*lc)[4], bool lim, int i,
-                                            double x, double y, double val[4], double gx[4], double gy[4]) {
+                                            const double c[kNM][4], int i, double x, double y, double val[4],
+                                            double gx[4], double gy[4]) {
   const int n = m.nc;
   const double p2 = x * x - m.m2[i], p3 = x * y - m.m2[n + i], p4 = y * y - m.m2[2 * n + i];
   const double x2 = x + x, y2 = y + y;
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
-    double c[kNM];
-#pragma unroll
-    for (int q = 0; q < kNM; ++q) c[q] = CHAR && lim ? lc[q][v] : coef[(q * 4 + v) * n + i];
-    val[v] = W[v * n + i] + c[0] * x + c[1] * y + c[2] * p2 + c[3] * p3 + c[4] * p4;
-    gx[v] = c[0] + c[2] * x2 + c[3] * y;
-    gy[v] = c[1] + c[3] * x + c[4] * y2;
+    val[v] = W[v * n + i] + c[0][v] * x + c[1][v] * y + c[2][v] * p2 + c[3][v] * p3 + c[4][v] * p4;
+    gx[v] = c[0][v] + c[2][v] * x2 + c[3][v] * y;
+    gy[v] = c[1][v] + c[3][v] * x + c[4][v] * y2;
   }
+}
+__device__ __forceinline__ void load_coef(int n, const double *__restrict__ coef, int i, double c[kNM][4]) {
+#pragma unroll
+  for (int q = 0; q < kNM; ++q)
+#pragma unroll
+    for (int v = 0; v < 4; ++v) c[q][v] = coef[(q * 4 + v) * n + i];
 }
 
 // Compact WENO on characteristic variables (Section 4, shock reflection),
@@ -413,23 +421,28 @@ __device__ void char_side(const MeshT<T> &m, const ParamsT<T> &P, const T *__res
                         T(0.5) * b1 } };
   const T h = T(1) / m.ih[i];
   T lin[5][2][4];
-  int nk = 0;
-  auto add = [&](int j) {
+  unsigned on = 1;
+  auto add = [&](int k, int j) {
     T gx[4], gy[4];
+#pragma unroll
     for (int a = 0; a < 4; ++a) { gx[a] = Wx[a * n + j]; gy[a] = Wx[(4 + a) * n + j]; }
+#pragma unroll
     for (int a = 0; a < 4; ++a) {
       T sx = T(0), sy = T(0);
+#pragma unroll
       for (int b = 0; b < 4; ++b) { sx += L[a][b] * gx[b]; sy += L[a][b] * gy[b]; }
-      lin[nk][0][a] = h * sx;
-      lin[nk][1][a] = h * sy;
+      lin[k][0][a] = h * sx;
+      lin[k][1][a] = h * sy;
     }
-    ++nk;
   };
-  add(i);
+  add(0, i);
+#pragma unroll
   for (int sl = 0; sl < kMaxFace; ++sl) {
-    if (m.cface[sl * n + i] == kNoFace) continue;
     const int j = m.cnbr[sl * n + i];
-    if (j >= 0) add(j);
+    if (m.cface[sl * n + i] != kNoFace && j >= 0) {
+      add(1 + sl, j);
+      on |= 2u << sl;
+    }
   }
   T cq[kNM][4];
   for (int q = 0; q < kNM; ++q) {
@@ -441,7 +454,7 @@ __device__ void char_side(const MeshT<T> &m, const ParamsT<T> &P, const T *__res
       cq[q][a] = acc;
     }
   }
-  weno_combine(P, m.m2[i], m.m2[n + i], m.m2[2 * n + i], nk, lin, cq);
+  weno_combine(P, m.m2[i], m.m2[n + i], m.m2[2 * n + i], on, lin, cq);
   for (int q = 0; q < kNM; ++q)
     for (int b = 0; b < 4; ++b) {
       T acc = T(0);
@@ -476,10 +489,10 @@ __device__ __forceinline__ void lo_ghost(const ParamsT<T> &P, int tag, T nx, T n
 // face; writes the weighted sums F0, F1, Wc, Wt (global frame) per face:
 //   out[(k*4 + v)*nf + f], k = 0 F0, 1 F1, 2 Wc, 3 Wt.
 // Two forms.  face_raw_at: both Gauss points of a face in one thread, raw
-// moments in the face frame; the full flux, and the FP32 of the mixed path
-// (whose rounding it fixes: the implicit solves of a V-cycle carry a changed
-// FP32 rounding into every cell, and the mixed results are to stay what they
-// are).  face_smooth_at: the FP64 smooth flux.
+// moments in the face frame: the FP32 of the mixed path (whose rounding it
+// fixes: the implicit solves of a V-cycle carry a changed FP32 rounding into
+// every cell, and the mixed results are to stay what they are).  face_point_at:
+// FP64.
 template <typename T, bool FULL, bool CHAR>
 __device__ __forceinline__ void face_raw_at(const MeshT<T> &m, const ParamsT<T> &P, const T *__restrict__ W,
                                         const T *__restrict__ Wx, const T *__restrict__ coef, T *__restrict__ out,
@@ -572,7 +585,7 @@ __device__ __forceinline__ void face_raw_at(const MeshT<T> &m, const ParamsT<T> 
   for (int k = 0; k < 4; ++k)
     for (int v = 0; v < 4; ++v) out[(k * 4 + v) * nf + f] = acc[k][v];
 }
-// The FP64 smooth flux.  One thread evaluates Gauss point k of face f; in the
+// The FP64 flux.  One thread evaluates Gauss point k of face f; in the
 // pair of lanes of a face lane 0 collects and stores F0 and F1, lane 1 Wc and
 // Wt.  GB300's FP64 units take 64 clocks of a sub-core per warp instruction
 // whatever the number of active lanes, so the FP64 instructions of a thread
@@ -580,8 +593,10 @@ __device__ __forceinline__ void face_raw_at(const MeshT<T> &m, const ParamsT<T> 
 // the global frame before the moments need them, the moments close about the
 // mean velocity (gks_smooth), erf and exp share one argument (half01), and
 // one point per thread halves the serial chain of a small mesh.  Bound by the
-// FP64 pipe.  Before (face_raw_at) and now: 319 -> 140 us on 90,368 faces,
-// 66 -> 23 us on 208.
+// FP64 pipe.  Smooth flux, before (face_raw_at) and now: 319 -> 140 us on
+// 90,368 faces, 66 -> 23 us on 208; full flux (gks_full): 167 -> 75 us on 10,088
+// faces; with characteristic WENO, each lane limiting one side, 217 -> 85 us on
+// 7,350.
 __device__ __forceinline__ void pair_sum_store(const double F0[4], const double F1[4], const double Wc[4],
                                                const double Wt[4], int k, unsigned pair, double *__restrict__ out,
                                                int nf, int f) {
@@ -595,38 +610,49 @@ __device__ __forceinline__ void pair_sum_store(const double F0[4], const double 
 #pragma unroll
   for (int q = 0; q < 8; ++q) out[(k * 8 + q) * nf + f] = 0.5 * a[q];
 }
-template <bool CHAR>
-__device__ __forceinline__ void face_smooth_at(const MeshT<double> &m, const ParamsT<double> &P,
-                                               const double *__restrict__ W, const double *__restrict__ Wx,
-                                               const double *__restrict__ coef, double *__restrict__ out, const int f,
-                                               const int k) {
+template <bool FULL, bool CHAR>
+__device__ __forceinline__ void face_point_at(const MeshT<double> &m, const ParamsT<double> &P,
+                                              const double *__restrict__ W, const double *__restrict__ Wx,
+                                              const double *__restrict__ coef, double *__restrict__ out,
+                                              const Ctl *ctl, const unsigned long long *dt_bits, const int f,
+                                              const int k) {
   const int sid = m.fsid[f];
   if (sid < 0) return;   // free face space of a batch
-  if (P.slim && P.slim[sid] != 0) return;   // the other flux class's launch
+  if (P.slim && (P.slim[sid] != 0) != FULL) return;   // the other flux class's launch
   const unsigned pair = 3u << (threadIdx.x & 30);      // the lanes of this face
   const int nf = m.nf;
   const int c0 = m.fc0[f], c1 = m.fc1[f];
   const double nx = m.fn[f], ny = m.fn[nf + f], ajump = m.fjump[f];
-  // characteristic WENO: the two sides' polynomials limited for this face
-  double cs0[CHAR ? kNM : 1][4], cs1[CHAR ? kNM : 1][4];
-  bool lim0 = false, lim1 = false;
+  // the two sides' polynomials.  Characteristic WENO limits them for this
+  // face: lane k that of side k, exchanged within the pair
+  double cL[kNM][4], cR[kNM][4];
   if constexpr (CHAR) {
     double wref[4];
     for (int v = 0; v < 4; ++v) wref[v] = c1 >= 0 ? 0.5 * (W[v * m.nc + c0] + W[v * m.nc + c1]) : W[v * m.nc + c0];
-    lim0 = m.wenok[c0] != 0;
-    if (lim0) char_side(m, P, W, Wx, coef, c0, wref, nx, ny, cs0);
-    lim1 = c1 >= 0 && m.wenok[c1] != 0;
-    if (lim1) char_side(m, P, W, Wx, coef, c1, wref, nx, ny, cs1);
+    const int ci = k && c1 >= 0 ? c1 : c0;
+    double own[kNM][4];
+    if (m.wenok[ci]) char_side(m, P, W, Wx, coef, ci, wref, nx, ny, own);
+    else load_coef(m.nc, coef, ci, own);
+#pragma unroll
+    for (int q = 0; q < kNM; ++q)
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        const double other = __shfl_xor_sync(pair, own[q][v], 1);
+        cL[q][v] = k ? other : own[q][v];
+        cR[q][v] = k ? own[q][v] : other;
+      }
+  } else {
+    load_coef(m.nc, coef, c0, cL);
+    if (c1 >= 0) load_coef(m.nc, coef, c1, cR);
   }
-  // the two sides: value and scaled gradient, global frame
+  // value and scaled gradient, global frame
   double wL[4], gL[2][4], wR[4], gR[2][4], wl[4], wr[4];
-  side_scaled<CHAR>(m, W, coef, cs0, lim0, c0, m.fxi[(2 * k) * nf + f], m.fxi[(2 * k + 1) * nf + f], wL, gL[0], gL[1]);
+  side_scaled(m, W, cL, c0, m.fxi[(2 * k) * nf + f], m.fxi[(2 * k + 1) * nf + f], wL, gL[0], gL[1]);
   D::rot_in(nx, ny, wL, wl);
   const double ihL = m.ih[c0];
   double ihR = ihL;
   if (c1 >= 0) {
-    side_scaled<CHAR>(m, W, coef, cs1, lim1, c1, m.fxi[(4 + 2 * k) * nf + f], m.fxi[(5 + 2 * k) * nf + f], wR, gR[0],
-                      gR[1]);
+    side_scaled(m, W, cR, c1, m.fxi[(4 + 2 * k) * nf + f], m.fxi[(5 + 2 * k) * nf + f], wR, gR[0], gR[1]);
     D::rot_in(nx, ny, wR, wr);
     ihR = m.ih[c1];
   } else {
@@ -650,12 +676,9 @@ __device__ __forceinline__ void face_smooth_at(const MeshT<double> &m, const Par
       D::rot_in(nx, ny, wR, wr);
     }
   }
-  // W^c from the two half ranges; its slopes: the mean of the sides plus,
-  // along n, alpha / delta times the jump
-  double wc[4], Wc[4], G[2][4], F0[4], F1[4], Wt[4];
-  D::half_state<double, false>(P.kc, wl, +1, wc);
-  D::half_state<double, true>(P.kc, wr, -1, wc);
-  D::rot_out(nx, ny, wc, Wc);
+  // slopes of the equilibrium at W^c: the mean of the sides plus, along n,
+  // alpha / delta times the jump
+  double Wc[4], G[2][4], F0[4], F1[4], Wt[4];
   const double hl = 0.5 * ihL, hr = 0.5 * ihR, ax = ajump * nx, ay = ajump * ny;
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
@@ -663,19 +686,47 @@ __device__ __forceinline__ void face_smooth_at(const MeshT<double> &m, const Par
     G[0][v] = hl * gL[0][v] + hr * gR[0][v] + ax * d;
     G[1][v] = hl * gL[1][v] + hr * gR[1][v] + ay * d;
   }
-  D::gks_smooth(P.kc, P.mu[sid], nx, ny, Wc, G, F0, F1, Wt);
+  if constexpr (FULL) {
+    // each side's derivatives along n and t in the face frame
+    double dnl[4], dtl[4], dnr[4], dtr[4], t0[4], t1[4];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      t0[v] = ihL * (nx * gL[0][v] + ny * gL[1][v]);
+      t1[v] = ihL * (nx * gL[1][v] - ny * gL[0][v]);
+    }
+    D::rot_in(nx, ny, t0, dnl);
+    D::rot_in(nx, ny, t1, dtl);
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      t0[v] = ihR * (nx * gR[0][v] + ny * gR[1][v]);
+      t1[v] = ihR * (nx * gR[1][v] - ny * gR[0][v]);
+    }
+    D::rot_in(nx, ny, t0, dnr);
+    D::rot_in(nx, ny, t1, dtr);
+    const double dt = dt_of(ctl, dt_bits, sid, P.cfl_hi);   // the full flux integrates over the step
+    D::gks_full(P.kc, P.mu[sid], dt, P.tau_c1, P.tau_c2, nx, ny, wl, wr, dnl, dtl, dnr, dtr, G, F0, F1, Wc, Wt);
+  } else {
+    // W^c from the two half ranges
+    double wc[4];
+    D::half_state<double, false>(P.kc, wl, +1, wc);
+    D::half_state<double, true>(P.kc, wr, -1, wc);
+    D::rot_out(nx, ny, wc, Wc);
+    D::gks_smooth(P.kc, P.mu[sid], nx, ny, Wc, G, F0, F1, Wt);
+  }
   pair_sum_store(F0, F1, Wc, Wt, k, pair, out, nf, f);
 }
 // threads a face takes
-template <typename T, bool FULL> __host__ __device__ constexpr int face_threads() { return FULL || is_f32<T>() ? 1 : 2; }
+template <typename T> __host__ __device__ constexpr int face_threads() { return is_f32<T>() ? 1 : 2; }
 template <typename T, bool FULL, bool CHAR>
 __global__ void __launch_bounds__(kMaxShapeBlock) k_face(MeshT<T> m, ParamsT<T> P, const T *W,
                                                          const T *Wx, const T *coef,
                                                          T *out, const Ctl *ctl,
                                                          const unsigned long long *dt_bits) {
   pdl_enter();
-  if constexpr (face_threads<T, FULL>() == 2)
-    for_items(2 * m.nf, [&](int i) { face_smooth_at<CHAR>(m, P, W, Wx, coef, out, i >> 1, i & 1); });
+  if constexpr (!is_f32<T>())
+    for_items(2 * m.nf, [&](int i) {
+      face_point_at<FULL, CHAR>(m, P, W, Wx, coef, out, ctl, dt_bits, i >> 1, i & 1);
+    });
   else
     for_items(m.nf, [&](int f) { face_raw_at<T, FULL, CHAR>(m, P, W, Wx, coef, out, ctl, dt_bits, f); });
   pdl_exit();

@@ -183,39 +183,54 @@ __device__ __forceinline__ void farfield_ghost(const ParamsT<T> &P, int tag, con
 // second derivatives, each multi-index once.  w ~ gamma / (beta + eps)^2,
 // gamma_0 = g0, the rest (1 - g0)/nk; result
 // (w_0 / gamma_0)(P2 - sum gamma_k P1_k) + sum w_k P1_k.
+// Candidate 0 is the cell's own; candidate 1 + s, of face slot s, counts where
+// bit 1 + s of on is set (slots by a constant index: no local memory).
+__device__ __forceinline__ float quot(float a, float b) { return a / b; }
+__device__ __forceinline__ double quot(double a, double b) { return a * dev::d_rcp(b); }
 template <typename T>
-__device__ __forceinline__ void weno_combine3(const ParamsT<T> &P, const T M[6], int nk, const T lin[7][3][NV],
+__device__ __forceinline__ void weno_combine3(const ParamsT<T> &P, const T M[6], unsigned on, const T lin[7][3][NV],
                                               T c[kNM3][NV]) {
+  const int nk = __popc(on);
   const T g0 = P.weno_g0, eps = P.weno_eps;
-  const T gk = (T(1) - g0) / T(nk);
+  const T gk = quot(T(1) - g0, T(nk));
   // symmetric M: xx xy xz yy yz zz
   const T Mx[3][3] = { { M[0], M[1], M[2] }, { M[1], M[3], M[4] }, { M[2], M[4], M[5] } };
+#pragma unroll
   for (int v = 0; v < NV; ++v) {
     const T q[kNM3] = { c[0][v], c[1][v], c[2][v], c[3][v], c[4][v], c[5][v], c[6][v], c[7][v], c[8][v] };
     const T G[3][3] = { { T(2) * q[3], q[4], q[5] }, { q[4], T(2) * q[6], q[7] }, { q[5], q[7], T(2) * q[8] } };
     T b0 = q[0] * q[0] + q[1] * q[1] + q[2] * q[2];
+#pragma unroll
     for (int d = 0; d < 3; ++d)
+#pragma unroll
       for (int a = 0; a < 3; ++a)
+#pragma unroll
         for (int e = 0; e < 3; ++e) b0 += G[d][a] * Mx[a][e] * G[d][e];
     b0 += T(4) * q[3] * q[3] + q[4] * q[4] + q[5] * q[5] + T(4) * q[6] * q[6] + q[7] * q[7] + T(4) * q[8] * q[8];
-    const T w0 = g0 / ((b0 + eps) * (b0 + eps));
+    const T w0 = quot(g0, (b0 + eps) * (b0 + eps));
     T ws = w0, wk[7];
     T l[3] = { T(0), T(0), T(0) };
+#pragma unroll
     for (int k = 0; k < 7; ++k) {
-      if (k >= nk) break;
+      if (!(on >> k & 1)) continue;
       const T b = lin[k][0][v] * lin[k][0][v] + lin[k][1][v] * lin[k][1][v] + lin[k][2][v] * lin[k][2][v];
-      wk[k] = gk / ((b + eps) * (b + eps));
+      wk[k] = quot(gk, (b + eps) * (b + eps));
       ws += wk[k];
+#pragma unroll
       for (int d = 0; d < 3; ++d) l[d] += gk * lin[k][d][v];
     }
-    const T iws = T(1) / ws;
-    const T f0 = w0 * iws / g0;
+    const T iws = quot(T(1), ws);
+    const T f0 = quot(w0 * iws, g0);
     T sel[3] = { T(0), T(0), T(0) };
+#pragma unroll
     for (int k = 0; k < 7; ++k) {
-      if (k >= nk) break;
+      if (!(on >> k & 1)) continue;
+#pragma unroll
       for (int d = 0; d < 3; ++d) sel[d] += wk[k] * iws * lin[k][d][v];
     }
+#pragma unroll
     for (int d = 0; d < 3; ++d) c[d][v] = f0 * (q[d] - l[d]) + sel[d];
+#pragma unroll
     for (int r = 3; r < kNM3; ++r) c[r][v] = f0 * q[r];
   }
 }
@@ -243,12 +258,15 @@ __device__ __forceinline__ void recon_at(const MeshT<T> &m, const ParamsT<T> &P,
     for (int v = 0; v < NV; ++v) c[q][v] = o0 * gi[0][v] + o1 * gi[1][v] + o2 * gi[2][v];
   }
   T lin[WENO ? 7 : 1][3][NV];
-  int nk = 1;
+  unsigned on = 1;
   if constexpr (WENO) {
     const T h = T(1) / m.ih[i];
+#pragma unroll
     for (int v = 0; v < NV; ++v)
+#pragma unroll
       for (int d = 0; d < 3; ++d) lin[0][d][v] = h * gi[d][v];
   }
+#pragma unroll (WENO ? kMaxFace3 : 1)
   for (int s = 0; s < kMaxFace3; ++s) {
     const int fs = m.cface[s * n + i];
     if (fs == kNoFace) continue;
@@ -263,9 +281,11 @@ __device__ __forceinline__ void recon_at(const MeshT<T> &m, const ParamsT<T> &P,
       }
       if constexpr (WENO) {
         const T h = T(1) / m.ih[i];
+#pragma unroll
         for (int v = 0; v < NV; ++v)
-          for (int d = 0; d < 3; ++d) lin[nk][d][v] = h * b[d][v];
-        ++nk;
+#pragma unroll
+          for (int d = 0; d < 3; ++d) lin[1 + s][d][v] = h * b[d][v];
+        on |= 2u << s;
       }
     } else {
       const int f = fs >= 0 ? fs : ~fs;
@@ -288,7 +308,7 @@ __device__ __forceinline__ void recon_at(const MeshT<T> &m, const ParamsT<T> &P,
   if constexpr (WENO) {
     if (wenok[i]) {
       const T M[6] = { m.m2[i], m.m2[n + i], m.m2[2 * n + i], m.m2[3 * n + i], m.m2[4 * n + i], m.m2[5 * n + i] };
-      weno_combine3(P, M, nk, lin, c);
+      weno_combine3(P, M, on, lin, c);
     }
   }
 #pragma unroll
@@ -361,8 +381,8 @@ __device__ __forceinline__ void recon_point(const MeshT<T> &m, const T *__restri
 // out[f][k*5 + v], k = 0 F0, 1 F1, 2 Wc, 3 Wt, weighted sums, global frame:
 // one run of kFO values per face (AoS), so that the cells gathering a face
 // read it in one piece.
-// Two forms, as in 2-D: face_raw_at (raw moments in the face frame: the full
-// flux and the FP32 of the mixed path) and face_smooth_at (FP64 smooth flux).
+// Two forms, as in 2-D: face_raw_at (raw moments in the face frame: the FP32
+// of the mixed path) and face_points_at (FP64).
 template <typename T, bool FULL>
 __device__ __forceinline__ void face_raw_at(const MeshT<T> &m, const ParamsT<T> &P, const T *__restrict__ W,
                                         const T *__restrict__ coef, T *__restrict__ out, const Ctl *ctl,
@@ -462,12 +482,13 @@ __device__ __forceinline__ void face_raw_at(const MeshT<T> &m, const ParamsT<T> 
     for (int v = 0; v < NV; ++v) o[k * NV + v] = acc[k][v];
   vstore<T, kFO>(out + static_cast<size_t>(f) * kFO, o);
 }
-// The FP64 smooth flux by the 2-D face_smooth_at's scheme.  LANES threads
-// share a face's 3 or 4 Gauss points.
-template <int LANES>
-__device__ __forceinline__ void face_smooth_at(const MeshT<double> &m, const ParamsT<double> &P,
+// The FP64 flux by the 2-D face_point_at's scheme.  LANES threads share a
+// face's 3 or 4 Gauss points.
+template <bool FULL, int LANES>
+__device__ __forceinline__ void face_points_at(const MeshT<double> &m, const ParamsT<double> &P,
                                                const double *__restrict__ W, const double *__restrict__ coef,
-                                               double *__restrict__ out, const int f, const int lane) {
+                                               double *__restrict__ out, const Ctl *ctl,
+                                               const unsigned long long *dt_bits, const int f, const int lane) {
   using T = double;
   const int nf = m.nf;
   const int c0 = m.fc0[f], c1 = m.fc1[f], ng = m.fng[f];
@@ -510,13 +531,9 @@ __device__ __forceinline__ void face_smooth_at(const MeshT<double> &m, const Par
       wall_ghost(P, tag, F, wL, gL, wR, gR);
       D3::rot_in(F, wR, wr);
     }
-    T F0[NV], F1[NV], Wc[NV], Wt[NV];
-    // W^c from the two half ranges; its slopes: the mean of the sides
-    // plus, along n, alpha / delta times the jump
-    T wc[NV], G[3][NV];
-    D3::half_state<T, false>(P.kc, wl, +1, wc);
-    D3::half_state<T, true>(P.kc, wr, -1, wc);
-    D3::rot_out(F, wc, Wc);
+    // slopes of the equilibrium at W^c: the mean of the sides plus, along
+    // n, alpha / delta times the jump
+    T Wc[NV], G[3][NV], F0[NV], F1[NV], Wt[NV];
     const T hl = T(0.5) * ihL, hr = T(0.5) * ihR;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
@@ -524,7 +541,31 @@ __device__ __forceinline__ void face_smooth_at(const MeshT<double> &m, const Par
 #pragma unroll
       for (int v = 0; v < NV; ++v) G[d][v] = hl * gL[d][v] + hr * gR[d][v] + aj * (wR[v] - wL[v]);
     }
-    D3::gks_smooth(P.kc, P.mu, F.e[0], Wc, G, F0, F1, Wt);
+    if constexpr (FULL) {
+      // each side's derivatives along the face axes, in the face frame
+      T dl[3][NV], dr[3][NV];
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        T t[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v)
+          t[v] = ihL * (F.e[a][0] * gL[0][v] + F.e[a][1] * gL[1][v] + F.e[a][2] * gL[2][v]);
+        D3::rot_in(F, t, dl[a]);
+#pragma unroll
+        for (int v = 0; v < NV; ++v)
+          t[v] = ihR * (F.e[a][0] * gR[0][v] + F.e[a][1] * gR[1][v] + F.e[a][2] * gR[2][v]);
+        D3::rot_in(F, t, dr[a]);
+      }
+      const T dt = dt_of(ctl, dt_bits, P.cfl_hi);   // the full flux integrates over the step
+      D3::gks_full(P.kc, P.mu, dt, P.tau_c1, P.tau_c2, F, wl, wr, dl, dr, G, F0, F1, Wc, Wt);
+    } else {
+      // W^c from the two half ranges
+      T wc[NV];
+      D3::half_state<T, false>(P.kc, wl, +1, wc);
+      D3::half_state<T, true>(P.kc, wr, -1, wc);
+      D3::rot_out(F, wc, Wc);
+      D3::gks_smooth(P.kc, P.mu, F.e[0], Wc, G, F0, F1, Wt);
+    }
     const T wk = m.fw[k * nf + f];
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
@@ -562,29 +603,23 @@ __device__ __forceinline__ void face_smooth_at(const MeshT<double> &m, const Par
 // in one thread: 358 and 2809 us).
 constexpr int64_t kFaceLanes4 = 100000;
 inline int face_lanes(int64_t n_faces) { return n_faces < kFaceLanes4 ? 4 : 1; }
-template <typename T>
+// FP32: one thread per face
+template <typename T, bool FULL>
 __global__ void __launch_bounds__(kMaxShapeBlock)
-    k_face(MeshT<T> m, ParamsT<T> P, const T *W, const T *coef,
-           T *out) {
+    k_face(MeshT<T> m, ParamsT<T> P, const T *W, const T *coef, T *out,
+           const Ctl *ctl, const unsigned long long *dt_bits) {
   pdl_enter();
-  for_items(m.nf, [&](int f) { face_raw_at<T, false>(m, P, W, coef, out, nullptr, nullptr, f); });
+  for_items(m.nf, [&](int f) { face_raw_at<T, FULL>(m, P, W, coef, out, ctl, dt_bits, f); });
   pdl_exit();
 }
-template <int LANES>
+// FP64
+template <bool FULL, int LANES>
 __global__ void __launch_bounds__(kMaxShapeBlock)
-    k_face_smooth(MeshT<double> m, ParamsT<double> P, const double *W,
-                  const double *coef, double *out) {
+    k_face_points(MeshT<double> m, ParamsT<double> P, const double *W, const double *coef,
+                  double *out, const Ctl *ctl, const unsigned long long *dt_bits) {
   pdl_enter();
-  for_items(LANES * m.nf, [&](int i) { face_smooth_at<LANES>(m, P, W, coef, out, i / LANES, i % LANES); });
-  pdl_exit();
-}
-// the full flux of Eq. (2nd-flux): the same face loop, with the step's dt
-template <typename T>
-__global__ void __launch_bounds__(kMaxShapeBlock)
-    k_face_full(MeshT<T> m, ParamsT<T> P, const T *W, const T *coef,
-                T *out, const Ctl *ctl, const unsigned long long *dt_bits) {
-  pdl_enter();
-  for_items(m.nf, [&](int f) { face_raw_at<T, true>(m, P, W, coef, out, ctl, dt_bits, f); });
+  for_items(LANES * m.nf,
+            [&](int i) { face_points_at<FULL, LANES>(m, P, W, coef, out, ctl, dt_bits, i / LANES, i % LANES); });
   pdl_exit();
 }
 

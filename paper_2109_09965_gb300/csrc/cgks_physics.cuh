@@ -333,9 +333,13 @@ __device__ __forceinline__ void half_state(const KC<T> &kc, const T W[NV], int s
 // traction mu (dU/dn + grad U_n - (2/N) div U n) with the heat flux
 // mu (N/2 + 1) d theta / dn.  About 110 FP64 instructions where the tables
 // of raw moments took about 650.
-template <typename T>
-__device__ __forceinline__ void gks_smooth(const KC<T> &kc, T mu_visc, T nx, T ny, const T Wc[NV],
-                                           const T G[2][NV], T F0[NV], T F1[NV], T Wt[NV]) {
+//
+// gks_centre: Fe the Euler flux of Wc, F1 = <u A psi> and Wt = <A psi> (times
+// rho), Hv the viscous part per unit viscosity.
+__device__ __forceinline__ void gks_centre(const KC<double> &kc, double nx, double ny, const double Wc[NV],
+                                           const double G[2][NV], bool visc, double Fe[NV], double F1[NV],
+                                           double Wt[NV], double Hv[NV], double &p) {
+  using T = double;
   const T c2 = kc.c2K, hN = kc.hN;
   const T rho = Wc[0], ir = d_rcp(rho);
   const T u = Wc[1] * ir, v = Wc[2] * ir, E = Wc[3] * ir;
@@ -353,7 +357,8 @@ __device__ __forceinline__ void gks_smooth(const KC<T> &kc, T mu_visc, T nx, T n
   const T ut = -(u * ux[0] + v * ux[1] + th * r[0] + Tx[0]);
   const T vt = -(u * vx[0] + v * vx[1] + th * r[1] + Tx[1]);
   const T Tt = -(u * Tx[0] + v * Tx[1] + c2 * th * div);
-  const T un = u * nx + v * ny, mn = rho * un, p = rho * th;
+  const T un = u * nx + v * ny, mn = rho * un;
+  p = rho * th;
   const T a0 = rho * rt, ek = u * ut + v * vt, ei = ek + hN * Tt;
   Wt[0] = a0;
   Wt[1] = u * a0 + rho * ut;
@@ -364,18 +369,26 @@ __device__ __forceinline__ void gks_smooth(const KC<T> &kc, T mu_visc, T nx, T n
   F1[1] = u * mt + mn * ut + nx * pt;
   F1[2] = v * mt + mn * vt + ny * pt;
   F1[3] = H * mt + mn * (ei + Tt);
-  F0[0] = mn;
-  F0[1] = mn * u + p * nx;
-  F0[2] = mn * v + p * ny;
-  F0[3] = mn * H;
-  if (mu_visc != T(0)) {
+  Fe[0] = mn;
+  Fe[1] = mn * u + p * nx;
+  Fe[2] = mn * v + p * ny;
+  Fe[3] = mn * H;
+  if (visc) {
     const T s = ux[1] + vx[0], d = c2 * div;
-    const T sx = mu_visc * ((T(2) * ux[0] - d) * nx + s * ny);
-    const T sy = mu_visc * (s * nx + (T(2) * vx[1] - d) * ny);
-    F0[1] -= sx;
-    F0[2] -= sy;
-    F0[3] -= u * sx + v * sy + mu_visc * (hN + T(1)) * (Tx[0] * nx + Tx[1] * ny);
+    Hv[0] = T(0);
+    Hv[1] = (T(2) * ux[0] - d) * nx + s * ny;
+    Hv[2] = s * nx + (T(2) * vx[1] - d) * ny;
+    Hv[3] = u * Hv[1] + v * Hv[2] + (hN + T(1)) * (Tx[0] * nx + Tx[1] * ny);
   }
+}
+__device__ __forceinline__ void gks_smooth(const KC<double> &kc, double mu_visc, double nx, double ny,
+                                           const double Wc[NV], const double G[2][NV], double F0[NV], double F1[NV],
+                                           double Wt[NV]) {
+  double Hv[NV], p;
+  gks_centre(kc, nx, ny, Wc, G, mu_visc != 0.0, F0, F1, Wt, Hv, p);
+  if (mu_visc != 0.0)
+#pragma unroll
+    for (int v = 1; v < NV; ++v) F0[v] -= mu_visc * Hv[v];
 }
 
 // ---------------- full flux, Eq. (2nd-flux) ----------------
@@ -526,6 +539,161 @@ __device__ void gks_full_point_local(const KC<T> &kc, T mu_visc, T ajump, T dt, 
     Wc[v] = T(2) * Wh[v] - Wd[v];
     Wt[v] = T(2) * (Wd[v] - Wh[v]) * idt;
   }
+}
+
+// ---- full flux, FP64 ----
+// Eq. (2nd-flux) from moments taken about the mean velocity in the tangential
+// and internal directions and over the half range of the normal one.  A
+// micro-slope along direction j is
+//   a_j = d_j rho / rho + c.d_j U / theta + ((c^2 + xi^2) / theta - N) phi_j / 2,
+// phi_j = d_j theta / theta; given the normal velocity u, its mean over the
+// other directions is the quadratic a0 + a1 u + a2 u^2 below, and the means of
+// S = u a_n + v a_t (+ A) times 1, c_t and c_t^2 + xi^2 are the polynomials
+// p, q and (N - 1) theta [p + phi_n u + phi_E] + 2 theta d_t U_t, so that only
+// the half moments <u^k>, k <= 6, enter.  About 200 FP64 instructions a side
+// where the moment tables took about 900.
+struct CentralSlope {
+  double a0, a1, a2;
+};
+__device__ __forceinline__ CentralSlope central_slope(double U, double ith, double r, double dU, double phi) {
+  CentralSlope a;
+  const double g = phi * ith;
+  a.a2 = 0.5 * g;
+  a.a1 = dU * ith - g * U;
+  a.a0 = r - 0.5 * phi - U * (a.a1 + a.a2 * U);
+  return a;
+}
+// One side's share of the rho-weighted moments, over u > 0 (sgn = +1) or u < 0
+// (-1); X[k] for k = 0: 1, 1: a.u, 2: a.u + A, of psi (P) and u psi (Q).
+// Returns the pressure.
+template <bool ADD>
+__device__ __forceinline__ double full_side(const KC<double> &kc, const double W[NV], const double dn[NV],
+                                            const double dt[NV], int sgn, double P[3][NV], double Q[3][NV]) {
+  const double c2 = kc.c2K, N1 = 2.0 * kc.hN - 1.0;
+  const double rho = W[0], ir = d_rcp(rho);
+  const double U = W[1] * ir, V = W[2] * ir, E = W[3] * ir;
+  const double th = c2 * (E - 0.5 * (U * U + V * V)), ith = d_rcp(th);
+  double sl, isp, mu[7];
+  sqrt_lambda(th, sl, isp);
+  half_moments<double, 6>(U, th, sl, isp, sgn, mu);
+  // derivatives of ln rho, U, V, theta along n and t, and in time (Euler)
+  const double rn = dn[0] * ir, rt = dt[0] * ir;
+  const double Un = dn[1] * ir - U * rn, Ut = dt[1] * ir - U * rt;
+  const double Vn = dn[2] * ir - V * rn, Vt = dt[2] * ir - V * rt;
+  const double Tn = c2 * (dn[3] * ir - E * rn - U * Un - V * Vn), Tt = c2 * (dt[3] * ir - E * rt - U * Ut - V * Vt);
+  const double div = Un + Vt;
+  const double r_ = -(U * rn + V * rt + div);
+  const double U_ = -(U * Un + V * Ut + th * rn + Tn);
+  const double V_ = -(U * Vn + V * Vt + th * rt + Tt);
+  const double T_ = -(U * Tn + V * Tt + c2 * th * div);
+  const double fn = Tn * ith, ft = Tt * ith, f_ = T_ * ith;
+  const CentralSlope an = central_slope(U, ith, rn, Un, fn), at = central_slope(U, ith, rt, Ut, ft),
+                     aA = central_slope(U, ith, r_, U_, f_);
+  const double Nt = N1 * th, e2 = V * V + Nt;
+  // S = u a_n + v a_t
+  const double p0 = V * at.a0 + Vt, p1 = an.a0 + V * at.a1, p2 = an.a1 + V * at.a2, p3 = an.a2;
+  const double q2 = 0.5 * ft, q1 = Vn + Ut - ft * U, q0 = V * Vt + th * (rt + q2) - U * (Ut - q2 * U);
+  const double k1 = Nt * fn, k0 = Nt * V * ft + 2.0 * th * Vt, kA = Nt * f_;
+  double S[4], A[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    S[k] = p0 * mu[k] + p1 * mu[k + 1] + p2 * mu[k + 2] + p3 * mu[k + 3];
+    A[k] = aA.a0 * mu[k] + aA.a1 * mu[k + 1] + aA.a2 * mu[k + 2];
+  }
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {   // weight 1 (P), u (Q)
+    double(*X)[NV] = k == 0 ? P : Q;
+    const double ct = q0 * mu[k] + q1 * mu[k + 1] + q2 * mu[k + 2], cA = V_ * mu[k];
+    const double x0[NV] = { mu[k], mu[k + 1], V * mu[k], 0.5 * (mu[k + 2] + e2 * mu[k]) };
+    const double x1[NV] = { S[k], S[k + 1], V * S[k] + ct,
+                            0.5 * (S[k + 2] + e2 * S[k] + k1 * mu[k + 1] + k0 * mu[k]) + V * ct };
+    const double x2[NV] = { A[k], A[k + 1], V * A[k] + cA, 0.5 * (A[k + 2] + e2 * A[k] + kA * mu[k]) + V * cA };
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      const double s = x1[v] + x2[v];
+      if (ADD) { X[0][v] += rho * x0[v]; X[1][v] += rho * x1[v]; X[2][v] += rho * s; }
+      else { X[0][v] = rho * x0[v]; X[1][v] = rho * x1[v]; X[2][v] = rho * s; }
+    }
+  }
+  return rho * th;
+}
+// Coefficients of Eq. (2nd-flux)'s pieces at time t for the flux integrated
+// over [0, t] (fi) and the state at t (wi): equilibrium 1, viscous part, A;
+// sides 1, a.u, a.u + A (see gks_full).  om = 1 - exp(-t / tau_n).
+__device__ __forceinline__ void full_coeffs(double t, double tau, double taun, double om, double fi[6], double wi[6]) {
+  const double e = 1.0 - om;
+  const double ie = taun * om, ite = taun * (ie - t * e);
+  const double c2 = ite + tau * ie - tau * t;
+  fi[0] = t - ie;
+  fi[1] = c2;
+  fi[2] = 0.5 * t * t - tau * t + tau * ie - c2;
+  fi[3] = ie;
+  fi[4] = -ite;
+  fi[5] = -tau * ie;
+  const double te = t * e;
+  wi[0] = om;
+  wi[1] = 0.0;
+  wi[2] = (t - tau + tau * e) - (te + tau * e - tau);
+  wi[3] = e;
+  wi[4] = -te;
+  wi[5] = -tau * e;
+}
+// The linear-in-time form of the time schemes from the integrals over [0, dt]
+// and [0, dt/2] (flux) and the values at dt/2 and dt (state): the six pieces'
+// coefficients for F0, F1, Wc, Wt.
+struct FullCoeffs {
+  double F0[6], F1[6], Wc[6], Wt[6];
+};
+__device__ __forceinline__ void full_time_fit(double dt, double tau, double taun, FullCoeffs &C) {
+  // exp(-dt / tau_n) from its value at dt/2: om(dt) = om (2 - om)
+  const double omh = taun > 0.0 ? -expm1(-0.5 * dt / taun) : 1.0, omd = omh * (2.0 - omh);
+  double fd[6], wd[6], fh[6], wh[6];
+  full_coeffs(dt, tau, taun, omd, fd, wd);
+  full_coeffs(0.5 * dt, tau, taun, omh, fh, wh);
+  const double idt = d_rcp(dt), i2 = 4.0 * idt * idt;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    C.F0[k] = (4.0 * fh[k] - fd[k]) * idt;
+    C.F1[k] = (fd[k] - 2.0 * fh[k]) * i2;
+    C.Wc[k] = 2.0 * wh[k] - wd[k];
+    C.Wt[k] = 2.0 * (wd[k] - wh[k]) * idt;
+  }
+}
+// Full gas-kinetic flux at one Gauss point (see gks_full_point_local): side
+// states and derivatives along n and t in the face frame, G the mean
+// derivatives of the sides plus the jump term in the global frame; results in
+// the global frame.
+__device__ __forceinline__ void gks_full(const KC<double> &kc, double mu_visc, double dt, double tc1, double tc2,
+                                         double nx, double ny, const double Wl[NV], const double Wr[NV],
+                                         const double dnl[NV], const double dtl[NV], const double dnr[NV],
+                                         const double dtr[NV], const double G[2][NV], double F0[NV], double F1[NV],
+                                         double Wc[NV], double Wt[NV]) {
+  double P[3][NV], Q[3][NV];
+  const double pl = full_side<false>(kc, Wl, dnl, dtl, +1, P, Q);
+  const double pr = full_side<true>(kc, Wr, dnr, dtr, -1, P, Q);
+  double W0[NV], Fe[NV], X2[NV], Y2[NV], Hv[NV], p;
+  rot_out(nx, ny, P[0], W0);
+  gks_centre(kc, nx, ny, W0, G, true, Fe, X2, Y2, Hv, p);
+  const double tau = mu_visc * d_rcp(p);
+  const double taun = tau + tc1 * dt + tc2 * dt * fabs(pl - pr) * d_rcp(pl + pr);
+  FullCoeffs C;
+  full_time_fit(dt, tau, taun, C);
+  auto combine = [&](const double c[6], const double X0[NV], const double *X1, const double Xc2[NV],
+                     const double X[3][NV], double out[NV]) {
+    double s[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) s[v] = c[3] * X[0][v] + c[4] * X[1][v] + c[5] * X[2][v];
+    rot_out(nx, ny, s, out);
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      out[v] += c[0] * X0[v] + c[2] * Xc2[v];
+      if (X1 && v > 0) out[v] += (c[1] * p) * X1[v];
+    }
+  };
+  combine(C.F0, Fe, Hv, X2, Q, F0);
+  combine(C.F1, Fe, Hv, X2, Q, F1);
+  combine(C.Wc, W0, nullptr, Y2, P, Wc);
+  combine(C.Wt, W0, nullptr, Y2, P, Wt);
 }
 
 // Cell-average primitives used by the low level (one set per cell and

@@ -212,9 +212,12 @@ __device__ __forceinline__ void half_state(const KC<T> &kc, const T W[NV], int s
 // interface state Wc and its derivatives G[j] along x, y, z, global frame,
 // n the face normal: the moments about the mean velocity in closed form, as
 // the 2-D dev::gks_smooth explains (N = K + 3 degrees of freedom).
-template <typename T>
-__device__ __forceinline__ void gks_smooth(const KC<T> &kc, T mu_visc, const T n[3], const T Wc[NV],
-                                           const T G[3][NV], T F0[NV], T F1[NV], T Wt[NV]) {
+// gks_centre: Fe the Euler flux of Wc, F1 = <u A psi> and Wt = <A psi> (times
+// rho), Hv the viscous part per unit viscosity.
+__device__ __forceinline__ void gks_centre(const KC<double> &kc, const double n[3], const double Wc[NV],
+                                           const double G[3][NV], bool visc, double Fe[NV], double F1[NV],
+                                           double Wt[NV], double Hv[NV], double &p) {
+  using T = double;
   const T c2 = kc.c2K, hN = kc.hN;
   const T rho = Wc[0], ir = dev::d_rcp(rho);
   const T u[3] = { Wc[1] * ir, Wc[2] * ir, Wc[3] * ir };
@@ -235,7 +238,8 @@ __device__ __forceinline__ void gks_smooth(const KC<T> &kc, T mu_visc, const T n
   for (int k = 0; k < 3; ++k)
     ut[k] = -(u[0] * du[0][k] + u[1] * du[1][k] + u[2] * du[2][k] + th * r[k] + Tx[k]);
   const T Tt = -(u[0] * Tx[0] + u[1] * Tx[1] + u[2] * Tx[2] + c2 * th * div);
-  const T un = u[0] * n[0] + u[1] * n[1] + u[2] * n[2], mn = rho * un, p = rho * th;
+  const T un = u[0] * n[0] + u[1] * n[1] + u[2] * n[2], mn = rho * un;
+  p = rho * th;
   const T a0 = rho * rt, ei = u[0] * ut[0] + u[1] * ut[1] + u[2] * ut[2] + hN * Tt;
   Wt[0] = a0;
 #pragma unroll
@@ -243,28 +247,36 @@ __device__ __forceinline__ void gks_smooth(const KC<T> &kc, T mu_visc, const T n
   Wt[4] = E * a0 + rho * ei;
   const T mt = Wt[1] * n[0] + Wt[2] * n[1] + Wt[3] * n[2], pt = th * a0 + rho * Tt;
   F1[0] = mt;
-  F0[0] = mn;
+  Fe[0] = mn;
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     F1[1 + k] = u[k] * mt + mn * ut[k] + n[k] * pt;
-    F0[1 + k] = mn * u[k] + p * n[k];
+    Fe[1 + k] = mn * u[k] + p * n[k];
   }
   F1[4] = H * mt + mn * (ei + Tt);
-  F0[4] = mn * H;
-  if (mu_visc != T(0)) {
-    T w = mu_visc * (hN + T(1)) * (Tx[0] * n[0] + Tx[1] * n[1] + Tx[2] * n[2]);
+  Fe[4] = mn * H;
+  if (visc) {
+    Hv[0] = T(0);
+    Hv[4] = (hN + T(1)) * (Tx[0] * n[0] + Tx[1] * n[1] + Tx[2] * n[2]);
     const T d = c2 * div;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       T s = -d * n[k];
 #pragma unroll
       for (int j = 0; j < 3; ++j) s += (du[j][k] + du[k][j]) * n[j];
-      s *= mu_visc;
-      F0[1 + k] -= s;
-      w += u[k] * s;
+      Hv[1 + k] = s;
+      Hv[4] += u[k] * s;
     }
-    F0[4] -= w;
   }
+}
+__device__ __forceinline__ void gks_smooth(const KC<double> &kc, double mu_visc, const double n[3],
+                                           const double Wc[NV], const double G[3][NV], double F0[NV], double F1[NV],
+                                           double Wt[NV]) {
+  double Hv[NV], p;
+  gks_centre(kc, n, Wc, G, mu_visc != 0.0, F0, F1, Wt, Hv, p);
+  if (mu_visc != 0.0)
+#pragma unroll
+    for (int v = 1; v < NV; ++v) F0[v] -= mu_visc * Hv[v];
 }
 
 // ---------------- full flux, Eq. (2nd-flux), 3-D ----------------
@@ -411,6 +423,114 @@ __device__ void gks_full_point_local(const KC<T> &kc, T mu_visc, T ajump, T dt, 
     Wc[v] = T(2) * Wh[v] - Wd[v];
     Wt[v] = T(2) * (Wd[v] - Wh[v]) * idt;
   }
+}
+
+// ---- full flux, FP64: the 2-D dev::gks_full with two tangents ----
+// One side's share of the rho-weighted moments over u > 0 (sgn = +1) or u < 0
+// (-1); X[k] for k = 0: 1, 1: a.u, 2: a.u + A, of psi (P) and u psi (Q).
+// Returns the pressure.
+template <bool ADD>
+__device__ __forceinline__ double full_side(const KC<double> &kc, const double W[NV], const double d[3][NV], int sgn,
+                                            double P[3][NV], double Q[3][NV]) {
+  const double c2 = kc.c2K, N1 = 2.0 * kc.hN - 1.0;
+  const double rho = W[0], ir = dev::d_rcp(rho);
+  const double u[3] = { W[1] * ir, W[2] * ir, W[3] * ir }, E = W[4] * ir, U = u[0];
+  const double th = c2 * (E - 0.5 * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2])), ith = dev::d_rcp(th);
+  double sl, isp, mu[7];
+  dev::sqrt_lambda(th, sl, isp);
+  half_moments<double, 6>(U, th, sl, isp, sgn, mu);
+  // derivatives of ln rho, u_k, theta along the axes j (R[j][k] = d_j u_k), and in time (Euler)
+  double r[3], R[3][3], T[3], r_ = 0.0, u_[3], T_ = 0.0, f[3];
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    r[j] = d[j][0] * ir;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) R[j][k] = d[j][1 + k] * ir - u[k] * r[j];
+    T[j] = c2 * (d[j][4] * ir - E * r[j] - u[0] * R[j][0] - u[1] * R[j][1] - u[2] * R[j][2]);
+    f[j] = T[j] * ith;
+  }
+  const double div = R[0][0] + R[1][1] + R[2][2];
+  r_ = -(u[0] * r[0] + u[1] * r[1] + u[2] * r[2] + div);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) u_[k] = -(u[0] * R[0][k] + u[1] * R[1][k] + u[2] * R[2][k] + th * r[k] + T[k]);
+  T_ = -(u[0] * T[0] + u[1] * T[1] + u[2] * T[2] + c2 * th * div);
+  const double f_ = T_ * ith;
+  const dev::CentralSlope a0 = dev::central_slope(U, ith, r[0], R[0][0], f[0]),
+                          a1 = dev::central_slope(U, ith, r[1], R[1][0], f[1]),
+                          a2 = dev::central_slope(U, ith, r[2], R[2][0], f[2]),
+                          aA = dev::central_slope(U, ith, r_, u_[0], f_);
+  const double Nt = N1 * th, e2 = u[1] * u[1] + u[2] * u[2] + Nt;
+  // S = u a_n + v a_1 + w a_2
+  const double h0 = R[1][1] + R[2][2];
+  const double p0 = u[1] * a1.a0 + u[2] * a2.a0 + h0, p1 = a0.a0 + u[1] * a1.a1 + u[2] * a2.a1,
+               p2 = a0.a1 + u[1] * a1.a2 + u[2] * a2.a2, p3 = a0.a2;
+  double q0[2], q1[2], q2[2];
+#pragma unroll
+  for (int t = 0; t < 2; ++t) {
+    q2[t] = 0.5 * f[1 + t];
+    q1[t] = R[0][1 + t] + R[1 + t][0] - f[1 + t] * U;
+    q0[t] = u[1] * R[1][1 + t] + u[2] * R[2][1 + t] + th * (r[1 + t] + q2[t]) - U * (R[1 + t][0] - q2[t] * U);
+  }
+  const double k1 = Nt * f[0], k0 = Nt * (u[1] * f[1] + u[2] * f[2]) + 2.0 * th * h0, kA = Nt * f_;
+  double S[4], A[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    S[k] = p0 * mu[k] + p1 * mu[k + 1] + p2 * mu[k + 2] + p3 * mu[k + 3];
+    A[k] = aA.a0 * mu[k] + aA.a1 * mu[k + 1] + aA.a2 * mu[k + 2];
+  }
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {   // weight 1 (P), u (Q)
+    double(*X)[NV] = k == 0 ? P : Q;
+    double ct[2], cA[2];
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      ct[t] = q0[t] * mu[k] + q1[t] * mu[k + 1] + q2[t] * mu[k + 2];
+      cA[t] = u_[1 + t] * mu[k];
+    }
+    const double x0[NV] = { mu[k], mu[k + 1], u[1] * mu[k], u[2] * mu[k], 0.5 * (mu[k + 2] + e2 * mu[k]) };
+    const double x1[NV] = { S[k], S[k + 1], u[1] * S[k] + ct[0], u[2] * S[k] + ct[1],
+                            0.5 * (S[k + 2] + e2 * S[k] + k1 * mu[k + 1] + k0 * mu[k]) + u[1] * ct[0] + u[2] * ct[1] };
+    const double x2[NV] = { A[k], A[k + 1], u[1] * A[k] + cA[0], u[2] * A[k] + cA[1],
+                            0.5 * (A[k + 2] + e2 * A[k] + kA * mu[k]) + u[1] * cA[0] + u[2] * cA[1] };
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      const double s = x1[v] + x2[v];
+      if (ADD) { X[0][v] += rho * x0[v]; X[1][v] += rho * x1[v]; X[2][v] += rho * s; }
+      else { X[0][v] = rho * x0[v]; X[1][v] = rho * x1[v]; X[2][v] = rho * s; }
+    }
+  }
+  return rho * th;
+}
+__device__ __forceinline__ void gks_full(const KC<double> &kc, double mu_visc, double dt, double tc1, double tc2,
+                                         const Frame<double> &F, const double Wl[NV], const double Wr[NV],
+                                         const double dl[3][NV], const double dr[3][NV], const double G[3][NV],
+                                         double F0[NV], double F1[NV], double Wc[NV], double Wt[NV]) {
+  double P[3][NV], Q[3][NV];
+  const double pl = full_side<false>(kc, Wl, dl, +1, P, Q);
+  const double pr = full_side<true>(kc, Wr, dr, -1, P, Q);
+  double W0[NV], Fe[NV], X2[NV], Y2[NV], Hv[NV], p;
+  rot_out(F, P[0], W0);
+  gks_centre(kc, F.e[0], W0, G, true, Fe, X2, Y2, Hv, p);
+  const double tau = mu_visc * dev::d_rcp(p);
+  const double taun = tau + tc1 * dt + tc2 * dt * fabs(pl - pr) * dev::d_rcp(pl + pr);
+  dev::FullCoeffs C;
+  dev::full_time_fit(dt, tau, taun, C);
+  auto combine = [&](const double c[6], const double X0[NV], const double *X1, const double Xc2[NV],
+                     const double X[3][NV], double out[NV]) {
+    double s[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) s[v] = c[3] * X[0][v] + c[4] * X[1][v] + c[5] * X[2][v];
+    rot_out(F, s, out);
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      out[v] += c[0] * X0[v] + c[2] * Xc2[v];
+      if (X1 && v > 0) out[v] += (c[1] * p) * X1[v];
+    }
+  };
+  combine(C.F0, Fe, Hv, X2, Q, F0);
+  combine(C.F1, Fe, Hv, X2, Q, F1);
+  combine(C.Wc, W0, nullptr, Y2, P, Wc);
+  combine(C.Wt, W0, nullptr, Y2, P, Wt);
 }
 
 // cell primitives of the low level: rho, u, v, w, p, 1/(2 lambda),

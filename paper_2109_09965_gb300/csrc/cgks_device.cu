@@ -555,6 +555,8 @@ void fill_shared_params(const Shared &sh, ParamsT<T> &P) {
   P.kc.c4K = static_cast<T>(4.0 / (K + 2.0));
   P.kc.hN = static_cast<T>(0.5 * (K + 2.0));
   P.kc.sq2g = static_cast<T>(std::sqrt(2.0 * sh.gamma));
+  const double N = 2.0 / (sh.gamma - 1.0), Nr = std::round(N);
+  P.kc.iN = std::fabs(N - Nr) < 1e-12 * N && Nr <= 64.0 ? static_cast<int>(Nr) : 0;
   P.flux_lo = sh.flux_lo;
   P.flux_hi = sh.flux_hi;
   P.tau_c1 = static_cast<T>(sh.tau_c1);

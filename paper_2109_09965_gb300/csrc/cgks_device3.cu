@@ -350,6 +350,8 @@ void fill_params(const cgks_params &p, ParamsT<T> &P) {
   P.kc.c4K = static_cast<T>(4.0 / (K + 3.0));
   P.kc.hN = static_cast<T>(0.5 * (K + 3.0));
   P.kc.sq2g = static_cast<T>(std::sqrt(2.0 * p.gamma));
+  const double N = 2.0 / (p.gamma - 1.0), Nr = std::round(N);
+  P.kc.iN = std::fabs(N - Nr) < 1e-12 * N && Nr <= 64.0 ? static_cast<int>(Nr) : 0;
   P.flux_lo = p.flux_lo;
   P.tau_c1 = static_cast<T>(p.tau_c1);
   P.tau_c2 = static_cast<T>(p.tau_c2);

@@ -184,7 +184,7 @@ template <typename T>
 __device__ __forceinline__ void farfield_ghost(const ParamsT<T> &P, int tag, T nx, T ny, const T wl[4], T wg[4]) {
   T une = P.bc_u[2 * tag] * nx + P.bc_u[2 * tag + 1] * ny;
   T ute = -P.bc_u[2 * tag] * ny + P.bc_u[2 * tag + 1] * nx;
-  D::ghost_farfield(P.gamma, P.bc_rho[tag], une, ute, P.bc_p[tag], wl, wg);
+  D::ghost_farfield(P.kc, P.gamma, P.bc_rho[tag], une, ute, P.bc_p[tag], wl, wg);
 }
 
 // prescribed state of a Dirichlet boundary in the face frame

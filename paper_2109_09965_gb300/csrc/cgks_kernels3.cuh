@@ -172,7 +172,7 @@ __device__ __forceinline__ void farfield_ghost(const ParamsT<T> &P, int tag, con
 #pragma unroll
   for (int a = 0; a < 3; ++a)
     ue[a] = F.e[a][0] * P.bc_u[3 * tag] + F.e[a][1] * P.bc_u[3 * tag + 1] + F.e[a][2] * P.bc_u[3 * tag + 2];
-  D3::ghost_farfield(P.gamma, P.bc_rho[tag], ue, P.bc_p[tag], wl, wg);
+  D3::ghost_farfield(P.kc, P.gamma, P.bc_rho[tag], ue, P.bc_p[tag], wl, wg);
 }
 
 // Compact WENO (conservative variables), 3-D form of the 2-D weno_combine:
@@ -502,6 +502,14 @@ __device__ __forceinline__ void face_points_at(const MeshT<double> &m, const Par
   const int tag = c1 < 0 ? -1 - c1 : 0;
   const bool farfield = c1 < 0 && P.bc_kind[tag] == CGKS_BC_FARFIELD;
   const T ihL = m.ih[c0], ihR = c1 >= 0 ? m.ih[c1] : ihL;
+  T wff[NV];   // the far-field state, one for the face
+  if (farfield) {
+    T wm[NV], wi[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) wm[v] = W[v * m.nc + c0];
+    D3::rot_in(F, wm, wi);
+    farfield_ghost(P, tag, F, wi, wff);
+  }
 #pragma unroll 1
   for (int k = lane; k < ng; k += LANES) {
     T x0[3], wL[NV], gL[3][NV], wR[NV], gR[3][NV];
@@ -517,11 +525,8 @@ __device__ __forceinline__ void face_points_at(const MeshT<double> &m, const Par
       recon_scaled(m, W, coef, c1, x1, wR, gR);
       D3::rot_in(F, wR, wr);
     } else if (farfield) {
-      T wm[NV], wi[NV];
 #pragma unroll
-      for (int v = 0; v < NV; ++v) wm[v] = W[v * m.nc + c0];
-      D3::rot_in(F, wm, wi);
-      farfield_ghost(P, tag, F, wi, wr);
+      for (int v = 0; v < NV; ++v) wr[v] = wff[v];
       D3::rot_out(F, wr, wR);
 #pragma unroll
       for (int d = 0; d < 3; ++d)

@@ -640,10 +640,33 @@ __device__ __forceinline__ void ghost_noslip(T gamma, const T uw[3], const T W[N
   }
 }
 
+// FP64 far-field state, see dev::far_state
+__device__ __forceinline__ void ghost_farfield(const KC<double> &kc, double gamma, double re, const double ue[3],
+                                               double pe, const double W[NV], double Wg[NV]) {
+  const double ri = W[0], ir = dev::d_rcp(ri);
+  const double ui[3] = { W[1] * ir, W[2] * ir, W[3] * ir };
+  const double pi = (gamma - 1.0) * (W[4] - 0.5 * ri * (ui[0] * ui[0] + ui[1] * ui[1] + ui[2] * ui[2]));
+  const double ci = dev::d_sqrt3(gamma * pi * ir), ce = dev::d_sqrt3(gamma * pe * dev::d_rcp(re));
+  double rb, ub[3], pb;
+  if (ui[0] <= -ci) {
+    rb = re; ub[0] = ue[0]; ub[1] = ue[1]; ub[2] = ue[2]; pb = pe;
+  } else if (ui[0] >= ci) {
+    rb = ri; ub[0] = ui[0]; ub[1] = ui[1]; ub[2] = ui[2]; pb = pi;
+  } else {
+    const dev::FarState f = dev::far_state(kc, ri, pi, ui[0], ci, re, pe, ue[0], ce);
+    rb = f.r; ub[0] = f.un; pb = f.p;
+    ub[1] = f.out ? ui[1] : ue[1];
+    ub[2] = f.out ? ui[2] : ue[2];
+  }
+  Wg[0] = rb; Wg[1] = rb * ub[0]; Wg[2] = rb * ub[1]; Wg[3] = rb * ub[2];
+  Wg[4] = pb * kc.hN + 0.5 * rb * (ub[0] * ub[0] + ub[1] * ub[1] + ub[2] * ub[2]);
+}
+
 // Riemann invariants normal to the face: interior W and free stream
 // (re, une, ut1e, ut2e, pe), local frame
 template <typename T>
-__device__ __forceinline__ void ghost_farfield(T gamma, T re, const T ue[3], T pe, const T W[NV], T Wg[NV]) {
+__device__ __forceinline__ void ghost_farfield(const KC<T> &, T gamma, T re, const T ue[3], T pe, const T W[NV],
+                                               T Wg[NV]) {
   const T ri = W[0], ir = T(1) / ri;
   const T ui[3] = { W[1] * ir, W[2] * ir, W[3] * ir };
   const T pi = (gamma - T(1)) * (W[4] - T(0.5) * ri * (ui[0] * ui[0] + ui[1] * ui[1] + ui[2] * ui[2]));

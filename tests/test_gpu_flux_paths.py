@@ -117,3 +117,20 @@ def test_one_and_four_lanes_per_cell_round_alike():
         assert np.array_equal(srv.poll(i)[1], s.get_state()[0])
         s.close()
     srv.close()
+
+
+@pytest.mark.parametrize("gamma", [5 / 3, 1.4, 1.33, 1.1])
+@pytest.mark.parametrize("dim", [2, 3])
+def test_far_field_state_at_whole_and_other_exponents(dim, gamma):
+    """Subsonic in- and outflow at the far field: the boundary density goes
+    with y^N, N = 2/(gamma - 1), by repeated squaring where N is a whole
+    number (3, 5, 20) and by pow at 1.33."""
+    if dim == 2:
+        mesh = MG.box(9, 7, jitter=0.15, seed=2, cells="tri", tags=(0, 0, 0, 0))
+        u = (0.3, 0.1)
+    else:
+        mesh = MG.box3(3, 3, 3, jitter=0.1, seed=2, cells="prism", tags=(0,) * 6)
+        u = (0.3, 0.1, -0.1)
+    p = (gamma - 1) / (GAM - 1) / GAM                          # of the state's energy
+    spec = dict(gamma=gamma, mu=0.005, cfl_hi=0.3, bcs=[dict(kind="farfield", rho=1.0, u=u, p=p)])
+    compare(mesh, spec, state(mesh, 0.2, 0.4), "fp64", 2)

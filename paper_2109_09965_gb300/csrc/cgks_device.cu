@@ -73,7 +73,7 @@ struct Member {
 
 // device tables of a batch (views into its arena)
 struct DevArrays {
-  double *vol, *ivol, *per, *ih, *m2, *op, *fn, *fS, *fjump, *fxi, *snx, *sny, *fidl = nullptr;
+  double *vol, *ivol, *per, *ih, *m2, *op, *fn, *fS, *fjump, *fxi, *snx, *sny, *sS, *fidl = nullptr;
   double *mu, *bcuw, *bcrho, *bcu, *bcp;
   int *cface, *cnbr, *fc0, *fc1, *csid, *fsid, *bckind;
   unsigned char *ccol, *wenok;
@@ -280,18 +280,16 @@ void enqueue_hi_step(Batch *b, double *Wout, TF *Wout_m, bool want_res) {
   double *part = want_res ? b->partial : nullptr;
   const dim3 g(nblk(b->N, kCellBlock)), blk(kCellBlock);
   enqueue_hi_eval<TF>(b, B.W, B.Wx, B.FA);
+  auto update = [&](auto kern, const TF *FB, double *Wo, double *Wxo, double *pt, double *R, TF *Wom, TF *Wxom) {
+    launch(b, KI_UPDATE, kern, g, blk, b->dm, b->dp, (const double *)b->W, (const TF *)B.FA, FB, (const Ctl *)b->ctl,
+           (const unsigned long long *)b->dt_bits, b->status, Wo, Wxo, pt, R, Wom, Wxom);
+  };
   if (b->sh.time_scheme == CGKS_S1O2) {
-    launch(b, KI_UPDATE, k_update<TF>, g, blk, b->dm, b->dp, (int)kS1O2, (const double *)b->W, (const TF *)B.FA,
-           (const TF *)B.FA, (const Ctl *)b->ctl, (const unsigned long long *)b->dt_bits, b->status, Wout, b->Wx,
-           part, b->Rp0, Wout_m, mirror<TF>(B.Wx));
+    update(k_update<TF, kS1O2>, B.FA, Wout, b->Wx, part, b->Rp0, Wout_m, mirror<TF>(B.Wx));
   } else {
-    launch(b, KI_UPDATE, k_update<TF>, g, blk, b->dm, b->dp, (int)kS2O4Stage, (const double *)b->W, (const TF *)B.FA,
-           (const TF *)B.FA, (const Ctl *)b->ctl, (const unsigned long long *)b->dt_bits, b->status, b->Ws, b->Wxs,
-           (double *)nullptr, (double *)nullptr, mirror<TF>(B.Ws), mirror<TF>(B.Wxs));
+    update(k_update<TF, kS2O4Stage>, B.FA, b->Ws, b->Wxs, nullptr, nullptr, mirror<TF>(B.Ws), mirror<TF>(B.Wxs));
     enqueue_hi_eval<TF>(b, B.Ws, B.Wxs, B.FB);
-    launch(b, KI_UPDATE, k_update<TF>, g, blk, b->dm, b->dp, (int)kS2O4Final, (const double *)b->W, (const TF *)B.FA,
-           (const TF *)B.FB, (const Ctl *)b->ctl, (const unsigned long long *)b->dt_bits, b->status, Wout, b->Wx,
-           part, b->Rp0, Wout_m, mirror<TF>(B.Wx));
+    update(k_update<TF, kS2O4Final>, B.FB, Wout, b->Wx, part, b->Rp0, Wout_m, mirror<TF>(B.Wx));
   }
   if (want_res) enqueue_res(b);
 }
@@ -434,7 +432,7 @@ void enqueue_cycle_t(Batch *b) {
   enqueue_hi_step<TF>(b, b->Wn, mirror<TF>(B.Wn), false);
   // 2: R_p0 = time-averaged high-order net flux at W^{n+1}
   enqueue_hi_eval<TF>(b, B.Wn, B.Wx, B.FB);
-  launch(b, KI_UPDATE, k_update<TF>, dim3(nblk(b->N, kCellBlock)), dim3(kCellBlock), b->dm, b->dp, (int)kResidual,
+  launch(b, KI_UPDATE, k_update<TF, kResidual>, dim3(nblk(b->N, kCellBlock)), dim3(kCellBlock), b->dm, b->dp,
          (const double *)b->Wn, (const TF *)B.FB, (const TF *)B.FB, (const Ctl *)b->ctl,
          (const unsigned long long *)b->dt_bits, b->status, (double *)nullptr, (double *)nullptr, (double *)nullptr,
          b->Rp0, (TF *)nullptr, (TF *)nullptr);
@@ -589,7 +587,7 @@ void plan_arena(Batch *b, int64_t N, int64_t F, int S, int64_t L, bool mixed, st
   P8(&b->U, 4 * N); P8(&b->Rp0, 4 * N); P8(&b->Src, 4 * N); P8(&b->stage, 12 * N);
   P8(&b->partial, 2 * std::max<int64_t>(N / kCellBlock, 1)); P8(&b->last, 4); P8(&b->res, S);
   P8(&d.vol, N); P8(&d.ivol, N); P8(&d.per, N); P8(&d.ih, N); P8(&d.m2, 3 * N); P8(&d.op, kNCol * kNM * N);
-  P8(&d.snx, kMaxFace * N); P8(&d.sny, kMaxFace * N);
+  P8(&d.snx, kMaxFace * N); P8(&d.sny, kMaxFace * N); P8(&d.sS, kMaxFace * N);
   P8(&d.fn, 2 * F); P8(&d.fS, F); P8(&d.fjump, F); P8(&d.fxi, 8 * F); P8(&d.fidl, F);
   P8(&d.mu, S); P8(&d.bcuw, 2 * T); P8(&d.bcrho, T); P8(&d.bcu, 2 * T); P8(&d.bcp, T);
   PI(&d.cface, kMaxFace * N); PI(&d.cnbr, kMaxFace * N); PI(&d.fc0, F); PI(&d.fc1, F); PI(&d.csid, N); PI(&d.fsid, F);
@@ -713,7 +711,7 @@ int create_batch(const Shared &sh, int64_t Ncap, int64_t Fcap, int S, cudaStream
   MeshT<double> &dm = b->dm;
   dm.nc = static_cast<int>(Ncap); dm.nf = static_cast<int>(Fcap);
   dm.vol = d.vol; dm.ivol = d.ivol; dm.per = d.per; dm.ih = d.ih; dm.m2 = d.m2; dm.op = d.op;
-  dm.fn = d.fn; dm.fS = d.fS; dm.fjump = d.fjump; dm.fxi = d.fxi; dm.snx = d.snx; dm.sny = d.sny;
+  dm.fn = d.fn; dm.fS = d.fS; dm.fjump = d.fjump; dm.fxi = d.fxi; dm.snx = d.snx; dm.sny = d.sny; dm.shs = d.sS;
   dm.fidl = d.fidl;
   dm.cface = d.cface; dm.cnbr = d.cnbr; dm.fc0 = d.fc0; dm.fc1 = d.fc1; dm.csid = d.csid; dm.fsid = d.fsid;
   dm.ccol = d.ccol; dm.wenok = d.wenok;
@@ -775,7 +773,8 @@ int insert_solve(Batch *b, int s, const Member &m, int64_t cell_off, int64_t fac
   if (cudaGetLastError() != cudaSuccess) return CGKS_ECUDA;
   // local tables (np cells, nf faces) with global indices
   std::vector<double> vol(np, 1.0), ivol(np, 1.0), per(np, 4.0), ih(np, 1.0), m2(3 * np, 0.0),
-      op(kNCol * kNM * np, 0.0), snx(kMaxFace * np, 0.0), sny(kMaxFace * np, 0.0), shs(kMaxFace * np, 0.0);
+      op(kNCol * kNM * np, 0.0), snx(kMaxFace * np, 0.0), sny(kMaxFace * np, 0.0), shs(kMaxFace * np, 0.0),
+      nxs(kMaxFace * np, 0.0), nys(kMaxFace * np, 0.0), sS(kMaxFace * np, 0.0);   // FP64: n S/2 and S per slot
   std::vector<double> fn(2 * nf), fS(nf), fjump(nf), fxi(8 * nf), fidl(nf);
   std::vector<int> cface(kMaxFace * np, kNoFace), cnbr(kMaxFace * np, -1), csid(np, -1), perm(np, 0), fc0(nf),
       fc1(nf), fsid(nf, s);
@@ -803,10 +802,9 @@ int insert_solve(Batch *b, int s, const Member &m, int64_t cell_off, int64_t fac
       snx[sl * np + i] = sg * hm.fn[f];
       sny[sl * np + i] = sg * hm.fn[nf + f];
       shs[sl * np + i] = 0.5 * hm.fS[f];
-      if (!b->mixed) {   // FP64 sweeps take n S/2
-        snx[sl * np + i] *= shs[sl * np + i];
-        sny[sl * np + i] *= shs[sl * np + i];
-      }
+      nxs[sl * np + i] = snx[sl * np + i] * shs[sl * np + i];
+      nys[sl * np + i] = sny[sl * np + i] * shs[sl * np + i];
+      sS[sl * np + i] = hm.fS[f];
     }
   }
   for (int c = 0; c < hm.n_colours; ++c)
@@ -842,7 +840,7 @@ int insert_solve(Batch *b, int s, const Member &m, int64_t cell_off, int64_t fac
   DevArrays &d = b->d;
   const int64_t T = kTagsPerSolve;
   up(d.vol, vol, np, N, co); up(d.ivol, ivol, np, N, co); up(d.per, per, np, N, co); up(d.ih, ih, np, N, co);
-  up(d.m2, m2, np, N, co); up(d.op, op, np, N, co); up(d.snx, snx, np, N, co); up(d.sny, sny, np, N, co);
+  up(d.m2, m2, np, N, co); up(d.op, op, np, N, co); up(d.snx, nxs, np, N, co); up(d.sny, nys, np, N, co); up(d.sS, sS, np, N, co);
   up(d.cface, cface, np, N, co); up(d.cnbr, cnbr, np, N, co);
   up(d.csid, csid, np, N, co); up(b->perm, perm, np, N, co); up(d.ccol, ccol, np, N, co);
   up(d.wenok, wenok, np, N, co);
@@ -1269,9 +1267,9 @@ int wall_loads_t(cgks_solver *s, int32_t tag, int64_t max_faces, int64_t *n_face
   if (b->sh.flux_hi == CGKS_FLUX_FULL) enqueue_dt(b, -1.0);   // the full flux integrates over a step
   enqueue_hi_eval<TF>(b, B.W, B.Wx, B.FA);
   const int64_t F = b->F, nf = hm.n_faces, off = b->mem[0].face_off;
-  std::vector<TF> F0(4 * static_cast<size_t>(F));
-  for (int v = 0; v < 4; ++v)
-    CK(cudaMemcpyAsync(F0.data() + v * F, B.FA + v * F, sizeof(TF) * F, cudaMemcpyDeviceToHost, s->stream));
+  // the face outputs, one run of kFO values per face: F0 is the first 4
+  std::vector<TF> FO(kFO * static_cast<size_t>(F));
+  CK(cudaMemcpyAsync(FO.data(), B.FA, sizeof(TF) * FO.size(), cudaMemcpyDeviceToHost, s->stream));
   CK(cudaStreamSynchronize(s->stream));
   int64_t k = 0;
   for (int64_t f = 0; f < nf; ++f) {
@@ -1285,8 +1283,8 @@ int wall_loads_t(cgks_solver *s, int32_t tag, int64_t max_faces, int64_t *n_face
       nrm[2 * k] = hm.fn[f];
       nrm[2 * k + 1] = hm.fn[nf + f];
       S[k] = hm.fS[f];
-      traction[2 * k] = static_cast<double>(F0[1 * F + off + f]);
-      traction[2 * k + 1] = static_cast<double>(F0[2 * F + off + f]);
+      traction[2 * k] = static_cast<double>(FO[kFO * (off + f) + 1]);
+      traction[2 * k + 1] = static_cast<double>(FO[kFO * (off + f) + 2]);
     }
     ++k;
   }

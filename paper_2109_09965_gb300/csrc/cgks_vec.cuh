@@ -72,4 +72,22 @@ __device__ __forceinline__ void widen(const double x[N], double y[N]) {
   for (int k = 0; k < N; ++k) y[k] = x[k];
 }
 
+// FP64 -> TF, rounded to nearest even as the conversion instruction does; to
+// FP32 with integer instructions for the same reason (values whose FP32 form is
+// normal, and zeros; the rest by the instruction).
+template <typename TF> __device__ __forceinline__ TF narrow(double x);
+template <> __device__ __forceinline__ double narrow<double>(double x) { return x; }
+template <> __device__ __forceinline__ float narrow<float>(double x) {
+  const unsigned hi = static_cast<unsigned>(__double2hiint(x)), lo = static_cast<unsigned>(__double2loint(x));
+  const unsigned sign = hi & 0x80000000u, mag = hi & 0x7fffffffu;
+  if (mag - 0x38100000u < 0x0fd00000u) {   // FP32 exponents 1 to 253: rounding cannot overflow
+    unsigned b = ((mag - 0x38000000u) << 3) | (lo >> 29);
+    const unsigned rest = lo & 0x1fffffffu;
+    b += rest > 0x10000000u - (b & 1u);    // above half, or half and odd
+    return __uint_as_float(sign | b);
+  }
+  if ((mag | lo) == 0u) return __uint_as_float(sign);
+  return static_cast<float>(x);
+}
+
 }  // namespace cgks

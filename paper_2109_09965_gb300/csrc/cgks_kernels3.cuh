@@ -884,11 +884,18 @@ __device__ __forceinline__ void lo_ghost(const ParamsT<T> &P, int tag, const D3:
 }
 
 // KFVS (or Lax-Friedrichs) flux, lambda_p = max of both sides
+__device__ __forceinline__ float third(float x) { return x / 3.0f; }
+__device__ __forceinline__ double third(double x) { return x * (1.0 / 3.0); }
 template <typename T>
 __device__ __forceinline__ void lo_face_at(const MeshT<T> &m, const ParamsT<T> &P, const T *__restrict__ base,
                                            T *__restrict__ Flo, const int f) {
   const int c0 = m.fc0[f], c1 = m.fc1[f];
-  const D3::Frame<T> F = frame_of(m, f);
+  // FP32 and boundary faces take the whole frame, an inner FP64 face its normal
+  D3::Frame<T> F;
+  if (is_f32<T>() || c1 < 0) F = frame_of(m, f);
+  else
+#pragma unroll
+    for (int d = 0; d < 3; ++d) F.e[0][d] = m.fe[d * m.nf + f];
   T ra[kBase], rb[kBase];
   vload<T, kBase>(base + static_cast<size_t>(c0) * kBase, ra);
   const D3::Prim<T> a = base_prim(ra);
@@ -906,7 +913,7 @@ __device__ __forceinline__ void lo_face_at(const MeshT<T> &m, const ParamsT<T> &
   }
   T la3[3], lb3[3];
 #pragma unroll
-  for (int k = 0; k < 3; ++k) {
+  for (int k = 0; k < (is_f32<T>() ? 3 : 1); ++k) {
     la3[k] = a.u * F.e[k][0] + a.v * F.e[k][1] + a.w * F.e[k][2];
     lb3[k] = b.u * F.e[k][0] + b.v * F.e[k][1] + b.w * F.e[k][2];
   }
@@ -931,6 +938,18 @@ __device__ __forceinline__ void lo_face_at(const MeshT<T> &m, const ParamsT<T> &
                        (wb[4] + b.p) * unb };
 #pragma unroll
     for (int v = 0; v < NV; ++v) Fg[v] = T(0.5) * (Fa[v] + Fb[v]) - T(0.5) * lmax * (wb[v] - wa[v]);
+  } else if constexpr (!is_f32<T>()) {
+    // KFVS without the face frame, as in 2-D
+    const T una = la3[0], unb = lb3[0];
+    T m0a, m1a, m0b, m1b;
+    dev::half01(una, a.sl, a.isp, +1, m0a, m1a);
+    dev::half01(unb, b.sl, b.isp, -1, m0b, m1b);
+    const T ja = a.rho * m1a, jb = b.rho * m1b, pa = a.p * m0a, pb = b.p * m0b, pn = pa + pb;
+    Fg[0] = ja + jb;
+    Fg[1] = ja * a.u + jb * b.u + pn * nx;
+    Fg[2] = ja * a.v + jb * b.v + pn * ny;
+    Fg[3] = ja * a.w + jb * b.w + pn * nz;
+    Fg[4] = m1a * (wa[4] + T(0.5) * a.p) + m1b * (wb[4] + T(0.5) * b.p) + T(0.5) * (pa * una + pb * unb);
   } else {
     T Fl[NV];
     D3::kfvs(P.K, a.rho, la3[0], la3[1], la3[2], a.i2l, a.sl, a.isp, b.rho, lb3[0], lb3[1], lb3[2], b.i2l, b.sl,
@@ -944,7 +963,7 @@ __device__ __forceinline__ void lo_face_at(const MeshT<T> &m, const ParamsT<T> &
     const T md = P.mu * m.fidl[f];
     const T du[3] = { b.u - a.u, b.v - a.v, b.w - a.w };
     const T nn[3] = { nx, ny, nz };
-    const T dn = (du[0] * nx + du[1] * ny + du[2] * nz) / T(3);
+    const T dn = third(du[0] * nx + du[1] * ny + du[2] * nz);
     const T um[3] = { T(0.5) * (a.u + b.u), T(0.5) * (a.v + b.v), T(0.5) * (a.w + b.w) };
     T work = T(0);
 #pragma unroll
@@ -953,7 +972,9 @@ __device__ __forceinline__ void lo_face_at(const MeshT<T> &m, const ParamsT<T> &
       Fg[1 + d] -= tau;
       work += tau * um[d];
     }
-    const T qn = -md * P.gamma / (P.gamma - T(1)) * (b.p * irb - a.p * ira);
+    T qn;   // gamma / (gamma - 1) = N / 2 + 1
+    if constexpr (is_f32<T>()) qn = -md * P.gamma / (P.gamma - T(1)) * (b.p * irb - a.p * ira);
+    else qn = -md * (P.kc.hN + T(1)) * (b.p * irb - a.p * ira);
     Fg[4] -= work - qn;
   }
   // one run per face (AoS): the flux and lambda_p, read together by the

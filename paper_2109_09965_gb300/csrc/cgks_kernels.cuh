@@ -1151,18 +1151,18 @@ __device__ __forceinline__ void lo_rhs_at(const MeshT<double> &m, const ParamsT<
   // dt_i = CFL_lo |Omega| / sum;  D_i = |Omega| / dt_i + sum / 2 (padding cells: 0)
   const double id = sum > 0.0 ? D::d_rcp(sum * (P.icfl_lo + 0.5)) : 0.0;
   invD[i] = narrow<TF>(id);
-  TF d[4];
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
     double src;
     if (first) { src = Rp0[v * n + i] - R[v]; Src[v * n + i] = src; }
     else src = ld<CG>(&Src[v * n + i]);
-    const double r = R[v] + src;
-    Rk[v * n + i] = narrow<TF>(r);
-    d[v] = narrow<TF>(r * id);
+    R[v] += src;
+    Rk[v * n + i] = narrow<TF>(R[v]);
   }
   if (g.c0) {
-    TF b[4];
+    TF b[4], d[4];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) d[v] = narrow<TF>(R[v] * id);
     vload<TF, 4, CG>(base + static_cast<size_t>(i) * kBase, b);
     store_delta(gamma, b, d, delta, i);
   } else {

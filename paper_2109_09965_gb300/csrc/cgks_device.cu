@@ -20,6 +20,7 @@
 #include <string>
 #include <vector>
 
+#include "cgks_insert.cuh"
 #include "cgks_internal.h"
 #include "cgks_kernels.cuh"
 #include "cgks_persistent.cuh"
@@ -69,17 +70,6 @@ struct Member {
   cgks_params params{};
   int64_t cell_off = 0, n_pad = 0, face_off = 0;
   bool active = false;
-};
-
-// device tables of a batch (views into its arena)
-struct DevArrays {
-  double *vol, *ivol, *per, *ih, *m2, *op, *fn, *fS, *fjump, *fxi, *snx, *sny, *sS, *fidl = nullptr;
-  double *mu, *bcuw, *bcrho, *bcu, *bcp;
-  int *cface, *cnbr, *fc0, *fc1, *csid, *fsid, *bckind;
-  unsigned char *ccol, *wenok;
-  float *f_ivol = nullptr, *f_ih = nullptr, *f_m2 = nullptr, *f_op = nullptr, *f_fn = nullptr, *f_fS = nullptr,
-        *f_fjump = nullptr, *f_fidl = nullptr, *f_fxi = nullptr, *f_snx = nullptr, *f_sny = nullptr, *f_shs = nullptr, *f_mu = nullptr,
-        *f_bcuw = nullptr, *f_bcrho = nullptr, *f_bcu = nullptr, *f_bcp = nullptr;
 };
 
 // A batch is a slot table over one device arena: capacity for Ncap cells,
@@ -584,7 +574,7 @@ void plan_arena(Batch *b, int64_t N, int64_t F, int S, int64_t L, bool mixed, st
   auto PV = [&](void **x, size_t bytes) { pieces.push_back({ x, bytes }); };
   const int64_t T = kTagsPerSolve * static_cast<int64_t>(S);
   P8(&b->W, 4 * N); P8(&b->Wx, 8 * N); P8(&b->Wn, 4 * N); P8(&b->Ws, 4 * N); P8(&b->Wxs, 8 * N);
-  P8(&b->U, 4 * N); P8(&b->Rp0, 4 * N); P8(&b->Src, 4 * N); P8(&b->stage, 12 * N);
+  P8(&b->U, 4 * N); P8(&b->Rp0, 4 * N); P8(&b->Src, 4 * N);
   P8(&b->partial, 2 * std::max<int64_t>(N / kCellBlock, 1)); P8(&b->last, 4); P8(&b->res, S);
   P8(&d.vol, N); P8(&d.ivol, N); P8(&d.per, N); P8(&d.ih, N); P8(&d.m2, 3 * N); P8(&d.op, kNCol * kNM * N);
   P8(&d.snx, kMaxFace * N); P8(&d.sny, kMaxFace * N); P8(&d.sS, kMaxFace * N);
@@ -694,6 +684,10 @@ int create_batch(const Shared &sh, int64_t Ncap, int64_t Fcap, int S, cudaStream
     char *cur = static_cast<char *>(b->arena);
     for (auto &pc : pieces) { *pc.dst = cur; cur += (pc.bytes + 255) & ~size_t(255); }
   }
+  // states are loaded, handed out and solves placed between cycles, 12 doubles
+  // per cell of one solve, in the face outputs' memory: 16 values per face and
+  // at least 3/2 faces per cell
+  b->stage = b->mixed ? reinterpret_cast<double *>(b->bf.FA) : b->bd.FA;
   if (!b->mixed) {
     Bufs<double> &X = b->bd;
     X.W = b->W; X.Wx = b->Wx; X.Wn = b->Wn; X.Ws = b->Ws; X.Wxs = b->Wxs;
@@ -771,103 +765,45 @@ int insert_solve(Batch *b, int s, const Member &m, int64_t cell_off, int64_t fac
   cudaStream_t st = b->stream;
   clear_cells(b, co, co + np);
   if (cudaGetLastError() != cudaSuccess) return CGKS_ECUDA;
-  // local tables (np cells, nf faces) with global indices
-  std::vector<double> vol(np, 1.0), ivol(np, 1.0), per(np, 4.0), ih(np, 1.0), m2(3 * np, 0.0),
-      op(kNCol * kNM * np, 0.0), snx(kMaxFace * np, 0.0), sny(kMaxFace * np, 0.0), shs(kMaxFace * np, 0.0),
-      nxs(kMaxFace * np, 0.0), nys(kMaxFace * np, 0.0), sS(kMaxFace * np, 0.0);   // FP64: n S/2 and S per slot
-  std::vector<double> fn(2 * nf), fS(nf), fjump(nf), fxi(8 * nf), fidl(nf);
-  std::vector<int> cface(kMaxFace * np, kNoFace), cnbr(kMaxFace * np, -1), csid(np, -1), perm(np, 0), fc0(nf),
-      fc1(nf), fsid(nf, s);
-  std::vector<unsigned char> ccol(np, 255), wenok(np, 0);
-  std::vector<char> wall(kTagsPerSolve, 0);
-  for (int t = 0; t < p.n_bc; ++t) wall[t] = is_wall_kind(p.bc[t].kind);
-  std::vector<double> ops;
-  std::vector<unsigned char> qok;
-  build_operator(hm, wall, ops, &qok);
-  for (int64_t i = 0; i < nc; ++i) wenok[i] = qok[i];
-  for (int64_t i = 0; i < nc; ++i) {
-    vol[i] = hm.vol[i]; ivol[i] = 1.0 / hm.vol[i]; per[i] = hm.per[i]; ih[i] = 1.0 / hm.h[i];
-    for (int q = 0; q < 3; ++q) m2[q * np + i] = hm.m2[q * nc + i];
-    for (int q = 0; q < kNCol * kNM; ++q) op[q * np + i] = ops[q * nc + i];
-    csid[i] = s;
-    perm[i] = hm.perm[i];
-    for (int sl = 0; sl < kMaxFace; ++sl) {
-      const int32_t fs = hm.cface[sl * nc + i];
-      if (fs == kNoFace) continue;
-      const int32_t f = fs >= 0 ? fs : ~fs;
-      const double sg = fs >= 0 ? 1.0 : -1.0;
-      cface[sl * np + i] = fs >= 0 ? static_cast<int>(f + fo) : ~static_cast<int>(f + fo);
-      const int32_t j = hm.cnbr[sl * nc + i];
-      cnbr[sl * np + i] = j >= 0 ? static_cast<int>(j + co) : -1;
-      snx[sl * np + i] = sg * hm.fn[f];
-      sny[sl * np + i] = sg * hm.fn[nf + f];
-      shs[sl * np + i] = 0.5 * hm.fS[f];
-      nxs[sl * np + i] = snx[sl * np + i] * shs[sl * np + i];
-      nys[sl * np + i] = sny[sl * np + i] * shs[sl * np + i];
-      sS[sl * np + i] = hm.fS[f];
-    }
-  }
-  for (int c = 0; c < hm.n_colours; ++c)
-    for (int32_t i = hm.colour_start[c]; i < hm.colour_start[c + 1]; ++i) ccol[i] = static_cast<unsigned char>(c);
-  for (int64_t f = 0; f < nf; ++f) {
-    fc0[f] = static_cast<int>(hm.fc0[f] + co);
-    const int32_t c1 = hm.fc1[f];
-    fc1[f] = c1 >= 0 ? static_cast<int>(c1 + co) : -1 - (s * kTagsPerSolve + (-1 - c1));
-    fn[f] = hm.fn[f]; fn[nf + f] = hm.fn[nf + f];
-    fS[f] = hm.fS[f];
-    fjump[f] = hm.fdelta[f] > 0.0 ? p.alpha / hm.fdelta[f] : 0.0;
-    fidl[f] = hm.fdelta[f] > 0.0 ? 1.0 / hm.fdelta[f] : 0.0;
-    for (int q = 0; q < 8; ++q) fxi[q * nf + f] = hm.fxi[q * nf + f];
-  }
-  std::vector<double> mu(1, p.mu), bc_uw(2 * kTagsPerSolve, 0.0), bc_rho(kTagsPerSolve, 1.0),
-      bc_u(2 * kTagsPerSolve, 0.0), bc_p(kTagsPerSolve, 1.0);
-  std::vector<int> bc_kind(kTagsPerSolve, CGKS_BC_SLIP);
+  Place pl;
+  std::memset(&pl, 0, sizeof(pl));
+  pl.slot = s;
+  pl.nc = static_cast<int>(nc); pl.np = static_cast<int>(np); pl.nf = static_cast<int>(nf);
+  pl.co = static_cast<int>(co); pl.fo = static_cast<int>(fo); pl.N = static_cast<int>(N); pl.F = static_cast<int>(F);
+  pl.n_colours = hm.n_colours;
+  for (int c = 0; c <= hm.n_colours; ++c) pl.colour_start[c] = hm.colour_start[c];
+  pl.alpha = p.alpha;
+  pl.mu = p.mu;
   for (int t = 0; t < kTagsPerSolve; ++t) {
     const cgks_bc &bc = p.bc[t];
-    bc_kind[t] = t < p.n_bc ? bc.kind : CGKS_BC_SLIP;
-    bc_uw[2 * t] = bc.u_wall[0]; bc_uw[2 * t + 1] = bc.u_wall[1];
-    bc_rho[t] = bc.rho; bc_u[2 * t] = bc.u[0]; bc_u[2 * t + 1] = bc.u[1]; bc_p[t] = bc.p;
+    if (t < p.n_bc && is_wall_kind(bc.kind)) pl.wall |= 1u << t;
+    pl.kind[t] = t < p.n_bc ? bc.kind : CGKS_BC_SLIP;
+    for (int q = 0; q < 2; ++q) { pl.uw[2 * t + q] = bc.u_wall[q]; pl.u[2 * t + q] = bc.u[q]; }
+    pl.rho[t] = bc.rho; pl.p[t] = bc.p;
   }
-  // component-sliced uploads: host [comps][len] -> device [comps][stride] at off
+  // the mesh as it is, [comps][n] -> [comps][stride] at an offset
   bool ok = true;
-  auto up = [&](auto *dst, const auto &src, int64_t len, int64_t stride, int64_t off) {
+  auto up = [&](auto *dst, const auto &src, int64_t n, int64_t stride) {
     using E = typename std::decay_t<decltype(src)>::value_type;
-    const int64_t comps = static_cast<int64_t>(src.size()) / std::max<int64_t>(len, 1);
-    for (int64_t q = 0; q < comps && ok && len > 0; ++q)
-      ok = cudaMemcpyAsync(dst + q * stride + off, src.data() + q * len, sizeof(E) * len, cudaMemcpyHostToDevice,
-                           st) == cudaSuccess;
+    static_assert(sizeof(E) == sizeof(*dst), "uploaded as it is");
+    const size_t row = sizeof(E) * n;
+    ok = ok && (n == 0 || cudaMemcpy2DAsync(dst, sizeof(E) * stride, src.data(), row, row, src.size() / n,
+                                            cudaMemcpyHostToDevice, st) == cudaSuccess);
   };
   DevArrays &d = b->d;
-  const int64_t T = kTagsPerSolve;
-  up(d.vol, vol, np, N, co); up(d.ivol, ivol, np, N, co); up(d.per, per, np, N, co); up(d.ih, ih, np, N, co);
-  up(d.m2, m2, np, N, co); up(d.op, op, np, N, co); up(d.snx, nxs, np, N, co); up(d.sny, nys, np, N, co); up(d.sS, sS, np, N, co);
-  up(d.cface, cface, np, N, co); up(d.cnbr, cnbr, np, N, co);
-  up(d.csid, csid, np, N, co); up(b->perm, perm, np, N, co); up(d.ccol, ccol, np, N, co);
-  up(d.wenok, wenok, np, N, co);
-  up(d.fn, fn, nf, F, fo); up(d.fS, fS, nf, F, fo); up(d.fjump, fjump, nf, F, fo); up(d.fxi, fxi, nf, F, fo);
-  up(d.fidl, fidl, nf, F, fo);
-  up(d.fc0, fc0, nf, F, fo); up(d.fc1, fc1, nf, F, fo); up(d.fsid, fsid, nf, F, fo);
-  up(d.mu, mu, 1, 1, s); up(d.bcuw, bc_uw, 2 * T, 0, 2 * T * s); up(d.bcrho, bc_rho, T, 0, T * s);
-  up(d.bcu, bc_u, 2 * T, 0, 2 * T * s); up(d.bcp, bc_p, T, 0, T * s); up(d.bckind, bc_kind, T, 0, T * s);
-  if (ok && b->mixed) {
-    auto f32 = [](const std::vector<double> &v) { return std::vector<float>(v.begin(), v.end()); };
-    std::vector<std::vector<float>> keep;   // alive until the stream syncs
-    auto upf = [&](float *dst, const std::vector<double> &src, int64_t len, int64_t stride, int64_t off) {
-      keep.push_back(f32(src));
-      up(dst, keep.back(), len, stride, off);
-    };
-    upf(d.f_ivol, ivol, np, N, co); upf(d.f_ih, ih, np, N, co); upf(d.f_m2, m2, np, N, co);
-    upf(d.f_op, op, np, N, co); upf(d.f_snx, snx, np, N, co); upf(d.f_sny, sny, np, N, co);
-    upf(d.f_shs, shs, np, N, co);
-    upf(d.f_fn, fn, nf, F, fo); upf(d.f_fS, fS, nf, F, fo); upf(d.f_fjump, fjump, nf, F, fo);
-    upf(d.f_fidl, fidl, nf, F, fo);
-    upf(d.f_fxi, fxi, nf, F, fo);
-    upf(d.f_mu, mu, 1, 1, s); upf(d.f_bcuw, bc_uw, 2 * T, 0, 2 * T * s); upf(d.f_bcrho, bc_rho, T, 0, T * s);
-    upf(d.f_bcu, bc_u, 2 * T, 0, 2 * T * s); upf(d.f_bcp, bc_p, T, 0, T * s);
-    ok = ok && cudaStreamSynchronize(st) == cudaSuccess;
-  }
+  double *xc = b->stage, *c2 = b->stage + 2 * nc;
+  up(d.vol + co, hm.vol, nc, N); up(d.per + co, hm.per, nc, N); up(d.ih + co, hm.h, nc, N); up(d.m2 + co, hm.m2, nc, N);
+  up(d.cface + co, hm.cface, nc, N); up(d.cnbr + co, hm.cnbr, nc, N); up(b->perm + co, hm.perm, nc, N);
+  up(xc, hm.xc, nc, nc); up(c2, hm.c2, nc, nc);
+  up(d.fn + fo, hm.fn, nf, F); up(d.fS + fo, hm.fS, nf, F); up(d.fidl + fo, hm.fdelta, nf, F);
+  up(d.fxi + fo, hm.fxi, nf, F); up(d.fc0 + fo, hm.fc0, nf, F); up(d.fc1 + fo, hm.fc1, nf, F);
+  if (!ok) return CGKS_ECUDA;
+  k_insert_cells<<<nblk(np, 64), 64, 0, st>>>(pl, d, b->perm, xc, c2);
+  k_insert_faces<<<std::max(nblk(nf, 128), 1), 128, 0, st>>>(pl, d);
+  b->launches += 2;
+  ok = cudaGetLastError() == cudaSuccess;
   ok = ok && cudaMemsetAsync(b->status + s, 0, sizeof(int), st) == cudaSuccess &&
-       cudaStreamSynchronize(st) == cudaSuccess;   // host tables go out of scope
+       cudaStreamSynchronize(st) == cudaSuccess;   // the mesh may go out of scope
   if (!ok) return CGKS_ECUDA;
   Member &M = b->mem[s];
   M = m;
@@ -1337,11 +1273,11 @@ int cgks_mesh_create(int dim, int64_t n_nodes, const double *xyz, int64_t n_cell
   if (!out) return CGKS_EINVAL;
   *out = nullptr;
   if (dim != 2 && dim != 3) return CGKS_EINVAL;
-  cgks_mesh *m = new (std::nothrow) cgks_mesh();
-  if (!m) return CGKS_ENOMEM;
-  m->dim = dim;
+  cgks_mesh *m = nullptr;
   int rc;
   try {
+    m = new cgks_mesh();
+    m->dim = dim;
     if (dim == 2)
       rc = build_host_mesh(n_nodes, xyz, n_cells, cell_type, cell_ptr, cell_nodes, n_bfaces, bface_ptr, bface_nodes,
                            bface_tag, m->h);
@@ -1439,11 +1375,7 @@ int cgks_solver_create(const cgks_mesh *m, const cgks_params *p, cgks_solver **o
     return CGKS_OK;
   }
   std::vector<Member> mem(1);
-  try {
-    mem[0].mesh = std::make_shared<HostMesh>(m->h);
-  } catch (const std::bad_alloc &) {
-    return fail(CGKS_ENOMEM);
-  }
+  mem[0].mesh = m->hp;
   mem[0].params = *p;
   rc = build_batch(shared_from(p), std::move(mem), s->stream, &s->b);
   if (rc) return fail(rc);
@@ -1829,7 +1761,7 @@ int cgks_server_submit(cgks_server *v, const cgks_mesh *m, const cgks_params *p,
   std::unique_ptr<cgks_server::Req> r(new (std::nothrow) cgks_server::Req());
   if (!r) return CGKS_ENOMEM;
   try {
-    r->mesh = std::make_shared<HostMesh>(m->h);
+    r->mesh = m->hp;
     r->W0.assign(W0, W0 + 4 * m->h.n_cells);
   } catch (const std::bad_alloc &) {
     return CGKS_ENOMEM;

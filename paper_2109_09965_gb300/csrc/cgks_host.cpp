@@ -30,40 +30,6 @@ inline uint64_t edge_key(int64_t a, int64_t b) {
   return (static_cast<uint64_t>(a) << 32) ^ static_cast<uint64_t>(b);
 }
 
-// Solve min ||A c - b|| for every unit b by modified Gram-Schmidt:
-// A = Q R, pinv = R^{-1} Q^T  (rows x 5 -> 5 x rows).
-bool mgs_pinv(int rows, const double *A, double *pinv) {
-  double Q[64][kNM], R[kNM][kNM];
-  for (int r = 0; r < rows; ++r)
-    for (int c = 0; c < kNM; ++c) Q[r][c] = A[r * kNM + c];
-  std::memset(R, 0, sizeof R);
-  for (int j = 0; j < kNM; ++j) {
-    for (int i = 0; i < j; ++i) {
-      double d = 0.0;
-      for (int r = 0; r < rows; ++r) d += Q[r][i] * Q[r][j];
-      R[i][j] = d;
-      for (int r = 0; r < rows; ++r) Q[r][j] -= d * Q[r][i];
-    }
-    double nrm = 0.0;
-    for (int r = 0; r < rows; ++r) nrm += Q[r][j] * Q[r][j];
-    nrm = std::sqrt(nrm);
-    if (!(nrm > 1e-13)) return false;
-    R[j][j] = nrm;
-    for (int r = 0; r < rows; ++r) Q[r][j] /= nrm;
-  }
-  // pinv[q][r] = sum_k Rinv[q][k] Q[r][k]; back substitution per row r
-  for (int r = 0; r < rows; ++r) {
-    double y[kNM];
-    for (int q = kNM - 1; q >= 0; --q) {
-      double v = Q[r][q];
-      for (int k = q + 1; k < kNM; ++k) v -= R[q][k] * y[k];
-      y[q] = v / R[q][q];
-    }
-    for (int q = 0; q < kNM; ++q) pinv[q * rows + r] = y[q];
-  }
-  return true;
-}
-
 }  // namespace
 
 int build_host_mesh(int64_t nn, const double *xy, int64_t nc, const uint8_t *ctype,
@@ -293,84 +259,6 @@ int build_host_mesh(int64_t nn, const double *xy, int64_t nc, const uint8_t *cty
   for (int64_t b = 0; b < nbf; ++b) tag_seen[btag[b]] = 1;
   for (int t = 0; t < CGKS_MAX_BC; ++t) if (tag_seen[t]) M.bface_tags_used.push_back(t);
   return CGKS_OK;
-}
-
-void build_operator(const HostMesh &M, const std::vector<char> &tag_is_wall, std::vector<double> &op,
-                    std::vector<unsigned char> *quad_ok) {
-  const int64_t nc = M.n_cells, nf = M.n_faces;
-  op.assign(static_cast<size_t>(kNCol * kNM) * nc, 0.0);
-  if (quad_ok) quad_ok->assign(nc, 0);
-  for (int64_t i = 0; i < nc; ++i) {
-    const double hi = M.h[i], xi0 = M.xc[i], yi0 = M.xc[nc + i];
-    const double mi[3] = { M.m2[i], M.m2[nc + i], M.m2[2 * nc + i] };
-    double A[64 * kNM];
-    int rows = 0;
-    int row_col[64];                      // operator column of each row
-    int nslots = 0;
-    for (int s = 0; s < kMaxFace; ++s) {
-      int32_t fs = M.cface[s * nc + i];
-      if (fs == kNoFace) continue;
-      int32_t f = fs >= 0 ? fs : ~fs;
-      int32_t j = M.cnbr[s * nc + i];
-      double dx, dy, Ixx, Ixy, Iyy;     // centre offset and central moments of the stencil cell
-      if (j >= 0) {
-        dx = M.xc[j] - xi0; dy = M.xc[nc + j] - yi0;
-        Ixx = M.c2[j]; Ixy = M.c2[nc + j]; Iyy = M.c2[2 * nc + j];
-      } else {
-        int tag = -1 - M.fc1[f];
-        if (!tag_is_wall[tag]) continue;
-        // mirror image of cell i across the wall line
-        double nx = M.fn[f], ny = M.fn[nf + f];
-        double px = xi0 + M.fxi[0 * nf + f] * hi, py = yi0 + M.fxi[1 * nf + f] * hi;  // a point on the wall
-        double d = (xi0 - px) * nx + (yi0 - py) * ny;
-        dx = -2.0 * d * nx; dy = -2.0 * d * ny;
-        double R[2][2] = { { 1 - 2 * nx * nx, -2 * nx * ny }, { -2 * nx * ny, 1 - 2 * ny * ny } };
-        double C[2][2] = { { M.c2[i], M.c2[nc + i] }, { M.c2[nc + i], M.c2[2 * nc + i] } };
-        double T[2][2];
-        for (int a = 0; a < 2; ++a) for (int b = 0; b < 2; ++b) {
-          double v = 0.0;
-          for (int p = 0; p < 2; ++p) for (int q = 0; q < 2; ++q) v += R[a][p] * C[p][q] * R[b][q];
-          T[a][b] = v;
-        }
-        Ixx = T[0][0]; Ixy = T[0][1]; Iyy = T[1][1];
-      }
-      double ex = dx / hi, ey = dy / hi, h2 = hi * hi;
-      double mq[3] = { Ixx / h2 + ex * ex, Ixy / h2 + ex * ey, Iyy / h2 + ey * ey };
-      double r0[kNM] = { ex, ey, mq[0] - mi[0], mq[1] - mi[1], mq[2] - mi[2] };
-      double r1[kNM] = { 1.0, 0.0, 2.0 * ex, ey, 0.0 };
-      double r2[kNM] = { 0.0, 1.0, 0.0, ex, 2.0 * ey };
-      for (int q = 0; q < kNM; ++q) {
-        A[rows * kNM + q] = r0[q]; A[(rows + 1) * kNM + q] = r1[q]; A[(rows + 2) * kNM + q] = r2[q];
-      }
-      row_col[rows] = 3 * s; row_col[rows + 1] = 3 * s + 1; row_col[rows + 2] = 3 * s + 2;
-      rows += 3;
-      ++nslots;
-    }
-    double *out = op.data();
-    auto put = [&](int col, int q, double v) { out[(static_cast<int64_t>(col) * kNM + q) * nc + i] = v; };
-    if (nslots < 2) {
-      // linear reconstruction from the own mean gradient
-      put(kNCol - 2, 0, hi);
-      put(kNCol - 1, 1, hi);
-      continue;
-    }
-    double o0[kNM] = { 1.0, 0.0, 0.0, 0.0, 0.0 }, o1[kNM] = { 0.0, 1.0, 0.0, 0.0, 0.0 };
-    for (int q = 0; q < kNM; ++q) { A[rows * kNM + q] = o0[q]; A[(rows + 1) * kNM + q] = o1[q]; }
-    row_col[rows] = kNCol - 2; row_col[rows + 1] = kNCol - 1;
-    rows += 2;
-    double pinv[kNM * 64];
-    if (!mgs_pinv(rows, A, pinv)) {
-      put(kNCol - 2, 0, hi);
-      put(kNCol - 1, 1, hi);
-      continue;
-    }
-    for (int r = 0; r < rows; ++r) {
-      int col = row_col[r];
-      bool grad_col = (col % 3) != 0 || col >= 3 * kMaxFace;
-      for (int q = 0; q < kNM; ++q) put(col, q, pinv[q * rows + r] * (grad_col ? hi : 1.0));
-    }
-    if (quad_ok) (*quad_ok)[i] = 1;
-  }
 }
 
 }  // namespace cgks

@@ -3,6 +3,7 @@
 #pragma once
 
 #include <cstdint>
+#include <memory>
 #include <vector>
 
 #include "../../include/cgks.h"
@@ -42,15 +43,6 @@ struct HostMesh {
   std::vector<double> fxi;           // [8][nf] scaled Gauss offsets: side0 (k0 x,y, k1 x,y), side1 (...)
   std::vector<int32_t> bface_tags_used;
 };
-
-// Compact least-squares reconstruction operator of every cell, [kNCol*kNM][n]
-// (column-major per cell: op[(col*kNM + q)*n + i]), with h_i folded into the
-// gradient columns.  tag_is_wall[t] selects the boundary tags whose mirror
-// ghost cells enter the fit.
-// quad_ok (optional): per cell 1 when the stencil gave a least-squares
-// quadratic, 0 when it fell back to the linear polynomial of the own gradient
-void build_operator(const HostMesh &m, const std::vector<char> &tag_is_wall, std::vector<double> &op,
-                    std::vector<unsigned char> *quad_ok = nullptr);
 
 // Returns CGKS_OK or CGKS_EMESH / CGKS_EINVAL.
 int build_host_mesh(int64_t n_nodes, const double *xy, int64_t n_cells, const uint8_t *ctype,
@@ -100,6 +92,7 @@ void build_operator3(const HostMesh3 &m, const std::vector<char> &tag_is_wall, s
 
 struct cgks_mesh {
   int dim = 2;
-  cgks::HostMesh h;
+  const std::shared_ptr<cgks::HostMesh> hp = std::make_shared<cgks::HostMesh>();   // the solves on it share it
+  cgks::HostMesh &h = *hp;
   cgks::HostMesh3 h3;
 };

@@ -134,3 +134,14 @@ def test_far_field_state_at_whole_and_other_exponents(dim, gamma):
     p = (gamma - 1) / (GAM - 1) / GAM                          # of the state's energy
     spec = dict(gamma=gamma, mu=0.005, cfl_hi=0.3, bcs=[dict(kind="farfield", rho=1.0, u=u, p=p)])
     compare(mesh, spec, state(mesh, 0.2, 0.4), "fp64", 2)
+
+
+@pytest.mark.parametrize("nx, ny", [(1, 1), (2, 1), (3, 1), (9, 7), (16, 8), (43, 3)])
+def test_device_tables_of_small_and_ragged_meshes(nx, ny):
+    """The reconstruction operator formed on the device: cells with no, one and
+    two stencil cells (linear fallback), wall mirrors on some sides, cell
+    counts around whole blocks (1 to 3, 63, 128, 129)."""
+    mesh = MG.box(nx, ny, jitter=0.1, seed=6, cells="quad", tags=(0, 1, 0, 1))
+    spec = dict(gamma=GAM, mu=0.01, cfl_hi=0.3,
+                bcs=[dict(kind="farfield", rho=1.0, u=(0.2, 0.0), p=1 / GAM), dict(kind="noslip")])
+    compare(mesh, spec, state(mesh, 0.1, 0.2), "fp64", 2)

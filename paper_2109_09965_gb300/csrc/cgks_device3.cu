@@ -9,6 +9,7 @@
 #include <cstring>
 #include <memory>
 #include <new>
+#include <numeric>
 #include <vector>
 
 #include "cgks_internal.h"
@@ -42,6 +43,13 @@ struct Geo3 {
 };
 
 struct Piece3 { void **dst; size_t bytes; };
+
+// one launch of the point relaxation over colour c
+struct SweepPass {
+  int c;
+  bool down;   // colours descending: only cells with a neighbour of a higher colour
+  bool end;    // of the last sweep: the last relaxation of these cells, ascending of those left out descending
+};
 }  // namespace
 
 struct Solver3 {
@@ -49,8 +57,8 @@ struct Solver3 {
   int64_t N = 0, F = 0;
   bool mixed = false;
   int n_colours = 0;
-  std::vector<int32_t> colour_start;
-  std::vector<int> sweep_seq;
+  std::vector<int32_t> colour_start, n_higher;
+  std::vector<SweepPass> passes;
   cudaStream_t stream = nullptr;
   void *arena = nullptr;
   size_t arena_bytes = 0;
@@ -198,8 +206,6 @@ void lo_solve(Solver3 *s) {
     launch(s, KI_LOCELL, k_lo_cell<TF>, gc, blk, static_cast<int>(s->N), fpar<TF>(s), first, (const double *)s->Wn,
            s->U, (const TF *)B.delta, base);
   };
-  std::vector<int> last(s->n_colours, -1);
-  for (size_t q = 0; q < s->sweep_seq.size(); ++q) last[s->sweep_seq[q]] = static_cast<int>(q);
   for (int k = 0; k < s->P.n_implicit; ++k) {
     if (k == 0 || !adv) cells(k == 0 ? 1 : 0);
     const int fs = s->tune.shape(TK_LOFACE), ss = s->tune.shape(TK_SWEEP);
@@ -209,17 +215,17 @@ void lo_solve(Solver3 *s) {
     });
     launch(s, KI_LORHS, k_lo_rhs<TF>, gc, blk, s->dm, s->dp, fpar<TF>(s).gamma, k == 0 ? 1 : 0, colour0_end,
            (const TF *)base, (const TF *)B.Flo, (const double *)s->Rp0, s->Src, B.Rk, B.invD, B.delta, B.lamS);
-    for (size_t q = 0; q < s->sweep_seq.size(); ++q) {
-      const int c = s->sweep_seq[q];
-      const int beg = s->colour_start[c], cnt = s->colour_start[c + 1] - beg;
+    for (const SweepPass &q : s->passes) {
+      const int beg = s->colour_start[q.c], nh = s->n_higher[q.c];
+      const int cnt = q.down ? nh : s->colour_start[q.c + 1] - beg;
+      const bool end = adv && q.end;
       tuned_launch(s->tune, TK_SWEEP, s->stream, [&] {
         const int lanes = sweep_lanes<TF>(cnt);
         auto go = [&](auto kern) {
           launch(s, KI_SWEEP, kern, dim3(nblk(static_cast<int64_t>(cnt) * lanes, shape_bs(ss))), dim3(shape_bs(ss)),
-                 fmesh<TF>(s), fpar<TF>(s), beg, cnt, (const TF *)base, (const TF *)B.Rk, (const TF *)B.invD,
+                 fmesh<TF>(s), fpar<TF>(s), beg, cnt, q.down ? beg : beg + nh, (const TF *)base, (const TF *)B.Rk, (const TF *)B.invD,
                  (const TF *)B.lamS, B.delta, s->U, next);
         };
-        const bool end = adv && last[c] == static_cast<int>(q);
         if (lanes == 1) {
           if (end) go(k_sweep<TF, true, 1>);
           else go(k_sweep<TF, false, 1>);
@@ -269,7 +275,7 @@ long long count_launches(const Solver3 *s, bool cycle) {
   if (!cycle) return 2 + hi + 1;
   const long long cells = last_pass_advances(s) ? 1 : s->P.n_implicit + 1;
   const long long lo =
-      s->P.n_implicit > 0 ? s->P.n_implicit * (2 + static_cast<long long>(s->sweep_seq.size())) + cells : 0;
+      s->P.n_implicit > 0 ? s->P.n_implicit * (2 + static_cast<long long>(s->passes.size())) + cells : 0;
   return 2 + hi + 3 + lo + 2;
 }
 
@@ -394,6 +400,27 @@ void s3_destroy(Solver3 *s) {
   delete s;
 }
 
+// Boundary faces are handed out by colour, then reverse Cuthill-McKee position
+// of their cell (and its own face order).
+static void sort_boundary_faces(Solver3 *s, const HostMesh3 &m) {
+  std::vector<int64_t> pos(m.n_cells);
+  for (int64_t k = 0; k < m.n_cells; ++k) pos[m.rcm[k]] = k;
+  std::vector<int32_t> &f = s->bf_face;
+  std::vector<size_t> at(f.size());
+  std::iota(at.begin(), at.end(), size_t(0));
+  std::stable_sort(at.begin(), at.end(), [&](size_t a, size_t b) {
+    const int64_t x = m.perm[m.fc0[f[a]]], y = m.perm[m.fc0[f[b]]];
+    return m.colour[x] != m.colour[y] ? m.colour[x] < m.colour[y] : pos[x] < pos[y];
+  });
+  const std::vector<int32_t> face = f, tag = s->bf_tag;
+  const std::vector<double> geo = s->bf_geo;
+  for (size_t k = 0; k < at.size(); ++k) {
+    f[k] = face[at[k]];
+    s->bf_tag[k] = tag[at[k]];
+    std::copy_n(&geo[7 * at[k]], 7, &s->bf_geo[7 * k]);
+  }
+}
+
 int s3_create(const HostMesh3 &m, const cgks_params *p, cudaStream_t stream, Timer *timer, Solver3 **out) {
   *out = nullptr;
   std::unique_ptr<Solver3> S(new (std::nothrow) Solver3());
@@ -414,19 +441,24 @@ int s3_create(const HostMesh3 &m, const cgks_params *p, cudaStream_t stream, Tim
                             m.fS[f] };
     s->bf_geo.insert(s->bf_geo.end(), geo, geo + 7);
   }
+  sort_boundary_faces(s, m);
   s->stream = stream;
   s->timer = timer;
   s->tune.on = p->autotune != 0;
   if (s->N * kNCol3 * kNM3 > INT32_MAX || s->F * 24 > INT32_MAX) return CGKS_EINVAL;
-  {
-    std::vector<int> seq;
-    const int C = m.n_colours;
-    for (int sw = 0; sw < p->n_sweeps; ++sw) {
-      for (int c = 0; c < C; ++c) if (seq.empty() || seq.back() != c) seq.push_back(c);
-      for (int c = C - 1; c >= 0; --c) if (seq.empty() || seq.back() != c) seq.push_back(c);
-    }
-    if (!seq.empty()) seq.erase(seq.begin());
-    s->sweep_seq = seq;
+  s->n_higher = m.n_higher;
+  // The passes after the first (colour 0, done with the right-hand side) of
+  // n_sweeps x (colours ascending, colours descending).  A relaxation whose
+  // inputs have not changed since the cell's last one gives the same values
+  // and is left out.  Ascending, every cell has neighbours of all lower colours
+  // (greedy colouring), which were relaxed since.  Descending, only neighbours
+  // of higher colours were, so cells without any rest: 162,000 of the 300,000
+  // cells of the middle colours of a 512,000-cell sphere.
+  for (int sw = 0; sw < p->n_sweeps; ++sw) {
+    const bool end = sw == p->n_sweeps - 1;
+    for (int c = 1; c < m.n_colours; ++c) s->passes.push_back({ c, false, end });
+    for (int c = m.n_colours - 2; c >= 0; --c)
+      if (m.n_higher[c] > 0) s->passes.push_back({ c, true, end });
   }
   std::vector<Piece3> pc;
   plan(s, pc);

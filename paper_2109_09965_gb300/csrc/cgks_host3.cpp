@@ -313,9 +313,18 @@ int build_host_mesh3(int64_t nn, const double *xyz, int64_t nc, const uint8_t *c
   for (int64_t c = 0; c < nc; ++c) M.colour_start[M.colour[c] + 1]++;
   for (int c = 0; c < ncol; ++c) M.colour_start[c + 1] += M.colour_start[c];
   {
-    std::vector<int32_t> fill(M.colour_start.begin(), M.colour_start.end() - 1);
+    auto higher = [&](int64_t v) {
+      if (M.colour[v] == 0) return true;
+      for (int64_t w : adj[v])
+        if (M.colour[w] > M.colour[v]) return true;
+      return false;
+    };
+    M.n_higher.assign(ncol, 0);
+    for (int64_t v : M.rcm) M.n_higher[M.colour[v]] += higher(v);
+    std::vector<int32_t> first(M.colour_start.begin(), M.colour_start.end() - 1), rest = first;
+    for (int c = 0; c < ncol; ++c) rest[c] += M.n_higher[c];
     for (int64_t v : M.rcm) {
-      const int32_t pos = fill[M.colour[v]]++;
+      const int32_t pos = (higher(v) ? first : rest)[M.colour[v]]++;
       M.perm[pos] = static_cast<int32_t>(v);
       M.iperm[v] = pos;
     }

@@ -57,12 +57,14 @@ constexpr int kMaxFace3 = 6;   // faces per cell (hexahedron)
 constexpr int kNCol3 = 4 * kMaxFace3 + 3;  // 4 per face slot (mean, 3 gradients) + own gradient
 constexpr int kMaxGP3 = 4;     // Gauss points per face (quadrilateral)
 
-// 3-D mesh in the library's internal orders (as HostMesh).
+// 3-D mesh in the library's internal orders (as HostMesh; inside a colour the
+// cells with a neighbour of a higher colour come first).
 struct HostMesh3 {
   int64_t n_cells = 0, n_faces = 0, n_bfaces = 0;
   int n_colours = 0;
   std::vector<int64_t> rcm;
   std::vector<int32_t> colour, perm, iperm, colour_start;
+  std::vector<int32_t> n_higher;   // [n_colours] cells with a neighbour of a higher colour (colour 0: all)
   // cells, internal order
   std::vector<double> vol, h, asum;  // volume, |Omega|^(1/3), sum of face areas
   std::vector<double> xc;            // [3][n] centroid

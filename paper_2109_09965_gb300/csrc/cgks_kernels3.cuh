@@ -1077,8 +1077,9 @@ __global__ void __launch_bounds__(kCellBlock) k_lo_rhs(MeshT<double> m, ParamsT<
 // its rounding.
 // LANES: one thread per cell, or eight (one per face slot, six used) where a
 // colour has too few cells to fill the device (sweep_lanes).
-// LAST: the cell's last relaxation of the implicit step also advances U and
-// writes the next step's base record (second buffer).
+// LAST: the cell's last relaxation of the implicit step, from cell adv on (the
+// others are relaxed once more), also advances U and writes the next step's
+// base record (second buffer).
 template <typename T>
 struct SlotData {
   static constexpr int NB = is_f32<T>() ? 8 : 5;   // part of a base record a sweep reads
@@ -1132,8 +1133,8 @@ constexpr int kOneLane64 = 4864, kOneLane32 = 14000;
 template <typename T> int sweep_lanes(int cnt) { return cnt >= (is_f32<T>() ? kOneLane32 : kOneLane64) ? 1 : kSweepLanes; }
 template <typename T, bool LAST, int LANES>
 __global__ void __launch_bounds__(kMaxShapeBlock)
-    k_sweep(MeshT<T> m, ParamsT<T> P, int begin, int count, const T *base, const T *Rk, const T *invD, const T *lamS,
-            T *delta, double *U, T *base_next) {
+    k_sweep(MeshT<T> m, ParamsT<T> P, int begin, int count, int adv, const T *base, const T *Rk, const T *invD,
+            const T *lamS, T *delta, double *U, T *base_next) {
   const int n = m.nc;
   constexpr int ND = del_run<T>();
   const int g = static_cast<int>(blockIdx.x * blockDim.x + threadIdx.x) / LANES;
@@ -1179,7 +1180,7 @@ __global__ void __launch_bounds__(kMaxShapeBlock)
       }
     }
     store_delta(P.gamma, bi, d, delta, i);
-    if constexpr (LAST) {
+    if (LAST && i >= adv) {
       double u[NV];
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
@@ -1232,7 +1233,7 @@ __global__ void __launch_bounds__(kMaxShapeBlock)
     }
     if constexpr (LAST) {
       us += static_cast<double>(ds);
-      if (i >= 0 && s < NV) U[s * n + i] = us;
+      if (i >= adv && s < NV) U[s * n + i] = us;
       double u[NV];
 #pragma unroll
       for (int v = 0; v < NV; ++v) u[v] = __shfl_sync(0xffffffffu, us, v, LANES);
@@ -1240,7 +1241,7 @@ __global__ void __launch_bounds__(kMaxShapeBlock)
       base_record(P, u, rec);
 #pragma unroll
       for (int v = 0; v < LANES; ++v)
-        if (i >= 0 && s == v) {
+        if (i >= adv && s == v) {
           const T two[2] = { rec[2 * v], rec[2 * v + 1] };
           T *o = base_next + static_cast<size_t>(i) * kBase + 2 * v;
           o[0] = two[0];

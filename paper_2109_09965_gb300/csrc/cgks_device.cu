@@ -231,7 +231,7 @@ void enqueue_hi_eval(Batch *b, const TF *W, const TF *Wx, TF *Fout) {
   const bool weno = b->sh.weno_eps > 0.0 && !chr, full = b->sh.flux_hi == CGKS_FLUX_FULL;
   const int rs = b->tune.shape(TK_RECON), fs = b->tune.shape(TK_FACE);
   auto recon = [&](auto kern) {
-    launch(b, KI_RECON, kern, dim3(nblk(b->N, shape_bs(rs))), dim3(shape_bs(rs)), fmesh<TF>(b),
+    launch(b, KI_RECON, kern, dim3(nblk(var_items<4 / recon_vars<TF>()>(b->N), shape_bs(rs))), dim3(shape_bs(rs)), fmesh<TF>(b),
            fparams<TF>(b), W, Wx, B.coef);
   };
   auto face = [&](auto kern, int threads) {   // threads: of a face

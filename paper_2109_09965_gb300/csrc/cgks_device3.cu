@@ -145,7 +145,7 @@ void hi_eval(Solver3 *s, const TF *W, const TF *Wx, TF *Fout) {
   const bool weno = s->P.weno_eps > 0.0, full = s->P.flux_hi == CGKS_FLUX_FULL;
   const int rs = s->tune.shape(TK_RECON), fs = s->tune.shape(TK_FACE);
   tuned_launch(s->tune, TK_RECON, s->stream, [&] {
-    const dim3 gr(nblk(s->N, shape_bs(rs))), blk(shape_bs(rs));
+    const dim3 gr(nblk((s->N + 31) / 32 * 32 * (NV / recon_vars<TF>()), shape_bs(rs))), blk(shape_bs(rs));
     if (weno)
       launch(s, KI_RECON, k_recon_weno<TF>, gr, blk, fmesh<TF>(s), fpar<TF>(s), W, Wx, B.coef,
              (const unsigned char *)s->g.wenok);

@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(kCellBlock) k_dt(MeshT<double> m, ParamsT<doub
   pdl_exit();
 }
 
-// Wall ghost of a state and its gradient (global frame), through the face frame.
+// FP32: wall ghost of a state and its gradient (global frame), through the face frame.
 template <typename T>
 __device__ __forceinline__ void wall_ghost_global(const ParamsT<T> &P, int tag, T nx, T ny, const T w[4],
                                                   const T gx[4], const T gy[4], T wg[4], T ggx[4], T ggy[4]) {
@@ -225,14 +225,14 @@ __host__ __device__ __forceinline__ bool is_wall_kind(int k) { return k == CGKS_
 // bit 1 + s of on is set (slots by a constant index: no local memory).
 __device__ __forceinline__ float quot(float a, float b) { return a / b; }
 __device__ __forceinline__ double quot(double a, double b) { return a * D::d_rcp(b); }
-template <typename T>
+template <typename T, int NC>
 __device__ __forceinline__ void weno_combine(const ParamsT<T> &P, T mxx, T mxy, T myy, unsigned on,
-                                             const T lin[5][2][4], T c[kNM][4]) {
+                                             const T (&lin)[5][2][NC], T (&c)[kNM][NC]) {
   const int nk = __popc(on);
   const T g0 = P.weno_g0, eps = P.weno_eps;
   const T gk = quot(T(1) - g0, T(nk));
 #pragma unroll
-  for (int v = 0; v < 4; ++v) {
+  for (int v = 0; v < NC; ++v) {
     const T c0 = c[0][v], c1 = c[1][v], c2 = c[2][v], c3 = c[3][v], c4 = c[4][v];
     const T b0 = c0 * c0 + c1 * c1 + (T(4) * c2 * c2 + c3 * c3) * mxx + (c3 * c3 + T(4) * c4 * c4) * myy +
                  (T(4) * c2 * c3 + T(4) * c3 * c4) * mxy + T(4) * c2 * c2 + c3 * c3 + T(4) * c4 * c4;
@@ -269,54 +269,87 @@ __device__ __forceinline__ void weno_combine(const ParamsT<T> &P, T mxx, T mxy, 
 
 // K1: compact least-squares quadratic of every cell.
 //   coef[(q*4 + v)*nc + i], q over (xi, eta, xi^2, xi eta, eta^2).
-template <typename T, bool WENO>
+// NC: conserved variables per thread.  FP64: one, the warps of a block on the
+// same 32 cells each taking another, because an FP64 launch takes as long as
+// the warps of one sub-core (608 of them) issue one after another, and one
+// thread per cell left most sub-cores idle below 20,000 cells; the operator
+// is then read from the cache by three of the four.  FP32: all four, the reads
+// of the operator bound it.  us per launch, FP64, before / now (with the wall
+// mirrors as linear maps): 128 cells 32.8 / 15.3, 2,048 31.1 / 14.4, 6,354 with
+// nonlinear weights 38.2 / 20.7, 57,344 46.9 / 45.8.
+template <typename T> __host__ __device__ constexpr int recon_vars() { return is_f32<T>() ? 4 : 1; }
+// threads of a launch over n cells with a warp per variable of 32 cells
+template <int VARS> __host__ __device__ constexpr int64_t var_items(int64_t n) { return (n + 31) / 32 * 32 * VARS; }
+template <typename T, bool WENO, int NC>
 __device__ __forceinline__ void recon_at(const MeshT<T> &m, const ParamsT<T> &P, const T *__restrict__ W,
-                                         const T *__restrict__ Wx, T *__restrict__ coef, const int i) {
-  const int n = m.nc;
-  T wi[4], gxi[4], gyi[4];
-  for (int v = 0; v < 4; ++v) { wi[v] = W[v * n + i]; gxi[v] = Wx[v * n + i]; gyi[v] = Wx[(4 + v) * n + i]; }
-  T c[kNM][4];
+                                         const T *__restrict__ Wx, T *__restrict__ coef, const int i,
+                                         const int comp) {
+  const int n = m.nc, vo = NC == 4 ? 0 : comp;
+  T wi[NC], gxi[NC], gyi[NC];
+#pragma unroll
+  for (int v = 0; v < NC; ++v) {
+    wi[v] = W[(vo + v) * n + i];
+    gxi[v] = Wx[(vo + v) * n + i];
+    gyi[v] = Wx[(4 + vo + v) * n + i];
+  }
+  T c[kNM][NC];
+#pragma unroll
   for (int q = 0; q < kNM; ++q) {
     T o0 = m.op[((kNCol - 2) * kNM + q) * n + i], o1 = m.op[((kNCol - 1) * kNM + q) * n + i];
-    for (int v = 0; v < 4; ++v) c[q][v] = o0 * gxi[v] + o1 * gyi[v];
+#pragma unroll
+    for (int v = 0; v < NC; ++v) c[q][v] = o0 * gxi[v] + o1 * gyi[v];
   }
   // linear WENO candidates: h times the cell-mean gradients of the cell and its face neighbours
-  T lin[WENO ? 5 : 1][2][4];
+  T lin[WENO ? 5 : 1][2][NC];
   unsigned on = 1;
   if constexpr (WENO) {
     const T hi = T(1) / m.ih[i];
-    for (int v = 0; v < 4; ++v) { lin[0][0][v] = hi * gxi[v]; lin[0][1][v] = hi * gyi[v]; }
+#pragma unroll
+    for (int v = 0; v < NC; ++v) { lin[0][0][v] = hi * gxi[v]; lin[0][1][v] = hi * gyi[v]; }
   }
 #pragma unroll
   for (int s = 0; s < kMaxFace; ++s) {
     int fs = m.cface[s * n + i];
     if (fs == kNoFace) continue;
     int j = m.cnbr[s * n + i];
-    T b0[4], b1[4], b2[4];
+    T b0[NC], b1[NC], b2[NC];
     if (j >= 0) {
-      for (int v = 0; v < 4; ++v) {
-        b0[v] = W[v * n + j] - wi[v];
-        b1[v] = Wx[v * n + j];
-        b2[v] = Wx[(4 + v) * n + j];
+#pragma unroll
+      for (int v = 0; v < NC; ++v) {
+        b0[v] = W[(vo + v) * n + j] - wi[v];
+        b1[v] = Wx[(vo + v) * n + j];
+        b2[v] = Wx[(4 + vo + v) * n + j];
       }
       if constexpr (WENO) {
         const T hi = T(1) / m.ih[i];
-        for (int v = 0; v < 4; ++v) { lin[1 + s][0][v] = hi * b1[v]; lin[1 + s][1][v] = hi * b2[v]; }
+#pragma unroll
+        for (int v = 0; v < NC; ++v) { lin[1 + s][0][v] = hi * b1[v]; lin[1 + s][1][v] = hi * b2[v]; }
         on |= 2u << s;
       }
     } else {
       int f = fs >= 0 ? fs : ~fs;
       int tag = -1 - m.fc1[f];
       if (!is_wall_kind(P.bc_kind[tag])) continue;
-      T wg[4];
-      wall_ghost_global(P, tag, m.fn[f], m.fn[m.nf + f], wi, gxi, gyi, wg, b1, b2);
-      for (int v = 0; v < 4; ++v) b0[v] = wg[v] - wi[v];
+      if constexpr (NC == 4) {
+        T wg[4];
+        wall_ghost_global(P, tag, m.fn[f], m.fn[m.nf + f], wi, gxi, gyi, wg, b1, b2);
+#pragma unroll
+        for (int v = 0; v < 4; ++v) b0[v] = wg[v] - wi[v];
+      } else {   // the mirror image mixes the variables
+        const double nn[2] = { m.fn[f], m.fn[m.nf + f] };
+        double b[2];
+        D::WallMap<2>(P.bc_kind[tag], P.bc_uw + 2 * tag, nn).one(comp, W + i, Wx + i, n, b0[0], b);
+        b1[0] = b[0];
+        b2[0] = b[1];
+      }
     }
+#pragma unroll
     for (int q = 0; q < kNM; ++q) {
       T o0 = m.op[((3 * s) * kNM + q) * n + i];
       T o1 = m.op[((3 * s + 1) * kNM + q) * n + i];
       T o2 = m.op[((3 * s + 2) * kNM + q) * n + i];
-      for (int v = 0; v < 4; ++v) c[q][v] += o0 * b0[v] + o1 * b1[v] + o2 * b2[v];
+#pragma unroll
+      for (int v = 0; v < NC; ++v) c[q][v] += o0 * b0[v] + o1 * b1[v] + o2 * b2[v];
     }
   }
   // cells whose stencil fell back to the linear polynomial of their own
@@ -324,8 +357,10 @@ __device__ __forceinline__ void recon_at(const MeshT<T> &m, const ParamsT<T> &P,
   // in the operator and keep it; the others may be limited
   if constexpr (WENO)
     if (m.wenok[i]) weno_combine(P, m.m2[i], m.m2[n + i], m.m2[2 * n + i], on, lin, c);
+#pragma unroll
   for (int q = 0; q < kNM; ++q)
-    for (int v = 0; v < 4; ++v) coef[(q * 4 + v) * n + i] = c[q][v];
+#pragma unroll
+    for (int v = 0; v < NC; ++v) coef[(q * 4 + vo + v) * n + i] = c[q][v];
 }
 template <typename T, bool WENO>
 __global__ void __launch_bounds__(kMaxShapeBlock) k_recon(MeshT<T> m, ParamsT<T> P,
@@ -333,12 +368,15 @@ __global__ void __launch_bounds__(kMaxShapeBlock) k_recon(MeshT<T> m, ParamsT<T>
                                                                         const T *Wx,
                                                                         T *coef) {
   pdl_enter();
-  for_items(m.nc, [&](int i) {
+  constexpr int NC = recon_vars<T>(), G = 4 / NC;   // threads per cell
+  for_items(static_cast<int>(var_items<G>(m.nc)), [&](int t) {
+    const int i = G == 1 ? t : t / (32 * G) * 32 + t % 32, comp = t / 32 % G;
+    if (i >= m.nc) return;
     if (P.slim) {
       const int sid = m.csid[i];
       if (sid >= 0 && (P.slim[sid] != 0) != WENO) return;
     }
-    recon_at<T, WENO>(m, P, W, Wx, coef, i);
+    recon_at<T, WENO, NC>(m, P, W, Wx, coef, i, comp);
   });
   pdl_exit();
 }
@@ -476,8 +514,14 @@ __device__ void char_side(const MeshT<T> &m, const ParamsT<T> &P, const T *__res
 template <typename T>
 __device__ __forceinline__ void lo_ghost(const ParamsT<T> &P, int tag, T nx, T ny, const T w[4], T wg[4]) {
   T wl[4], z[4] = { T(0), T(0), T(0), T(0) }, wgl[4], a[4], b[4];
-  D::rot_in(nx, ny, w, wl);
   int kind = P.bc_kind[tag];
+  if constexpr (!is_f32<T>())
+    if (is_wall_kind(kind)) {
+      const double nn[2] = { nx, ny };
+      D::WallMap<2>(kind, P.bc_uw + 2 * tag, nn).apply(w, wg);
+      return;
+    }
+  D::rot_in(nx, ny, w, wl);
   if (kind == CGKS_BC_FARFIELD) {
     farfield_ghost(P, tag, nx, ny, wl, wgl);
   } else if (kind == CGKS_BC_DIRICHLET) {
@@ -687,7 +731,10 @@ __device__ __forceinline__ void face_point_at(const MeshT<double> &m, const Para
     } else if (kind == CGKS_BC_OUTFLOW) {
       for (int v = 0; v < 4; ++v) { wR[v] = wL[v]; wr[v] = wl[v]; gR[0][v] = gL[0][v]; gR[1][v] = gL[1][v]; }
     } else {
-      wall_ghost_global(P, tag, nx, ny, wL, gL[0], gL[1], wR, gR[0], gR[1]);   // linear in the gradient
+      const double nn[2] = { nx, ny };
+      const D::WallMap<2> mirror(kind, P.bc_uw + 2 * tag, nn);
+      mirror.apply(wL, wR);
+      mirror.apply_gradient(gL, gR);
       D::rot_in(nx, ny, wR, wr);
     }
   }

@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(kCellBlock) k_dt(MeshT<double> m, ParamsT<doub
   pdl_exit();
 }
 
-// wall ghost of a state and its gradient (global), through the face frame
+// FP32: wall ghost of a state and its gradient (global), through the face frame
 template <typename T>
 __device__ __forceinline__ void wall_ghost(const ParamsT<T> &P, int tag, const D3::Frame<T> &F, const T w[NV],
                                            const T g[3][NV], T wg[NV], T gg[3][NV]) {
@@ -194,16 +194,16 @@ __device__ __forceinline__ void farfield_ghost(const ParamsT<T> &P, int tag, con
 // bit 1 + s of on is set (slots by a constant index: no local memory).
 __device__ __forceinline__ float quot(float a, float b) { return a / b; }
 __device__ __forceinline__ double quot(double a, double b) { return a * dev::d_rcp(b); }
-template <typename T>
-__device__ __forceinline__ void weno_combine3(const ParamsT<T> &P, const T M[6], unsigned on, const T lin[7][3][NV],
-                                              T c[kNM3][NV]) {
+template <typename T, int NC>
+__device__ __forceinline__ void weno_combine3(const ParamsT<T> &P, const T M[6], unsigned on, const T (&lin)[7][3][NC],
+                                              T (&c)[kNM3][NC]) {
   const int nk = __popc(on);
   const T g0 = P.weno_g0, eps = P.weno_eps;
   const T gk = quot(T(1) - g0, T(nk));
   // symmetric M: xx xy xz yy yz zz
   const T Mx[3][3] = { { M[0], M[1], M[2] }, { M[1], M[3], M[4] }, { M[2], M[4], M[5] } };
 #pragma unroll
-  for (int v = 0; v < NV; ++v) {
+  for (int v = 0; v < NC; ++v) {
     const T q[kNM3] = { c[0][v], c[1][v], c[2][v], c[3][v], c[4][v], c[5][v], c[6][v], c[7][v], c[8][v] };
     const T G[3][3] = { { T(2) * q[3], q[4], q[5] }, { q[4], T(2) * q[6], q[7] }, { q[5], q[7], T(2) * q[8] } };
     T b0 = q[0] * q[0] + q[1] * q[1] + q[2] * q[2];
@@ -242,54 +242,67 @@ __device__ __forceinline__ void weno_combine3(const ParamsT<T> &P, const T M[6],
   }
 }
 
-// K1: compact quadratic per cell: coef[(q*5 + v)][n], 9 monomials
-template <typename T, bool WENO>
+// K1: compact quadratic per cell: coef[(q*5 + v)][n], 9 monomials.  FP64: one
+// thread per cell and variable, FP32: per cell (as in 2-D).  us per launch,
+// FP64, before / now (with the wall mirrors as linear maps): 9,177 hexahedra
+// 120.5 / 48.4, a sphere of 128,000 cells 318.9 / 280.5.
+template <typename T> __host__ __device__ constexpr int recon_vars() { return is_f32<T>() ? NV : 1; }
+// f(cell, variable) over the items of a launch, a warp per variable of 32 cells
+template <typename T, typename F>
+__device__ __forceinline__ void for_recon(const int n, F &&f) {
+  constexpr int G = NV / recon_vars<T>();
+  for_items((n + 31) / 32 * 32 * G, [&](int t) {
+    const int i = G == 1 ? t : t / (32 * G) * 32 + t % 32;
+    if (i < n) f(i, t / 32 % G);
+  });
+}
+template <typename T, bool WENO, int NC>
 __device__ __forceinline__ void recon_at(const MeshT<T> &m, const ParamsT<T> &P, const T *__restrict__ W,
                                          const T *__restrict__ Wx, T *__restrict__ coef,
-                                         const unsigned char *__restrict__ wenok, const int i) {
-  const int n = m.nc;
-  T wi[NV], gi[3][NV];
+                                         const unsigned char *__restrict__ wenok, const int i, const int comp) {
+  const int n = m.nc, vo = NC == NV ? 0 : comp;
+  T wi[NC], gi[3][NC];
 #pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    wi[v] = W[v * n + i];
+  for (int v = 0; v < NC; ++v) {
+    wi[v] = W[(vo + v) * n + i];
 #pragma unroll
-    for (int d = 0; d < 3; ++d) gi[d][v] = Wx[(d * NV + v) * n + i];
+    for (int d = 0; d < 3; ++d) gi[d][v] = Wx[(d * NV + vo + v) * n + i];
   }
-  T c[kNM3][NV];
+  T c[kNM3][NC];
 #pragma unroll
   for (int q = 0; q < kNM3; ++q) {
     const T o0 = m.op[((4 * kMaxFace3) * kNM3 + q) * n + i];
     const T o1 = m.op[((4 * kMaxFace3 + 1) * kNM3 + q) * n + i];
     const T o2 = m.op[((4 * kMaxFace3 + 2) * kNM3 + q) * n + i];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) c[q][v] = o0 * gi[0][v] + o1 * gi[1][v] + o2 * gi[2][v];
+    for (int v = 0; v < NC; ++v) c[q][v] = o0 * gi[0][v] + o1 * gi[1][v] + o2 * gi[2][v];
   }
-  T lin[WENO ? 7 : 1][3][NV];
+  T lin[WENO ? 7 : 1][3][NC];
   unsigned on = 1;
   if constexpr (WENO) {
     const T h = T(1) / m.ih[i];
 #pragma unroll
-    for (int v = 0; v < NV; ++v)
+    for (int v = 0; v < NC; ++v)
 #pragma unroll
       for (int d = 0; d < 3; ++d) lin[0][d][v] = h * gi[d][v];
   }
-#pragma unroll (WENO ? kMaxFace3 : 1)
+#pragma unroll (WENO || NC == 1 ? kMaxFace3 : 1)
   for (int s = 0; s < kMaxFace3; ++s) {
     const int fs = m.cface[s * n + i];
     if (fs == kNoFace) continue;
     const int j = m.cnbr[s * n + i];
-    T b0[NV], b[3][NV];
+    T b0[NC], b[3][NC];
     if (j >= 0) {
 #pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        b0[v] = W[v * n + j] - wi[v];
+      for (int v = 0; v < NC; ++v) {
+        b0[v] = W[(vo + v) * n + j] - wi[v];
 #pragma unroll
-        for (int d = 0; d < 3; ++d) b[d][v] = Wx[(d * NV + v) * n + j];
+        for (int d = 0; d < 3; ++d) b[d][v] = Wx[(d * NV + vo + v) * n + j];
       }
       if constexpr (WENO) {
         const T h = T(1) / m.ih[i];
 #pragma unroll
-        for (int v = 0; v < NV; ++v)
+        for (int v = 0; v < NC; ++v)
 #pragma unroll
           for (int d = 0; d < 3; ++d) lin[1 + s][d][v] = h * b[d][v];
         on |= 2u << s;
@@ -298,18 +311,26 @@ __device__ __forceinline__ void recon_at(const MeshT<T> &m, const ParamsT<T> &P,
       const int f = fs >= 0 ? fs : ~fs;
       const int tag = -1 - m.fc1[f];
       if (P.bc_kind[tag] == CGKS_BC_FARFIELD) continue;
-      const D3::Frame<T> F = frame_of(m, f);
-      T wg[NV];
-      wall_ghost(P, tag, F, wi, gi, wg, b);
+      if constexpr (NC == NV) {
+        const D3::Frame<T> F = frame_of(m, f);
+        T wg[NV];
+        wall_ghost(P, tag, F, wi, gi, wg, b);
 #pragma unroll
-      for (int v = 0; v < NV; ++v) b0[v] = wg[v] - wi[v];
+        for (int v = 0; v < NV; ++v) b0[v] = wg[v] - wi[v];
+      } else {   // the mirror image mixes the variables
+        const double nn[3] = { m.fe[f], m.fe[m.nf + f], m.fe[2 * m.nf + f] };
+        double g[3];
+        dev::WallMap<3>(P.bc_kind[tag], P.bc_uw + 3 * tag, nn).one(comp, W + i, Wx + i, n, b0[0], g);
+#pragma unroll
+        for (int d = 0; d < 3; ++d) b[d][0] = g[d];
+      }
     }
 #pragma unroll
     for (int q = 0; q < kNM3; ++q) {
       const T o0 = m.op[((4 * s) * kNM3 + q) * n + i], o1 = m.op[((4 * s + 1) * kNM3 + q) * n + i];
       const T o2 = m.op[((4 * s + 2) * kNM3 + q) * n + i], o3 = m.op[((4 * s + 3) * kNM3 + q) * n + i];
 #pragma unroll
-      for (int v = 0; v < NV; ++v) c[q][v] += o0 * b0[v] + o1 * b[0][v] + o2 * b[1][v] + o3 * b[2][v];
+      for (int v = 0; v < NC; ++v) c[q][v] += o0 * b0[v] + o1 * b[0][v] + o2 * b[1][v] + o3 * b[2][v];
     }
   }
   if constexpr (WENO) {
@@ -321,13 +342,13 @@ __device__ __forceinline__ void recon_at(const MeshT<T> &m, const ParamsT<T> &P,
 #pragma unroll
   for (int q = 0; q < kNM3; ++q)
 #pragma unroll
-    for (int v = 0; v < NV; ++v) coef[(q * NV + v) * n + i] = c[q][v];
+    for (int v = 0; v < NC; ++v) coef[(q * NV + vo + v) * n + i] = c[q][v];
 }
 template <typename T>
 __global__ void __launch_bounds__(kMaxShapeBlock)
     k_recon(MeshT<T> m, ParamsT<T> P, const T *W, const T *Wx, T *coef) {
   pdl_enter();
-  for_items(m.nc, [&](int i) { recon_at<T, false>(m, P, W, Wx, coef, nullptr, i); });
+  for_recon<T>(m.nc, [&](int i, int comp) { recon_at<T, false, recon_vars<T>()>(m, P, W, Wx, coef, nullptr, i, comp); });
   pdl_exit();
 }
 // with the compact WENO step; wenok[i] = 1 where the stencil gave a quadratic
@@ -336,7 +357,7 @@ __global__ void __launch_bounds__(kMaxShapeBlock)
     k_recon_weno(MeshT<T> m, ParamsT<T> P, const T *W, const T *Wx, T *coef,
                  const unsigned char *wenok) {
   pdl_enter();
-  for_items(m.nc, [&](int i) { recon_at<T, true>(m, P, W, Wx, coef, wenok, i); });
+  for_recon<T>(m.nc, [&](int i, int comp) { recon_at<T, true, recon_vars<T>()>(m, P, W, Wx, coef, wenok, i, comp); });
   pdl_exit();
 }
 
@@ -540,7 +561,9 @@ __device__ __forceinline__ void face_points_at(const MeshT<double> &m, const Par
 #pragma unroll
         for (int v = 0; v < NV; ++v) gR[d][v] = T(0);
     } else {
-      wall_ghost(P, tag, F, wL, gL, wR, gR);
+      const dev::WallMap<3> mirror(P.bc_kind[tag], P.bc_uw + 3 * tag, F.e[0]);
+      mirror.apply(wL, wR);
+      mirror.apply_gradient(gL, gR);
       D3::rot_in(F, wR, wr);
     }
     // slopes of the equilibrium at W^c: the mean of the sides plus, along
@@ -859,9 +882,14 @@ __global__ void __launch_bounds__(kCellBlock) k_lo_cell(int n, ParamsT<TF> P, in
 template <typename T>
 __device__ __forceinline__ void lo_ghost(const ParamsT<T> &P, int tag, const D3::Frame<T> &F, const T w[NV],
                                          T wg[NV]) {
+  const int kind = P.bc_kind[tag];
+  if constexpr (!is_f32<T>())
+    if (kind != CGKS_BC_FARFIELD) {
+      dev::WallMap<3>(kind, P.bc_uw + 3 * tag, F.e[0]).apply(w, wg);
+      return;
+    }
   T wl[NV], wgl[NV];
   D3::rot_in(F, w, wl);
-  const int kind = P.bc_kind[tag];
   if (kind == CGKS_BC_FARFIELD) {
     farfield_ghost(P, tag, F, wl, wgl);
   } else {

@@ -293,6 +293,8 @@ void enqueue_hi_step(Batch *b, double *Wout, TF *Wout_m, bool want_res) {
 bool last_pass_advances(const Batch *b) {
   return b->sh.sweep_order != CGKS_SWEEP_PARTITIONED && b->sh.n_sweeps > 0 && b->n_colours > 1;
 }
+// the low-order fluxes and the right-hand side in one launch
+bool merged_rhs(const Batch *b) { return b->N <= (b->mixed ? merge_cells<float>() : merge_cells<double>()); }
 template <typename TF>
 void enqueue_lo_fused(Batch *b) {
   Bufs<TF> &B = bufs<TF>(b);
@@ -356,12 +358,19 @@ void enqueue_lo_solve(Batch *b) {
   for (int k = 0; k < b->sh.n_implicit; ++k) {
     if (k == 0 || !adv) cells(k == 0 ? 1 : 0);
     const int fsh = b->tune.shape(TK_LOFACE);
+    const bool merged = merged_rhs(b);
     tuned_launch(b->tune, TK_LOFACE, b->stream, [&] {
-      launch(b, KI_LOFACE, k_lo_face<TF>, dim3(nblk(b->F, shape_bs(fsh))), dim3(shape_bs(fsh)),
-             fmesh<TF>(b), fparams<TF>(b), (const TF *)base, B.Flo);
+      if (merged)
+        launch(b, KI_LOFACE, k_lo_flux_rhs<TF>, dim3(nblk(kMaxFace * b->N, shape_bs(fsh))), dim3(shape_bs(fsh)),
+               fmesh<TF>(b), fparams<TF>(b), b->dm, b->dp, k == 0 ? 1 : 0, colour0, (const TF *)base,
+               (const double *)b->Rp0, b->Src, B.Rk, B.invD, del0, B.lamS);
+      else
+        launch(b, KI_LOFACE, k_lo_face<TF>, dim3(nblk(b->F, shape_bs(fsh))), dim3(shape_bs(fsh)),
+               fmesh<TF>(b), fparams<TF>(b), (const TF *)base, B.Flo);
     });
-    launch(b, KI_LORHS, k_lo_rhs<TF>, gc, blk, b->dm, b->dp, fparams<TF>(b).gamma, k == 0 ? 1 : 0, colour0,
-           (const TF *)base, (const TF *)B.Flo, (const double *)b->Rp0, b->Src, B.Rk, B.invD, del0, B.lamS);
+    if (!merged)
+      launch(b, KI_LORHS, k_lo_rhs<TF>, gc, blk, b->dm, b->dp, fparams<TF>(b).gamma, k == 0 ? 1 : 0, colour0,
+             (const TF *)base, (const TF *)B.Flo, (const double *)b->Rp0, b->Src, B.Rk, B.invD, del0, B.lamS);
     if (part) {
       TF *in = del0, *out = del0 == B.delta ? B.delta2 : B.delta;
       for (int sw = 0; sw < b->sh.n_sweeps; ++sw) {
@@ -458,7 +467,7 @@ long long count_launches(const Batch *b, bool cycle) {
                                ? static_cast<long long>(b->sh.n_sweeps)
                                : static_cast<long long>(b->sweep_seq.size());
   const long long cells = last_pass_advances(b) ? 1 : b->sh.n_implicit + 1;
-  long long lo = b->lo_fused_ok ? 1 : b->sh.n_implicit > 0 ? b->sh.n_implicit * (2 + sweeps) + cells : 0;
+  long long lo = b->lo_fused_ok ? 1 : b->sh.n_implicit > 0 ? b->sh.n_implicit * ((merged_rhs(b) ? 1 : 2) + sweeps) + cells : 0;
   return dt + hi + per_eval + 1 + lo + 2;
 }
 

@@ -191,8 +191,8 @@ __device__ __forceinline__ void wall_ghost_global(const ParamsT<T> &P, int tag, 
 
 template <typename T>
 __device__ __forceinline__ void farfield_ghost(const ParamsT<T> &P, int tag, T nx, T ny, const T wl[4], T wg[4]) {
-  T une = P.bc_u[2 * tag] * nx + P.bc_u[2 * tag + 1] * ny;
-  T ute = -P.bc_u[2 * tag] * ny + P.bc_u[2 * tag + 1] * nx;
+  T une = D::dot2(P.bc_u[2 * tag], nx, P.bc_u[2 * tag + 1], ny);
+  T ute = D::dot2(-P.bc_u[2 * tag], ny, P.bc_u[2 * tag + 1], nx);
   D::ghost_farfield(P.kc, P.gamma, P.bc_rho[tag], une, ute, P.bc_p[tag], wl, wg);
 }
 
@@ -200,10 +200,10 @@ __device__ __forceinline__ void farfield_ghost(const ParamsT<T> &P, int tag, T n
 template <typename T>
 __device__ __forceinline__ void dirichlet_ghost(const ParamsT<T> &P, int tag, T nx, T ny, T wg[4]) {
   const T r = P.bc_rho[tag], p = P.bc_p[tag];
-  const T un = P.bc_u[2 * tag] * nx + P.bc_u[2 * tag + 1] * ny;
-  const T ut = -P.bc_u[2 * tag] * ny + P.bc_u[2 * tag + 1] * nx;
+  const T un = D::dot2(P.bc_u[2 * tag], nx, P.bc_u[2 * tag + 1], ny);
+  const T ut = D::dot2(-P.bc_u[2 * tag], ny, P.bc_u[2 * tag + 1], nx);
   wg[0] = r; wg[1] = r * un; wg[2] = r * ut;
-  wg[3] = p / (P.gamma - T(1)) + T(0.5) * r * (un * un + ut * ut);
+  wg[3] = p / (P.gamma - T(1)) + T(0.5) * r * D::dot2(un, un, ut, ut);
 }
 
 __host__ __device__ __forceinline__ bool is_wall_kind(int k) { return k == CGKS_BC_SLIP || k == CGKS_BC_NOSLIP; }
@@ -1065,10 +1065,10 @@ __device__ __forceinline__ LoFaceGeo<T> lo_face_geo(const MeshT<T> &m, const Par
 }
 __device__ __forceinline__ float third(float x) { return x / 3.0f; }
 __device__ __forceinline__ double third(double x) { return x * (1.0 / 3.0); }
+// the flux (out of c0) and, in o[4], lambda_p
 template <typename T, bool CG>
-__device__ __forceinline__ void lo_face_at(const MeshT<T> &m, const ParamsT<T> &P, const LoFaceGeo<T> &g,
-                                           const T *base, T *__restrict__ Flo, const int f) {
-  if (g.sid < 0) return;   // free face space of a batch
+__device__ __forceinline__ void lo_flux_at(const MeshT<T> &m, const ParamsT<T> &P, const LoFaceGeo<T> &g,
+                                           const T *base, const int f, T o[lo_run<T>()]) {
   const int c1 = g.c1;
   const T nx = g.nx, ny = g.ny, mu = g.mu;
   T ra[kBase], rb[kBase];
@@ -1086,7 +1086,7 @@ __device__ __forceinline__ void lo_face_at(const MeshT<T> &m, const ParamsT<T> &
     lo_ghost(P, -1 - c1, nx, ny, wa, wb);
     b = D::prim_of(wb, P.gamma, P.kc);
   }
-  const T una = a.u * nx + a.v * ny, unb = b.u * nx + b.v * ny;
+  const T una = D::dot2(a.u, nx, a.v, ny), unb = D::dot2(b.u, nx, b.v, ny);
   T la = fabs(una) + a.c, lb = fabs(unb) + b.c, ira = T(0), irb = T(0);
   if (mu != T(0)) {
     ira = D::d_rcp(a.rho);
@@ -1100,10 +1100,15 @@ __device__ __forceinline__ void lo_face_at(const MeshT<T> &m, const ParamsT<T> &
     // Lax-Friedrichs alternative of Section 3 with the implicit operator's
     // lambda_p: (F_n(U_l) + F_n(U_r)) / 2 - lambda_p (U_r - U_l) / 2
     // (products rounded by themselves: the mixed path's FP32 results stay what they are)
-    const T Fa[4] = { mul_rn(a.rho, una), wa[1] * una + a.p * nx, wa[2] * una + a.p * ny, mul_rn(wa[3] + a.p, una) };
-    const T Fb[4] = { mul_rn(b.rho, unb), wb[1] * unb + b.p * nx, wb[2] * unb + b.p * ny, mul_rn(wb[3] + b.p, unb) };
+    const T Fa[4] = { mul_rn(a.rho, una), D::dot2(wa[1], una, a.p, nx), D::dot2(wa[2], una, a.p, ny),
+                      mul_rn(wa[3] + a.p, una) };
+    const T Fb[4] = { mul_rn(b.rho, unb), D::dot2(wb[1], unb, b.p, nx), D::dot2(wb[2], unb, b.p, ny),
+                      mul_rn(wb[3] + b.p, unb) };
 #pragma unroll
-    for (int v = 0; v < 4; ++v) F[v] = T(0.5) * (Fa[v] + Fb[v]) - T(0.5) * lmax * (wb[v] - wa[v]);
+    for (int v = 0; v < 4; ++v) {
+      if constexpr (is_f32<T>()) F[v] = T(0.5) * (Fa[v] + Fb[v]) - T(0.5) * lmax * (wb[v] - wa[v]);
+      else F[v] = D::dot2(T(0.5), Fa[v] + Fb[v], -(T(0.5) * lmax), wb[v] - wa[v]);
+    }
   } else if constexpr (is_f32<T>()) {
     const T uta = -a.u * ny + a.v * nx, utb = -b.u * ny + b.v * nx;
     T Fl[4];
@@ -1116,11 +1121,13 @@ __device__ __forceinline__ void lo_face_at(const MeshT<T> &m, const ParamsT<T> &
     T m0a, m1a, m0b, m1b;
     D::half01(una, a.sl, a.isp, +1, m0a, m1a);
     D::half01(unb, b.sl, b.isp, -1, m0b, m1b);
-    const T ja = a.rho * m1a, jb = b.rho * m1b, pa = a.p * m0a, pb = b.p * m0b, pn = pa + pb;
+    const T ja = D::prod(a.rho, m1a), jb = D::prod(b.rho, m1b), pa = D::prod(a.p, m0a), pb = D::prod(b.p, m0b);
+    const T pn = pa + pb;
     F[0] = ja + jb;
-    F[1] = ja * a.u + jb * b.u + pn * nx;
-    F[2] = ja * a.v + jb * b.v + pn * ny;
-    F[3] = m1a * (wa[3] + T(0.5) * a.p) + m1b * (wb[3] + T(0.5) * b.p) + T(0.5) * (pa * una + pb * unb);
+    F[1] = fma(pn, nx, D::dot2(ja, a.u, jb, b.u));
+    F[2] = fma(pn, ny, D::dot2(ja, a.v, jb, b.v));
+    F[3] = fma(T(0.5), D::dot2(pa, una, pb, unb),
+               D::dot2(m1a, fma(T(0.5), a.p, wa[3]), m1b, fma(T(0.5), b.p, wb[3])));
   }
   if (P.lo_viscous && mu > T(0)) {
     // first-order viscous flux: normal gradients from the two cell states
@@ -1128,23 +1135,28 @@ __device__ __forceinline__ void lo_face_at(const MeshT<T> &m, const ParamsT<T> &
     //   tau.n = mu / delta (du + (n.du) n / 3),  q.n = -kappa (T_r - T_l) / delta
     const T md = mu * m.fidl[f];
     const T dux = b.u - a.u, duy = b.v - a.v;
-    const T dn = third(dux * nx + duy * ny);
-    const T tx = md * (dux + dn * nx), ty = md * (duy + dn * ny);
+    const T dn = third(D::dot2(dux, nx, duy, ny));
+    const T tx = D::prod(md, dux + dn * nx), ty = D::prod(md, duy + dn * ny);
     T qn;   // gamma / (gamma - 1) = N / 2 + 1
     if constexpr (is_f32<T>()) qn = -md * P.gamma / (P.gamma - T(1)) * (b.p * irb - a.p * ira);
-    else qn = -md * (P.kc.hN + T(1)) * (b.p * irb - a.p * ira);
+    else qn = D::prod(-md * (P.kc.hN + T(1)), D::dot2(b.p, irb, -a.p, ira));
     F[1] -= tx;
     F[2] -= ty;
-    F[3] -= tx * (T(0.5) * (a.u + b.u)) + ty * (T(0.5) * (a.v + b.v)) - qn;
+    F[3] -= D::dot2(tx, T(0.5) * (a.u + b.u), ty, T(0.5) * (a.v + b.v)) - qn;
   }
-  constexpr int N = lo_run<T>();
-  T o[N];
 #pragma unroll
   for (int v = 0; v < 4; ++v) o[v] = F[v];
   o[4] = lmax;
 #pragma unroll
-  for (int v = 5; v < N; ++v) o[v] = T(0);
-  vstore<T, N>(Flo + static_cast<size_t>(f) * N, o);
+  for (int v = 5; v < lo_run<T>(); ++v) o[v] = T(0);
+}
+template <typename T, bool CG>
+__device__ __forceinline__ void lo_face_at(const MeshT<T> &m, const ParamsT<T> &P, const LoFaceGeo<T> &g,
+                                           const T *base, T *__restrict__ Flo, const int f) {
+  if (g.sid < 0) return;   // free face space of a batch
+  T o[lo_run<T>()];
+  lo_flux_at<T, CG>(m, P, g, base, f, o);
+  vstore<T, lo_run<T>()>(Flo + static_cast<size_t>(f) * lo_run<T>(), o);
 }
 template <typename T>
 __global__ void __launch_bounds__(kMaxShapeBlock) k_lo_face(MeshT<T> m, ParamsT<T> P, const T *base, T *Flo) {
@@ -1209,7 +1221,7 @@ __device__ __forceinline__ void lo_rhs_at(const MeshT<double> &m, const ParamsT<
   if (g.c0) {
     TF b[4], d[4];
 #pragma unroll
-    for (int v = 0; v < 4; ++v) d[v] = narrow<TF>(R[v] * id);
+    for (int v = 0; v < 4; ++v) d[v] = narrow<TF>(__dmul_rn(R[v], id));
     vload<TF, 4, CG>(base + static_cast<size_t>(i) * kBase, b);
     store_delta(gamma, b, d, delta, i);
   } else {
@@ -1234,6 +1246,89 @@ __global__ void __launch_bounds__(kCellBlock) k_lo_rhs(MeshT<double> m, ParamsT<
   lo_rhs_at<TF, false>(m, P, gamma, g, first, base, Flo, Rp0, Src, Rk, invD, delta, lamS, i);
   pdl_exit();
 }
+
+// K5b and K6 in one launch, four lanes per cell, one per face slot: the lane
+// forms its slot's flux, then the sums of one variable.  Every face is
+// evaluated twice, with the same bits, but a launch and its wait are saved and
+// the chain of FP64 instructions that a small launch waits for shrinks (the
+// sums of one variable, 20 instructions, where one thread took 60).
+// us per V-cycle, two launches / one: mixed 2,048 cells 183 / 169, FP64 321 / 302.
+template <typename TF>
+__global__ void __launch_bounds__(kMaxShapeBlock) k_lo_flux_rhs(MeshT<TF> fm, ParamsT<TF> fP, MeshT<double> m,
+                                                                ParamsT<double> P, int first, int colour0,
+                                                                const TF *base, const double *Rp0, double *Src,
+                                                                TF *Rk, TF *invD, TF *delta, TF *lamS) {
+  const int t = static_cast<int>(blockIdx.x * blockDim.x + threadIdx.x);
+  const int i = t / kMaxFace, s = t % kMaxFace, n = m.nc;
+  const bool in = i < n;
+  // mesh data first (nothing in a cycle writes it), then wait for the predecessor
+  const int fs = in ? m.cface[s * n + i] : kNoFace, f = fs >= 0 ? fs : ~fs;
+  const double S = in ? m.shs[s * n + i] : 0.0;
+  const bool c0 = in && colour0 && m.ccol[i] == 0, there = fs != kNoFace;
+  LoFaceGeo<TF> g;
+  if (there) g = lo_face_geo(fm, fP, f);
+  pdl_enter();
+  double x[5] = { 0.0, 0.0, 0.0, 0.0, 0.0 };
+  TF lam = TF(0);
+  if (there) {
+    TF o[lo_run<TF>()];
+    lo_flux_at<TF, false>(fm, fP, g, base, f, o);
+    widen<5>(o, x);
+    if constexpr (is_f32<TF>()) lam = o[4];
+    else lam = o[4] * (0.5 * S);
+  }
+  // lane s sums variable s, in the order of the slots
+  double R = 0.0, sum = 0.0;
+#pragma unroll
+  for (int q = 0; q < kMaxFace; ++q) {
+    double y[5];
+#pragma unroll
+    for (int v = 0; v < 5; ++v) y[v] = __shfl_sync(0xffffffffu, x[v], q, kMaxFace);
+    const double Sq = __shfl_sync(0xffffffffu, S, q, kMaxFace);
+    const int fq = __shfl_sync(0xffffffffu, fs, q, kMaxFace);
+    const double xv = s == 0 ? y[0] : s == 1 ? y[1] : s == 2 ? y[2] : y[3];
+    if (fq != kNoFace) {
+      R += (fq >= 0 ? -Sq : Sq) * xv;
+      sum += y[4] * Sq;
+    }
+  }
+  const double id = sum > 0.0 ? D::d_rcp(sum * (P.icfl_lo + 0.5)) : 0.0;
+  if (in) {
+    double src;
+    if (first) { src = Rp0[s * n + i] - R; Src[s * n + i] = src; }
+    else src = Src[s * n + i];
+    R += src;
+    Rk[s * n + i] = narrow<TF>(R);
+    lamS[s * n + i] = lam;
+    if (s == 0) invD[i] = narrow<TF>(id);
+  }
+  const TF ds = c0 ? narrow<TF>(__dmul_rn(R, id)) : TF(0);
+  if constexpr (is_f32<TF>()) {
+    if (in) delta[static_cast<size_t>(i) * 4 + s] = ds;
+  } else {
+    TF d[4], rec[8];
+#pragma unroll
+    for (int v = 0; v < 8; ++v) rec[v] = TF(0);
+#pragma unroll
+    for (int v = 0; v < 4; ++v) d[v] = __shfl_sync(0xffffffffu, ds, v, 4);
+    if (c0) {
+      TF b[4];
+      vload<TF, 4>(base + static_cast<size_t>(i) * kBase, b);
+      delta_record(fP.gamma, b, d, rec);
+    }
+    const TF lo = s == 0 ? rec[0] : s == 1 ? rec[2] : s == 2 ? rec[4] : rec[6];
+    const TF hi = s == 0 ? rec[1] : s == 1 ? rec[3] : s == 2 ? rec[5] : rec[7];
+    const TF two[2] = { lo, hi };
+    if (in) vstore<TF, 2>(delta + static_cast<size_t>(i) * 8 + 2 * s, two);
+  }
+  pdl_exit();
+}
+// Cells up to which the merged launch is the shorter one: in FP64 while its
+// four lanes per cell give a sub-core (608) one or two warps, 4,864 to 9,728
+// cells; in FP32 until evaluating every face twice costs more than a launch.
+// us per V-cycle, split / merged: FP64 4,050 cells 314 / 296, 8,192 347 / 355;
+// FP32 25,088 cells 210 / 204, 34,848 215 / 222.
+template <typename T> __host__ __device__ constexpr int64_t merge_cells() { return is_f32<T>() ? 30000 : 6656; }
 
 // The cells of one colour form one contiguous range per solve.  A sweep
 // launch covers up to kMaxRanges ranges, carried in the kernel parameters

@@ -33,19 +33,27 @@ template <typename T> __device__ __forceinline__ T d_pi();
 template <> __device__ __forceinline__ double d_pi<double>() { return 3.141592653589793238462643; }
 template <> __device__ __forceinline__ float d_pi<float>() { return 3.14159265358979f; }
 
+// a b and a b + c d with the roundings spelled out in FP64, so that code
+// compiled into two kernels gives the same bits in both; FP32 as the compiler
+// fuses them.
+__device__ __forceinline__ float prod(float a, float b) { return a * b; }
+__device__ __forceinline__ double prod(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float dot2(float a, float b, float c, float d) { return a * b + c * d; }
+__device__ __forceinline__ double dot2(double a, double b, double c, double d) { return fma(c, d, __dmul_rn(a, b)); }
+
 // Rotate a conservative vector between global and face frames.
 template <typename T>
 __device__ __forceinline__ void rot_in(T nx, T ny, const T g[NV], T l[NV]) {
   l[0] = g[0];
-  l[1] = g[1] * nx + g[2] * ny;
-  l[2] = -g[1] * ny + g[2] * nx;
+  l[1] = dot2(g[1], nx, g[2], ny);
+  l[2] = dot2(-g[1], ny, g[2], nx);
   l[3] = g[3];
 }
 template <typename T>
 __device__ __forceinline__ void rot_out(T nx, T ny, const T l[NV], T g[NV]) {
   g[0] = l[0];
-  g[1] = l[1] * nx - l[2] * ny;
-  g[2] = l[1] * ny + l[2] * nx;
+  g[1] = dot2(l[1], nx, -l[2], ny);
+  g[2] = dot2(l[1], ny, l[2], nx);
   g[3] = l[3];
 }
 
@@ -710,17 +718,17 @@ __device__ __forceinline__ float sound_speed(const KC<float> &, float gamma, flo
   return sqrtf(gamma * p * ir);
 }
 __device__ __forceinline__ double sound_speed(const KC<double> &kc, double, double, double, double i2l, double sl) {
-  return kc.sq2g * (i2l * sl);
+  return __dmul_rn(kc.sq2g, i2l * sl);
 }
 template <typename T>
 __device__ __forceinline__ Prim<T> prim_of(const T W[NV], T gamma, const KC<T> &kc) {
   Prim<T> q;
   const T ir = d_rcp(W[0]);
   q.rho = W[0];
-  q.u = W[1] * ir;
-  q.v = W[2] * ir;
-  const T eps = W[3] - T(0.5) * q.rho * (q.u * q.u + q.v * q.v);
-  q.p = (gamma - T(1)) * eps;
+  q.u = prod(W[1], ir);
+  q.v = prod(W[2], ir);
+  const T eps = W[3] - T(0.5) * q.rho * dot2(q.u, q.u, q.v, q.v);
+  q.p = prod(gamma - T(1), eps);
   q.i2l = kc.c2K * eps * ir;
   sqrt_lambda(q.i2l, q.sl, q.isp);
   q.c = sound_speed(kc, gamma, q.p, ir, q.i2l, q.sl);
@@ -941,8 +949,8 @@ __device__ __forceinline__ FarState far_state(const KC<double> &kc, double ri, d
 __device__ __forceinline__ void ghost_farfield(const KC<double> &kc, double gamma, double re, double une, double ute,
                                                double pe, const double W[NV], double Wg[NV]) {
   const double ri = W[0], ir = d_rcp(ri);
-  const double uni = W[1] * ir, uti = W[2] * ir;
-  const double pi = (gamma - 1.0) * (W[3] - 0.5 * ri * (uni * uni + uti * uti));
+  const double uni = prod(W[1], ir), uti = prod(W[2], ir);
+  const double pi = (gamma - 1.0) * (W[3] - 0.5 * ri * dot2(uni, uni, uti, uti));
   const double ci = d_sqrt3(gamma * pi * ir), ce = d_sqrt3(gamma * pe * d_rcp(re));
   double rb, unb, utb, pb;
   if (uni <= -ci) {
@@ -955,7 +963,7 @@ __device__ __forceinline__ void ghost_farfield(const KC<double> &kc, double gamm
     utb = f.out ? uti : ute;
   }
   Wg[0] = rb; Wg[1] = rb * unb; Wg[2] = rb * utb;
-  Wg[3] = pb * kc.hN + 0.5 * rb * (unb * unb + utb * utb);   // 1 / (gamma - 1) = N / 2
+  Wg[3] = dot2(pb, kc.hN, 0.5 * rb, dot2(unb, unb, utb, utb));   // 1 / (gamma - 1) = N / 2
 }
 
 // 1-D Riemann invariants normal to the face between the interior state W

@@ -145,3 +145,30 @@ def test_device_tables_of_small_and_ragged_meshes(nx, ny):
     spec = dict(gamma=GAM, mu=0.01, cfl_hi=0.3,
                 bcs=[dict(kind="farfield", rho=1.0, u=(0.2, 0.0), p=1 / GAM), dict(kind="noslip")])
     compare(mesh, spec, state(mesh, 0.1, 0.2), "fp64", 2)
+
+
+@pytest.mark.parametrize("precision, big", [("fp64", 64), ("mixed", 130)])   # 8,192 cells; 33,800
+@pytest.mark.parametrize("opts", [dict(), dict(lo_viscous=1), dict(flux_lo="lf")])
+def test_merged_and_separate_right_hand_sides_round_alike(opts, precision, big):
+    """A small solve forms fluxes and right-hand side in one launch, and beside
+    a large one in two: the same bits, at walls, far field and slip."""
+    from paper_2109_09965_gb300 import cgks
+    far = dict(kind="farfield", rho=1.0, u=(0.2, 0.05), p=1 / GAM)
+    box = MG.box(13, 9, jitter=0.15, seed=5, cells="mixed", quad_mask=lambda i, j: (2 * i + j) % 5 == 0,
+                 tags=(0, 1, 2, 1))
+    cav = dict(gamma=GAM, mu=0.15 / 1000, bcs=[dict(kind="noslip"), dict(kind="noslip", uw=(0.15, 0.0))])
+    work = [(box, dict(gamma=GAM, mu=0.01, bcs=[far, dict(kind="slip"), dict(kind="noslip", uw=(0.1, 0.0))])),
+            (MG.cavity(20, seed=2), cav), (MG.cavity(big, seed=1), cav)]
+    srv = cgks.Server(3 << 30, precision=precision, max_active=4, max_cycles=100, **opts)
+    gms = [cgks.Mesh(m) for m, _ in work]
+    states = [state(m, 0.0, 0.1) for m, _ in work]
+    ids = [srv.submit(g, spec, W, 1e-300, 3) for g, (_, spec), W in zip(gms, work, states)]
+    while srv.step():
+        pass
+    for g, (_, spec), W, i in zip(gms, work, states, ids):
+        s = cgks.Solver(g, dict(spec, precision=precision, **opts))
+        s.set_state(W)
+        s.pmg_cycle(3)
+        assert np.array_equal(srv.poll(i)[1], s.get_state()[0])
+        s.close()
+    srv.close()

@@ -286,7 +286,7 @@ __device__ __forceinline__ void recon_at(const MeshT<T> &m, const ParamsT<T> &P,
 #pragma unroll
       for (int d = 0; d < 3; ++d) lin[0][d][v] = h * gi[d][v];
   }
-#pragma unroll (WENO || NC == 1 ? kMaxFace3 : 1)
+#pragma unroll (WENO || NC == 1 ? kMaxFace3 : 2)   // 2: loads of two slots in flight, 162 -> 151 us (512,000 cells)
   for (int s = 0; s < kMaxFace3; ++s) {
     const int fs = m.cface[s * n + i];
     if (fs == kNoFace) continue;
@@ -638,9 +638,12 @@ __device__ __forceinline__ void face_points_at(const MeshT<double> &m, const Par
 // in one thread: 358 and 2809 us).
 constexpr int64_t kFaceLanes4 = 100000;
 inline int face_lanes(int64_t n_faces) { return n_faces < kFaceLanes4 ? 4 : 1; }
-// FP32: one thread per face
+// FP32: one thread per face.  Bound by latency at two warps a scheduler (255
+// registers); the smooth flux is shorter with 128 and four warps, in spite of
+// some spills: 512,000 cells 411 -> 377 us a launch (112: 390, 144: 427); the
+// full flux is not (128,000 cells 241; 128 registers 252, 168: 248).
 template <typename T, bool FULL>
-__global__ void __launch_bounds__(kMaxShapeBlock)
+__global__ void __maxnreg__(FULL ? 255 : 128)
     k_face(MeshT<T> m, ParamsT<T> P, const T *W, const T *coef, T *out,
            const Ctl *ctl, const unsigned long long *dt_bits) {
   pdl_enter();

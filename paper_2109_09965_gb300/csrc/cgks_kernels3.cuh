@@ -117,24 +117,28 @@ __global__ void k_reset_dt(Ctl *ctl, unsigned long long *dt_bits, double dt_fixe
 __global__ void __launch_bounds__(kCellBlock) k_dt(MeshT<double> m, ParamsT<double> P, const double *W,
                                                    unsigned long long *dt_bits) {
   pdl_enter();
-  __shared__ double wmin[kCellBlock / 32];
+  // the minimum on the bits, positive doubles sort like integers (a NaN sorts
+  // last): comparisons of doubles take the FP64 pipe
+  __shared__ unsigned long long wmin[kCellBlock / 32];
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   double d = INFINITY;
   if (i < m.nc) {
     const int n = m.nc;
-    const double rho = W[i], ir = 1.0 / rho;
-    const double u = W[n + i] * ir, v = W[2 * n + i] * ir, w = W[3 * n + i] * ir;
-    const double p = (P.gamma - 1.0) * (W[4 * n + i] - 0.5 * rho * (u * u + v * v + w * w));
+    const double rho = W[i], ir = dev::d_rcp(rho);
+    const double u = W[n + i] * ir, v = W[2 * n + i] * ir, w = W[3 * n + i] * ir, q2 = u * u + v * v + w * w;
+    const double p = (P.gamma - 1.0) * (W[4 * n + i] - 0.5 * rho * q2);
     const double hh = m.hdt[i];
-    const double speed = sqrt(u * u + v * v + w * w) + sqrt(P.gamma * p * ir) + 2.0 * (P.mu * ir) / hh;
-    d = hh / speed;
+    const double speed = dev::sqrt_fast(q2) + dev::sqrt_fast(P.gamma * p * ir);
+    d = hh * hh * dev::d_rcp(fma(hh, speed, 2.0 * (P.mu * ir)));   // hh / (speed + 2 nu / hh)
   }
-  for (int o = 16; o > 0; o >>= 1) d = fmin(d, __shfl_down_sync(0xffffffffu, d, o));
-  if ((threadIdx.x & 31) == 0) wmin[threadIdx.x >> 5] = d;
+  unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(d));
+  for (int o = 16; o > 0; o >>= 1) b = min(b, __shfl_down_sync(0xffffffffu, b, o));
+  if ((threadIdx.x & 31) == 0) wmin[threadIdx.x >> 5] = b;
   __syncthreads();
   if (threadIdx.x == 0) {
-    for (int k = 1; k < kCellBlock / 32; ++k) d = fmin(d, wmin[k]);
-    if (d < INFINITY) atomicMin(dt_bits, static_cast<unsigned long long>(__double_as_longlong(d)));
+    for (int w = 1; w < kCellBlock / 32; ++w) b = min(b, wmin[w]);
+    constexpr unsigned long long kInf = 0x7ff0000000000000ull;
+    if (b < kInf) atomicMin(dt_bits, b);
   }
   pdl_exit();
 }
@@ -699,8 +703,8 @@ __global__ void __launch_bounds__(kCellBlock) k_update(MeshT<double> m, ParamsT<
       const int fs = fsl[s];
       if (fs == kNoFace) continue;
       const size_t at = static_cast<size_t>(fs >= 0 ? fs : ~fs) * kFO;
-      // the slot's area and sgn S n_f from the per-cell slot arrays (coalesced)
-      const double h = 2.0 * m.shs[s * n + i], S = fs >= 0 ? h : -h;
+      // half the slot's area and sgn S n_f from the per-cell slot arrays (coalesced)
+      const double h = m.shs[s * n + i], S = fs >= 0 ? h : -h;
       // the face's run of F0, F1, Wc, Wt (and the second stage's, when used);
       // the residual reads the leading F0, F1 part only
       constexpr int kRes = (2 * NV + VecOf<TF>::W - 1) / VecOf<TF>::W * VecOf<TF>::W;
@@ -718,7 +722,7 @@ __global__ void __launch_bounds__(kCellBlock) k_update(MeshT<double> m, ParamsT<
       double nn[3] = { 0.0, 0.0, 0.0 };
       if constexpr (mode != kResidual)
 #pragma unroll
-        for (int d = 0; d < 3; ++d) nn[d] = 2.0 * m.sn[(3 * s + d) * n + i];
+        for (int d = 0; d < 3; ++d) nn[d] = m.sn[(3 * s + d) * n + i];
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         double f1 = a[NV + v];
@@ -737,9 +741,9 @@ __global__ void __launch_bounds__(kCellBlock) k_update(MeshT<double> m, ParamsT<
     }
     if (Rout)
 #pragma unroll
-      for (int v = 0; v < NV; ++v) Rout[v * n + i] = R[v];
+      for (int v = 0; v < NV; ++v) Rout[v * n + i] = 2.0 * R[v];
     if constexpr (mode != kResidual) {
-      const double iv = m.ivol[i], k = dt * iv;
+      const double iv2 = 2.0 * m.ivol[i], k = dt * iv2;
       const double old = Wbase[i];   // Wout may be Wbase (explicit steps update in place)
       double w[NV];
 #pragma unroll
@@ -749,7 +753,7 @@ __global__ void __launch_bounds__(kCellBlock) k_update(MeshT<double> m, ParamsT<
         if (Wout_m) Wout_m[v * n + i] = narrow<TF>(w[v]);
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-          const double x = g[d][v] * iv;
+          const double x = g[d][v] * iv2;
           Wxout[(d * NV + v) * n + i] = x;
           if (Wxout_m) Wxout_m[(d * NV + v) * n + i] = narrow<TF>(x);
         }

@@ -922,6 +922,8 @@ struct FarState {
   double un, r, p;
 };
 __device__ __forceinline__ double d_sqrt3(double x) { return x * d_rsqrt3(x); }
+// the same with the library's root for zero and everything out of the normal range
+__device__ __forceinline__ double sqrt_fast(double x) { return x > 1e-290 && x < 1e290 ? d_sqrt3(x) : sqrt(x); }
 __device__ __forceinline__ FarState far_state(const KC<double> &kc, double ri, double pi, double ui, double ci,
                                               double re, double pe, double ue, double ce) {
   const double N = 2.0 * kc.hN;

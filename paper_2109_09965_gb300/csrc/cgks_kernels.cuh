@@ -265,9 +265,11 @@ __device__ __forceinline__ void weno_combine(const ParamsT<T> &P, T mxx, T mxy, 
 #pragma unroll
     for (int k = 0; k < 5; ++k)
       if (on >> k & 1) {
-        sel0 += wk[k] * iws * lin[k][0][v];
-        sel1 += wk[k] * iws * lin[k][1][v];
+        const T w = is_f32<T>() ? wk[k] * iws : wk[k];
+        sel0 += w * lin[k][0][v];
+        sel1 += w * lin[k][1][v];
       }
+    if constexpr (!is_f32<T>()) { sel0 *= iws; sel1 *= iws; }
     c[0][v] = f0 * (c0 - lin0) + sel0;
     c[1][v] = f0 * (c1 - lin1) + sel1;
     c[2][v] = f0 * c2;
@@ -312,7 +314,7 @@ __device__ __forceinline__ void recon_at(const MeshT<T> &m, const ParamsT<T> &P,
   T lin[WENO ? 5 : 1][2][NC];
   unsigned on = 1;
   if constexpr (WENO) {
-    const T hi = T(1) / m.ih[i];
+    const T hi = quot(T(1), m.ih[i]);
 #pragma unroll
     for (int v = 0; v < NC; ++v) { lin[0][0][v] = hi * gxi[v]; lin[0][1][v] = hi * gyi[v]; }
   }
@@ -330,7 +332,7 @@ __device__ __forceinline__ void recon_at(const MeshT<T> &m, const ParamsT<T> &P,
         b2[v] = Wx[(4 + vo + v) * n + j];
       }
       if constexpr (WENO) {
-        const T hi = T(1) / m.ih[i];
+        const T hi = quot(T(1), m.ih[i]);
 #pragma unroll
         for (int v = 0; v < NC; ++v) { lin[1 + s][0][v] = hi * b1[v]; lin[1 + s][1][v] = hi * b2[v]; }
         on |= 2u << s;
@@ -452,6 +454,97 @@ __device__ __forceinline__ void load_coef(int n, const double *__restrict__ coef
 // weno_combine per characteristic field and projected back.  Right
 // eigenvectors (columns): u_n - c, entropy, shear, u_n + c; the left ones
 // in closed form with b1 = (gamma - 1)/c^2, b2 = b1 |u|^2 / 2.
+// The fields of a conservative vector and back, FP64: the eigenvectors' products
+// with what they share taken once (12 and 13 instructions, as matrices 16).
+struct CharFrame {
+  double u, v, q2h, H, c, un, ut, nx, ny;              // q2h = |u|^2 / 2
+  double b1, b1u, b1v, b2, cn, cnx, cny;               // of the left ones; cn = un / (2 c), ...
+  __device__ __forceinline__ CharFrame(double gamma, const double w[4], double nx_, double ny_) : nx(nx_), ny(ny_) {
+    const double ir = D::d_rcp(w[0]);
+    u = w[1] * ir;
+    v = w[2] * ir;
+    const double q2 = u * u + v * v, p = (gamma - 1.0) * (w[3] - 0.5 * w[0] * q2), c2 = gamma * p * ir;
+    const double ic = D::d_rsqrt3(c2);
+    c = c2 * ic;
+    q2h = 0.5 * q2;
+    H = (w[3] + p) * ir;
+    un = u * nx + v * ny;
+    ut = v * nx - u * ny;
+    b1 = (gamma - 1.0) * ic * ic;
+    b1u = b1 * u;
+    b1v = b1 * v;
+    b2 = b1 * q2h;
+    const double h = 0.5 * ic;
+    cn = un * h;
+    cnx = nx * h;
+    cny = ny * h;
+  }
+  // the left eigenvectors times s
+  __device__ __forceinline__ CharFrame scaled(double s) const {
+    CharFrame f(*this);
+    f.b1 *= s; f.b1u *= s; f.b1v *= s; f.b2 *= s; f.cn *= s; f.cnx *= s; f.cny *= s;
+    f.ut *= s; f.nx *= s; f.ny *= s;
+    return f;
+  }
+  __device__ __forceinline__ void fields(double one, const double x[4], double a[4]) const {
+    const double s = b2 * x[0] - b1u * x[1] - b1v * x[2] + b1 * x[3];
+    const double d = cnx * x[1] + cny * x[2] - cn * x[0];
+    a[0] = 0.5 * s - d;
+    a[1] = one * x[0] - s;
+    a[2] = nx * x[2] - ny * x[1] - ut * x[0];
+    a[3] = 0.5 * s + d;
+  }
+  __device__ __forceinline__ void conservative(const double a[4], double x[4]) const {
+    const double s = a[0] + a[3], d = c * (a[3] - a[0]);
+    x[0] = s + a[1];
+    x[1] = u * x[0] + nx * d - ny * a[2];
+    x[2] = v * x[0] + ny * d + nx * a[2];
+    x[3] = H * s + q2h * a[1] + un * d + ut * a[2];
+  }
+};
+__device__ __forceinline__ void char_side(const MeshT<double> &m, const ParamsT<double> &P, const double *W,
+                                          const double *Wx, const double *coef, int i, const double wref[4],
+                                          double nx, double ny, double out[kNM][4]) {
+  const int n = m.nc;
+  const CharFrame f(P.gamma, wref, nx, ny);
+  const double h = quot(1.0, m.ih[i]);
+  double lin[5][2][4];
+  unsigned on = 1;
+  {
+    const CharFrame g = f.scaled(h);
+    auto add = [&](int k, int j) {
+      double x[4], a[4];
+#pragma unroll
+      for (int d = 0; d < 2; ++d) {
+#pragma unroll
+        for (int b = 0; b < 4; ++b) x[b] = Wx[(4 * d + b) * n + j];
+        g.fields(h, x, a);
+#pragma unroll
+        for (int b = 0; b < 4; ++b) lin[k][d][b] = a[b];
+      }
+    };
+    add(0, i);
+#pragma unroll
+    for (int s = 0; s < kMaxFace; ++s) {
+      const int j = m.cnbr[s * n + i];
+      if (m.cface[s * n + i] != kNoFace && j >= 0) {
+        add(1 + s, j);
+        on |= 2u << s;
+      }
+    }
+  }
+  double cq[kNM][4];
+#pragma unroll
+  for (int q = 0; q < kNM; ++q) {
+    double x[4];
+#pragma unroll
+    for (int b = 0; b < 4; ++b) x[b] = coef[(q * 4 + b) * n + i];
+    f.fields(1.0, x, cq[q]);
+  }
+  weno_combine(P, m.m2[i], m.m2[n + i], m.m2[2 * n + i], on, lin, cq);
+#pragma unroll
+  for (int q = 0; q < kNM; ++q) f.conservative(cq[q], out[q]);
+}
 template <typename T>
 __device__ void char_side(const MeshT<T> &m, const ParamsT<T> &P, const T *__restrict__ W, const T *__restrict__ Wx,
                           const T *__restrict__ coef, int i, const T wref[4], T nx, T ny, T out[kNM][4]) {

@@ -287,7 +287,7 @@ __device__ __forceinline__ void recon_at(const MeshT<T> &m, const ParamsT<T> &P,
   T lin[WENO ? 7 : 1][3][NC];
   unsigned on = 1;
   if constexpr (WENO) {
-    const T h = T(1) / m.ih[i];
+    const T h = quot(T(1), m.ih[i]);
 #pragma unroll
     for (int v = 0; v < NC; ++v)
 #pragma unroll
@@ -307,7 +307,7 @@ __device__ __forceinline__ void recon_at(const MeshT<T> &m, const ParamsT<T> &P,
         for (int d = 0; d < 3; ++d) b[d][v] = Wx[(d * NV + vo + v) * n + j];
       }
       if constexpr (WENO) {
-        const T h = T(1) / m.ih[i];
+        const T h = quot(T(1), m.ih[i]);
 #pragma unroll
         for (int v = 0; v < NC; ++v)
 #pragma unroll

@@ -471,14 +471,13 @@ FACES3 = {2: [(0, 2, 1), (0, 1, 3), (1, 2, 3), (2, 0, 3)],
           3: [(0, 2, 1), (3, 4, 5), (0, 1, 4, 3), (1, 2, 5, 4), (2, 0, 3, 5)],
           4: [(0, 3, 2, 1), (0, 1, 4), (1, 2, 4), (2, 3, 4), (3, 0, 4)],
           5: [(0, 3, 2, 1), (4, 5, 6, 7), (0, 1, 5, 4), (1, 2, 6, 5), (2, 3, 7, 6), (3, 0, 4, 7)]}
-# FP64 operations per Gauss point of the 3-D smooth flux: 2395 for the
-# kinetic flux (630 add, 1749 mul, 8 div, 4 sqrt, 2 exp, 2 erfc; counted by
-# instantiating the kernels' templated physics on a counting number type)
-# + ~825 for the two quadratic evaluations, frame rotations and sums.
-FLOPS_PER_GP3 = 3220
-# per interior neighbour of a relaxed cell: U + dU 5, Euler flux 31, bracket
-# and accumulation 30, weight 1; 5 multiplications by 1/D per cell
-SWEEP3_FLOPS_PER_NEIGHBOUR, SWEEP3_FLOPS_PER_CELL = 67, 5
+# FP64 operations per Gauss point of the 3-D smooth flux: 600 instructions as
+# counted on the 128,000-cell sphere (two quadratic evaluations, the flux from
+# moments about the mean velocity, sums), a fused multiply-add being two.
+FLOPS_PER_GP3 = 1200
+# the relaxation's increment form: 22 instructions per interior neighbour of a
+# relaxed cell, 33 per cell
+SWEEP3_FLOPS_PER_NEIGHBOUR, SWEEP3_FLOPS_PER_CELL = 44, 66
 
 
 def topology3(mesh, gm):
@@ -518,17 +517,20 @@ def work_model3(mesh, gm, spec, precision, _cache={}):
     _, colour = gm.ordering()
     colour = np.asarray(colour)
     C = int(colour.max()) + 1
+    # passes (colour, descending): a descending pass relaxes the cells with a
+    # neighbour of a higher colour; the first pass is the right-hand side's
+    up = np.zeros(mesh.n_cells, bool)
+    up[a[colour[b] > colour[a]]] = True
+    up[b[colour[a] > colour[b]]] = True
     seq = []
     for _ in range(spec["n_sweeps"]):
-        for c in list(range(C)) + list(range(C - 1, -1, -1)):
-            if not seq or seq[-1] != c:
-                seq.append(c)
-    seq = seq[1:]
+        seq += [(c, False) for c in range(1, C)]
+        seq += [(c, True) for c in range(C - 2, -1, -1) if c == 0 or (up & (colour == c)).any()]
     ni = spec["n_implicit"]
     w = 8 if precision == "fp64" else 4
     by_c = {}
-    for c in range(C):
-        incol = colour == c
+    for c, down in sorted(set(seq)):
+        incol = (colour == c) & (up | (not down) | (c == 0))
         slots = int(nb[incol].sum())
         # distinct neighbours of the colour's cells
         na = b[incol[a]]
@@ -536,9 +538,9 @@ def work_model3(mesh, gm, spec, precision, _cache={}):
         uniq = np.unique(np.concatenate([na, nbb])).size
         flops = SWEEP3_FLOPS_PER_NEIGHBOUR * slots + SWEEP3_FLOPS_PER_CELL * int(incol.sum())
         own = int(incol.sum()) * 11 * w
-        per_slot = slots * (4 + 5 * w + (4 + 5 * w if precision == "fp64" else 0))
-        nbr = uniq * (10 * w + (4 * w if precision == "mixed" else 0))
-        by_c[c] = (flops, own + per_slot + nbr)
+        per_slot = slots * (4 + 5 * w)              # neighbour, normal, area, lambda
+        nbr = uniq * (15 * w if precision == "fp64" else 16 * w)   # base and increment records
+        by_c[c, down] = (flops, own + per_slot + nbr)
     n, F = mesh.n_cells, gm.n_faces
     gps = 3 * T + 4 * Q
     return {"sweep_flops": ni * sum(by_c[c][0] for c in seq),
@@ -546,9 +548,9 @@ def work_model3(mesh, gm, spec, precision, _cache={}):
             "bytes": {"k_sweep": ni * sum(by_c[c][1] for c in seq),
                       "k_recon": 2 * n * ((20 + 243 + 45) * w + 48),
                       "k_face": 2 * (n * 56 * w + F * (47 * w + 12)),
-                      "k_lo_face": ni * (n * 15 * w + F * (6 * w + 9 * w + 12 + (10 * w if precision == "fp64" else 0))),
+                      "k_lo_face": ni * (n * 15 * w + F * (6 * w + 9 * w + 12)),
                       "k_lo_rhs": ni * (F * 7 * w + n * (24 + 5 * 8 + 16 * w + 6 * w)),
-                      "k_lo_cell": (ni + 1) * n * (10 * 8 + 5 * w + 10 * w),
+                      "k_lo_cell": n * (5 * 8 + 16 * w),
                       "k_prolong": n * 20 * 8},
             "gauss_points": gps, "colours": C, "sweep_launches": ni * len(seq)}
 
@@ -784,21 +786,18 @@ def topology(mesh, gm):
     return nb, nbrs, np.asarray(colour), n_int, len(edges)
 
 
-# FP64 operations (add, mul, div each 1) of the relaxation term of one
-# interior neighbour: U + dU (4), Euler normal flux (23), the bracket
-# ((F - F_cache) - lambda (U + dU - U)) scaled by S/2 and accumulated (24),
-# S/2 weight (1); plus 4 multiplications by 1/D per cell.
-SWEEP_FLOPS_PER_NEIGHBOUR = 52
-SWEEP_FLOPS_PER_CELL = 4
-# other low-order phases (FP64 operations): KFVS flux of a face with its two
-# spectral radii and Euler cache ~120; right-hand side of a cell ~50 (face
-# sums, 1/D); cell primitives ~25 (1 division, 2 square roots)
-LO_FACE_FLOPS, LO_RHS_FLOPS, LO_CELL_FLOPS = 120, 50, 25
-# FP64 operations per Gauss point of the 2-D smooth flux: 1163 for the
-# kinetic flux (302 add, 827 mul, 26 div, 4 sqrt, 2 exp, 2 erfc; counted on
-# an operation-counting number type) + ~330 for the two quadratic
-# evaluations, rotations and sums (2 Gauss points per face)
-FLOPS_PER_GP2 = 1490
+# FP64 operations as the kernels issue them, a fused multiply-add counted as
+# two.  Relaxation in increment form: 17 instructions per interior neighbour,
+# 21 per cell.
+SWEEP_FLOPS_PER_NEIGHBOUR = 34
+SWEEP_FLOPS_PER_CELL = 42
+# other low-order phases (instructions counted on the 57,344-cell cylinder, x 2):
+# KFVS flux of a face with its spectral radii 96, right-hand side of a cell 48,
+# base record of a cell 24
+LO_FACE_FLOPS, LO_RHS_FLOPS, LO_CELL_FLOPS = 192, 96, 48
+# per Gauss point of the 2-D smooth flux (2 per face): 338 instructions (two
+# quadratic evaluations, the flux from moments about the mean velocity, sums)
+FLOPS_PER_GP2 = 676
 FP64_PEAK_TFLOPS = 1.25    # GB300: 152 SMs x 2.07 GHz x 2 FP64 FMA/clk x 2 flops (recipe table)
 
 
@@ -825,8 +824,8 @@ def work_model(mesh, gm, spec, precision):
         uniq = len({j for i in cells for j in nbrs[i]})
         flops = SWEEP_FLOPS_PER_NEIGHBOUR * slots + SWEEP_FLOPS_PER_CELL * len(cells)
         own = len(cells) * 9 * w
-        per_slot = slots * (4 + 4 * w + (4 + 4 * w if precision == "fp64" else 0))
-        nbr = uniq * (8 * w + (3 * w if precision == "mixed" else 0))
+        per_slot = slots * (4 + 4 * w)              # neighbour, normal, area, lambda
+        nbr = uniq * 12 * w                         # base and increment records
         by_c[c] = (flops, own + per_slot + nbr)
     sweep_flops = ni * sum(by_c[c][0] for c in seq)
     sweep_bytes = ni * sum(by_c[c][1] for c in seq)
@@ -842,12 +841,12 @@ def work_model(mesh, gm, spec, precision):
         # face sums (16 per face in a stage update, 4 in the residual mode),
         # geometry, W in, W/Wx out; ev launches per cycle
         "k_update": F * (16 * (ev - 1) + 4) * w + ev * (F * 3 * d + n * (16 + 2 * 4 * d + 2 * 8 * d)),
-        "k_lo_face": ni * (n * 13 * w + F * (5 * w + 3 * w + 12 + (8 * w if precision == "fp64" else 0))),
+        "k_lo_face": ni * (n * 13 * w + F * (5 * w + 3 * w + 12)),
         "k_lo_rhs": ni * (F * 6 * w + n * (16 + 4 * d + 13 * w + 4 * w)),
-        "k_lo_cell": (ni + 1) * n * (8 * d + 4 * w + 9 * w),
+        "k_lo_cell": n * (4 * d + 12 * w),
         "k_prolong": n * (4 * 3 + 4) * d,
     }
-    lo_flops = sweep_flops + ni * (LO_FACE_FLOPS * F + LO_RHS_FLOPS * n) + (ni + 1) * LO_CELL_FLOPS * n
+    lo_flops = sweep_flops + ni * (LO_FACE_FLOPS * F + LO_RHS_FLOPS * n) + ni * LO_CELL_FLOPS * n
     bytes_["k_lo_solve"] = sum(bytes_[k] for k in ("k_sweep", "k_lo_face", "k_lo_rhs", "k_lo_cell"))
     return {"sweep_flops": sweep_flops, "lo_flops": lo_flops, "bytes": bytes_, "colours": C,
             "sweep_launches": ni * len(seq), "face_flops": ev * F * 2 * FLOPS_PER_GP2}

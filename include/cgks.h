@@ -269,7 +269,7 @@ const char *cgks_strerror(int status);
  * A server keeps every admitted solve's state on the device and advances
  * all of them with one batched V-cycle per cgks_server_step: their cells
  * and faces are concatenated into one index space (each solve's cells
- * padded to a multiple of 256), so every kernel of the cycle runs once for
+ * padded to a multiple of 64), so every kernel of the cycle runs once for
  * the whole batch.  Requests are admitted first-come-first-served while the
  * sum of their device footprints stays within hbm_budget and fewer than
  * max_active are running; a solve retires when its density residual Res
@@ -394,9 +394,9 @@ int cgks_wall_loads(cgks_solver *s, int32_t tag, int64_t max_faces, int64_t *n_f
  * Four kernels take a launch shape: the compact reconstruction, the
  * gas-kinetic face flux, the low-order (KFVS) face flux and the colour
  * sweep, in that order (CGKS_TUNE_KERNELS).  A shape (CGKS_TUNE_SHAPES of
- * them, index 0..4) is a block size, a number of items (cells or faces;
- * cells per lane group for the sweep) per thread and a minimum number of
- * resident blocks per SM (a register cap); cgks_tune_shape describes one.
+ * them, index 0..4) is a block size, a number of items per thread (1) and a
+ * minimum number of resident blocks per SM (1: no register cap);
+ * cgks_tune_shape describes one.
  * Each item is computed by the same arithmetic under every shape, so the
  * shape never changes a result, only the time.
  * With autotune on, the first 3 x CGKS_TUNE_SHAPES V-cycles (or explicit

@@ -1178,7 +1178,11 @@ __global__ void __launch_bounds__(kMaxShapeBlock)
   const int g = static_cast<int>(blockIdx.x * blockDim.x + threadIdx.x) / LANES;
   const int i = g < count ? begin + g : -1;
   if constexpr (LANES == 1) {
-    constexpr int CH = is_f32<T>() ? 6 : 3;   // slots whose loads are in flight together (registers)
+    // slots whose loads are in flight together: all six took 137 registers in
+    // FP32, six warps an SM (V-cycle's sweeps, 512,000 cells mixed: 1412 us with
+    // six, 1313 with three, 1273 with two, 1300 with one; FP64, 128,000: 1305
+    // with three, 1297 with two)
+    constexpr int CH = 2;
     if (i < 0) { pdl_enter(); return; }   // waits too: this grid ends after its predecessor
     // the neighbours (mesh data) before the wait for the predecessor
     int nb[kMaxFace3];

@@ -910,7 +910,7 @@ enum UpdMode { kS1O2 = 0, kS2O4Stage = 1, kS2O4Final = 2, kResidual = 3 };
 // accumulated in FP64): runs are widened and mirrors rounded with integer
 // instructions, areas and normals come from the cell's slots (coalesced), the
 // mode is a template argument so that only the values it needs are read.
-// us per launch, before and now: 57,344 cells mixed 30.2 -> 17.2, FP64 22.7 -> 17.3.
+// us per launch, before and now: 57,344 cells mixed 30.2 -> 16.6, FP64 22.7 -> 16.9.
 template <typename TF, int mode>
 __global__ void __launch_bounds__(kCellBlock) k_update(MeshT<double> m, ParamsT<double> P, const double *Wbase,
                                                        const TF *FA, const TF *FB, const Ctl *ctl,
@@ -1139,7 +1139,7 @@ __global__ void __launch_bounds__(kCellBlock) k_lo_cell(int n, ParamsT<TF> P, in
 // K5b: first-order KFVS (or Lax-Friedrichs) flux and the spectral radius
 // lambda_p = max of both sides.  FP64 is bound by its pipe, so it has no face
 // frame, no division and no pow.  us per launch, FP64, before and now: 57,344
-// cells 68 -> 28.4, a 128,000-cell sphere (3-D) 220 -> 96.6.
+// cells 68 -> 28.4, a 128,000-cell sphere (3-D) 220 -> 93.5.
 template <typename T>
 struct LoFaceGeo {
   int sid, c0, c1;

@@ -642,7 +642,8 @@ __device__ __forceinline__ void face_points_at(const MeshT<double> &m, const Par
 // point of a triangle; four on a small one spread its few faces over the FP64
 // units (608 sub-cores).  28,850 faces (hexahedra): 174 us with 4, 191 with 1;
 // 282,880 (mostly triangles): 1281 us with 4, 1162 with 1 (before, raw moments
-// in one thread: 358 and 2809 us).
+// in one thread: 358 and 2809 us).  With the far field hoisted and the wall
+// mirrors linear the better ones take 145 and 1074 us.
 constexpr int64_t kFaceLanes4 = 100000;
 inline int face_lanes(int64_t n_faces) { return n_faces < kFaceLanes4 ? 4 : 1; }
 // FP32: one thread per face.  Bound by latency at two warps a scheduler (255
@@ -674,7 +675,7 @@ enum UpdMode { kS1O2 = 0, kS2O4Stage = 1, kS2O4Final = 2, kResidual = 3 };
 //   R = -sum sgn S (a0 F0A + a1 F1(A, B));  W_out = W_base + dt/|Omega| R;
 //   Wx_out = 1/|Omega| sum sgn S n (WcA + b1 Wt)
 // In the mixed path the runs are widened and the mirrors rounded with integer
-// instructions (the FP64 pipe bounds the kernel): 223 -> 127 us a launch on
+// instructions (the FP64 pipe bounds the kernel): 223 -> 119 us a launch on
 // 512,000 cells.
 // The mode is a template argument so that each variant holds only the runs
 // it reads: the residual reads F0 and F1 of one buffer, the stages one
@@ -1038,7 +1039,7 @@ __global__ void __launch_bounds__(kMaxShapeBlock)
 // FP64 times S/2), first colour pass (dU = R / D on colour 0, zero elsewhere)
 // The FP64 pipe bounds it in both precisions (a cell's fluxes are summed in
 // FP64): FP32 fluxes are widened with integer instructions and only colour 0
-// forms R / D.  512,000 cells mixed: 107 -> 80.4 us a launch.
+// forms R / D.  512,000 cells mixed: 107 -> 78.4 us a launch.
 template <typename TF>
 __global__ void __launch_bounds__(kCellBlock) k_lo_rhs(MeshT<double> m, ParamsT<double> P, TF gamma, int first,
                                                        int colour0_end, const TF *base,
@@ -1166,7 +1167,8 @@ constexpr int kSweepLanes = 8;
 // 4,864 cells.  Event-timed, us per launch, eight / one: colours of 3,960 cells
 // 11.7 / 13.3; 15,360 25.0 / 14.6; 25,000 to 51,463 42.6 / 18.8 (before: 41.4).
 // FP32 is bound by the latency of its gathers and then by their number: 3,960
-// 6.5 / 7.7; 12,779 7.2 / 7.7; 15,360 8.3 / 8.0; 211,181 17.0 / 15.9.
+// 6.5 / 7.7; 12,779 7.2 / 7.7; 15,360 8.3 / 8.0; 211,181 17.0 / 15.9
+// (one thread with the loads of all six slots in flight; less now).
 constexpr int kOneLane64 = 4864, kOneLane32 = 14000;
 template <typename T> int sweep_lanes(int cnt) { return cnt >= (is_f32<T>() ? kOneLane32 : kOneLane64) ? 1 : kSweepLanes; }
 template <typename T, bool LAST, int LANES>

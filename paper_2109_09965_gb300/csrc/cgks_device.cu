@@ -122,6 +122,7 @@ struct Batch {
   int n_lim = 0, n_smooth = 0;       // active solves of each class
   int64_t ptab_cap = 0;              // ints ptab holds
   int n_parts = 0;
+  int part_lanes = 1;                // lanes per cell of the partitioned sweep
   int lo_grid = 0;
   bool lo_fused_ok = false;
   Tuner tune;                          // launch shapes of the tunable kernels
@@ -374,10 +375,13 @@ void enqueue_lo_solve(Batch *b) {
     if (part) {
       TF *in = del0, *out = del0 == B.delta ? B.delta2 : B.delta;
       for (int sw = 0; sw < b->sh.n_sweeps; ++sw) {
-        launch_cluster(b, KI_SWEEP, k_sweep_part<TF>, dim3(b->n_parts * kPartCluster), dim3(kPartBlock),
-                       kPartCluster, fmesh<TF>(b), fparams<TF>(b), (const int *)b->ptab, b->n_colours,
-                       (const TF *)base, (const TF *)B.Rk, (const TF *)B.invD, (const TF *)B.lamS, (const TF *)in,
-                       out);
+        auto go = [&](auto kern) {
+          launch_cluster(b, KI_SWEEP, kern, dim3(b->n_parts * kPartCluster), dim3(kPartBlock), kPartCluster,
+                         fmesh<TF>(b), fparams<TF>(b), (const int *)b->ptab, b->n_colours, (const TF *)base,
+                         (const TF *)B.Rk, (const TF *)B.invD, (const TF *)B.lamS, (const TF *)in, out);
+        };
+        if (b->part_lanes == 4) go(k_sweep_part<TF, 4>);
+        else go(k_sweep_part<TF, 1>);
         std::swap(in, out);
       }
       continue;
@@ -953,6 +957,9 @@ int finalize_batch(Batch *b) {
       }
     }
     b->n_parts = static_cast<int>(tab.size() / (2 * std::max(C, 1)));
+    int run = 0;   // the longest
+    for (size_t k = 0; k < tab.size(); k += 2) run = std::max(run, tab[k + 1] - tab[k]);
+    b->part_lanes = b->mixed ? part_lanes<float>(run) : part_lanes<double>(run);
     if (static_cast<int64_t>(tab.size()) > b->ptab_cap) return CGKS_EINVAL;
     if (!tab.empty())
       CK(cudaMemcpyAsync(b->ptab, tab.data(), sizeof(int) * tab.size(), cudaMemcpyHostToDevice, b->stream));

@@ -1568,6 +1568,50 @@ __device__ __forceinline__ void sweep_cell(const MeshT<T> &m, T gamma, const Slo
   }
   store_delta(gamma, bi, d, out, i);
 }
+// Four lanes per cell (i < 0: none), lane s one slot: the new increment's
+// component s is returned, the delta record written to out; CG and CGD as for
+// slot_load.  Whole warps call it.
+template <typename T, bool CG, bool CGD, typename DelOf>
+__device__ __forceinline__ T sweep_quad(const MeshT<T> &m, T gamma, const SlotGeo<T> &geo, const int i, const int s,
+                                        const T *base, const T *Rk, const T *invD, const T *lamS, DelOf &&del_of,
+                                        T *out) {
+  const int n = m.nc;
+  T bi[4] = { T(0), T(0), T(0), T(0) }, r = T(0), iD = T(0);
+  if (i >= 0) {
+    r = ld<CG>(&Rk[s * n + i]);
+    iD = ld<CG>(&invD[i]);
+    if constexpr (!is_f32<T>()) vload<T, 4, CG>(base + static_cast<size_t>(i) * kBase, bi);
+  }
+  T c[4] = { T(0), T(0), T(0), T(0) };
+  if (geo.j >= 0) {
+    SlotData<T> x;
+    slot_load<T, CG, CGD>(m, i, s, geo.j, base, lamS, del_of(geo.j), x);
+    slot_bracket(gamma, geo, x, c);
+  }
+  // lane s needs component s summed over the group: a transposing
+  // reduction (3 additions per lane instead of an all-reduce of 4 values);
+  // every lane stays to the shuffles, absent cells and slots add 0
+  const bool b0 = s & 1, b1 = s & 2;
+  const T k0 = add_rn(b0 ? c[1] : c[0], __shfl_xor_sync(0xffffffffu, b0 ? c[0] : c[1], 1));   // component b0
+  const T k1 = add_rn(b0 ? c[3] : c[2], __shfl_xor_sync(0xffffffffu, b0 ? c[2] : c[3], 1));   // component b0 + 2
+  const T mine = add_rn(b1 ? k1 : k0, __shfl_xor_sync(0xffffffffu, b1 ? k0 : k1, 2));
+  const T ds = (r - mine) * iD;
+  if constexpr (is_f32<T>()) {
+    if (i >= 0) out[static_cast<size_t>(i) * 4 + s] = ds;
+  } else {
+    T d[4], rec[8];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) d[v] = __shfl_sync(0xffffffffu, ds, v, 4);
+    delta_record(gamma, bi, d, rec);
+    if (i >= 0) {
+      const T lo = s == 0 ? rec[0] : s == 1 ? rec[2] : s == 2 ? rec[4] : rec[6];
+      const T hi = s == 0 ? rec[1] : s == 1 ? rec[3] : s == 2 ? rec[5] : rec[7];
+      const T two[2] = { lo, hi };
+      vstore<T, 2>(out + static_cast<size_t>(i) * 8 + 2 * s, two);
+    }
+  }
+  return ds;
+}
 // Lanes per cell of a sweep over cnt cells.  An FP64 launch takes as long as
 // the warps of one sub-core (608 of them) issue one after another: about 43
 // instructions for each 8 cells with four lanes, 91 for each 32 with one, so
@@ -1621,44 +1665,11 @@ __global__ void __launch_bounds__(kMaxShapeBlock) k_sweep(MeshT<T> m, ParamsT<T>
     const int s = threadIdx.x & (kMaxFace - 1);
     const SlotGeo<T> geo = slot_geo(m, i, s);
     pdl_enter();
-    T bi[4] = { T(0), T(0), T(0), T(0) }, r = T(0), iD = T(0);
-    double us = 0.0;
-    if (i >= 0) {
-      r = Rk[s * n + i];
-      iD = invD[i];
-      if constexpr (!is_f32<T>()) vload<T, 4>(base + static_cast<size_t>(i) * kBase, bi);
-      if (LAST) us = U[s * n + i];
-    }
-    T c[4] = { T(0), T(0), T(0), T(0) };
-    if (geo.j >= 0) {
-      SlotData<T> x;
-      slot_load<T, false, false>(m, i, s, geo.j, base, lamS, delta, x);
-      slot_bracket(P.gamma, geo, x, c);
-    }
-    // lane s needs component s summed over the group: a transposing
-    // reduction (3 additions per lane instead of an all-reduce of 4 values);
-    // every lane stays to the shuffles, absent cells and slots add 0
-    const bool b0 = s & 1, b1 = s & 2;
-    const T k0 = add_rn(b0 ? c[1] : c[0], __shfl_xor_sync(0xffffffffu, b0 ? c[0] : c[1], 1));   // component b0
-    const T k1 = add_rn(b0 ? c[3] : c[2], __shfl_xor_sync(0xffffffffu, b0 ? c[2] : c[3], 1));   // component b0 + 2
-    const T mine = add_rn(b1 ? k1 : k0, __shfl_xor_sync(0xffffffffu, b1 ? k0 : k1, 2));
-    const T ds = (r - mine) * iD;
-    if constexpr (is_f32<T>()) {
-      if (i >= 0) delta[static_cast<size_t>(i) * 4 + s] = ds;
-    } else {
-      T d[4], rec[8];
-#pragma unroll
-      for (int v = 0; v < 4; ++v) d[v] = __shfl_sync(0xffffffffu, ds, v, 4);
-      delta_record(P.gamma, bi, d, rec);
-      if (i >= 0) {
-        const T lo = s == 0 ? rec[0] : s == 1 ? rec[2] : s == 2 ? rec[4] : rec[6];
-        const T hi = s == 0 ? rec[1] : s == 1 ? rec[3] : s == 2 ? rec[5] : rec[7];
-        const T two[2] = { lo, hi };
-        vstore<T, 2>(delta + static_cast<size_t>(i) * 8 + 2 * s, two);
-      }
-    }
+    const double us0 = LAST && i >= 0 ? U[s * n + i] : 0.0;
+    const T ds = sweep_quad<T, false, false>(m, P.gamma, geo, i, s, base, Rk, invD, lamS,
+                                             [&](int) -> const T * { return delta; }, delta);
     if constexpr (LAST) {
-      us += static_cast<double>(ds);
+      const double us = us0 + static_cast<double>(ds);
       if (i >= 0) U[s * n + i] = us;
       double u[4];
 #pragma unroll
@@ -1693,6 +1704,15 @@ __global__ void __launch_bounds__(kMaxShapeBlock) k_sweep(MeshT<T> m, ParamsT<T>
 constexpr int kPartBlock = 256;        // threads per CTA: one cell per thread and pass
 constexpr int kPartCluster = 8;        // CTAs per partition (portable cluster size)
 constexpr int kMaxPartColours = 16;
+// Lanes per cell, from the longest run of cells that one colour has in a
+// partition.  A cluster takes 2,048 cells a pass with one lane and 512 with
+// four, which need half the registers (twice the clusters at once) and half
+// the chain; past two to three such passes one lane is the shorter.  us per
+// V-cycle, one / four lanes: FP64 runs of 127 cells 5504 / 1921, 1,020
+// 1714 / 1306, 1,365 738 / 779, 2,000 1290 / 1406 (8,192 cells for the third,
+// else 57,344); mixed 1415 / 487, 424 / 357, 319 / 297, 330 / 344 (18,432 for
+// the last).
+template <typename T> int part_lanes(int run) { return run <= (is_f32<T>() ? 1536 : 1280) ? 4 : 1; }
 
 __device__ __forceinline__ unsigned cluster_ctarank() {
   unsigned r;
@@ -1712,7 +1732,7 @@ __device__ __forceinline__ void cluster_sync() {
 
 // ptab [Q][C][2]: first and end cell (internal index) of colour c in
 // partition q; C colours
-template <typename T>
+template <typename T, int LANES>
 __global__ void __launch_bounds__(kPartBlock) k_sweep_part(MeshT<T> m, ParamsT<T> P, const int *__restrict__ ptab,
                                                            int C, const T *base,
                                                            const T *Rk, const T *invD,
@@ -1732,19 +1752,26 @@ __global__ void __launch_bounds__(kPartBlock) k_sweep_part(MeshT<T> m, ParamsT<T
     const bool fwd = step < C;
     const int c = fwd ? step : 2 * C - 2 - step;
     const int b = sb[c], e = se[c];
-    for (int i = b + static_cast<int>(rank) * kPartBlock + static_cast<int>(threadIdx.x); i < e;
-         i += static_cast<int>(K) * kPartBlock) {
-      SlotGeo<T> g[kMaxFace];
+    // the increments of j: this sweep's where its colour is done, else those at its start
+    auto del_of = [&](int j) -> const T * {
+      const int cj = m.ccol[j];
+      const bool fresh = cj < C && j >= sb[cj] && j < se[cj] && (!fwd || cj < c);
+      return fresh ? delta_out : delta_in;
+    };
+    constexpr int kCells = kPartBlock / LANES;   // of a CTA's pass
+    // (LANES == 4: the 8 cells of a warp iterate together)
+    const int lead = static_cast<int>(LANES == 1 ? threadIdx.x : threadIdx.x / 32 * 8);
+    for (int i0 = b + static_cast<int>(rank) * kCells + lead; i0 < e; i0 += static_cast<int>(K) * kCells) {
+      if constexpr (LANES == 1) {
+        SlotGeo<T> g[kMaxFace];
 #pragma unroll
-      for (int k = 0; k < kMaxFace; ++k) g[k] = slot_geo(m, i, k);
-      T d[4];
-      sweep_cell<T, false, true>(m, P.gamma, g, i, base, Rk, invD, lamS,
-                                 [&](int j) -> const T * {
-                                   const int cj = m.ccol[j];
-                                   const bool fresh = cj < C && j >= sb[cj] && j < se[cj] && (!fwd || cj < c);
-                                   return fresh ? delta_out : delta_in;
-                                 },
-                                 delta_out, d);
+        for (int k = 0; k < kMaxFace; ++k) g[k] = slot_geo(m, i0, k);
+        T d[4];
+        sweep_cell<T, false, true>(m, P.gamma, g, i0, base, Rk, invD, lamS, del_of, delta_out, d);
+      } else {
+        const int at = i0 + static_cast<int>(threadIdx.x % 32 / 4), i = at < e ? at : -1, k = threadIdx.x % 4;
+        sweep_quad<T, false, true>(m, P.gamma, slot_geo(m, i, k), i, k, base, Rk, invD, lamS, del_of, delta_out);
+      }
     }
     if (step + 1 < steps) cluster_sync();
   }

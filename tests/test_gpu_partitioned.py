@@ -111,3 +111,21 @@ def test_partitioned_rejections(libs):
     with pytest.raises(cgks.CgksError):
         cgks.Solver(cgks.Mesh(m3), dict(gamma=GAM, sweep_order="partitioned",
                                         bcs=[dict(kind="farfield", rho=1.0, u=(0.1, 0.0, 0.0), p=1 / GAM)]))
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("part_cells, n_parts", [(2600, 4), (3500, 3), (4096, 2)])
+def test_one_and_four_lanes_per_cell_match_oracle(libs, part_cells, n_parts, precision):
+    """Partitions whose colours hold about 1,010, 1,350 and 2,020 cells, on the
+    sides of the lengths (1,280 in FP64, 1,536 in mixed) from which the sweep
+    takes one lane per cell instead of four: one and several passes of a
+    cluster, whole and ragged ones."""
+    mesh = MG.cavity(64)
+    spec = dict(gamma=GAM, mu=0.15 / 1000, cfl_hi=0.4,
+                bcs=[dict(kind="noslip"), dict(kind="noslip", uw=(0.15, 0.0))])
+    W = np.tile(exact.cons_from_prim(GAM, 1.0, 0.0, 0.0, 1 / GAM), (mesh.n_cells, 1))
+    g, o, n = pair_part(libs, mesh, spec, (W, None), part_cells, precision)
+    assert n == n_parts
+    g.pmg_cycle(2)
+    o.pmg_cycles(2)
+    assert rel(g.get_state()[0], o.get_state()[0]) < (TOL if precision == "fp64" else 1e-5)

@@ -1537,22 +1537,22 @@ __device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(
 
 // One thread per cell: the new increment of cell i in d, its delta record
 // written to out.  The neighbours' delta records are read from del_of(j)
-// (through L2 when CGD is set), the rest through L2 when CG is.
-template <typename T, bool CG, bool CGD, typename DelOf>
+// (through L2 when CGD is set).
+template <typename T, bool CGD, typename DelOf>
 __device__ __forceinline__ void sweep_cell(const MeshT<T> &m, T gamma, const SlotGeo<T> g[kMaxFace], const int i,
                                            const T *base, const T *Rk, const T *invD, const T *lamS, DelOf &&del_of,
                                            T *out, T d[4]) {
   const int n = m.nc;
   T r[4], bi[4] = { T(0), T(0), T(0), T(0) };
 #pragma unroll
-  for (int v = 0; v < 4; ++v) r[v] = ld<CG>(&Rk[v * n + i]);
-  if constexpr (!is_f32<T>()) vload<T, 4, CG>(base + static_cast<size_t>(i) * kBase, bi);
-  const T iD = ld<CG>(&invD[i]);
+  for (int v = 0; v < 4; ++v) r[v] = Rk[v * n + i];
+  if constexpr (!is_f32<T>()) vload<T, 4>(base + static_cast<size_t>(i) * kBase, bi);
+  const T iD = invD[i];
   // every neighbour's loads are in flight before the first is used
   SlotData<T> x[kMaxFace];
 #pragma unroll
   for (int s = 0; s < kMaxFace; ++s)
-    if (g[s].j >= 0) slot_load<T, CG, CGD>(m, i, s, g[s].j, base, lamS, del_of(g[s].j), x[s]);
+    if (g[s].j >= 0) slot_load<T, false, CGD>(m, i, s, g[s].j, base, lamS, del_of(g[s].j), x[s]);
   T c[kMaxFace][4];
 #pragma unroll
   for (int s = 0; s < kMaxFace; ++s) {
@@ -1647,7 +1647,7 @@ __global__ void __launch_bounds__(kMaxShapeBlock) k_sweep(MeshT<T> m, ParamsT<T>
     for (int s = 0; s < kMaxFace; ++s) geo[s] = slot_geo(m, i, s);
     pdl_enter();
     T d[4];
-    sweep_cell<T, false, false>(m, P.gamma, geo, i, base, Rk, invD, lamS, [&](int) -> const T * { return delta; },
+    sweep_cell<T, false>(m, P.gamma, geo, i, base, Rk, invD, lamS, [&](int) -> const T * { return delta; },
                                 delta, d);
     if constexpr (LAST) {
       double u[4];
@@ -1767,7 +1767,7 @@ __global__ void __launch_bounds__(kPartBlock) k_sweep_part(MeshT<T> m, ParamsT<T
 #pragma unroll
         for (int k = 0; k < kMaxFace; ++k) g[k] = slot_geo(m, i0, k);
         T d[4];
-        sweep_cell<T, false, true>(m, P.gamma, g, i0, base, Rk, invD, lamS, del_of, delta_out, d);
+        sweep_cell<T, true>(m, P.gamma, g, i0, base, Rk, invD, lamS, del_of, delta_out, d);
       } else {
         const int at = i0 + static_cast<int>(threadIdx.x % 32 / 4), i = at < e ? at : -1, k = threadIdx.x % 4;
         sweep_quad<T, false, true>(m, P.gamma, slot_geo(m, i, k), i, k, base, Rk, invD, lamS, del_of, delta_out);

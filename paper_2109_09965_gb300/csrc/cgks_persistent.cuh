@@ -1,8 +1,8 @@
 // Persistent fused low-order solve (included by cgks_device.cu only).
 //
 // One cooperative launch runs the whole low-order level of a V-cycle
-// (Section 3, steps 3-4): n_implicit backward-Euler steps, each = cell
-// primitives (and U += dU), KFVS faces, right-hand side with the first
+// (Section 3, steps 3-4): n_implicit backward-Euler steps, each = base
+// records (and U += dU), KFVS faces, right-hand side with the first
 // colour pass, then the remaining colour passes of Algorithm 1, and the
 // final U += dU.  Phases are separated by a grid barrier instead of kernel
 // boundaries.  Every value produced inside the launch is read with
@@ -10,8 +10,8 @@
 // functions of the per-phase kernels of cgks_kernels.cuh.
 //
 // Measured on GB300 (57k-cell cylinder V-cycle): slower than the per-phase
-// kernels replayed from a CUDA graph (FP64 2.22 vs 1.89 ms, mixed 0.54 vs
-// 0.42 ms): the resident grid holds fewer warps per SM than the separate
+// kernels replayed from a CUDA graph (FP64 1.34 vs 0.91 ms, mixed 0.48 vs
+// 0.28 ms): the resident grid holds fewer warps per SM than the separate
 // launches and the graph already hides their launch gaps, so the library
 // uses it only when asked (cgks_params.low_order_fused).
 //
@@ -130,14 +130,16 @@ __global__ void __launch_bounds__(kPersistBlock, 2) k_lo_solve(const __grid_cons
     for (int q = 0; q < a.n_seq; ++q) {
       const int c = a.seq[q];
       const int total = a.cr.rpre[a.cr.rstart[c + 1] + c];
-      for (int g = tid; g < total; g += nth) {
-        const int i = colour_cell(a.cr, c, g);
-        TF d[4];
-        SlotGeo<TF> geo[kMaxFace];
-#pragma unroll
-        for (int s = 0; s < kMaxFace; ++s) geo[s] = slot_geo(a.fm, i, s);
-        sweep_cell<TF, true, true>(a.fm, a.fp.gamma, geo, i, a.base, a.Rk, a.invD, a.lamS,
-                                   [&](int) -> const TF * { return a.delta; }, a.delta, d);
+      // Four lanes per cell, 8 cells of a warp iterating together.  One thread per
+      // cell spilled in FP64 and left most of the resident warps idle below 20,000
+      // cells of a colour: us per V-cycle, one / four, 2,048 cells FP64 878 / 714,
+      // mixed 425 / 368; 57,344 1638 / 1336, 522 / 475; 131,072 2220 / 2261,
+      // 681 / 684.
+      const int s = threadIdx.x % 4;
+      for (int g0 = tid / 32 * 8; g0 < total; g0 += nth / 4) {
+        const int g = g0 + static_cast<int>(threadIdx.x % 32 / 4), i = g < total ? colour_cell(a.cr, c, g) : -1;
+        sweep_quad<TF, true, true>(a.fm, a.fp.gamma, slot_geo(a.fm, i, s), i, s, a.base, a.Rk, a.invD, a.lamS,
+                                   [&](int) -> const TF * { return a.delta; }, a.delta);
       }
       if (!grid_barrier(a.gb, a.spin_limit, a.err, a.n_err)) return;
     }

@@ -253,6 +253,28 @@ def test_fused_low_order_equals_per_phase_launches(name, precision):
     np.testing.assert_allclose(out[0][1], out[1][1], rtol=100 * tol)
 
 
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_fused_low_order_with_more_cells_than_lane_groups(precision):
+    """51,200 cells: each colour has more cells (25,600) than the resident grid
+    has groups of four lanes (at most 2 x 256 / 4 per SM, 19,456), so warps take
+    several turns, the last one ragged."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    from paper_2109_09965_gb300 import cgks
+    mesh = MG.cavity(160)
+    spec = dict(gamma=GAM, mu=0.15 / 1000, cfl_hi=0.4,
+                bcs=[dict(kind="noslip"), dict(kind="noslip", uw=(0.15, 0.0))])
+    W = np.tile(exact.cons_from_prim(GAM, 1.0, 0.0, 0.0, 1 / GAM), (mesh.n_cells, 1))
+    out = []
+    for fused in (1, 0):
+        s = cgks.Solver(cgks.Mesh(mesh), dict(spec, precision=precision, low_order_fused=fused))
+        s.set_state(W)
+        s.pmg_cycle(2)
+        out.append(s.get_state()[0])
+    assert rel(*out) < (1e-13 if precision == "fp64" else 1e-5)
+
+
 def test_fused_barrier_timeout_reports_status_and_recovers():
     """A grid-barrier wait of the persistent low-order launch that runs out
     (a spin limit of one poll, so the first blocks to arrive give up) ends

@@ -1218,30 +1218,39 @@ int wall_loads_t(cgks_solver *s, int32_t tag, int64_t max_faces, int64_t *n_face
   Bufs<TF> &B = bufs<TF>(b);
   if (b->sh.flux_hi == CGKS_FLUX_FULL) enqueue_dt(b, -1.0);   // the full flux integrates over a step
   enqueue_hi_eval<TF>(b, B.W, B.Wx, B.FA);
-  const int64_t F = b->F, nf = hm.n_faces, off = b->mem[0].face_off;
-  // the face outputs, one run of kFO values per face: F0 is the first 4
-  std::vector<TF> FO(kFO * static_cast<size_t>(F));
-  CK(cudaMemcpyAsync(FO.data(), B.FA, sizeof(TF) * FO.size(), cudaMemcpyDeviceToHost, s->stream));
-  CK(cudaStreamSynchronize(s->stream));
-  int64_t k = 0;
-  for (int64_t f = 0; f < nf; ++f) {
-    if (hm.fc1[f] != -1 - tag) continue;
-    if (k < max_faces) {
-      const int c0 = hm.fc0[f];
-      const double h = hm.h[c0];
-      // face midpoint: the mean of its two Gauss points (offsets from c0 scaled by 1/h)
-      x[2 * k] = hm.xc[c0] + 0.5 * h * (hm.fxi[0 * nf + f] + hm.fxi[2 * nf + f]);
-      x[2 * k + 1] = hm.xc[hm.n_cells + c0] + 0.5 * h * (hm.fxi[1 * nf + f] + hm.fxi[3 * nf + f]);
-      nrm[2 * k] = hm.fn[f];
-      nrm[2 * k + 1] = hm.fn[nf + f];
-      S[k] = hm.fS[f];
-      traction[2 * k] = static_cast<double>(FO[kFO * (off + f) + 1]);
-      traction[2 * k + 1] = static_cast<double>(FO[kFO * (off + f) + 2]);
-    }
-    ++k;
+  const int64_t nf = hm.n_faces, off = b->mem[0].face_off;
+  std::vector<int> face;
+  for (int64_t f = 0; f < nf; ++f)
+    if (hm.fc1[f] == -1 - tag) face.push_back(static_cast<int>(f));
+  const int64_t n = static_cast<int64_t>(face.size()), m = std::min(n, max_faces);
+  // only the tag's momentum fluxes leave the device: packed into FB, scratch
+  // between cycles (16 values per face), behind the list of faces
+  std::vector<TF> t(2 * static_cast<size_t>(m));
+  if (m > 0) {
+    int *list = reinterpret_cast<int *>(B.FB);
+    TF *packed = B.FB + (m * sizeof(int) + 15) / 16 * 16 / sizeof(TF);
+    CK(cudaMemcpyAsync(list, face.data(), sizeof(int) * m, cudaMemcpyHostToDevice, s->stream));
+    k_pack_traction<TF><<<nblk(m, 128), 128, 0, s->stream>>>(static_cast<int>(m), static_cast<int>(off), list,
+                                                             (const TF *)B.FA, packed);
+    CK(cudaGetLastError());
+    b->launches++;
+    CK(cudaMemcpyAsync(t.data(), packed, sizeof(TF) * t.size(), cudaMemcpyDeviceToHost, s->stream));
   }
-  *n_faces = k;
-  return k <= max_faces ? CGKS_OK : CGKS_EINVAL;
+  CK(cudaStreamSynchronize(s->stream));
+  for (int64_t k = 0; k < m; ++k) {
+    const int64_t f = face[k];
+    const int c0 = hm.fc0[f];
+    const double h = hm.h[c0];
+    // face midpoint: the mean of its two Gauss points (offsets from c0 scaled by 1/h)
+    x[2 * k] = hm.xc[c0] + 0.5 * h * (hm.fxi[0 * nf + f] + hm.fxi[2 * nf + f]);
+    x[2 * k + 1] = hm.xc[hm.n_cells + c0] + 0.5 * h * (hm.fxi[1 * nf + f] + hm.fxi[3 * nf + f]);
+    nrm[2 * k] = hm.fn[f];
+    nrm[2 * k + 1] = hm.fn[nf + f];
+    S[k] = hm.fS[f];
+    for (int d = 0; d < 2; ++d) traction[2 * k + d] = static_cast<double>(t[2 * k + d]);
+  }
+  *n_faces = n;
+  return n <= max_faces ? CGKS_OK : CGKS_EINVAL;
 }
 
 extern "C" {

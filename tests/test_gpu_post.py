@@ -150,3 +150,34 @@ def test_wall_loads_match_oracle_3d(cg, oracles, precision):
         np.testing.assert_allclose(g["S"], r["S"][k], rtol=1e-13)
         err = np.abs(g["traction"] - r["traction"][k]).max() / np.abs(r["traction"]).max()
         assert err < tol, (tag, err)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_wall_loads_leave_the_solve_alone_and_fill_what_fits(cg, precision):
+    """A call between two-stage steps and V-cycles changes nothing that follows
+    (it packs its result in their scratch); arrays too small take the first
+    faces and EINVAL; a tag without faces gives none."""
+    import ctypes as C
+    mesh = MG.cavity(13)
+    spec = dict(gamma=GAM, mu=0.15 / 100, cfl_hi=0.3, time_scheme="S2O4", precision=precision,
+                bcs=[dict(kind="noslip"), dict(kind="noslip", uw=(0.15, 0.0)), dict(kind="slip")])
+    W = np.tile(exact.cons_from_prim(GAM, 1.0, 0.0, 0.0, 1 / GAM), (mesh.n_cells, 1))
+    end = []
+    for look in (False, True):
+        s = cg.Solver(cg.Mesh(mesh), spec)
+        s.set_state(W)
+        for _ in range(3):
+            s.explicit_steps(2)
+            s.pmg_cycle(1)
+            if look:
+                loads = s.wall_loads(1)
+        end.append(s.get_state())
+    assert np.array_equal(end[0][0], end[1][0]) and np.array_equal(end[0][1], end[1][1])
+    m = loads["S"].size
+    assert m == 13 and s.wall_loads(2)["S"].size == 0
+    n = C.c_int64(0)
+    x, nn, S, t = np.zeros((5, 2)), np.zeros((5, 2)), np.zeros(5), np.zeros((5, 2))
+    p = [a.ctypes.data_as(C.c_void_p) for a in (x, nn, S, t)]
+    assert cg.lib().cgks_wall_loads(s._h, 1, 5, C.byref(n), *p) == cg.EINVAL and n.value == m
+    for a, k in ((x, "x"), (nn, "n"), (S, "S"), (t, "traction")):
+        assert np.array_equal(a, loads[k][:5])

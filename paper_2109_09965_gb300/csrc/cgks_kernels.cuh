@@ -292,8 +292,8 @@ template <typename T> __host__ __device__ constexpr int recon_vars() { return is
 // threads of a launch over n cells with a warp per variable of 32 cells
 template <int VARS> __host__ __device__ constexpr int64_t var_items(int64_t n) { return (n + 31) / 32 * 32 * VARS; }
 template <typename T, bool WENO, int NC>
-__device__ __forceinline__ void recon_at(const MeshT<T> &m, const ParamsT<T> &P, const T *__restrict__ W,
-                                         const T *__restrict__ Wx, T *__restrict__ coef, const int i,
+__device__ __forceinline__ void recon_at(const MeshT<T> &m, const ParamsT<T> &P, const T *W,
+                                         const T *Wx, T *__restrict__ coef, const int i,
                                          const int comp) {
   const int n = m.nc, vo = NC == 4 ? 0 : comp;
   T wi[NC], gxi[NC], gyi[NC];
@@ -394,7 +394,7 @@ __global__ void __launch_bounds__(kMaxShapeBlock) k_recon(MeshT<T> m, ParamsT<T>
 
 // value and gradient of the quadratic of cell i at scaled offset (x, y)
 template <typename T>
-__device__ __forceinline__ void recon_point(const MeshT<T> &m, const T *__restrict__ W, const T *__restrict__ coef,
+__device__ __forceinline__ void recon_point(const MeshT<T> &m, const T *W, const T *coef,
                                             int i, T x, T y, T val[4], T gx[4], T gy[4]) {
   const int n = m.nc;
   T ih = m.ih[i];
@@ -411,7 +411,7 @@ __device__ __forceinline__ void recon_point(const MeshT<T> &m, const T *__restri
 // value and gradient at scaled offset (x, y) of a polynomial of cell i with
 // the given coefficients c[q][v]
 template <typename T>
-__device__ __forceinline__ void poly_point(const MeshT<T> &m, const T *__restrict__ W, const T c[kNM][4], int i, T x,
+__device__ __forceinline__ void poly_point(const MeshT<T> &m, const T *W, const T c[kNM][4], int i, T x,
                                            T y, T val[4], T gx[4], T gy[4]) {
   const int n = m.nc;
   T ih = m.ih[i];
@@ -425,7 +425,7 @@ __device__ __forceinline__ void poly_point(const MeshT<T> &m, const T *__restric
 
 // the same from given coefficients, the gradient left in the cell's scaled
 // coordinates (to be multiplied by 1/h)
-__device__ __forceinline__ void side_scaled(const MeshT<double> &m, const double *__restrict__ W,
+__device__ __forceinline__ void side_scaled(const MeshT<double> &m, const double *W,
                                             const double c[kNM][4], int i, double x, double y, double val[4],
                                             double gx[4], double gy[4]) {
   const int n = m.nc;
@@ -438,7 +438,7 @@ __device__ __forceinline__ void side_scaled(const MeshT<double> &m, const double
     gy[v] = c[1][v] + c[3][v] * x + c[4][v] * y2;
   }
 }
-__device__ __forceinline__ void load_coef(int n, const double *__restrict__ coef, int i, double c[kNM][4]) {
+__device__ __forceinline__ void load_coef(int n, const double *coef, int i, double c[kNM][4]) {
 #pragma unroll
   for (int q = 0; q < kNM; ++q)
 #pragma unroll
@@ -547,8 +547,8 @@ __device__ __forceinline__ void char_side(const MeshT<double> &m, const ParamsT<
   for (int q = 0; q < kNM; ++q) f.conservative(cq[q], out[q]);
 }
 template <typename T>
-__device__ void char_side(const MeshT<T> &m, const ParamsT<T> &P, const T *__restrict__ W, const T *__restrict__ Wx,
-                          const T *__restrict__ coef, int i, const T wref[4], T nx, T ny, T out[kNM][4]) {
+__device__ void char_side(const MeshT<T> &m, const ParamsT<T> &P, const T *W, const T *Wx,
+                          const T *coef, int i, const T wref[4], T nx, T ny, T out[kNM][4]) {
   const int n = m.nc;
   const T g = P.gamma;
   const T ir = T(1) / wref[0];
@@ -651,8 +651,8 @@ __device__ __forceinline__ void lo_ghost(const ParamsT<T> &P, int tag, T nx, T n
 // every cell, and the mixed results are to stay what they are).  face_point_at:
 // FP64.
 template <typename T, bool FULL, bool CHAR>
-__device__ __forceinline__ void face_raw_at(const MeshT<T> &m, const ParamsT<T> &P, const T *__restrict__ W,
-                                        const T *__restrict__ Wx, const T *__restrict__ coef, T *__restrict__ out,
+__device__ __forceinline__ void face_raw_at(const MeshT<T> &m, const ParamsT<T> &P, const T *W,
+                                        const T *Wx, const T *coef, T *__restrict__ out,
                                         const Ctl *ctl, const unsigned long long *dt_bits, const int f) {
   const int sid = m.fsid[f];
   if (sid < 0) return;   // free face space of a batch
@@ -774,8 +774,8 @@ __device__ __forceinline__ void pair_sum_store(const double F0[4], const double 
 }
 template <bool FULL, bool CHAR>
 __device__ __forceinline__ void face_point_at(const MeshT<double> &m, const ParamsT<double> &P,
-                                              const double *__restrict__ W, const double *__restrict__ Wx,
-                                              const double *__restrict__ coef, double *__restrict__ out,
+                                              const double *W, const double *Wx,
+                                              const double *coef, double *__restrict__ out,
                                               const Ctl *ctl, const unsigned long long *dt_bits, const int f,
                                               const int k) {
   const int sid = m.fsid[f];
@@ -1111,7 +1111,7 @@ __device__ __forceinline__ void store_delta(float, const float *, const float d[
 // K5a: per-cell start of an implicit step: U = W_p0 (first step) or
 // U += dU (Algorithm 1's update, in FP64), then the base record of U.
 template <typename TF, bool CG>
-__device__ __forceinline__ void lo_cell_at(int n, const ParamsT<TF> &P, int first, const double *__restrict__ Wp0,
+__device__ __forceinline__ void lo_cell_at(int n, const ParamsT<TF> &P, int first, const double *Wp0,
                                            double *U, const TF *delta, TF *base, int i) {
   TF d[4] = { TF(0), TF(0), TF(0), TF(0) };
   if (!first) vload<TF, 4, CG>(delta + static_cast<size_t>(i) * del_run<TF>(), d);
@@ -1290,7 +1290,7 @@ __device__ __forceinline__ RhsGeo rhs_geo(const MeshT<double> &m, int i, int col
 }
 template <typename TF, bool CG>
 __device__ __forceinline__ void lo_rhs_at(const MeshT<double> &m, const ParamsT<double> &P, TF gamma, const RhsGeo &g,
-                                          int first, const TF *base, const TF *Flo, const double *__restrict__ Rp0,
+                                          int first, const TF *base, const TF *Flo, const double *Rp0,
                                           double *Src, TF *Rk, TF *invD, TF *delta, TF *lamS, int i) {
   const int n = m.nc;
   constexpr int N = lo_run<TF>();

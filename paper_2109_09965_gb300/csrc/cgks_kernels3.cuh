@@ -264,8 +264,8 @@ __device__ __forceinline__ void for_recon(const int n, F &&f) {
   });
 }
 template <typename T, bool WENO, int NC>
-__device__ __forceinline__ void recon_at(const MeshT<T> &m, const ParamsT<T> &P, const T *__restrict__ W,
-                                         const T *__restrict__ Wx, T *__restrict__ coef,
+__device__ __forceinline__ void recon_at(const MeshT<T> &m, const ParamsT<T> &P, const T *W,
+                                         const T *Wx, T *__restrict__ coef,
                                          const unsigned char *__restrict__ wenok, const int i, const int comp) {
   const int n = m.nc, vo = NC == NV ? 0 : comp;
   T wi[NC], gi[3][NC];
@@ -370,7 +370,7 @@ __global__ void __launch_bounds__(kMaxShapeBlock)
 
 // value and gradient of cell i's quadratic at scaled offset x; the gradient
 // is left in the cell's scaled coordinates (times 1/h = ih for the physical one)
-__device__ __forceinline__ void recon_scaled(const MeshT<double> &m, const double *__restrict__ W, const double *__restrict__ coef,
+__device__ __forceinline__ void recon_scaled(const MeshT<double> &m, const double *W, const double *coef,
                                              int i, const double x[3], double val[NV], double g[3][NV]) {
   const int n = m.nc;
   const double a = x[0], b = x[1], e = x[2];
@@ -392,7 +392,7 @@ __device__ __forceinline__ void recon_scaled(const MeshT<double> &m, const doubl
 
 // value and gradient of cell i's quadratic at scaled offset x
 template <typename T>
-__device__ __forceinline__ void recon_point(const MeshT<T> &m, const T *__restrict__ W, const T *__restrict__ coef,
+__device__ __forceinline__ void recon_point(const MeshT<T> &m, const T *W, const T *coef,
                                             int i, const T x[3], T val[NV], T g[3][NV]) {
   const int n = m.nc;
   const T ih = m.ih[i];
@@ -419,8 +419,8 @@ __device__ __forceinline__ void recon_point(const MeshT<T> &m, const T *__restri
 // Two forms, as in 2-D: face_raw_at (raw moments in the face frame: the FP32
 // of the mixed path) and face_points_at (FP64).
 template <typename T, bool FULL>
-__device__ __forceinline__ void face_raw_at(const MeshT<T> &m, const ParamsT<T> &P, const T *__restrict__ W,
-                                        const T *__restrict__ coef, T *__restrict__ out, const Ctl *ctl,
+__device__ __forceinline__ void face_raw_at(const MeshT<T> &m, const ParamsT<T> &P, const T *W,
+                                        const T *coef, T *__restrict__ out, const Ctl *ctl,
                                         const unsigned long long *dt_bits, const int f) {
   const int nf = m.nf;
   T dt = T(0);
@@ -521,7 +521,7 @@ __device__ __forceinline__ void face_raw_at(const MeshT<T> &m, const ParamsT<T> 
 // face's 3 or 4 Gauss points.
 template <bool FULL, int LANES>
 __device__ __forceinline__ void face_points_at(const MeshT<double> &m, const ParamsT<double> &P,
-                                               const double *__restrict__ W, const double *__restrict__ coef,
+                                               const double *W, const double *coef,
                                                double *__restrict__ out, const Ctl *ctl,
                                                const unsigned long long *dt_bits, const int f, const int lane) {
   using T = double;
@@ -926,7 +926,7 @@ __device__ __forceinline__ void lo_ghost(const ParamsT<T> &P, int tag, const D3:
 __device__ __forceinline__ float third(float x) { return x / 3.0f; }
 __device__ __forceinline__ double third(double x) { return x * (1.0 / 3.0); }
 template <typename T>
-__device__ __forceinline__ void lo_face_at(const MeshT<T> &m, const ParamsT<T> &P, const T *__restrict__ base,
+__device__ __forceinline__ void lo_face_at(const MeshT<T> &m, const ParamsT<T> &P, const T *base,
                                            T *__restrict__ Flo, const int f) {
   const int c0 = m.fc0[f], c1 = m.fc1[f];
   // FP32 and boundary faces take the whole frame, an inner FP64 face its normal

@@ -471,13 +471,13 @@ FACES3 = {2: [(0, 2, 1), (0, 1, 3), (1, 2, 3), (2, 0, 3)],
           3: [(0, 2, 1), (3, 4, 5), (0, 1, 4, 3), (1, 2, 5, 4), (2, 0, 3, 5)],
           4: [(0, 3, 2, 1), (0, 1, 4), (1, 2, 4), (2, 3, 4), (3, 0, 4)],
           5: [(0, 3, 2, 1), (4, 5, 6, 7), (0, 1, 5, 4), (1, 2, 6, 5), (2, 3, 7, 6), (3, 0, 4, 7)]}
-# FP64 operations per Gauss point of the 3-D smooth flux: 600 instructions as
-# counted on the 128,000-cell sphere (two quadratic evaluations, the flux from
-# moments about the mean velocity, sums), a fused multiply-add being two.
-FLOPS_PER_GP3 = 1200
-# the relaxation's increment form: 22 instructions per interior neighbour of a
-# relaxed cell, 33 per cell
-SWEEP3_FLOPS_PER_NEIGHBOUR, SWEEP3_FLOPS_PER_CELL = 44, 66
+# FP64 operations of the 3-D kernels (additions, multiplications, and two for a
+# fused multiply-add; executed ones counted by ncu on the 128,000-cell sphere).
+# Smooth flux, per Gauss point: two quadratic evaluations, the flux from moments
+# about the mean velocity, sums.  Relaxation in increment form: per interior
+# neighbour, per cell, and per cell whose state advances with it.
+FLOPS_PER_GP3 = 984
+SWEEP3_FLOPS_PER_NEIGHBOUR, SWEEP3_FLOPS_PER_CELL, SWEEP3_FLOPS_ADVANCE = 40, 43, 38
 
 
 def topology3(mesh, gm):
@@ -522,35 +522,42 @@ def work_model3(mesh, gm, spec, precision, _cache={}):
     up = np.zeros(mesh.n_cells, bool)
     up[a[colour[b] > colour[a]]] = True
     up[b[colour[a] > colour[b]]] = True
+    up[colour == 0] = True
     seq = []
     for _ in range(spec["n_sweeps"]):
         seq += [(c, False) for c in range(1, C)]
-        seq += [(c, True) for c in range(C - 2, -1, -1) if c == 0 or (up & (colour == c)).any()]
+        seq += [(c, True) for c in range(C - 2, -1, -1) if (up & (colour == c)).any()]
     ni = spec["n_implicit"]
     w = 8 if precision == "fp64" else 4
     by_c = {}
     for c, down in sorted(set(seq)):
-        incol = (colour == c) & (up | (not down) | (c == 0))
+        incol = (colour == c) & (up | (not down))
         slots = int(nb[incol].sum())
         # distinct neighbours of the colour's cells
         na = b[incol[a]]
         nbb = a[incol[b]]
         uniq = np.unique(np.concatenate([na, nbb])).size
         flops = SWEEP3_FLOPS_PER_NEIGHBOUR * slots + SWEEP3_FLOPS_PER_CELL * int(incol.sum())
-        own = int(incol.sum()) * 11 * w
-        per_slot = slots * (4 + 5 * w)              # neighbour, normal, area, lambda
-        nbr = uniq * (15 * w if precision == "fp64" else 16 * w)   # base and increment records
+        # right-hand side, 1/D, own base (FP64), increment record out; per slot the
+        # neighbour, normal (FP32: and area), lambda; the base and increment records
+        own = int(incol.sum()) * (20 if precision == "fp64" else 14) * w
+        per_slot = slots * (4 + (4 if precision == "fp64" else 5) * w)
+        nbr = uniq * (15 if precision == "fp64" else 16) * w
         by_c[c, down] = (flops, own + per_slot + nbr)
     n, F = mesh.n_cells, gm.n_faces
     gps = 3 * T + 4 * Q
-    return {"sweep_flops": ni * sum(by_c[c][0] for c in seq),
+    # every cell's last relaxation of an implicit step advances U (FP64) and
+    # writes the next step's base record
+    adv = n if seq and C > 1 else 0
+    adv_bytes = adv * (2 * 5 * 8 + 16 * w)
+    return {"sweep_flops": ni * (sum(by_c[c][0] for c in seq) + SWEEP3_FLOPS_ADVANCE * adv),
             "face_flops": 2 * gps * FLOPS_PER_GP3,     # two evaluations per V-cycle
-            "bytes": {"k_sweep": ni * sum(by_c[c][1] for c in seq),
+            "bytes": {"k_sweep": ni * (sum(by_c[c][1] for c in seq) + adv_bytes),
                       "k_recon": 2 * n * ((20 + 243 + 45) * w + 48),
                       "k_face": 2 * (n * 56 * w + F * (47 * w + 12)),
                       "k_lo_face": ni * (n * 15 * w + F * (6 * w + 9 * w + 12)),
-                      "k_lo_rhs": ni * (F * 7 * w + n * (24 + 5 * 8 + 16 * w + 6 * w)),
-                      "k_lo_cell": n * (5 * 8 + 16 * w),
+                      "k_lo_rhs": ni * (F * 6 * w + n * (24 + 6 * 8 + 5 * 8 + (22 if w == 8 else 20) * w)),
+                      "k_lo_cell": (1 if adv else ni + 1) * n * (2 * 5 * 8 + 16 * w),
                       "k_prolong": n * 20 * 8},
             "gauss_points": gps, "colours": C, "sweep_launches": ni * len(seq)}
 
@@ -786,18 +793,17 @@ def topology(mesh, gm):
     return nb, nbrs, np.asarray(colour), n_int, len(edges)
 
 
-# FP64 operations as the kernels issue them, a fused multiply-add counted as
-# two.  Relaxation in increment form: 17 instructions per interior neighbour,
-# 21 per cell.
-SWEEP_FLOPS_PER_NEIGHBOUR = 34
-SWEEP_FLOPS_PER_CELL = 42
-# other low-order phases (instructions counted on the 57,344-cell cylinder, x 2):
-# KFVS flux of a face with its spectral radii 96, right-hand side of a cell 48,
-# base record of a cell 24
-LO_FACE_FLOPS, LO_RHS_FLOPS, LO_CELL_FLOPS = 192, 96, 48
-# per Gauss point of the 2-D smooth flux (2 per face): 338 instructions (two
-# quadratic evaluations, the flux from moments about the mean velocity, sums)
-FLOPS_PER_GP2 = 676
+# FP64 operations of the 2-D kernels (additions, multiplications, and two for a
+# fused multiply-add; executed ones counted by ncu on the 57,344-cell cylinder).
+# Relaxation in increment form: per interior neighbour, per cell, and per cell
+# whose state advances with it.
+SWEEP_FLOPS_PER_NEIGHBOUR, SWEEP_FLOPS_PER_CELL, SWEEP_FLOPS_ADVANCE = 30, 32, 35
+# other low-order phases: KFVS flux of a face with its spectral radii,
+# right-hand side of a cell, base record of a cell
+LO_FACE_FLOPS, LO_RHS_FLOPS, LO_CELL_FLOPS = 144, 69, 32
+# per Gauss point of the 2-D smooth flux (2 per face): two quadratic
+# evaluations, the flux from moments about the mean velocity, sums
+FLOPS_PER_GP2 = 539
 FP64_PEAK_TFLOPS = 1.25    # GB300: 152 SMs x 2.07 GHz x 2 FP64 FMA/clk x 2 flops (recipe table)
 
 
@@ -823,13 +829,18 @@ def work_model(mesh, gm, spec, precision):
         slots = int(nb[cells].sum())
         uniq = len({j for i in cells for j in nbrs[i]})
         flops = SWEEP_FLOPS_PER_NEIGHBOUR * slots + SWEEP_FLOPS_PER_CELL * len(cells)
-        own = len(cells) * 9 * w
-        per_slot = slots * (4 + 4 * w)              # neighbour, normal, area, lambda
-        nbr = uniq * 12 * w                         # base and increment records
+        # right-hand side, 1/D, own base (FP64), increment record out; per slot the
+        # neighbour, normal (FP32: and area), lambda; the base and increment records
+        own = len(cells) * (17 if precision == "fp64" else 9) * w
+        per_slot = slots * (4 + (3 if precision == "fp64" else 4) * w)
+        nbr = uniq * 12 * w
         by_c[c] = (flops, own + per_slot + nbr)
-    sweep_flops = ni * sum(by_c[c][0] for c in seq)
-    sweep_bytes = ni * sum(by_c[c][1] for c in seq)
     d = 8
+    # every cell's last relaxation of an implicit step advances U (FP64) and
+    # writes the next step's base record
+    adv = n if seq and C > 1 else 0
+    sweep_flops = ni * (sum(by_c[c][0] for c in seq) + SWEEP_FLOPS_ADVANCE * adv)
+    sweep_bytes = ni * (sum(by_c[c][1] for c in seq) + adv * (2 * 4 * d + 12 * w))
     # high-order evaluations per cycle: the step (1 in S1O2, 2 in S2O4) and R_p0
     ev = 2 if spec.get("time_scheme", "S1O2") == "S1O2" else 3
     bytes_ = {
@@ -842,26 +853,28 @@ def work_model(mesh, gm, spec, precision):
         # geometry, W in, W/Wx out; ev launches per cycle
         "k_update": F * (16 * (ev - 1) + 4) * w + ev * (F * 3 * d + n * (16 + 2 * 4 * d + 2 * 8 * d)),
         "k_lo_face": ni * (n * 13 * w + F * (5 * w + 3 * w + 12)),
-        "k_lo_rhs": ni * (F * 6 * w + n * (16 + 4 * d + 13 * w + 4 * w)),
-        "k_lo_cell": n * (4 * d + 12 * w),
+        "k_lo_rhs": ni * (F * 5 * w + n * (16 + 4 * d + 4 * d + (17 if w == 8 else 13) * w)),
+        "k_lo_cell": (1 if adv else ni + 1) * n * (2 * 4 * d + 12 * w),   # W_p0 or U in, U and base record out
         "k_prolong": n * (4 * 3 + 4) * d,
     }
-    lo_flops = sweep_flops + ni * (LO_FACE_FLOPS * F + LO_RHS_FLOPS * n) + ni * LO_CELL_FLOPS * n
+    lo_flops = sweep_flops + ni * (LO_FACE_FLOPS * F + LO_RHS_FLOPS * n) + LO_CELL_FLOPS * n
     bytes_["k_lo_solve"] = sum(bytes_[k] for k in ("k_sweep", "k_lo_face", "k_lo_rhs", "k_lo_cell"))
     return {"sweep_flops": sweep_flops, "lo_flops": lo_flops, "bytes": bytes_, "colours": C,
             "sweep_launches": ni * len(seq), "face_flops": ev * F * 2 * FLOPS_PER_GP2}
 
 
 # DRAM bytes (read + write) per launch of a workload's dominant kernel from
-# one ncu capture of that workload and kernel (--clock-control none, a few
-# launches, averaged over the colours of a V-cycle for k_sweep).  An entry
-# is removed when its kernel changes; a workload with no entry reports
-# traffic null.
+# one ncu capture of that workload and kernel (--clock-control none, caches
+# flushed before each launch, averaged over the launches of a V-cycle;
+# profiles/kernel_captures.md).  An entry is removed when its kernel changes; a
+# workload with no entry reports traffic null.
 NCU_TRAFFIC = {
-    # 57,344-cell cylinder, per V-cycle 6 x (6 big-colour + 2 small-colour)
-    # launches: (6 x 9.62 MB + 2 x 0.88 MB) / 8 and (6 x 3.78 MB + 2 x 0.78 MB) / 8
-    ("cylinder57k", "k_sweep", "fp64"): 7.43e6,
-    ("cylinder57k", "k_sweep", "mixed"): 3.03e6,
+    # 57,344-cell cylinder, 48 launches of a V-cycle: 24 of a large colour 11.15 MB
+    # (mixed 4.36), 12 that also advance the state 12.07 (5.28), 12 of the small
+    # colour 0.29 (0.22)
+    ("cylinder57k", "k_sweep", "fp64"): 8.67e6,
+    ("cylinder57k", "k_sweep", "mixed"): 3.55e6,
+    ("cylinder57k", "k_face", "fp64"): 21.95e6,
 }
 
 

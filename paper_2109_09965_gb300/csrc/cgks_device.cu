@@ -88,6 +88,7 @@ struct Batch {
   bool mixed = false;
   int n_colours = 0;
   std::vector<int> sweep_seq;        // colour order after the first pass
+  std::vector<int> sweep_last;       // [n_colours] position of a colour's last visit in it
   std::vector<int> list_off;         // [n_colours + 1] offsets into the sweep cell list
   std::vector<Ranges> ranges[kNShape];  // per sweep shape, per colour: per-solve cell ranges (n = 0: the list)
   std::vector<int> lanes;               // [n_colours] lanes per cell of the colour's sweeps
@@ -353,9 +354,6 @@ void enqueue_lo_solve(Batch *b) {
     launch(b, KI_LOCELL, k_lo_cell<TF>, gc, blk, static_cast<int>(b->Ncap), fparams<TF>(b), first,
            (const double *)b->Wn, b->U, (const TF *)B.delta, base);
   };
-  // the last visit of each colour in the sequence
-  std::vector<int> last(b->n_colours, -1);
-  for (size_t q = 0; q < b->sweep_seq.size(); ++q) last[b->sweep_seq[q]] = static_cast<int>(q);
   for (int k = 0; k < b->sh.n_implicit; ++k) {
     if (k == 0 || !adv) cells(k == 0 ? 1 : 0);
     const int fsh = b->tune.shape(TK_LOFACE);
@@ -399,7 +397,7 @@ void enqueue_lo_solve(Batch *b) {
                  use_list ? (const int *)b->list + b->list_off[c] : (const int *)nullptr, cnt, (const TF *)base,
                  (const TF *)B.Rk, (const TF *)B.invD, (const TF *)B.lamS, B.delta, b->U, next);
         };
-        const bool end = adv && last[c] == static_cast<int>(q);
+        const bool end = adv && b->sweep_last[c] == static_cast<int>(q);
         if constexpr (!is_f32<TF>()) {
           if (b->lanes[c] == 1) {
             if (end) go(k_sweep<TF, true, 1>);
@@ -882,6 +880,8 @@ int finalize_batch(Batch *b) {
   }
   if (!seq.empty()) seq.erase(seq.begin());
   b->sweep_seq = seq;
+  b->sweep_last.assign(C, -1);
+  for (size_t q = 0; q < seq.size(); ++q) b->sweep_last[seq[q]] = static_cast<int>(q);
   for (auto &rs : b->ranges) rs.assign(C, Ranges{});
   b->list_off.assign(C + 1, 0);
   b->lanes.assign(C, 4);

@@ -94,9 +94,11 @@ template <> __device__ __forceinline__ float d_rsqrt<float>(float x) { return rs
 
 // Reciprocal and reciprocal square root.  GB300 issues two FP64 lanes per
 // clock per SM, so the number of FP64 instructions is what an FP64 kernel
-// costs: the FP64 forms take the hardware's estimate (relative error 2^-22)
-// and one third-order step of Newton's family (Householder's iteration),
-// whose error is of the order of the cube, 2^-66.
+// costs: the FP64 forms take the hardware's estimate (20 mantissa bits; e below is
+// at most 2^-19.9 for 1/x and 2^-19.0 for 1/sqrt(x), measured) and one third-order
+// step of Newton's family (Householder's iteration), which leaves e^3 = 2^-59.8 and
+// 5/16 e^3 = 2^-58.7: with the roundings, relative errors below 1.1 and 2 units
+// (2^-53), where the IEEE quotient is correctly rounded.
 //   1/x:        e = 1 - x r,    r <- r + r (e + e^2)             3 FP64
 //   1/sqrt(x):  e = 1 - x r^2,  r <- r + r e (1/2 + 3/8 e)       5 FP64
 // against 8-9 for the IEEE quotient and the library's rsqrt.  Normal
@@ -132,9 +134,13 @@ __device__ __forceinline__ void sqrt_lambda(double i2l, double &sl, double &isp)
 // u > 0 (sgn = +1) or u < 0 (-1), z = sl U.  In FP64, for |z| < 1 (normal Mach
 // number below 1.19), erf(z) / (2 z) and exp(-z^2) come from polynomials in
 // t = z^2, the interpolants at the Chebyshev nodes of [0, 1] (degrees 11 and
-// 12, relative errors 8e-18): 24 FP64 instructions in place of about 90 of the
-// library pair; beyond, and for NaN, the library's functions.  FP32 keeps the
-// library's: its arithmetic is not what the mixed path waits for.
+// 12; with the coefficients rounded to double relative errors 4e-17 and 1e-16,
+// before the roundings of the evaluation): 24 FP64 instructions in place of about
+// 90 of the library pair; beyond, and for NaN, the library's functions.  <1> is
+// then 0.5 plus a product, exact to a few units of 2^-53 absolutely; where it is
+// small (0.08 at |z| = 1) that is several units relative to itself, but the other
+// side's share of the same sum is near 1.  FP32 keeps the library's: its
+// arithmetic is not what the mixed path waits for.
 __device__ __forceinline__ void half01(double U, double sl, double isp, int sgn, double &m0, double &m1) {
   const double z = sl * U, t = z * z;
   double ex;

@@ -55,7 +55,7 @@ struct SweepPass {
 struct Solver3 {
   cgks_params P{};
   int64_t N = 0, F = 0;
-  bool mixed = false;
+  bool mixed = false, quads = false;   // quads: quadrilateral faces
   int n_colours = 0;
   std::vector<int32_t> colour_start, n_higher;
   std::vector<SweepPass> passes;
@@ -159,7 +159,7 @@ void hi_eval(Solver3 *s, const TF *W, const TF *Wx, TF *Fout) {
     if constexpr (is_f32<TF>()) {
       if (full) go(1, k_face<TF, true>);
       else go(1, k_face<TF, false>);
-    } else if (face_lanes(s->F) == 4) {
+    } else if (face_lanes(s->F, s->quads) == 4) {
       if (full) go(4, k_face_points<true, 4>);
       else go(4, k_face_points<false, 4>);
     } else {
@@ -446,6 +446,7 @@ int s3_create(const HostMesh3 &m, const cgks_params *p, cudaStream_t stream, Tim
   s->timer = timer;
   s->tune.on = p->autotune != 0;
   if (s->N * kNCol3 * kNM3 > INT32_MAX || s->F * 24 > INT32_MAX) return CGKS_EINVAL;
+  s->quads = std::any_of(m.fng.begin(), m.fng.end(), [](int32_t n) { return n == 4; });
   s->n_higher = m.n_higher;
   // The passes after the first (colour 0, done with the right-hand side) of
   // n_sweeps x (colours ascending, colours descending).  A relaxation whose

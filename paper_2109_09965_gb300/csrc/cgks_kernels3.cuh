@@ -638,14 +638,21 @@ __device__ __forceinline__ void face_points_at(const MeshT<double> &m, const Par
     }
   }
 }
-// Threads per face: one on a large mesh wastes no lane on the missing fourth
-// point of a triangle; four on a small one spread its few faces over the FP64
-// units (608 sub-cores).  28,850 faces (hexahedra): 174 us with 4, 191 with 1;
-// 282,880 (mostly triangles): 1281 us with 4, 1162 with 1 (before, raw moments
-// in one thread: 358 and 2809 us).  With the far field hoisted and the wall
-// mirrors linear the better ones take 145 and 1074 us.
-constexpr int64_t kFaceLanes4 = 100000;
-inline int face_lanes(int64_t n_faces) { return n_faces < kFaceLanes4 ? 4 : 1; }
+// Threads per face, FP64.  A launch takes as long as the warps of one sub-core
+// (608 of them) issue one after another: per 32 faces one warp of 3 or 4 points
+// with one thread, 4 warps of a point with four.  Four lose nothing where there
+// are quadrilaterals (a warp with one among its faces takes 4 points either way)
+// and are the finer quantum, one is a little shorter on large meshes; on
+// triangles alone the fourth lane idles, and one thread is shorter from two
+// warps of the four-lane form a sub-core on (9,728 faces).  us per launch, smooth
+// flux, one / four: hexahedra 13,056 faces 86 / 76, 61,236 319 / 287, 92,256
+// 409 / 420, 196,800 851 / 856; prisms 41,600 248 / 199, 112,896 483 / 507;
+// sphere shells (prisms and tetrahedra) 51,520 261 / 238, 70,720 306 / 321, 98,560
+// 477 / 446, 142,080 590 / 630; tetrahedra 9,234 68 / 53, 12,600 69 / 76, 50,688
+// 195 / 242, 113,778 372 / 516.  (Raw moments in one thread took 358 us on 28,850
+// faces of hexahedra and 2809 us on 282,880 of a shell; now 145 and 1074.)
+constexpr int64_t kFaceLanes4 = 100000, kFaceLanes4Tri = 9728;
+inline int face_lanes(int64_t n_faces, bool quads) { return n_faces < (quads ? kFaceLanes4 : kFaceLanes4Tri) ? 4 : 1; }
 // FP32: one thread per face.  Bound by latency at two warps a scheduler (255
 // registers); the smooth flux is shorter with 128 and four warps, in spite of
 // some spills: 512,000 cells 411 -> 377 us a launch (112: 390, 144: 427); the

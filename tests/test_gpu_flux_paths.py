@@ -82,6 +82,19 @@ def test_one_thread_per_face_matches_the_oracle(flux, precision):
     compare(mesh, spec, state(mesh, 0.2, 0.3), precision, 0)
 
 
+@pytest.mark.parametrize("flux", ["smooth", "full"])
+@pytest.mark.parametrize("n, faces", [(9, 9234), (10, 12600)])
+def test_triangles_on_both_sides_of_one_thread_per_face(n, faces, flux):
+    """Tetrahedra alone: four threads share a face up to 9,728 faces, one takes
+    it beyond."""
+    mesh = MG.box3(n, n, n, jitter=0.1, seed=3, cells="tet", tags=(0, 0, 0, 0, 1, 1))
+    spec = dict(gamma=GAM, mu=0.002, cfl_hi=0.3, flux_hi=flux,
+                bcs=[dict(kind="farfield", rho=1.0, u=(0.3, 0.0, 0.0), p=1 / GAM), dict(kind="slip")])
+    from paper_2109_09965_gb300 import cgks
+    assert cgks.Mesh(mesh).n_faces == faces
+    compare(mesh, spec, state(mesh, 0.2, 0.3), "fp64", 0)
+
+
 @pytest.mark.parametrize("precision", ["fp64", "mixed"])
 @pytest.mark.parametrize("scheme", [dict(n_sweeps=0), dict(n_sweeps=1), dict(n_implicit=1), dict(n_implicit=3, n_sweeps=3)])
 def test_low_level_passes_that_advance_the_state(scheme, precision):

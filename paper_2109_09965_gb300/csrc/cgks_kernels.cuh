@@ -1427,10 +1427,12 @@ __global__ void __launch_bounds__(kMaxShapeBlock) k_lo_flux_rhs(MeshT<TF> fm, Pa
   pdl_exit();
 }
 // Cells up to which the merged launch is the shorter one: in FP64 while its
-// four lanes per cell give a sub-core (608) one or two warps, 4,864 to 9,728
-// cells; in FP32 until evaluating every face twice costs more than a launch.
-// us per V-cycle, split / merged: FP64 4,050 cells 314 / 296, 8,192 347 / 355;
-// FP32 25,088 cells 210 / 204, 34,848 215 / 222.
+// four lanes per cell give a sub-core (608) one or two warps (4,864 to 9,728
+// cells), in FP32 until evaluating every face twice costs more than a launch;
+// the lines lie in the ranges where both sides take the same.  us per V-cycle,
+// split / merged (cavities): FP64 4,608 cells 310 / 298, 5,832 315 / 316, 6,498
+// 319 / 319, 7,200 326 / 329, 8,192 333 / 346; mixed 20,000 199 / 192, 26,450
+// 201 / 198, 29,768 213 / 211, 33,800 214 / 216, 41,472 230 / 240.
 template <typename T> __host__ __device__ constexpr int64_t merge_cells() { return is_f32<T>() ? 30000 : 6656; }
 
 // The cells of one colour form one contiguous range per solve.  A sweep

@@ -1629,8 +1629,8 @@ int cgks_launches_per_call(const cgks_solver *s, int cycle) {
 int cgks_tune_shape(int32_t shape, int32_t *block, int32_t *per_thread, int32_t *min_blocks) {
   if (shape < 0 || shape >= kNShape) return CGKS_EINVAL;
   if (block) *block = shape_bs(shape);
-  if (per_thread) *per_thread = shape_ipt(shape);
-  if (min_blocks) *min_blocks = shape_minb(shape);
+  if (per_thread) *per_thread = 1;
+  if (min_blocks) *min_blocks = 1;   // no register cap
   return CGKS_OK;
 }
 

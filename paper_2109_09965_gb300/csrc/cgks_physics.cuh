@@ -19,19 +19,12 @@ namespace dev {
 
 constexpr int NV = 4;
 
+// the library's, in the FP32 forms (the FP64 ones have their own arithmetic below)
 __device__ __forceinline__ float d_erfc(float x) { return erfcf(x); }
-template <typename T> __device__ __forceinline__ T d_exp(T x);
-template <> __device__ __forceinline__ double d_exp<double>(double x) { return exp(x); }
-template <> __device__ __forceinline__ float d_exp<float>(float x) { return expf(x); }
-template <typename T> __device__ __forceinline__ T d_expm1(T x);
-template <> __device__ __forceinline__ double d_expm1<double>(double x) { return expm1(x); }
-template <> __device__ __forceinline__ float d_expm1<float>(float x) { return expm1f(x); }
-template <typename T> __device__ __forceinline__ T d_sqrt(T x);
-template <> __device__ __forceinline__ double d_sqrt<double>(double x) { return sqrt(x); }
-template <> __device__ __forceinline__ float d_sqrt<float>(float x) { return sqrtf(x); }
-template <typename T> __device__ __forceinline__ T d_pi();
-template <> __device__ __forceinline__ double d_pi<double>() { return 3.141592653589793238462643; }
-template <> __device__ __forceinline__ float d_pi<float>() { return 3.14159265358979f; }
+__device__ __forceinline__ float d_exp(float x) { return expf(x); }
+__device__ __forceinline__ float d_expm1(float x) { return expm1f(x); }
+__device__ __forceinline__ float d_sqrt(float x) { return sqrtf(x); }
+__device__ __forceinline__ float d_rsqrt(float x) { return rsqrtf(x); }
 
 // a b and a b + c d with the roundings spelled out in FP64, so that code
 // compiled into two kernels gives the same bits in both; FP32 as the compiler
@@ -87,10 +80,6 @@ __device__ __forceinline__ Maxw<T> maxw(const T W[NV], T c2K) {
   g.lam = T(0.5) / g.i2l;
   return g;
 }
-
-template <typename T> __device__ __forceinline__ T d_rsqrt(T x);
-template <> __device__ __forceinline__ double d_rsqrt<double>(double x) { return rsqrt(x); }
-template <> __device__ __forceinline__ float d_rsqrt<float>(float x) { return rsqrtf(x); }
 
 // Reciprocal and reciprocal square root.  GB300 issues two FP64 lanes per
 // clock per SM, so the number of FP64 instructions is what an FP64 kernel

@@ -21,9 +21,6 @@ constexpr int kMaxShapeBlock = 256;   // the largest block of any shape
 __host__ __device__ constexpr int shape_bs(int s) {
   return s == 1 ? 64 : s == 2 ? 256 : s == 3 ? 96 : s == 4 ? 192 : 128;
 }
-__host__ __device__ constexpr int shape_ipt(int) { return 1; }
-// minimum resident blocks per SM; 1 = no register cap
-__host__ __device__ constexpr int shape_minb(int) { return 1; }
 
 // tunable kernels
 enum TuneKernel { TK_RECON = 0, TK_FACE, TK_LOFACE, TK_SWEEP, TK_COUNT };

@@ -212,7 +212,7 @@ __device__ __forceinline__ void dirichlet_ghost(const ParamsT<T> &P, int tag, T 
   const T un = D::dot2(P.bc_u[2 * tag], nx, P.bc_u[2 * tag + 1], ny);
   const T ut = D::dot2(-P.bc_u[2 * tag], ny, P.bc_u[2 * tag + 1], nx);
   wg[0] = r; wg[1] = r * un; wg[2] = r * ut;
-  wg[3] = p / (P.gamma - T(1)) + T(0.5) * r * D::dot2(un, un, ut, ut);
+  wg[3] = D::mad(T(0.5) * r, D::dot2(un, un, ut, ut), p / (P.gamma - T(1)));
 }
 
 __host__ __device__ __forceinline__ bool is_wall_kind(int k) { return k == CGKS_BC_SLIP || k == CGKS_BC_NOSLIP; }
@@ -1194,8 +1194,8 @@ __device__ __forceinline__ void lo_flux_at(const MeshT<T> &m, const ParamsT<T> &
   if (mu != T(0)) {
     ira = D::d_rcp(a.rho);
     irb = D::d_rcp(b.rho);
-    la += T(2) * (mu * ira) * g.S * g.iva;
-    lb += T(2) * (mu * irb) * g.S * g.ivb;
+    la = D::mad(T(2) * (mu * ira) * g.S, g.iva, la);
+    lb = D::mad(T(2) * (mu * irb) * g.S, g.ivb, lb);
   }
   const T lmax = la > lb ? la : lb;
   T F[4];
@@ -1239,7 +1239,7 @@ __device__ __forceinline__ void lo_flux_at(const MeshT<T> &m, const ParamsT<T> &
     const T md = mu * m.fidl[f];
     const T dux = b.u - a.u, duy = b.v - a.v;
     const T dn = third(D::dot2(dux, nx, duy, ny));
-    const T tx = D::prod(md, dux + dn * nx), ty = D::prod(md, duy + dn * ny);
+    const T tx = D::prod(md, D::mad(dn, nx, dux)), ty = D::prod(md, D::mad(dn, ny, duy));
     T qn;   // gamma / (gamma - 1) = N / 2 + 1
     if constexpr (is_f32<T>()) qn = -md * P.gamma / (P.gamma - T(1)) * (b.p * irb - a.p * ira);
     else qn = D::prod(-md * (P.kc.hN + T(1)), D::dot2(b.p, irb, -a.p, ira));
@@ -1305,8 +1305,8 @@ __device__ __forceinline__ void lo_rhs_at(const MeshT<double> &m, const ParamsT<
     vload<TF, N, CG>(Flo + static_cast<size_t>(fs >= 0 ? fs : ~fs) * N, fl);
     widen<5>(fl, x);
 #pragma unroll
-    for (int v = 0; v < 4; ++v) R[v] += Sg * x[v];
-    sum += x[4] * S;
+    for (int v = 0; v < 4; ++v) R[v] = D::mad(Sg, x[v], R[v]);
+    sum = D::mad(x[4], S, sum);
     if constexpr (is_f32<TF>()) lamS[s * n + i] = fl[4];
     else lamS[s * n + i] = fl[4] * (0.5 * S);
   }
@@ -1391,8 +1391,8 @@ __global__ void __launch_bounds__(kMaxShapeBlock) k_lo_flux_rhs(MeshT<TF> fm, Pa
     const int fq = __shfl_sync(0xffffffffu, fs, q, kMaxFace);
     const double xv = s == 0 ? y[0] : s == 1 ? y[1] : s == 2 ? y[2] : y[3];
     if (fq != kNoFace) {
-      R += (fq >= 0 ? -Sq : Sq) * xv;
-      sum += y[4] * Sq;
+      R = D::mad(fq >= 0 ? -Sq : Sq, xv, R);
+      sum = D::mad(y[4], Sq, sum);
     }
   }
   const double id = sum > 0.0 ? D::d_rcp(sum * (P.icfl_lo + 0.5)) : 0.0;

@@ -27,12 +27,17 @@ __device__ __forceinline__ float d_sqrt(float x) { return sqrtf(x); }
 __device__ __forceinline__ float d_rsqrt(float x) { return rsqrtf(x); }
 
 // a b and a b + c d with the roundings spelled out in FP64, so that code
-// compiled into two kernels gives the same bits in both; FP32 as the compiler
-// fuses them.
+// compiled into two kernels gives the same bits in both.  In FP32 they are what
+// the compiler makes of them (the mixed path's results keep those roundings):
+// that it fuses the low-level flux alike in the two kernels that hold it is
+// checked, not ensured (test_merged_and_separate_right_hand_sides_round_alike).
 __device__ __forceinline__ float prod(float a, float b) { return a * b; }
 __device__ __forceinline__ double prod(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ float dot2(float a, float b, float c, float d) { return a * b + c * d; }
 __device__ __forceinline__ double dot2(double a, double b, double c, double d) { return fma(c, d, __dmul_rn(a, b)); }
+// a b + c, one rounding
+__device__ __forceinline__ float mad(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double mad(double a, double b, double c) { return __fma_rn(a, b, c); }
 
 // Rotate a conservative vector between global and face frames.
 template <typename T>
@@ -722,7 +727,7 @@ __device__ __forceinline__ Prim<T> prim_of(const T W[NV], T gamma, const KC<T> &
   q.rho = W[0];
   q.u = prod(W[1], ir);
   q.v = prod(W[2], ir);
-  const T eps = W[3] - T(0.5) * q.rho * dot2(q.u, q.u, q.v, q.v);
+  const T eps = mad(T(-0.5) * q.rho, dot2(q.u, q.u, q.v, q.v), W[3]);
   q.p = prod(gamma - T(1), eps);
   q.i2l = kc.c2K * eps * ir;
   sqrt_lambda(q.i2l, q.sl, q.isp);
@@ -922,7 +927,7 @@ __device__ __forceinline__ double sqrt_fast(double x) { return x > 1e-290 && x <
 __device__ __forceinline__ FarState far_state(const KC<double> &kc, double ri, double pi, double ui, double ci,
                                               double re, double pe, double ue, double ce) {
   const double N = 2.0 * kc.hN;
-  const double Rp = ui + N * ci, Rm = ue - N * ce;
+  const double Rp = mad(N, ci, ui), Rm = mad(-N, ce, ue);
   FarState f;
   f.un = 0.5 * (Rp + Rm);
   f.out = f.un >= 0.0;
@@ -947,7 +952,7 @@ __device__ __forceinline__ void ghost_farfield(const KC<double> &kc, double gamm
                                                double pe, const double W[NV], double Wg[NV]) {
   const double ri = W[0], ir = d_rcp(ri);
   const double uni = prod(W[1], ir), uti = prod(W[2], ir);
-  const double pi = (gamma - 1.0) * (W[3] - 0.5 * ri * dot2(uni, uni, uti, uti));
+  const double pi = (gamma - 1.0) * mad(-0.5 * ri, dot2(uni, uni, uti, uti), W[3]);
   const double ci = d_sqrt3(gamma * pi * ir), ce = d_sqrt3(gamma * pe * d_rcp(re));
   double rb, unb, utb, pb;
   if (uni <= -ci) {

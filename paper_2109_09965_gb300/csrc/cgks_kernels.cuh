@@ -1113,14 +1113,18 @@ __device__ __forceinline__ void store_delta(float, const float *, const float d[
 template <typename TF, bool CG>
 __device__ __forceinline__ void lo_cell_at(int n, const ParamsT<TF> &P, int first, const double *Wp0,
                                            double *U, const TF *delta, TF *base, int i) {
-  TF d[4] = { TF(0), TF(0), TF(0), TF(0) };
-  if (!first) vload<TF, 4, CG>(delta + static_cast<size_t>(i) * del_run<TF>(), d);
-  double u[4];
+  double u[4];   // (all loads before the first store, which they might alias)
+  if (first) {
 #pragma unroll
-  for (int v = 0; v < 4; ++v) {
-    u[v] = first ? Wp0[v * n + i] : ld<CG>(&U[v * n + i]) + static_cast<double>(d[v]);
-    U[v * n + i] = u[v];
+    for (int v = 0; v < 4; ++v) u[v] = Wp0[v * n + i];
+  } else {
+    TF d[4];
+    vload<TF, 4, CG>(delta + static_cast<size_t>(i) * del_run<TF>(), d);
+#pragma unroll
+    for (int v = 0; v < 4; ++v) u[v] = ld<CG>(&U[v * n + i]) + static_cast<double>(d[v]);
   }
+#pragma unroll
+  for (int v = 0; v < 4; ++v) U[v * n + i] = u[v];
   TF r[kBase];
   base_record(P, u, r);
   vstore<TF, kBase>(base + static_cast<size_t>(i) * kBase, r);
@@ -1312,13 +1316,14 @@ __device__ __forceinline__ void lo_rhs_at(const MeshT<double> &m, const ParamsT<
   }
   // dt_i = CFL_lo |Omega| / sum;  D_i = |Omega| / dt_i + sum / 2 (padding cells: 0)
   const double id = sum > 0.0 ? D::d_rcp(sum * (P.icfl_lo + 0.5)) : 0.0;
+  double src[4];
+#pragma unroll
+  for (int v = 0; v < 4; ++v) src[v] = first ? Rp0[v * n + i] - R[v] : ld<CG>(&Src[v * n + i]);
   invD[i] = narrow<TF>(id);
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
-    double src;
-    if (first) { src = Rp0[v * n + i] - R[v]; Src[v * n + i] = src; }
-    else src = ld<CG>(&Src[v * n + i]);
-    R[v] += src;
+    if (first) Src[v * n + i] = src[v];
+    R[v] += src[v];
     Rk[v * n + i] = narrow<TF>(R[v]);
   }
   if (g.c0) {

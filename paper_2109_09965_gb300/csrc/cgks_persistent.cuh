@@ -10,8 +10,8 @@
 // functions of the per-phase kernels of cgks_kernels.cuh.
 //
 // Measured on GB300 (57k-cell cylinder V-cycle): slower than the per-phase
-// kernels replayed from a CUDA graph (FP64 1.34 vs 0.91 ms, mixed 0.48 vs
-// 0.28 ms): the resident grid holds fewer warps per SM than the separate
+// kernels replayed from a CUDA graph (FP64 1.31 vs 0.92 ms, mixed 0.47 vs
+// 0.26 ms): the resident grid holds fewer warps per SM than the separate
 // launches and the graph already hides their launch gaps, so the library
 // uses it only when asked (cgks_params.low_order_fused).
 //
